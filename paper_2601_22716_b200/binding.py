@@ -1,4 +1,4 @@
-"""Thin ctypes binding over liblords.so: argument marshalling only.
+"""Thin binding over liblords.so: argument marshalling only (native for the calls that take tensors, ctypes for the rest).
 
 Every function has the name of the C entry point it calls (include/lords.h).  Tensors
 are torch CUDA tensors used purely as device-memory handles; their ``data_ptr()`` and the
@@ -14,6 +14,7 @@ import numpy as np
 
 _PKG = Path(__file__).resolve().parent
 _LIBPATH = _PKG / "liblords.so"
+_NATIVEPATH = _PKG / "_native.so"
 _lib = None
 
 
@@ -43,21 +44,6 @@ def _load():
         "lords_unpack_codes": (ci, [p, i64, i64, ci, p]),
         "lords_init": (ci, [ci, sz]),
         "lords_shutdown": (ci, []),
-        "lords_linear_forward": (ci, [p, p, p, p, p, ci, ci, ci, ci, p, p]),
-        "lords_linear_forward_bits": (ci, [p, p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_linear_forward_f32": (ci, [p, p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_linear_forward_host": (ci, [p, p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_linear_forward_noalloc": (ci, [p, p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_quantize_codes": (ci, [p, p, p, p, ci, ci, ci, ci, p, p]),
-        "lords_transpose_codes": (ci, [p, ci, ci, ci, p, p]),
-        "lords_linear_backward_input": (ci, [p, p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_linear_backward_input_f32": (ci, [p, p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_linear_backward_factors": (ci, [p, p, p, p, p, p, ci, ci, ci, ci, ci, p, p, p]),
-        "lords_linear_backward_qat": (ci, [p, p, p, p, p, p, p, ci, ci, ci, ci, ci, p, p, p, p]),
-        "lords_blockscale_forward": (ci, [p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_blockscale_forward_f32": (ci, [p, p, p, p, ci, ci, ci, ci, ci, p, p]),
-        "lords_adapter_forward": (ci, [p, p, p, p, p, p, ci, ci, ci, ci, ci, ci, p, p]),
-        "lords_adapter_forward_f32": (ci, [p, p, p, p, p, p, ci, ci, ci, ci, ci, ci, p, p]),
         "lords_poll_status": (ci, [p]),
         "lords_read_status_detail": (ci, [p]),
         "lords_last_cuda_error": (ci, []),
@@ -156,107 +142,37 @@ def _cb_ptr(codebook, bits):
     return cb
 
 
-def lords_linear_forward(x, Qpacked, B, A, codebook, M, m, n, r, y, stream=None) -> None:
-    """4-bit entry point: device tensors x[M,n], Qpacked[m,n/2], B[m,r], A[r,n] -> y[M,m] (bf16)."""
-    cb = _cb_ptr(codebook, 4)
-    _check(_load().lords_linear_forward(x.data_ptr(), Qpacked.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                        cb.ctypes.data, M, m, n, r, y.data_ptr(), _stream_ptr(stream)),
-           "lords_linear_forward")
+# The calls that take tensors are native functions (csrc/lords_module.cc): a small layer runs in a few
+# microseconds, which is less than marshalling a dozen arguments in Python takes.
+_TENSOR_CALLS = ("lords_linear_forward", "lords_linear_forward_bits", "lords_linear_forward_f32", "lords_linear_forward_host",
+                 "lords_linear_forward_noalloc", "lords_quantize_codes", "lords_transpose_codes", "lords_linear_backward_input",
+                 "lords_linear_backward_input_f32", "lords_linear_backward_factors", "lords_linear_backward_qat",
+                 "lords_blockscale_forward", "lords_adapter_forward")
 
 
-def lords_linear_forward_bits(x, Qpacked, B, A, codebook, bits, M, m, n, r, y, stream=None) -> None:
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_linear_forward_bits(x.data_ptr(), Qpacked.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                             cb.ctypes.data, bits, M, m, n, r, y.data_ptr(),
-                                             _stream_ptr(stream)), "lords_linear_forward_bits")
+def _native():
+    """The native module with the tensor calls; its functions replace this module's placeholders."""
+    _load()      # reports a missing library first
+    if not _NATIVEPATH.exists():
+        raise ImportError(f"{_NATIVEPATH} is missing: build it with `python -m paper_2601_22716_b200.build`.")
+    from . import _native as mod
+    mod.setup(LordsError, _cb_ptr)
+    for name in _TENSOR_CALLS:
+        globals()[name] = getattr(mod, name)
+    return mod
 
 
-def lords_linear_forward_f32(x, Qpacked, B, A, codebook, bits, M, m, n, r, y32, stream=None) -> None:
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_linear_forward_f32(x.data_ptr(), Qpacked.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                            cb.ctypes.data, bits, M, m, n, r, y32.data_ptr(),
-                                            _stream_ptr(stream)), "lords_linear_forward_f32")
+def _placeholder(name):
+    def call(*args, **kwargs):
+        return getattr(_native(), name)(*args, **kwargs)
+    call.__name__ = call.__qualname__ = name
+    return call
 
 
-def lords_linear_forward_host(x_host, Qpacked, B, A, codebook, bits, M, m, n, r, y_host, stream=None) -> None:
-    """x_host / y_host are CPU tensors (pinned for asynchronous copies); weights are device tensors."""
-    cb = _cb_ptr(codebook, bits)
-    if x_host.is_cuda or y_host.is_cuda:
-        raise ValueError("x_host and y_host must be host tensors")
-    _check(_load().lords_linear_forward_host(x_host.data_ptr(), Qpacked.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                             cb.ctypes.data, bits, M, m, n, r, y_host.data_ptr(),
-                                             _stream_ptr(stream)), "lords_linear_forward_host")
-
-
-def lords_linear_forward_noalloc(x, Qpacked, B, A, codebook, bits, M, m, n, r, y, stream=None) -> None:
-    """Forward that never allocates and needs no lords_init (scratch lives in the library image)."""
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_linear_forward_noalloc(x.data_ptr(), Qpacked.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                                cb.ctypes.data, bits, M, m, n, r, y.data_ptr(),
-                                                _stream_ptr(stream)), "lords_linear_forward_noalloc")
-
-
-def lords_quantize_codes(W, B, A, codebook, bits, m, n, r, Qpacked, stream=None) -> None:
-    """Alg. 1 step 2.1 on the device: packed codes of the nearest levels of W / (B A)."""
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_quantize_codes(W.data_ptr(), B.data_ptr(), A.data_ptr(), cb.ctypes.data, bits, m, n, r,
-                                        Qpacked.data_ptr(), _stream_ptr(stream)), "lords_quantize_codes")
-
-
-def lords_transpose_codes(Qpacked, bits, m, n, Qt_packed, stream=None) -> None:
-    """Packed codes of Q^T (n rows of m codes) from the packed codes of Q, on the device."""
-    _check(_load().lords_transpose_codes(Qpacked.data_ptr(), bits, m, n, Qt_packed.data_ptr(), _stream_ptr(stream)),
-           "lords_transpose_codes")
-
-
-def lords_linear_backward_input(dy, Qt_packed, B, A, codebook, bits, M, m, n, r, dx, stream=None) -> None:
-    """dx = dy W^ (bf16 [M, n]) for a layer whose transposed codes Qt_packed were made by lords_transpose_codes."""
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_linear_backward_input(dy.data_ptr(), Qt_packed.data_ptr(), B.data_ptr(), A.data_ptr(), cb.ctypes.data,
-                                               bits, M, m, n, r, dx.data_ptr(), _stream_ptr(stream)),
-           "lords_linear_backward_input")
-
-
-def lords_linear_backward_input_f32(dy, Qt_packed, B, A, codebook, bits, M, m, n, r, dx32, stream=None) -> None:
-    """The same with the fp32 accumulator stored (float [M, n])."""
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_linear_backward_input_f32(dy.data_ptr(), Qt_packed.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                                   cb.ctypes.data, bits, M, m, n, r, dx32.data_ptr(), _stream_ptr(stream)),
-           "lords_linear_backward_input_f32")
-
-
-def lords_linear_backward_factors(dy, x, Qpacked, B, A, codebook, bits, M, m, n, r, dB, dA, stream=None) -> None:
-    """dB (float [m, r]) and dA (float [r, n]) of the layer with the codes fixed; either may be None."""
-    cb = _cb_ptr(codebook, bits)
-    _check(_load().lords_linear_backward_factors(dy.data_ptr(), x.data_ptr(), Qpacked.data_ptr(), B.data_ptr(), A.data_ptr(),
-                                                 cb.ctypes.data, bits, M, m, n, r,
-                                                 None if dB is None else dB.data_ptr(), None if dA is None else dA.data_ptr(),
-                                                 _stream_ptr(stream)), "lords_linear_backward_factors")
-
-
-def lords_linear_backward_qat(dy, x, W, Qpacked, B, A, codebook, bits, M, m, n, r, dW, dB, dA, stream=None) -> None:
-    """Straight-through gradients of quantisation-aware training (Eq. 4-5); any of dW, dB, dA may be None."""
-    cb = _cb_ptr(codebook, bits)
-    ptr = lambda t: None if t is None else t.data_ptr()
-    _check(_load().lords_linear_backward_qat(dy.data_ptr(), x.data_ptr(), W.data_ptr(), Qpacked.data_ptr(), B.data_ptr(),
-                                             A.data_ptr(), cb.ctypes.data, bits, M, m, n, r, ptr(dW), ptr(dB), ptr(dA),
-                                             _stream_ptr(stream)), "lords_linear_backward_qat")
-
-
-def lords_blockscale_forward(x, Qpacked, scales, codebook, bits, blk, M, m, n, y, stream=None, f32=False) -> None:
-    """Comparator (Eq. 2): y = x (L[Q] (.) (s (x) 1))^T; y is bf16 [M, m], or float with f32=True."""
-    cb = _cb_ptr(codebook, bits)
-    fn = _load().lords_blockscale_forward_f32 if f32 else _load().lords_blockscale_forward
-    _check(fn(x.data_ptr(), Qpacked.data_ptr(), scales.data_ptr(), cb.ctypes.data, bits, blk, M, m, n, y.data_ptr(),
-              _stream_ptr(stream)), "lords_blockscale_forward")
-
-
-def lords_adapter_forward(x, Qpacked, scales, A_l, B_l, codebook, bits, blk, M, m, n, r, y, stream=None, f32=False) -> None:
-    """Comparator (Sec. 3.4 / 4.4): the block-scaled layer plus an additive rank-r adapter, three launches."""
-    cb = _cb_ptr(codebook, bits)
-    fn = _load().lords_adapter_forward_f32 if f32 else _load().lords_adapter_forward
-    _check(fn(x.data_ptr(), Qpacked.data_ptr(), scales.data_ptr(), A_l.data_ptr(), B_l.data_ptr(), cb.ctypes.data, bits, blk,
-              M, m, n, r, y.data_ptr(), _stream_ptr(stream)), "lords_adapter_forward")
+for _name in _TENSOR_CALLS:
+    globals()[_name] = _placeholder(_name)      # a library that is built after the import is loaded by the first call
+if _LIBPATH.exists() and _NATIVEPATH.exists():
+    _native()
 
 
 def lords_poll_status(stream=None) -> int:
