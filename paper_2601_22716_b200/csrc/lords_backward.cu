@@ -477,19 +477,20 @@ __global__ void __launch_bounds__(kTcThreads, 2) lords_backward_tc_kernel(const 
         const uint32_t a_lo0 = (uint32_t)umma_desc_sw128(0, 1024, (uint32_t)kTcGAtom) | ((base & 0x3FFFFu) >> 4);
         const uint32_t b_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         const uint32_t b_lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | (((base + 2 * kTcGAtom) & 0x3FFFFu) >> 4);
+        const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
         if (scale_mma) {
             // S[128 x 64] = B_tile (K-major: a row is one row of B, 16 ranks = 32 bytes) * A_tile (MN-major: a row is one
             // rank, 16 ranks = 16 rows of 128 bytes), one MMA per 16 ranks, into the columns behind the accumulator
             constexpr uint32_t idesc_s = umma_idesc_f16(1, 0, 1, kTcRows, kTcCols);
             if (!mbar_wait(bar_s_full, 0, status, 44)) failed = true;
             tc_fence_after_sync();
-            if (lane == 0 && !failed) {
+            if (!__any_sync(0xffffffffu, failed)) {
                 const uint32_t sb_lo = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((s_btile & 0x3FFFFu) >> 4);
                 const uint32_t sa_lo = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((s_atile & 0x3FFFFu) >> 4);
                 for (int k = 0; k < r16 / 16; ++k)
-                    umma_f16_ss(tmem_base + kTcTmemCols, umma_desc_pack(sb_lo + k * 2, b_hi), umma_desc_pack(sa_lo + k * 128, b_hi),
-                                idesc_s, k > 0 ? 1u : 0u);
-                umma_commit(bar_s_done);
+                    umma_f16_ss(tmem_u + kTcTmemCols, umma_desc_pack(sb_lo + k * 2, b_hi), umma_desc_pack(sa_lo + k * 128, b_hi),
+                                idesc_s, k > 0 ? 1u : 0u, leader);
+                umma_commit(bar_s_done, leader);
             }
             __syncwarp();
         }
@@ -497,15 +498,13 @@ __global__ void __launch_bounds__(kTcThreads, 2) lords_backward_tc_kernel(const 
             const int s = c % kTcStages;
             if (!mbar_wait(bar_full + 8 * s, (uint32_t)((c / kTcStages) & 1), status, 42)) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t off = (uint32_t)((s * kTcStage) >> 4);
+            const uint32_t off = (uint32_t)((s * kTcStage) >> 4);
 #pragma unroll
-                for (int k = 0; k < kTcTok / 16; ++k)      // 16 tokens = 16 rows of 128 bytes
-                    umma_f16_ss(tmem_base, umma_desc_pack(a_lo0 + off + k * 128, a_hi), umma_desc_pack(b_lo0 + off + k * 128, b_hi),
-                                idesc, (c > 0 || k > 0) ? 1u : 0u);
-                umma_commit(bar_empty + 8 * s);
-                if (c == chunks - 1) umma_commit(bar_acc);
-            }
+            for (int k = 0; k < kTcTok / 16; ++k)      // 16 tokens = 16 rows of 128 bytes
+                umma_f16_ss(tmem_u, umma_desc_pack(a_lo0 + off + k * 128, a_hi), umma_desc_pack(b_lo0 + off + k * 128, b_hi),
+                            idesc, (c > 0 || k > 0) ? 1u : 0u, leader);
+            umma_commit(bar_empty + 8 * s, leader);
+            if (c == chunks - 1) umma_commit(bar_acc, leader);
             __syncwarp();
         }
     } else {

@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
                     // a stage is freed by work that stands behind the dependency point: pass it first, so that
                     // the bounded wait does not run while the previous launch (however long) still works
                     if (it == SQ) griddep_wait();
-                    if (!mbar_wait(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1), status, 1)) { failed = true; break; }
+                    if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1), status, 1)) { failed = true; break; }
                 }
                 const uint32_t bar = bar_q_full + 8 * sq;
                 mbar_expect_tx(bar, (uint32_t)C::QSTAGE);
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
             griddep_wait();   // x may be the previous launch's output
             for (int it = 0; it < pre; ++it) load_x(it);
             for (int it = S; it < total; ++it) {
-                if (!mbar_wait(bar_mma_done + 8 * ((it - S) % kAF), (uint32_t)(((it - S) / kAF) & 1), status, 2)) { failed = true; break; }
+                if (!mbar_wait<kWaitSlackNs>(bar_mma_done + 8 * ((it - S) % kAF), (uint32_t)(((it - S) / kAF) & 1), status, 2)) { failed = true; break; }
                 load_a(it);
                 load_x(it);
             }
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
         // H == 2: issuer j owns half j and takes every k-step.  H == 1: the two issuers take the
         // k-steps alternately, each into its own accumulator (the epilogue adds the two), which
         // doubles the rate at which MMAs leave the CTA.
-        const int j = warp - kIssuerWarp0;
+        const int j = (int)warp_uniform((uint32_t)(warp - kIssuerWarp0));
         const int h = H == 2 ? j : 0;
         constexpr int kStride = H == 2 ? 1 : 2;
         static_assert(H == 2 || S % 2 == 0, "with alternating issuers every ring barrier belongs to one of them");
@@ -375,23 +375,23 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
         const uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);  // fp16 x fp16 -> fp32, K-major
         const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         const uint32_t desc_lo = (uint32_t)umma_desc_sw128(0, 1024, 16);
-        const uint32_t acc = tmem_base + (uint32_t)(j * kNMax);
         const int first = H == 2 ? 0 : j;
+        tmem_base = warp_uniform(tmem_base);
+        const uint32_t acc = tmem_base + (uint32_t)(j * kNMax);
+        const uint32_t leader = elect_one();
         for (int it = first; it < total; it += kStride) {
             const int s = it % S;
-            if (!mbar_wait(bar_ax_ready + 8 * s, (uint32_t)((it / S) & 1), status, 3) ||
-                !mbar_wait(bar_ready + 8 * (h * S + s), (uint32_t)((it / S) & 1), status, 4)) { failed = true; break; }
+            if (!mbar_wait<kWaitSpin>(bar_ax_ready + 8 * s, (uint32_t)((it / S) & 1), status, 3) ||
+                !mbar_wait<kWaitSpin>(bar_ready + 8 * (h * S + s), (uint32_t)((it / S) & 1), status, 4)) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t wslot = tmem_base + kWCol + (uint32_t)((h * S + s) * kWSlotCols);
-                const uint32_t b_lo = desc_lo | ((ax_stage(s) & 0x3FFFFu) >> 4);
+            const uint32_t wslot = tmem_base + kWCol + (uint32_t)((h * S + s) * kWSlotCols);
+            const uint32_t b_lo = desc_lo | ((ax_stage(s) & 0x3FFFFu) >> 4);
 #pragma unroll
-                for (int k = 0; k < kStep / 16; ++k)
-                    umma_f16_ts(acc, wslot + k * 8, umma_desc_pack(b_lo + (k >> 2) * (kAtomBytes >> 4) + (k & 3) * 2, desc_hi),
-                                idesc, (it == first && k == 0) ? 0u : 1u);
-                umma_commit(bar_mma_done + 8 * (it % kAF));
-                if (it + kStride >= total) umma_commit(bar_acc_full + 8 * j);
-            }
+            for (int k = 0; k < kStep / 16; ++k)
+                umma_f16_ts(acc, wslot + k * 8, umma_desc_pack(b_lo + (k >> 2) * (kAtomBytes >> 4) + (k & 3) * 2, desc_hi),
+                            idesc, (it == first && k == 0) ? 0u : 1u, leader);
+            umma_commit(bar_mma_done + 8 * (it % kAF), leader);
+            if (it + kStride >= total) umma_commit(bar_acc_full + 8 * j, leader);
             __syncwarp();
         }
     } else if (warp >= kConvWarp0) {
@@ -654,11 +654,12 @@ template <int BITS, int NTOK, int H> struct DecodeVariant {
         }
         return cache[dev][cs] > 0 ? cache[dev][cs] : 0;
     }
-    static int launch(const DecodeParams &k, int tiles, int cs, cudaStream_t stream)
+    static int launch(const DecodeParams &k, int tiles, int cs, bool ordered, cudaStream_t stream)
     {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
         fill(cfg, attr, cs, tiles, stream);
+        if (ordered) attr[1].val.programmaticStreamSerializationAllowed = 0;
         LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_decode_kernel<BITS, NTOK, H>, k));
         return LORDS_OK;
     }
@@ -711,8 +712,8 @@ template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem
                      CU_TENSOR_MAP_SWIZZLE_NONE))
         return LORDS_ERR_CUDA;
     k.tiles = two ? tiles2 : tiles1;
-    return two ? DecodeVariant<BITS, NTOK, 2>::launch(k, tiles2, cs2, stream)
-               : DecodeVariant<BITS, NTOK, 1>::launch(k, tiles1, cs1, stream);
+    return two ? DecodeVariant<BITS, NTOK, 2>::launch(k, tiles2, cs2, p.ordered, stream)
+               : DecodeVariant<BITS, NTOK, 1>::launch(k, tiles1, cs1, p.ordered, stream);
 }
 
 }  // namespace
@@ -721,12 +722,8 @@ template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem
 // (3-bit), which makes every TMA row pitch a multiple of 16 bytes.  Anything else: LORDS_ERR_UNSUPPORTED.
 int launch_decode(const Problem &p, State &st, cudaStream_t stream)
 {
-    if (p.bits < 2 || p.bits > 4) return LORDS_ERR_UNSUPPORTED;
-    if (p.M > 2) return LORDS_ERR_UNSUPPORTED;
+    if (!decode_takes(p)) return LORDS_ERR_UNSUPPORTED;
     const int r_pad = (p.r + 15) / 16 * 16;
-    if (p.M * r_pad > kNMax) return LORDS_ERR_UNSUPPORTED;
-    if (p.n % (p.bits == 4 ? 32 : p.bits == 2 ? 64 : 128) != 0) return LORDS_ERR_UNSUPPORTED;
-
     DecodeParams k;
     k.x = p.x; k.B = p.B;
     for (int c = 0; c < 16; ++c) k.levels[c] = p.levels[c];

@@ -133,52 +133,36 @@ struct alignas(64) Dec16Params {
     int blk, nblk;
 };
 
-// 64 columns of one row: code pairs -> level pairs, times the matching pairs of S (sp, in and out).
+// The packed codes of one row's 64-column half, and the table address of its code pair P (columns 2P, 2P + 1).
 // 4-bit rows are 64 bytes and arrive 64-byte-swizzled (16-byte chunk c of row i sits at chunk
-// c ^ ((i >> 1) & 3)); 3-bit rows are 48 bytes, pair P at bit 6P of the row's bit stream.
-template <int BITS>
-__device__ __forceinline__ void dequant_half_row(uint32_t qrow, int row, int ch, uint32_t lut_lane, uint32_t (&sp)[32])
-{
-    if constexpr (BITS == 4) {
-        const uint32_t sw = (uint32_t)((row >> 1) & 3);
-        const uint4 c0 = lds_v4(qrow + (((2 * ch) ^ sw) << 4)), c1 = lds_v4(qrow + (((2 * ch + 1) ^ sw) << 4));
-        const uint32_t w[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
+// c ^ ((i >> 1) & 3)); 3-bit rows are 48 bytes, 2-bit rows 32 bytes as they are.
+template <int BITS> struct HalfRow {
+    uint32_t w[2 * BITS];
+    __device__ __forceinline__ void read(uint32_t qrow, int row, int ch)
+    {
+        if constexpr (BITS == 4) {
+            const uint32_t sw = (uint32_t)((row >> 1) & 3);
+            const uint4 c0 = lds_v4(qrow + (((2 * ch) ^ sw) << 4)), c1 = lds_v4(qrow + (((2 * ch + 1) ^ sw) << 4));
+            w[0] = c0.x; w[1] = c0.y; w[2] = c0.z; w[3] = c0.w; w[4] = c1.x; w[5] = c1.y; w[6] = c1.z; w[7] = c1.w;
+        } else if constexpr (BITS == 2) {
+            const uint4 c0 = lds_v4(qrow + 16 * ch);
+            w[0] = c0.x; w[1] = c0.y; w[2] = c0.z; w[3] = c0.w;
+        } else {
 #pragma unroll
-        for (int wi = 0; wi < 8; ++wi)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const uint32_t lv = lds_u32(__byte_perm(w[wi], lut_lane, 0x7604u | (uint32_t)(b << 4)));
-                const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), *reinterpret_cast<const __half2 *>(&sp[wi * 4 + b]));
-                sp[wi * 4 + b] = *reinterpret_cast<const uint32_t *>(&wv);
-            }
-    } else if constexpr (BITS == 2) {
-        // 32-byte rows: half ch is the 16 bytes at 16 ch, pair P at bit 4P of them
-        const uint4 c0 = lds_v4(qrow + 16 * ch);
-        const uint32_t w[4] = {c0.x, c0.y, c0.z, c0.w};
-#pragma unroll
-        for (int pp = 0; pp < 32; ++pp) {
-            const int off = 4 * (pp & 7);
-            const uint32_t sh = off >= 7 ? (w[pp >> 3] >> (off - 7)) : (w[pp >> 3] << (7 - off));
-            const uint32_t lv = lds_u32((sh & 0x780u) | lut_lane);
-            const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), *reinterpret_cast<const __half2 *>(&sp[pp]));
-            sp[pp] = *reinterpret_cast<const uint32_t *>(&wv);
-        }
-    } else {
-        // half ch = pairs 32 ch .. 32 ch + 31 = bits 192 ch .. of the 384-bit row = words 6 ch .. 6 ch + 5
-        const uint32_t base = qrow + 24 * ch;
-        const uint32_t w[6] = {lds_u32(base), lds_u32(base + 4), lds_u32(base + 8), lds_u32(base + 12), lds_u32(base + 16), lds_u32(base + 20)};
-#pragma unroll
-        for (int pp = 0; pp < 32; ++pp) {
-            const int bit = 6 * pp, wi = bit >> 5, off = bit & 31;
-            uint32_t sh;
-            if (off > 26) sh = __funnelshift_r(w[wi], w[wi + 1 < 6 ? wi + 1 : 5], off - 7);
-            else sh = off >= 7 ? (w[wi] >> (off - 7)) : (w[wi] << (7 - off));
-            const uint32_t lv = lds_u32((sh & 0x1F80u) | lut_lane);
-            const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), *reinterpret_cast<const __half2 *>(&sp[pp]));
-            sp[pp] = *reinterpret_cast<const uint32_t *>(&wv);
+            for (int k = 0; k < 6; ++k) w[k] = lds_u32(qrow + 24 * ch + 4 * k);
         }
     }
-}
+    __device__ __forceinline__ uint32_t address(int P, uint32_t lut_lane) const
+    {
+        if constexpr (BITS == 4) return __byte_perm(w[P >> 2], lut_lane, 0x7604u | (uint32_t)((P & 3) << 4));
+        const int bit = 2 * BITS * P, wi = bit >> 5, off = bit & 31;
+        constexpr uint32_t mask = BITS == 3 ? 0x1F80u : 0x780u;
+        uint32_t sh;
+        if (off + 2 * BITS > 32) sh = __funnelshift_r(w[wi], w[wi + 1 < 2 * BITS ? wi + 1 : wi], off - 7);
+        else sh = off >= 7 ? (w[wi] >> (off - 7)) : (w[wi] << (7 - off));
+        return (sh & mask) | lut_lane;
+    }
+};
 
 // BLOCK: the scale of an element is its row's block scale (Eq. 2: S = s (x) 1) instead of (BA)_ij: no
 // scale MMA, no factor tiles; a worker thread's 64 columns lie in one block (blk is a multiple of 64),
@@ -270,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
                     // a stage is freed by work that stands behind the dependency point: pass it first, so that
                     // the bounded wait does not run while the previous launch (however long) still works
                     if (it == SQ) griddep_wait();
-                    if (!mbar_wait(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1))) { failed = true; break; }
+                    if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1))) { failed = true; break; }
                 }
                 const uint32_t bar = bar_q_full + 8 * sq;
                 mbar_expect_tx(bar, (uint32_t)C::QSTAGE);
@@ -345,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             const uint32_t tx = (uint32_t)(2 * p.r_pad * 128);
             for (int it = 0; it < total; ++it) {
                 const int sa = it % C::SA;
-                if (it >= C::SA && !mbar_wait(bar_a_done + 8 * sa, (uint32_t)((it / C::SA - 1) & 1))) { failed = true; break; }
+                if (it >= C::SA && !mbar_wait<kWaitSlackNs>(bar_a_done + 8 * sa, (uint32_t)((it / C::SA - 1) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_a_full + 8 * sa;
                 mbar_expect_tx(bar, tx);
 #pragma unroll
@@ -361,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             griddep_wait();
             for (int it = 0; it < total; ++it) {
                 const int sx = it % WS;
-                if (it >= WS && !mbar_wait(bar_mma_done + 8 * ((it - WS) % WB), (uint32_t)(((it - WS) / WB) & 1))) { failed = true; break; }
+                if (it >= WS && !mbar_wait<kWaitSlackNs>(bar_mma_done + 8 * ((it - WS) % WB), (uint32_t)(((it - WS) / WB) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_x_full + 8 * sx;
                 mbar_expect_tx(bar, (uint32_t)kXStage);
 #pragma unroll
@@ -381,50 +365,50 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         const uint32_t b_lo = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((b_tile & 0x3FFFFu) >> 4);
         const uint32_t a_lo0 = (uint32_t)umma_desc_sw128(0, 1024, (uint32_t)C::AATOM) | ((a0 & 0x3FFFFu) >> 4);
         const int rsteps = p.r_pad / 16;
-        const int sj = warp - kScaleWarp0;
+        const int sj = (int)warp_uniform((uint32_t)(warp - kScaleWarp0));
+        tmem_base = warp_uniform(tmem_base);
+        const uint32_t leader = elect_one();
         static_assert(SD == 2 && C::SA % 2 == 0, "one scale issuer per S buffer; each factor-ring barrier belongs to one of them");
         if (b_by_tma && sj < total && !mbar_wait(bar_b_full, 0)) failed = true;
         for (int it = sj; !BLOCK && it < total && !failed; it += 2) {
             const int sa = it % C::SA, sd = it % SD;
-            if (!mbar_wait(bar_a_full + 8 * sa, (uint32_t)((it / C::SA) & 1))) { failed = true; break; }
-            if (it >= SD && !mbar_wait(bar_s_empty + 8 * sd, (uint32_t)((it / SD - 1) & 1))) { failed = true; break; }
+            if (!mbar_wait<kWaitSpin>(bar_a_full + 8 * sa, (uint32_t)((it / C::SA) & 1))) { failed = true; break; }
+            if (it >= SD && !mbar_wait<kWaitSpin>(bar_s_empty + 8 * sd, (uint32_t)((it / SD - 1) & 1))) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ASTAGE >> 4));
-                for (int k = 0; k < rsteps; ++k)
-                    umma_f16_ss(tmem_base + kSCol + (uint32_t)(sd * kStep), umma_desc_pack(b_lo + k * 2, desc_hi),
-                                umma_desc_pack(a_lo + k * 128, desc_hi), idesc_s, k > 0);
-                umma_commit(bar_s_full + 8 * sd);
-                umma_commit(bar_a_done + 8 * sa);
-            }
+            const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ASTAGE >> 4));
+            for (int k = 0; k < rsteps; ++k)
+                umma_f16_ss(tmem_base + kSCol + (uint32_t)(sd * kStep), umma_desc_pack(b_lo + k * 2, desc_hi),
+                            umma_desc_pack(a_lo + k * 128, desc_hi), idesc_s, k > 0, leader);
+            umma_commit(bar_s_full + 8 * sd, leader);
+            umma_commit(bar_a_done + 8 * sa, leader);
             __syncwarp();
         }
     } else if (warp >= kIssuerWarp0) {
         // ------------------------------------------------------------------ main-MMA issuers
         // Issuer j takes the k-steps of parity j into an accumulator of its own (the epilogue adds
         // the two), which doubles the rate at which MMAs leave the CTA.
-        const int j = warp - kIssuerWarp0;
+        const int j = (int)warp_uniform((uint32_t)(warp - kIssuerWarp0));
         uint32_t tmem_base;
         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
         constexpr uint32_t idesc_m = umma_idesc_f16(0, 0, 0, kRows, kTok);   // fp16, K-major
         const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         const uint32_t x_lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((x0 & 0x3FFFFu) >> 4);
+        tmem_base = warp_uniform(tmem_base);
+        const uint32_t leader = elect_one();
         const uint32_t acc = tmem_base + (uint32_t)(j * 32);
         for (int it = j; it < total; it += 2) {
             const int ws = it % WS;
-            if (!mbar_wait(bar_x_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1)) ||
-                !mbar_wait(bar_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1))) { failed = true; break; }
+            if (!mbar_wait<kWaitSpin>(bar_x_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1)) ||
+                !mbar_wait<kWaitSpin>(bar_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1))) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t wslot = tmem_base + kWCol + (uint32_t)(ws * 64);
-                const uint32_t x_lo = x_lo0 + (uint32_t)(ws * (kXStage >> 4));
+            const uint32_t wslot = tmem_base + kWCol + (uint32_t)(ws * 64);
+            const uint32_t x_lo = x_lo0 + (uint32_t)(ws * (kXStage >> 4));
 #pragma unroll
-                for (int k = 0; k < kStep / 16; ++k)
-                    umma_f16_ts(acc, wslot + k * 8, umma_desc_pack(x_lo + (k >> 2) * (kXAtom >> 4) + (k & 3) * 2, desc_hi),
-                                idesc_m, (it == j && k == 0) ? 0u : 1u);
-                umma_commit(bar_mma_done + 8 * (it % WB));
-                if (it + 2 >= total) umma_commit(bar_acc_full + 8 * j);
-            }
+            for (int k = 0; k < kStep / 16; ++k)
+                umma_f16_ts(acc, wslot + k * 8, umma_desc_pack(x_lo + (k >> 2) * (kXAtom >> 4) + (k & 3) * 2, desc_hi),
+                            idesc_m, (it == j && k == 0) ? 0u : 1u, leader);
+            umma_commit(bar_mma_done + 8 * (it % WB), leader);
+            if (it + 2 >= total) umma_commit(bar_acc_full + 8 * j, leader);
             __syncwarp();
         }
     } else if (warp >= kConvWarp0) {
@@ -464,37 +448,49 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
 
         for (int it = g; it < total; it += 2) {
             const int sq = it % SQ, sd = it % SD, ws = it % WS;
-            // this thread's 64 columns of S, as 32 fp16 pairs
+            // S and the codes have landed, and the W slot is free: the MMAs of step it - WS have completed
+            const uint32_t bar_first = BLOCK ? bar_q_full + 8 * sq : bar_s_full + 8 * sd, par_q = (uint32_t)((it / SQ) & 1);
+            if (!mbar_wait_warp3(bar_first, BLOCK ? par_q : (uint32_t)((it / SD) & 1), bar_q_full + 8 * sq, par_q,
+                                 bar_mma_done + 8 * ((it + WB - WS) % WB), (uint32_t)(((it - WS) / WB) & 1), it >= WS)) { failed = true; break; }
+            tc_fence_after_sync();
+            // 16 columns of S at a time, the next 16 on their way from TMEM while these are rounded to fp16 pairs and
+            // multiplied by the looked-up level pairs: the conversions, the look-ups and the TMEM loads of a warp overlap
             uint32_t sp[32];
+            HalfRow<BITS> codes;
             if constexpr (BLOCK) {
+                codes.read(q0 + sq * C::QSTAGE + row * C::QROW, row, ch);
                 const int i = row0 + row, blkidx = ((ks_a + it) * kStep + ch * 64) / p.blk;
                 const float sc = (i < p.m && blkidx < p.nblk) ? __uint_as_float((uint32_t)p.scales[(size_t)i * p.nblk + blkidx] << 16) : 0.0f;
                 const __half2 s2 = __floats2half2_rn(sc, sc);
 #pragma unroll
-                for (int pp = 0; pp < 32; ++pp) sp[pp] = *reinterpret_cast<const uint32_t *>(&s2);
+                for (int pp = 0; pp < 32; ++pp) {
+                    const uint32_t lv = lds_table(codes.address(pp, lut_lane));
+                    const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), s2);
+                    sp[pp] = *reinterpret_cast<const uint32_t *>(&wv);
+                }
             } else {
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_s_full + 8 * sd, (uint32_t)((it / SD) & 1)))) { failed = true; break; }
-            tc_fence_after_sync();
+                const uint32_t s_addr = lane_addr + kSCol + (uint32_t)(sd * kStep + ch * 64);
+                uint32_t s[2][16];
+                tmem_ld_32x16(s_addr, s[0]);
+                codes.read(q0 + sq * C::QSTAGE + row * C::QROW, row, ch);
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                uint32_t s[32];
-                tmem_ld_32x32(lane_addr + kSCol + (uint32_t)(sd * kStep + ch * 64 + hf * 32), s);
-                tmem_wait_ld();
+                for (int k = 0; k < 4; ++k) {
+                    tmem_wait_ld(s[k & 1]);
+                    if (k < 3) tmem_ld_32x16(s_addr + (uint32_t)(16 * (k + 1)), s[(k + 1) & 1]);
+                    else {
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar_s_empty + 8 * sd);      // S is in registers: the buffer may be refilled
+                    }
 #pragma unroll
-                for (int pp = 0; pp < 16; ++pp) {
-                    const __half2 sv = __floats2half2_rn(__uint_as_float(s[2 * pp]), __uint_as_float(s[2 * pp + 1]));
-                    sp[hf * 16 + pp] = *reinterpret_cast<const uint32_t *>(&sv);
+                    for (int e = 0; e < 8; ++e) {
+                        const uint32_t lv = lds_table(codes.address(8 * k + e, lut_lane));
+                        const __half2 sv = __floats2half2_rn(__uint_as_float(s[k & 1][2 * e]), __uint_as_float(s[k & 1][2 * e + 1]));
+                        const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), sv);
+                        sp[8 * k + e] = *reinterpret_cast<const uint32_t *>(&wv);
+                    }
                 }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_s_empty + 8 * sd);      // S is in registers: the buffer may be refilled
-            }
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_q_full + 8 * sq, (uint32_t)((it / SQ) & 1)))) { failed = true; break; }
-            dequant_half_row<BITS>(q0 + sq * C::QSTAGE + row * C::QROW, row, ch, lut_lane, sp);
-            // the W slot is free once the MMAs of step it - WS have completed
-            if (it >= WS && !__all_sync(0xffffffffu, mbar_wait(bar_mma_done + 8 * ((it - WS) % WB), (uint32_t)(((it - WS) / WB) & 1)))) { failed = true; break; }
-            tc_fence_after_sync();
             tmem_st_32x32(lane_addr + kWCol + (uint32_t)(ws * 64 + ch * 32), sp);
             tmem_wait_st();
             tc_fence_before_sync();
@@ -675,6 +671,7 @@ template <int BITS, int RP, bool BLOCK = false> int launch_variant(Dec16Params &
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     V::fill(cfg, attr, cs, tiles, stream);
+    if (p.ordered) attr[1].val.programmaticStreamSerializationAllowed = 0;
     LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_decode16_kernel<BITS, RP, BLOCK>, k));
     return LORDS_OK;
 }
@@ -687,10 +684,7 @@ template <int BITS, int RP, bool BLOCK = false> int launch_variant(Dec16Params &
 // Anything else: LORDS_ERR_UNSUPPORTED.
 int launch_decode16(const Problem &p, State &st, cudaStream_t stream)
 {
-    if (p.bits < 2 || p.bits > 4) return LORDS_ERR_UNSUPPORTED;
-    if (p.M > kTok) return LORDS_ERR_UNSUPPORTED;
-    if (p.r > 64) return LORDS_ERR_UNSUPPORTED;
-    if (p.n % (p.bits == 3 ? 128 : 64) != 0) return LORDS_ERR_UNSUPPORTED;
+    if (!decode16_takes(p)) return LORDS_ERR_UNSUPPORTED;
 
     Dec16Params k;
     k.B = p.B;

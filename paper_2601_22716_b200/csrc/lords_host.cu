@@ -144,7 +144,7 @@ static int validate(const void *x, const uint8_t *q, const void *B, const void *
 }
 
 static int forward_common(const void *x, const uint8_t *q, const void *B, const void *A, const float *cb,
-                          int bits, int M, int m, int n, int r, void *y, int y_f32, void *stream)
+                          int bits, int M, int m, int n, int r, void *y, int y_f32, void *stream, int ordered = 0)
 {
     int rc = validate(x, q, B, A, cb, bits, M, m, n, r, y);
     if (rc != LORDS_OK) return rc;
@@ -157,6 +157,7 @@ static int forward_common(const void *x, const uint8_t *q, const void *B, const 
     for (int c = 0; c < 16; ++c) p.levels[c] = c < (1 << bits) ? cb[c] : 0.0f;
     p.bits = bits; p.M = M; p.m = m; p.n = n; p.r = r;
     p.y = y; p.y_f32 = y_f32;
+    p.ordered = ordered;
     st.last_launches = 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
@@ -444,7 +445,8 @@ static int backward_input_common(const void *dy, const uint8_t *Qt, const void *
     int rc = launch_transpose_bf16_pair(static_cast<const uint16_t *>(A), r, n, At, static_cast<const uint16_t *>(B), m, r, Bt, s);
     if (rc != LORDS_OK) return rc;
     // the transposed layer has n out-features and m in-features; its "B" is A^T and its "A" is B^T
-    rc = forward_common(dy, Qt, At, Bt, cb, bits, M, n, m, r, dx, dx_f32, stream);
+    // (the factors have just been written on the stream)
+    rc = forward_common(dy, Qt, At, Bt, cb, bits, M, n, m, r, dx, dx_f32, stream, 1);
     if (rc != LORDS_OK) return rc;
     st.last_launches += 1;
     return LORDS_OK;

@@ -20,7 +20,16 @@ struct Problem {
     int bits, M, m, n, r;
     void *y;             // bf16 [M][m] or float [M][m]
     int y_f32;           // 1: store the fp32 accumulator
+    int ordered = 0;     // 1: the weights come from the launch just before: the first kernel must not begin ahead of its end
 };
+
+// Which calls the aligned tensor-core kernels take: TMA wants row pitches that are multiples of 16 bytes.
+inline bool decode_takes(const Problem &p)      // reassociated form: M * ceil16(r) accumulator columns, at most 64
+{
+    return p.M <= 2 && p.M * ((p.r + 15) / 16 * 16) <= 64 && p.n % (p.bits == 4 ? 32 : p.bits == 2 ? 64 : 128) == 0;
+}
+inline bool decode16_takes(const Problem &p) { return p.M <= 16 && p.r <= 64 && p.n % (p.bits == 3 ? 128 : 64) == 0; }
+inline bool umma_takes(const Problem &p) { return p.r <= 64 && p.n % (p.bits == 3 ? 128 : 64) == 0; }
 
 // Library-owned device memory and switches (one instance per process).
 struct State {
@@ -37,7 +46,7 @@ struct State {
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
     uint8_t *bw_scratch = nullptr;  // transposed factors for the input gradient
     size_t bw_scratch_bytes = 0;
-    int forced_path = 0;            // 0 auto, 1 simt, 2 decode (reassociated form), 3 umma (scale-MMA form), 4 decode16
+    int forced_path = 0;            // 0 auto, 1 simt, 2 decode (reassociated form), 3 umma (scale-MMA form), 4 decode16, 5 dense, 6 direct, 7 wide
     int forced_splitk = 0;          // 0 auto
     int forced_bn = 0;              // 0 auto; else the token tile of the scale-MMA kernel (32, 64, 128, 256)
     int last_cuda_error = 0;
@@ -62,6 +71,16 @@ int launch_simt(const Problem &p, State &st, cudaStream_t stream);
 // Tensor-core path (TMA + tcgen05/TMEM), scale matrix rebuilt per tile by a small MMA.
 // LORDS_ERR_UNSUPPORTED for shapes outside its rules.
 int launch_umma(const Problem &p, State &st, cudaStream_t stream);
+
+// Up to 16 tokens, ranks 65 .. 128: scale MMA on tcgen05, weights formed in registers.  LORDS_ERR_UNSUPPORTED otherwise.
+int launch_wide(const Problem &p, State &st, cudaStream_t stream);
+
+// Up to 16 tokens, any shape: weights formed in registers and multiplied there (warp-level MMAs).
+int launch_direct(const Problem &p, State &st, cudaStream_t stream);
+
+// Two-phase tensor-core path for any shape: W^ expanded once into scratch, then a dense product.
+// LORDS_ERR_WORKSPACE when the scratch memory does not hold it.
+int launch_dense(const Problem &p, State &st, cudaStream_t stream);
 
 // Tensor-core decode path (M <= 2), reassociated form with the scale factors folded into the
 // activation operand.  LORDS_ERR_UNSUPPORTED for shapes outside its rules.

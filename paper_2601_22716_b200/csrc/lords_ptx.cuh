@@ -92,23 +92,88 @@ __device__ __forceinline__ bool wait_limit_expired(WaitLimit &w, const int *stat
     return false;
 }
 
+// Up to 64 tries, SLEEP nanoseconds apart (0: as fast as the tries return).  Written out because a waiting warp takes issue slots
+// from the warps it waits for: four instructions a try, where the compiler's version of this loop took about fourteen
+// (in a decode kernel with ten waiting warps that was more than half of everything the SM issued).
+template <int SLEEP> __device__ __forceinline__ bool mbar_try_wait_64(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    if constexpr (SLEEP == 0)
+        asm volatile(
+            "{\n"
+            ".reg .pred p, q;\n"
+            ".reg .u32 c;\n"
+            "mov.u32 c, 64;\n"
+            "TRY:\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            "@p bra DONE;\n"
+            "sub.u32 c, c, 1;\n"
+            "setp.ne.u32 q, c, 0;\n"
+            "@q bra TRY;\n"
+            "DONE:\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+    else
+        asm volatile(
+            "{\n"
+            ".reg .pred p, q;\n"
+            ".reg .u32 c;\n"
+            "mov.u32 c, 64;\n"
+            "TRY:\n"
+            "nanosleep.u32 %3;\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            "@p bra DONE;\n"
+            "sub.u32 c, c, 1;\n"
+            "setp.ne.u32 q, c, 0;\n"
+            "@q bra TRY;\n"
+            "DONE:\n"
+            "selp.u32 %0, 1, 0, p;\n"
+            "}\n"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity), "n"(SLEEP)
+            : "memory");
+    return ok != 0;
+}
+
 // Bounded wait: gives up after kWaitLimitNs of polling (or as soon as the status word is set) and
 // reports failure, so that no role of a kernel can spin forever on a shared GPU.  Callers record
-// LORDS_ERR_TIMEOUT and drain.
+// LORDS_ERR_TIMEOUT and drain.  SLEEP: kWaitSleepNs ordinarily; kWaitSpin for the few warps whose latency is on every step's
+// path (MMA issuers); kWaitSlackNs for producers that run several steps ahead.
+constexpr int kWaitSpin = 0, kWaitSlackNs = 200;
+template <int SLEEP = (int)kWaitSleepNs>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const int *status = nullptr, uint32_t tag = 0)
 {
-    if (mbar_try_wait(bar, parity) || mbar_try_wait(bar, parity)) return true;
-    // a waiting warp sleeps between its tries, so that it does not take issue slots from the warps
-    // it is waiting for
+    if (mbar_try_wait(bar, parity)) return true;
     WaitLimit limit = wait_limit_start();
     for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 64; ++i) {
-            __nanosleep(kWaitSleepNs);
-            if (mbar_try_wait(bar, parity)) return true;
-        }
+        if (mbar_try_wait_64<SLEEP>(bar, parity)) return true;
         if (wait_limit_expired(limit, status, bar, parity, tag)) return false;
     }
+}
+
+// One or several barriers for a whole warp: the tries of several overlap, where one wait after the other costs about 110 cycles
+// each in a busy CTA even when every phase is long complete.  `need2` false: the third barrier is not waited for.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar0, uint32_t par0, const int *status = nullptr, uint32_t tag = 0)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar0, par0))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar0, par0, status, tag));
+}
+__device__ __forceinline__ bool mbar_wait_warp2(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, const int *status = nullptr, uint32_t tag = 0)
+{
+    const bool a = mbar_try_wait(bar0, par0), b = mbar_try_wait(bar1, par1);
+    if (__all_sync(0xffffffffu, a && b)) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar0, par0, status, tag) && mbar_wait(bar1, par1, status, tag + 1));
+}
+__device__ __forceinline__ bool mbar_wait_warp3(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2, bool need2,
+                                                const int *status = nullptr, uint32_t tag = 0)
+{
+    const bool a = mbar_try_wait(bar0, par0), b = mbar_try_wait(bar1, par1), c = !need2 || mbar_try_wait(bar2, par2);
+    if (__all_sync(0xffffffffu, a && b && c)) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar0, par0, status, tag) && mbar_wait(bar1, par1, status, tag + 1) &&
+                                       (!need2 || mbar_wait(bar2, par2, status, tag + 2)));
 }
 
 // ---- programmatic dependent launch ----------------------------------------------------------------
@@ -182,6 +247,16 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&v)[16])
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// The same, tied to the registers that the loads fill, so that nothing computed from them can be scheduled ahead of the wait.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
+                 :
+                 : "memory");
+}
+
 // 32 lanes x 32 consecutive 32-bit columns, registers -> TMEM: thread l writes lane (base_lane + l).
 __device__ __forceinline__ void tmem_st_32x32(uint32_t taddr, const uint32_t (&v)[32])
 {
@@ -211,6 +286,14 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
 {
     uint32_t v;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+// An entry of a table that never changes after set-up, at an address made from loaded data.  Not volatile: volatile loads keep their
+// order among themselves and with everything else that is volatile, which lines up every look-up with its use.
+__device__ __forceinline__ uint32_t lds_table(uint32_t addr)
+{
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
     return v;
 }
 __device__ __forceinline__ uint4 lds_v4(uint32_t addr)
@@ -324,34 +407,59 @@ __host__ __device__ constexpr uint32_t umma_idesc_f16(int ab_format, int a_mn, i
            | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.
+// One lane of the (converged) warp, always the same one: 1 for it, 0 for the others.
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n.reg .pred q;\n.reg .b32 r;\nelect.sync r|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}\n" : "=r"(p));
+    return p;
+}
+// A value that is the same in every lane, in a form that the compiler knows to be: operands of the instructions
+// below then live in uniform registers.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
+// The tcgen05 instructions of an issuing warp are executed by the whole converged warp under a predicate that is true for one lane
+// (`leader`, from elect_one) instead of inside a branch that one lane takes: in the branch every operand of every
+// instruction goes through a move from a vector to a uniform register, and one thread issued an MMA per 57
+// cycles whatever its size; under the predicate they leave at the tensor core's rate (128 x 16 x 16: 12 cycles, 128 x 32
+// x 16: 17, measured on an idle SM).  All operands must be the same in every lane.
+//
+// D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void umma_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate)
+                                            uint32_t accumulate, uint32_t leader)
 {
     asm volatile(
         "{\n"
-        ".reg .pred p;\n"
+        ".reg .pred p, q;\n"
         "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
         : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]
 __device__ __forceinline__ void umma_f16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate)
+                                            uint32_t accumulate, uint32_t leader)
 {
     asm volatile(
         "{\n"
-        ".reg .pred p;\n"
+        ".reg .pred p, q;\n"
         "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        "setp.ne.b32 q, %5, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
         : "memory");
 }
 // Arrive once on `bar` when every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint32_t bar)
+__device__ __forceinline__ void umma_commit(uint32_t bar, uint32_t leader)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %1, 0;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
+        "}\n" ::"r"(bar), "r"(leader)
+        : "memory");
 }
 
 }  // namespace ptx

@@ -219,19 +219,19 @@ __global__ void __launch_bounds__(kThreadsQ, 3) lords_quantize_kernel(const __gr
         const uint32_t b_lo = lbo_lo | ((b_tile & 0x3FFFFu) >> 4);
         const uint32_t a_lo0 = lbo_lo | ((a0 & 0x3FFFFu) >> 4);
         const int ksteps = p.r_pad / 16;
+        tmem_base = warp_uniform(tmem_base);
+        const uint32_t leader = elect_one();
         for (int it = 0; it < total; ++it) {
             const int sa = it % kSAQ, sd = it % kSDQ;
             if (!mbar_wait(bar_a_full + 8 * sa, (uint32_t)((it / kSAQ) & 1), status, 32)) { failed = true; break; }
             if (it >= kSDQ && !mbar_wait(bar_s_free + 8 * sd, (uint32_t)((it / kSDQ - 1) & 1), status, 33)) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (kATileBytesQ >> 4));
-                for (int k = 0; k < ksteps; ++k)
-                    umma_f16_ss(tmem_base + (uint32_t)(sd * kColsQ), umma_desc_pack(b_lo + k * 2, desc_hi),
-                                umma_desc_pack(a_lo + k * 128, desc_hi), idesc, k > 0);
-                umma_commit(bar_s_full + 8 * sd);
-                umma_commit(bar_a_free + 8 * sa);
-            }
+            const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (kATileBytesQ >> 4));
+            for (int k = 0; k < ksteps; ++k)
+                umma_f16_ss(tmem_base + (uint32_t)(sd * kColsQ), umma_desc_pack(b_lo + k * 2, desc_hi),
+                            umma_desc_pack(a_lo + k * 128, desc_hi), idesc, k > 0, leader);
+            umma_commit(bar_s_full + 8 * sd, leader);
+            umma_commit(bar_a_free + 8 * sa, leader);
             __syncwarp();
         }
         // no commit is still on its way to a barrier when the CTA ends

@@ -35,7 +35,6 @@ using namespace ptx;
 
 constexpr int BM = 128;                        // W^ rows per CTA = UMMA M
 constexpr int BK = 64;                         // in-feature columns per k-step
-constexpr int kRMaxUmma = 64;                  // largest rank this path takes (one swizzle atom of K)
 constexpr int kWorkWarps = 16;                 // two groups of eight
 constexpr int kGroupWarps = 8;
 constexpr int kIssuerWarp = kWorkWarps;        // 16: main MMAs
@@ -238,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                     if (next_q >= SQ) {
                         const uint32_t par = (uint32_t)((next_q / SQ - 1) & 1);
                         if (blocking) {
-                            if (!mbar_wait(bar_q_empty + 8 * sq, par)) return false;
+                            if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, par)) return false;
                         } else if (!mbar_try_wait(bar_q_empty + 8 * sq, par)) {
                             return true;
                         }
@@ -257,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
             for (int it = 0; it < total; ++it) {
                 const int sx = it % SX;
                 if (next_q <= (it >> 1) && !issue_q(true)) { failed = true; break; }   // the pair this k-step reads
-                if (it >= SX && !mbar_wait(bar_done + 8 * ((it - SX) % DR), (uint32_t)(((it - SX) / DR) & 1))) { failed = true; break; }
+                if (it >= SX && !mbar_wait<kWaitSlackNs>(bar_done + 8 * ((it - SX) % DR), (uint32_t)(((it - SX) / DR) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_x_full + 8 * sx;
                 mbar_expect_tx(bar, (uint32_t)C::XTILE);
                 tma_load_2d(x0 + sx * C::XTILE, &p.tm_x, (2 * pa + it) * BK, tok0, bar);
@@ -328,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                 // commit the workers wait for as well (this lane looks at every phase of those barriers
                 // in turn, and no slot barrier can run a phase ahead of it: the scale MMA of k-step
                 // j - SA + SD needs a factor tile that this lane has not loaded yet)
-                if (j >= SA && !mbar_wait(bar_s_full + 8 * ((j - SA) % SD), (uint32_t)(((j - SA) / SD) & 1))) { failed = true; break; }
+                if (j >= SA && !mbar_wait<kWaitSlackNs>(bar_s_full + 8 * ((j - SA) % SD), (uint32_t)(((j - SA) / SD) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_a_full + 8 * sa;
                 mbar_expect_tx(bar, tx);
                 tma_load_2d(a0 + sa * kATileBytes, &p.tm_a, (2 * pa + j) * BK, 0, bar);
@@ -346,19 +345,19 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
         const uint32_t b_lo = lbo_lo | ((b_tile & 0x3FFFFu) >> 4);
         const uint32_t a_lo0 = lbo_lo | ((a0 & 0x3FFFFu) >> 4);
         const int ksteps = p.r_pad / 16;
+        tmem_base = warp_uniform(tmem_base);
+        const uint32_t leader = elect_one();
         for (int j = 0; j < total; ++j) {
             const int sa = j % SA, sd = j % SD;
-            if (!mbar_wait(bar_a_full + 8 * sa, (uint32_t)((j / SA) & 1))) { failed = true; break; }
+            if (!mbar_wait<kWaitSpin>(bar_a_full + 8 * sa, (uint32_t)((j / SA) & 1))) { failed = true; break; }
             // the slot is free once the main MMAs of k-step j - SD have read their operand out of it
-            if (j >= SD && !mbar_wait(bar_done + 8 * ((j - SD) % DR), (uint32_t)(((j - SD) / DR) & 1))) { failed = true; break; }
+            if (j >= SD && !mbar_wait<kWaitSpin>(bar_done + 8 * ((j - SD) % DR), (uint32_t)(((j - SD) / DR) & 1))) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (kATileBytes >> 4));
-                for (int k = 0; k < ksteps; ++k)
-                    umma_f16_ss(tmem_base + C::SCOL + sd * 64, umma_desc_pack(b_lo + k * 2, desc_hi),
-                                umma_desc_pack(a_lo + k * 128, desc_hi), idesc_s, k > 0);
-                umma_commit(bar_s_full + 8 * sd);
-            }
+            const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (kATileBytes >> 4));
+            for (int k = 0; k < ksteps; ++k)
+                umma_f16_ss(tmem_base + C::SCOL + sd * 64, umma_desc_pack(b_lo + k * 2, desc_hi),
+                            umma_desc_pack(a_lo + k * 128, desc_hi), idesc_s, k > 0, leader);
+            umma_commit(bar_s_full + 8 * sd, leader);
             __syncwarp();
         }
     } else if (warp == kIssuerWarp) {
@@ -368,23 +367,23 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
         constexpr uint32_t idesc_m = umma_idesc_f16(0, 0, 0, BM, BN);     // fp16, K-major
         const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         const uint32_t x_lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((x0 & 0x3FFFFu) >> 4);
+        tmem_base = warp_uniform(tmem_base);
+        const uint32_t leader = elect_one();
         for (int it = 0; it < total; ++it) {
             const int sx = it % SX, ws = it % SD;
             // W^ of the k-step is in TMEM and its activation tile has landed
-            if (!mbar_wait(bar_w_full + 8 * ws, (uint32_t)((it / SD) & 1))) { failed = true; break; }
-            if (!mbar_wait(bar_x_full + 8 * sx, (uint32_t)((it / SX) & 1))) { failed = true; break; }
+            if (!mbar_wait<kWaitSpin>(bar_w_full + 8 * ws, (uint32_t)((it / SD) & 1))) { failed = true; break; }
+            if (!mbar_wait<kWaitSpin>(bar_x_full + 8 * sx, (uint32_t)((it / SX) & 1))) { failed = true; break; }
             tc_fence_after_sync();
-            if (lane == 0) {
-                const uint32_t wslot = tmem_base + C::SCOL + (uint32_t)(ws * 64);
-                const uint32_t x_lo = x_lo0 + (uint32_t)((sx * C::XTILE) >> 4);
+            const uint32_t wslot = tmem_base + C::SCOL + (uint32_t)(ws * 64);
+            const uint32_t x_lo = x_lo0 + (uint32_t)((sx * C::XTILE) >> 4);
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    // columns 0-31 of the k-step sit in slot columns 0-15, columns 32-63 in 32-47
-                    umma_f16_ts(tmem_base, wslot + (k >> 1) * 32 + (k & 1) * 8, umma_desc_pack(x_lo + k * 2, desc_hi), idesc_m,
-                                (it > 0 || k > 0) ? 1u : 0u);
-                umma_commit(bar_done + 8 * (it % DR));
-                if (it == total - 1) umma_commit(bar_acc_full);
-            }
+            for (int k = 0; k < BK / 16; ++k)
+                // columns 0-31 of the k-step sit in slot columns 0-15, columns 32-63 in 32-47
+                umma_f16_ts(tmem_base, wslot + (k >> 1) * 32 + (k & 1) * 8, umma_desc_pack(x_lo + k * 2, desc_hi), idesc_m,
+                            (it > 0 || k > 0) ? 1u : 0u, leader);
+            umma_commit(bar_done + 8 * (it % DR), leader);
+            if (it == total - 1) umma_commit(bar_acc_full, leader);
             __syncwarp();
         }
     } else {
@@ -607,11 +606,12 @@ template <int BITS, int BN, int RP> struct UmmaVariant {
         }
         return cache[dev][cs] > 0 ? cache[dev][cs] : 0;
     }
-    static int launch(const UmmaParams &k, int tiles, int cs, cudaStream_t stream)
+    static int launch(const UmmaParams &k, int tiles, int cs, bool ordered, cudaStream_t stream)
     {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
         fill(cfg, attr, cs, tiles, stream);
+        if (ordered) attr[1].val.programmaticStreamSerializationAllowed = 0;
         LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_umma_kernel<BITS, BN, RP>, k));
         return LORDS_OK;
     }
@@ -680,7 +680,7 @@ template <int BITS, int BN, int RP> int launch_variant(UmmaParams &k, const Prob
         const int early = (size_t)p.M * p.n <= ((size_t)8 << 20) ? 1 : 0;
         cudaLaunchAttribute pre_attr[1];
         pre_attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        pre_attr[0].val.programmaticStreamSerializationAllowed = early;
+        pre_attr[0].val.programmaticStreamSerializationAllowed = early && !p.ordered;
         cudaLaunchConfig_t pre_cfg = cudaLaunchConfig_t{};
         pre_cfg.gridDim = dim3((unsigned)((n_vec + 255) / 256));
         pre_cfg.blockDim = dim3(256);
@@ -699,7 +699,7 @@ template <int BITS, int BN, int RP> int launch_variant(UmmaParams &k, const Prob
         !make_map_2d(&k.tm_q, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.q, row_bytes, (uint64_t)p.m, (uint32_t)UCfg<BITS, BN, RP>::QROW, BM,
                      BITS == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE))
         return LORDS_ERR_CUDA;
-    rc = V::launch(k, clusters, cs, stream);
+    rc = V::launch(k, clusters, cs, p.ordered && UCfg<BITS, BN, RP>::kConvertInKernel, stream);
     if (rc != LORDS_OK) return rc;
     st.last_launches = UCfg<BITS, BN, RP>::kConvertInKernel ? 1 : 2;
     return LORDS_OK;
@@ -737,8 +737,7 @@ template <int BITS> int launch_bits(UmmaParams &k, const Problem &p, State &st, 
 // every TMA row pitch a multiple of 16 bytes.  Anything else: LORDS_ERR_UNSUPPORTED.
 int launch_umma(const Problem &p, State &st, cudaStream_t stream)
 {
-    if (p.bits < 2 || p.bits > 4) return LORDS_ERR_UNSUPPORTED;
-    if (p.r > kRMaxUmma || p.n % (p.bits == 3 ? 128 : 64) != 0) return LORDS_ERR_UNSUPPORTED;
+    if (!umma_takes(p)) return LORDS_ERR_UNSUPPORTED;
 
     UmmaParams k;
     k.B = p.B;
