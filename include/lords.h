@@ -316,7 +316,7 @@ int lords_last_cuda_error(void);
 /*
  * Measurement switches.  Keys: "path" = "auto" | "simt" | "decode" (reassociated-form kernel,
  * M <= 2) | "decode16" (scale-MMA form with 128-column k-steps, 3 <= M <= 16) | "umma" (scale-MMA
- * kernel for any M; "prefill" is an alias);
+ * kernel for any M; "prefill" is an alias) | "dense" (weights expanded to fp16 scratch, then a dense product; any shape) | "direct" (weights formed in registers; M <= 128) | "wide" (M <= 16, 64 < r <= 128);
  * "splitk" = "0" (auto) or a positive integer (CTAs sharing one tile's k-range); "bn" = "0" (auto)
  * or the token tile 32, 64, 128, 256 of the scale-MMA kernel for M > 16; "inject_status" = "0" or a
  * negative status code: writes that value into the device status word, as a kernel that gave up would
@@ -324,8 +324,9 @@ int lords_last_cuda_error(void);
  */
 int lords_set_option(const char *key, const char *value);
 
-/* Name of the path the most recent call dispatched to ("simt", "decode", "decode16", "umma"; "quantize",
- * "quantize_simt" for lords_quantize_codes). */
+/* Name of the path the most recent call dispatched to ("simt", "decode", "decode16", "umma", "wide", "direct", "dense";
+ * "quantize", "quantize_simt" for lords_quantize_codes).  A small layer that the direct kernel takes in place of the decode,
+ * 16-token or scale-MMA kernel reports the name of the path it stands in for. */
 const char *lords_last_path(void);
 
 /* Number of kernels the most recent forward call launched. */

@@ -143,6 +143,73 @@ static int validate(const void *x, const uint8_t *q, const void *B, const void *
     return LORDS_OK;
 }
 
+// Dispatch of a forward call.  A forced path takes the call or declines it (LORDS_ERR_UNSUPPORTED).  Automatically:
+//   - shapes whose row pitches TMA can express, ranks up to 64: the reassociated decode kernel (up to two tokens), the 16-token
+//     kernel, the scale-MMA kernel -- except where the layer is so small that their set-up (a 64 KB table, 27 warps,
+//     TMEM) is most of the call: there the direct kernel stands in for them, under their name (256 x 256: 4.6 -> 3.2 us,
+//     1024 x 2048: 6.1 -> 4.6; level at 2048 x 2048 with rank 32; the two-token kernel sets up less: level at 1024 x 1024;
+//     beyond 16 tokens while token groups x weights stay under 8 M: 1024 x 1024, 64 tokens 7.0 -> 5.9, 128 tokens 8.0 -> 7.5);
+//   - ranks above 64 with up to 16 tokens: the wide-rank kernel, or for small layers the direct kernel;
+//   - everything else: the direct kernel while token groups x weights stay under 32 M (4096 x 4094, 32 tokens: 28 us
+//     against 30; 37 tokens: 46 against 33), then the two-phase path; the CUDA cores for a handful of weights.
+static int dispatch(const Problem &p, State &st, cudaStream_t s)
+{
+    switch (st.forced_path) {
+        case 1: return launch_simt(p, st, s);
+        case 2: return launch_decode(p, st, s);
+        case 3: return launch_umma(p, st, s);
+        case 4: return launch_decode16(p, st, s);
+        case 5: return launch_dense(p, st, s);
+        case 6: return launch_direct(p, st, s);
+        case 7: return launch_wide(p, st, s);
+        default: break;
+    }
+    const long long weights = (long long)p.m * p.n, grouped = (p.M + 15) / 16 * weights;
+    int rc = LORDS_ERR_UNSUPPORTED;
+    if (decode_takes(p)) {
+        if (weights <= (1 << 19)) {
+            rc = launch_direct(p, st, s);
+            if (rc == LORDS_OK) st.last_path = "decode";
+        } else {
+            rc = launch_decode(p, st, s);
+        }
+        if (rc != LORDS_ERR_UNSUPPORTED) return rc;
+    }
+    if (decode16_takes(p)) {
+        if (weights <= (p.r <= 32 ? 3 << 20 : 1 << 20)) {
+            rc = launch_direct(p, st, s);
+            if (rc == LORDS_OK) st.last_path = "decode16";
+        } else {
+            rc = launch_decode16(p, st, s);
+        }
+        if (rc != LORDS_ERR_UNSUPPORTED) return rc;
+    }
+    if (umma_takes(p)) {
+        if (p.M <= 128 && grouped <= (8 << 20)) {
+            rc = launch_direct(p, st, s);
+            if (rc == LORDS_OK) st.last_path = "umma";
+        } else {
+            rc = launch_umma(p, st, s);
+        }
+        if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
+    }
+    if (weights > (1 << 13)) {
+        if (weights > (1 << 20)) {
+            rc = launch_wide(p, st, s);
+            if (rc != LORDS_ERR_UNSUPPORTED) return rc;
+        }
+        if (grouped <= (32 << 20)) {
+            rc = launch_direct(p, st, s);
+            if (rc != LORDS_ERR_UNSUPPORTED) return rc;
+        }
+        rc = launch_dense(p, st, s);
+        if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
+        rc = launch_direct(p, st, s);
+        if (rc != LORDS_ERR_UNSUPPORTED) return rc;
+    }
+    return launch_simt(p, st, s);
+}
+
 static int forward_common(const void *x, const uint8_t *q, const void *B, const void *A, const float *cb,
                           int bits, int M, int m, int n, int r, void *y, int y_f32, void *stream, int ordered = 0)
 {
@@ -161,25 +228,7 @@ static int forward_common(const void *x, const uint8_t *q, const void *B, const 
     st.last_launches = 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
-    // Dispatch.  Each tensor-core path declines (LORDS_ERR_UNSUPPORTED) shapes outside its rules;
-    // "auto" tries the decode kernels (M <= 2, then 3 <= M <= 16), then the scale-MMA kernel, then the
-    // CUDA-core path.
-    if (st.forced_path == 0 || st.forced_path == 2) {
-        rc = launch_decode(p, st, s);
-        if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
-        if (st.forced_path == 2) return rc;
-    }
-    if (st.forced_path == 0 || st.forced_path == 4) {
-        rc = launch_decode16(p, st, s);
-        if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
-        if (st.forced_path == 4) return rc;
-    }
-    if (st.forced_path == 0 || st.forced_path == 3) {
-        rc = launch_umma(p, st, s);
-        if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
-        if (st.forced_path == 3) return rc;
-    }
-    return launch_simt(p, st, s);
+    return dispatch(p, st, s);
 }
 
 }  // namespace lords
@@ -570,7 +619,10 @@ int lords_poll_status(void *stream)
     LORDS_CUDA_TRY(cudaStreamSynchronize(s));
     int word = 0;
     LORDS_CUDA_TRY(cudaMemcpy(&word, st.status_word, sizeof(int), cudaMemcpyDeviceToHost));
-    if (word != 0) LORDS_CUDA_TRY(cudaMemset(st.status_word, 0, sizeof(int)));
+    if (word != 0) {
+        LORDS_CUDA_TRY(cudaMemset(st.status_word, 0, sizeof(int)));
+        LORDS_CUDA_TRY(cudaMemset(st.counters, 0, sizeof(int) * (size_t)st.counter_slots));    // a kernel that gave up may have left some set
+    }
     return word;
 }
 
@@ -597,6 +649,9 @@ int lords_set_option(const char *key, const char *value)
         else if (std::strcmp(value, "decode") == 0) st.forced_path = 2;
         else if (std::strcmp(value, "umma") == 0 || std::strcmp(value, "prefill") == 0) st.forced_path = 3;
         else if (std::strcmp(value, "decode16") == 0) st.forced_path = 4;
+        else if (std::strcmp(value, "dense") == 0) st.forced_path = 5;
+        else if (std::strcmp(value, "direct") == 0) st.forced_path = 6;
+        else if (std::strcmp(value, "wide") == 0) st.forced_path = 7;
         else return LORDS_ERR_OPTION;
         return LORDS_OK;
     }
