@@ -29,8 +29,7 @@
 //          the two folds (register-blocked, operands from shared memory as 16-byte words) on the CUDA
 //          cores.  Taken when the row pitches suit TMA (m, n multiples of 8).
 // Either way every output element is summed in a fixed order without atomics: runs are bit-identical.
-// Bound: fp32 ALU, m n M fused multiply-adds for the tile product (twice with the walk), or, with the
-// tensor schedule, the 2 m n r multiply-adds of the folds.
+// Bound of the CUDA-core schedules: fp32 ALU, m n M fused multiply-adds for the tile product (twice with the walk).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -362,89 +361,116 @@ __global__ void __launch_bounds__(kBwThreads) lords_backward_tile_kernel(const B
     }
 }
 
-// Schedule "tensor": CTA (jt, it) handles rows it * 128 .. and columns jt * 64 .. of W.
-//   G[128 x 64] = sum_t g[t][i] x[t][j]:  both operands are MN-major in shared memory (a row of the tile
-//   is one token: 64 consecutive rows or columns of W), K = 16 tokens per MMA, 64 tokens per stage.
-// Warps 0..7: epilogue (level multiply, folds); 8: TMEM allocation and MMA issue; 9: TMA producer.
-constexpr int kTcRows = 128, kTcCols = 64, kTcTok = 64, kTcStages = 3;
-constexpr int kTcThreads = 320;
-constexpr int kTcGAtom = kTcTok * 128;                        // 64 tokens x 64 rows of W, bf16
-constexpr int kTcStage = 2 * kTcGAtom + kTcTok * 128;         // g: two atoms, x: one
-constexpr uint32_t kTcTmemCols = 64;
-// epilogue buffers (floats): rows of the dS tile and of the A slice are 68 floats apart, rows of the B slice
-// (stored [rank][row]) 132: multiples of four, so that four neighbouring values are one 16-byte word, and with
-// 16-byte words of consecutive rows in different banks
-constexpr int kTcDsPitch = kTcCols + 4, kTcFbPitch = kTcRows + 4;
+// Schedule "tensor": both products on the tensor cores.  A CTA owns 128 rows of W and walks over its share of the 128-column
+// tiles.  Per tile:
+//   G[128 x 128] = sum_t g[t][i] x[t][j]   operands as they lie in memory (MN-major: a shared-memory row is one token), 64 tokens
+//                                          per stage, accumulators in TMEM (two of them: the next tile's product
+//                                          runs while this one is worked on)
+//   dS = G (.) L[Q]                        eight epilogue warps, fp32
+//   dB[128 x r] += dS A_tile^T,  dA_tile^T[128 x r] = dS^T B_tile
+// The folds take dS as three bf16 terms, dS = hi + mid + lo exactly (8 bits of the significand each, split by truncation),
+// and the factors are bf16 as given, so every product is exact and the sums are fp32: the precision of the fp32
+// folds on the CUDA cores that this replaces, at the tensor cores' rate.  One shared-memory tile serves both folds,
+// K-major for dB and MN-major (transposed) for dA; likewise the A tile and the B tile.  dB stays in TMEM over the CTA's
+// tiles; dA_tile goes to scratch, one contribution per row block.
+// 4096 x 4096, r = 32, 512 tokens: 119 us with the folds on the CUDA cores (bound by shared memory at two multiply-adds per
+// word read), @@US@@ us now; what bounds it is the way of g and x from L2 (32 KB per 64 tokens of a tile) and the
+// level multiply with its three-way split (about ten instructions per weight).
+//
+// Warps 0..7: epilogue; 8: TMA of g and x; 9: main MMAs; 10: fold (and scale) MMAs; 11: TMA of the factor tiles.
+constexpr int kTcRows = 128, kTcCols = 128, kTcTok = 64;
+constexpr int kTcEpiWarps = 8;
+constexpr int kTcTmaWarp = 8, kTcMainWarp = 9, kTcFoldWarp = 10, kTcFactorWarp = 11;
+constexpr int kTcThreads = 12 * 32;
+constexpr int kTcGAtom = kTcTok * 128;                        // 64 tokens x 64 rows (or columns) of W, bf16
+constexpr int kTcStage = 4 * kTcGAtom;                        // g: two atoms, x: two
+constexpr int kTcDsAtom = kTcRows * 128;                      // 128 rows x 64 columns of one term of dS
+constexpr int kTcDsTerm = 2 * kTcDsAtom;
 
-struct alignas(64) BwTcParams {
-    CUtensorMap tm_g;     // bf16 [M][m], box {64, 64}, 128-byte swizzle (tokens past M read as zero)
-    CUtensorMap tm_x;     // bf16 [M][n], box {64, 64}, 128-byte swizzle
-    BwParams b;
-    float *part_dB;       // [n / 64 tiles][m][r4]
-    float *part_dA;       // [m / 128 tiles][r4][n]
-    int *status;
-    // quantisation-aware training (Eq. 4-5): the latent weight and, optionally, where dL/dW goes
-    const uint16_t *W;    // bf16 [m][n]
-    float *dW;            // float [m][n] or null
-    // QAT with a rank that is a multiple of 8 up to 64: S = B_tile A_tile by a scale MMA (Eq. 3), as in the forward kernels
-    CUtensorMap tm_b;     // bf16 [m][r], box {64 ranks, 128 rows}, 128-byte swizzle (ranks past r read as zero)
-    CUtensorMap tm_a;     // bf16 [r][n], box {64 columns, ceil16(r) ranks}, 128-byte swizzle
-    int scale_mma;
+// RA: ranks the factor tiles are sized for (64 or 128).  QAT: with the scale tile and the latent weight (Eq. 4-5).
+template <int RA, bool QAT> struct BwCfg {
+    static constexpr int NA = QAT && RA == 64 ? 2 : 1;        // A tiles in flight: S of the next tile needs its A tile early
+    static constexpr int STAGES = RA == 64 && !QAT ? 3 : 2;
+    static constexpr int NG = QAT && RA == 128 ? 1 : 2;       // accumulators of G
+    static constexpr int AATOM = RA * 128;                    // RA ranks x 64 columns
+    static constexpr int ATILE = 2 * AATOM;
+    static constexpr int BTILE = RA / 64 * kTcRows * 128;     // 128 rows x RA ranks, 64 ranks per atom
+    static constexpr int SMEM = 1024 + STAGES * kTcStage + 3 * kTcDsTerm + NA * ATILE + BTILE + 512;
+    static constexpr uint32_t S_COL = NG * kTcCols, DB_COL = S_COL + (QAT ? kTcCols : 0), DA_COL = DB_COL + RA;
+    static constexpr uint32_t TMEM = 512;
+    static_assert(SMEM <= 232448 && DA_COL + RA <= 512, "shared memory and TMEM");
 };
 
-constexpr int kTcBTile = kTcRows * 128;                       // scale MMA: B[128 rows][64 ranks] bf16
-constexpr int kTcATile = 64 * 128;                            // scale MMA: A[64 ranks][64 columns] bf16
+struct alignas(64) BwTcParams {
+    CUtensorMap tm_g;     // bf16 [M][m], box {64, 64}, 128-byte swizzle (tokens past M and rows past m read as zero)
+    CUtensorMap tm_x;     // bf16 [M][n], box {64, 64}, 128-byte swizzle
+    CUtensorMap tm_a;     // bf16 [r][n], box {64 columns, ceil16(r) ranks}, 128-byte swizzle (ranks past r read as zero)
+    CUtensorMap tm_b;     // bf16 [m][r], box {64 ranks, 128 rows}, 128-byte swizzle; used if rows of B are 16-byte multiples
+    BwParams b;
+    int r4, r_pad;
+    int col_tiles, splits;   // 128-column tiles; CTAs that share a row block
+    float *part_dB;       // [splits][m][r4] or null
+    float *part_dA;       // [row blocks][r4][n] or null
+    int *status;
+};
 
-__host__ __device__ constexpr int bw_tc_smem(int r4, bool qat)
+template <int RA, bool QAT>
+__global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const __grid_constant__ BwTcParams p)
 {
-    // the epilogue's buffers (dS tile, the two factor slices) reuse the stages once the MMAs are done;
-    // the operand tiles of the scale MMA (QAT) lie behind the barriers, on a 1024-byte boundary of their own
-    const int stages = kTcStages * kTcStage;
-    const int epi = kTcRows * kTcDsPitch * 4 + r4 * kTcDsPitch * 4 + r4 * kTcFbPitch * 4;
-    return 1024 + (stages > epi ? stages : epi) + 256 + (qat ? 1024 + kTcBTile + kTcATile : 0);
-}
-
-// QAT: the tile of g^T x is dL/dW^ itself (Eq. 4: stored as dL/dW if asked for), and the factor of
-// dL/dS is Q - W (/) S instead of Q (Eq. 5), with S = B A rebuilt per element from the factor slices.
-template <bool QAT>
-__global__ void __launch_bounds__(kTcThreads, 2) lords_backward_tc_kernel(const __grid_constant__ BwTcParams p)
-{
+    using C = BwCfg<RA, QAT>;
     extern __shared__ uint8_t tc_smem_raw[];
     const uint32_t base = (smem_u32(tc_smem_raw) + 1023u) & ~1023u;
-    uint8_t *base_ptr = tc_smem_raw + (base - smem_u32(tc_smem_raw));
-    const int r4 = (p.b.r + 3) & ~3;
-    const int stages_bytes = kTcStages * kTcStage;
-    const int epi_bytes = kTcRows * kTcDsPitch * 4 + r4 * kTcDsPitch * 4 + r4 * kTcFbPitch * 4;
-    const uint32_t bars = base + (uint32_t)(stages_bytes > epi_bytes ? stages_bytes : epi_bytes);
-    const uint32_t bar_full = bars, bar_empty = bars + 8 * kTcStages, bar_acc = bar_empty + 8 * kTcStages;
-    const uint32_t tmem_slot = bar_acc + 8;
-    const uint32_t bar_s_full = bar_acc + 16, bar_s_done = bar_acc + 24;     // scale MMA (QAT): operand tiles landed, S complete
-    const uint32_t s_btile = (bars + 256u + 1023u) & ~1023u, s_atile = s_btile + kTcBTile;
-    const bool scale_mma = QAT && p.scale_mma != 0;
-    constexpr uint32_t kTmemCols = QAT ? 2 * kTcTmemCols : kTcTmemCols;     // QAT: S in the columns behind the accumulator
-    const int r16 = (p.b.r + 15) & ~15;
-    // the level table in shared memory (16 floats behind the barriers): a lookup by a per-thread code is one
-    // conflict-free read there, where the same lookup in the kernel parameters is replayed once per distinct code
-    float *levels_s = reinterpret_cast<float *>(base_ptr + (bars - base) + 128);
-
+    const uint32_t ds0 = base + C::STAGES * kTcStage, a_s = ds0 + 3 * kTcDsTerm, b_s = a_s + C::NA * C::ATILE, bars = b_s + C::BTILE;
+    const uint32_t bar_full = bars, bar_empty = bar_full + 8 * C::STAGES, bar_g = bar_empty + 8 * C::STAGES, bar_g_free = bar_g + 16;
+    const uint32_t bar_a = bar_g_free + 16, bar_ds = bar_a + 16, bar_fold = bar_ds + 8, bar_b = bar_fold + 8, bar_s = bar_b + 8, bar_s_free = bar_s + 8;
+    const uint32_t tmem_slot = bar_s_free + 8, levels_s = bars + 256;      // sixteen floats
+    static_assert(16 * C::STAGES + 16 * 3 + 8 * 5 + 4 <= 256, "barrier area");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int jt = blockIdx.x, it = blockIdx.y;
-    const int i0 = it * kTcRows, j0 = jt * kTcCols;
+    const int rb = (int)blockIdx.x / p.splits, split = (int)blockIdx.x % p.splits;
+    const int i0 = rb * kTcRows;
+    const int t_a = (int)((long long)split * p.col_tiles / p.splits), total = (int)((long long)(split + 1) * p.col_tiles / p.splits) - t_a;
     const int chunks = (p.b.M + kTcTok - 1) / kTcTok;
+    const bool b_by_tma = (p.b.r & 7) == 0;
     const int *status = p.status;
     bool failed = false;
 
-    if (tid == 0) {
-        for (int s = 0; s < kTcStages; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
-        mbar_init(bar_acc, 1);
-        mbar_init(bar_s_full, 1);
-        mbar_init(bar_s_done, 1);
-        fence_mbar_init();
-    }
-    if (tid >= 32 && tid < 48) levels_s[tid - 32] = p.b.levels[tid - 32];
-    if (warp == 8) {
-        tmem_alloc(tmem_slot, kTmemCols);
+    if (warp == kTcTmaWarp) {
+        if (lane == 0) {
+            for (int s = 0; s < C::STAGES; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
+            for (int s = 0; s < 2; ++s) { mbar_init(bar_g + 8 * s, 1); mbar_init(bar_g_free + 8 * s, kTcEpiWarps); mbar_init(bar_a + 8 * s, 1); }
+            mbar_init(bar_ds, kTcEpiWarps);
+            mbar_init(bar_fold, 1);
+            mbar_init(bar_b, 1);
+            mbar_init(bar_s, 1);
+            mbar_init(bar_s_free, kTcEpiWarps);
+            fence_mbar_init();
+            tma_prefetch_desc(&p.tm_g);
+            tma_prefetch_desc(&p.tm_x);
+            tma_prefetch_desc(&p.tm_a);
+        }
+    } else if (warp == kTcFoldWarp) {
+        tmem_alloc(tmem_slot, C::TMEM);
         tmem_relinquish();
+    } else if (warp < kTcEpiWarps) {
+        if (tid < 16) sts_u32(levels_s + 4 * tid, __float_as_uint(p.b.levels[tid]));
+        if (!b_by_tma) {
+            // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m
+            const int rr = tid >> 1, i = i0 + rr;
+            for (int c = 0; c < RA / 16; ++c) {
+                const int chunk = (tid & 1) * (RA / 16) + c;
+                uint32_t w4[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int k = chunk * 8 + 2 * e;
+                    const uint32_t lo = (i < p.b.m && k < p.b.r) ? p.b.B[(size_t)i * p.b.r + k] : 0u;
+                    const uint32_t hi = (i < p.b.m && k + 1 < p.b.r) ? p.b.B[(size_t)i * p.b.r + k + 1] : 0u;
+                    w4[e] = lo | (hi << 16);
+                }
+                sts_v4(b_s + (uint32_t)((chunk >> 3) * kTcRows * 128 + (rr >> 3) * 1024 + (rr & 7) * 128 + (((chunk & 7) ^ (rr & 7)) << 4)),
+                       make_uint4(w4[0], w4[1], w4[2], w4[3]));
+            }
+            fence_proxy_async_smem();
+        }
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -452,347 +478,290 @@ __global__ void __launch_bounds__(kTcThreads, 2) lords_backward_tc_kernel(const 
     uint32_t tmem_base;
     asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
 
-    if (warp == 9) {
+    if (warp == kTcTmaWarp) {
+        // ------------------------------------------------------------------ g and x, 64 tokens per stage
         if (lane == 0) {
-            tma_prefetch_desc(&p.tm_g);
-            tma_prefetch_desc(&p.tm_x);
-            if (scale_mma) {
-                mbar_expect_tx(bar_s_full, (uint32_t)(kTcBTile + r16 * 128));
-                tma_load_2d(s_btile, &p.tm_b, 0, i0, bar_s_full);
-                tma_load_2d(s_atile, &p.tm_a, j0, 0, bar_s_full);
-            }
-            for (int c = 0; c < chunks; ++c) {
-                const int s = c % kTcStages;
-                if (c >= kTcStages && !mbar_wait(bar_empty + 8 * s, (uint32_t)((c / kTcStages - 1) & 1), status, 41)) { failed = true; break; }
-                const uint32_t bar = bar_full + 8 * s, st0 = base + (uint32_t)(s * kTcStage);
-                mbar_expect_tx(bar, (uint32_t)kTcStage);
-                tma_load_2d(st0, &p.tm_g, i0, c * kTcTok, bar);
-                tma_load_2d(st0 + kTcGAtom, &p.tm_g, i0 + 64, c * kTcTok, bar);
-                tma_load_2d(st0 + 2 * kTcGAtom, &p.tm_x, j0, c * kTcTok, bar);
+            int it = 0;
+            for (int t = 0; t < total && !failed; ++t) {
+                const int j0 = (t_a + t) * kTcCols;
+                for (int c = 0; c < chunks; ++c, ++it) {
+                    const int s = it % C::STAGES;
+                    if (it >= C::STAGES && !mbar_wait(bar_empty + 8 * s, (uint32_t)((it / C::STAGES - 1) & 1), status, 41)) { failed = true; break; }
+                    const uint32_t bar = bar_full + 8 * s, st0 = base + (uint32_t)(s * kTcStage);
+                    mbar_expect_tx(bar, (uint32_t)kTcStage);
+                    tma_load_2d(st0, &p.tm_g, i0, c * kTcTok, bar);
+                    tma_load_2d(st0 + kTcGAtom, &p.tm_g, i0 + 64, c * kTcTok, bar);
+                    tma_load_2d(st0 + 2 * kTcGAtom, &p.tm_x, j0, c * kTcTok, bar);
+                    tma_load_2d(st0 + 3 * kTcGAtom, &p.tm_x, j0 + 64, c * kTcTok, bar);
+                }
             }
         }
-    } else if (warp == 8) {
+        __syncwarp();
+    } else if (warp == kTcFactorWarp) {
+        // ------------------------------------------------------------------ the B tile once, an A tile per column tile
+        if (lane == 0) {
+            if (b_by_tma) {
+                mbar_expect_tx(bar_b, (uint32_t)C::BTILE);
+                for (int h = 0; h < RA / 64; ++h) tma_load_2d(b_s + (uint32_t)(h * kTcRows * 128), &p.tm_b, h * 64, i0, bar_b);
+            }
+            for (int t = 0; t < total; ++t) {
+                // its buffer is free when the folds of the tile NA before it have completed (with two buffers the folds cannot
+                // run a phase ahead of this wait: the scale MMA issued before them needs the tile loaded here)
+                if (t >= C::NA && !mbar_wait(bar_fold, (uint32_t)((t - C::NA) & 1), status, 46)) { failed = true; break; }
+                const uint32_t bar = bar_a + 8 * (t % C::NA), dst = a_s + (uint32_t)((t % C::NA) * C::ATILE);
+                const int j0 = (t_a + t) * kTcCols;
+                mbar_expect_tx(bar, (uint32_t)(2 * p.r_pad * 128));
+                tma_load_2d(dst, &p.tm_a, j0, 0, bar);
+                tma_load_2d(dst + C::AATOM, &p.tm_a, j0 + 64, 0, bar);
+            }
+        }
+        __syncwarp();
+    } else if (warp == kTcMainWarp) {
+        // ------------------------------------------------------------------ main MMAs
         constexpr uint32_t idesc = umma_idesc_f16(1, 1, 1, kTcRows, kTcCols);     // bf16, both operands MN-major
-        const uint32_t a_hi = (uint32_t)(umma_desc_sw128(0, 1024, (uint32_t)kTcGAtom) >> 32);
+        const uint32_t hi = (uint32_t)(umma_desc_sw128(0, 1024, (uint32_t)kTcGAtom) >> 32);
         const uint32_t a_lo0 = (uint32_t)umma_desc_sw128(0, 1024, (uint32_t)kTcGAtom) | ((base & 0x3FFFFu) >> 4);
-        const uint32_t b_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
-        const uint32_t b_lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | (((base + 2 * kTcGAtom) & 0x3FFFFu) >> 4);
         const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
-        if (scale_mma) {
-            // S[128 x 64] = B_tile (K-major: a row is one row of B, 16 ranks = 32 bytes) * A_tile (MN-major: a row is one
-            // rank, 16 ranks = 16 rows of 128 bytes), one MMA per 16 ranks, into the columns behind the accumulator
-            constexpr uint32_t idesc_s = umma_idesc_f16(1, 0, 1, kTcRows, kTcCols);
-            if (!mbar_wait(bar_s_full, 0, status, 44)) failed = true;
+        int it = 0;
+        for (int t = 0; t < total && !failed; ++t) {
+            const int gb = t % C::NG;
+            if (t >= C::NG && !mbar_wait_warp(bar_g_free + 8 * gb, (uint32_t)((t / C::NG - 1) & 1), status, 47)) { failed = true; break; }
             tc_fence_after_sync();
-            if (!__any_sync(0xffffffffu, failed)) {
-                const uint32_t sb_lo = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((s_btile & 0x3FFFFu) >> 4);
-                const uint32_t sa_lo = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((s_atile & 0x3FFFFu) >> 4);
-                for (int k = 0; k < r16 / 16; ++k)
-                    umma_f16_ss(tmem_u + kTcTmemCols, umma_desc_pack(sb_lo + k * 2, b_hi), umma_desc_pack(sa_lo + k * 128, b_hi),
-                                idesc_s, k > 0 ? 1u : 0u, leader);
-                umma_commit(bar_s_done, leader);
-            }
-            __syncwarp();
-        }
-        for (int c = 0; c < chunks && !failed; ++c) {
-            const int s = c % kTcStages;
-            if (!mbar_wait(bar_full + 8 * s, (uint32_t)((c / kTcStages) & 1), status, 42)) { failed = true; break; }
-            tc_fence_after_sync();
-            const uint32_t off = (uint32_t)((s * kTcStage) >> 4);
+            for (int c = 0; c < chunks; ++c, ++it) {
+                const int s = it % C::STAGES;
+                if (!mbar_wait_warp(bar_full + 8 * s, (uint32_t)((it / C::STAGES) & 1), status, 42)) { failed = true; break; }
+                tc_fence_after_sync();
+                const uint32_t a_lo = a_lo0 + (uint32_t)((s * kTcStage) >> 4), b_lo = a_lo + (2 * kTcGAtom >> 4);
 #pragma unroll
-            for (int k = 0; k < kTcTok / 16; ++k)      // 16 tokens = 16 rows of 128 bytes
-                umma_f16_ss(tmem_u, umma_desc_pack(a_lo0 + off + k * 128, a_hi), umma_desc_pack(b_lo0 + off + k * 128, b_hi),
-                            idesc, (c > 0 || k > 0) ? 1u : 0u, leader);
-            umma_commit(bar_empty + 8 * s, leader);
-            if (c == chunks - 1) umma_commit(bar_acc, leader);
-            __syncwarp();
+                for (int k = 0; k < kTcTok / 16; ++k)      // 16 tokens = 16 rows of 128 bytes
+                    umma_f16_ss(tmem_u + (uint32_t)(gb * kTcCols), umma_desc_pack(a_lo + k * 128, hi), umma_desc_pack(b_lo + k * 128, hi), idesc,
+                                (c > 0 || k > 0) ? 1u : 0u, leader);
+                umma_commit(bar_empty + 8 * s, leader);
+                if (c == chunks - 1) umma_commit(bar_g + 8 * gb, leader);
+            }
+        }
+    } else if (warp == kTcFoldWarp) {
+        // ------------------------------------------------------------------ fold MMAs, and for QAT the scale MMA of the next tile
+        const uint32_t idesc_b = umma_idesc_f16(1, 0, 0, kTcRows, 16) & ~(0x3Fu << 17) | ((uint32_t)(p.r_pad >> 3) << 17);    // dS K-major, A tile K-major
+        const uint32_t idesc_a = umma_idesc_f16(1, 1, 1, kTcCols, 16) & ~(0x3Fu << 17) | ((uint32_t)(p.r_pad >> 3) << 17);    // dS MN-major, B tile MN-major
+        constexpr uint32_t idesc_s = umma_idesc_f16(1, 0, 1, kTcRows, kTcCols);                                               // B tile K-major, A tile MN-major
+        const uint32_t hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
+        auto desc_lo = [&](uint32_t addr, uint32_t lbo) { return (uint32_t)umma_desc_sw128(0, 1024, lbo) | ((addr & 0x3FFFFu) >> 4); };
+        const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
+        if (b_by_tma && !mbar_wait_warp(bar_b, 0, status, 44)) failed = true;
+        auto scale = [&](int t) {
+            if (!mbar_wait_warp(bar_a + 8 * (t % C::NA), (uint32_t)((t / C::NA) & 1), status, 48) ||
+                (t > 0 && !mbar_wait_warp(bar_s_free, (uint32_t)((t - 1) & 1), status, 49))) { failed = true; return; }
+            tc_fence_after_sync();
+            const uint32_t sb = desc_lo(b_s, 16), sa = desc_lo(a_s + (uint32_t)((t % C::NA) * C::ATILE), (uint32_t)C::AATOM);
+            for (int k = 0; k < p.r_pad / 16; ++k)
+                umma_f16_ss(tmem_u + C::S_COL, umma_desc_pack(sb + (k >> 2) * (kTcRows * 128 >> 4) + (k & 3) * 2, hi), umma_desc_pack(sa + k * 128, hi),
+                            idesc_s, k > 0 ? 1u : 0u, leader);
+            umma_commit(bar_s, leader);
+        };
+        if (QAT && total > 0 && !failed) scale(0);
+        for (int t = 0; t < total && !failed; ++t) {
+            const int an = t % C::NA;
+            if (QAT && C::NA == 2 && t + 1 < total) scale(t + 1);
+            if (failed) break;
+            if (!mbar_wait_warp2(bar_a + 8 * an, (uint32_t)((t / C::NA) & 1), bar_ds, (uint32_t)(t & 1), status, 50)) { failed = true; break; }
+            tc_fence_after_sync();
+            const uint32_t a_tile = a_s + (uint32_t)(an * C::ATILE);
+            if (p.part_dB) {
+                const uint32_t db = desc_lo(a_tile, 16);
+#pragma unroll 1
+                for (int e = 0; e < 3; ++e) {
+                    const uint32_t da = desc_lo(ds0 + (uint32_t)(e * kTcDsTerm), 16);
+#pragma unroll
+                    for (int k = 0; k < kTcCols / 16; ++k)
+                        umma_f16_ss(tmem_u + C::DB_COL, umma_desc_pack(da + (k >> 2) * (kTcDsAtom >> 4) + (k & 3) * 2, hi),
+                                    umma_desc_pack(db + (k >> 2) * (C::AATOM >> 4) + (k & 3) * 2, hi), idesc_b, (t > 0 || e > 0 || k > 0) ? 1u : 0u, leader);
+                }
+            }
+            if (p.part_dA) {
+                const uint32_t db = desc_lo(b_s, (uint32_t)(kTcRows * 128));
+#pragma unroll 1
+                for (int e = 0; e < 3; ++e) {
+                    const uint32_t da = desc_lo(ds0 + (uint32_t)(e * kTcDsTerm), (uint32_t)kTcDsAtom);
+#pragma unroll
+                    for (int k = 0; k < kTcRows / 16; ++k)
+                        umma_f16_ss(tmem_u + C::DA_COL, umma_desc_pack(da + k * 128, hi), umma_desc_pack(db + k * 128, hi), idesc_a,
+                                    (e > 0 || k > 0) ? 1u : 0u, leader);
+                }
+            }
+            umma_commit(bar_fold, leader);
+            if (QAT && C::NA == 1 && t + 1 < total) scale(t + 1);
         }
     } else {
-        // ---- epilogue: thread = (row quadrant q, column half ch): row i0 + q * 32 + lane, 32 columns
-        const int q = warp & 3, ch = warp >> 2;
-        const int ri = q * 32 + lane, i = i0 + ri;
-        // the dS tile and the factor slices (widened to fp32)
-        float (*ds)[kTcDsPitch] = reinterpret_cast<float (*)[kTcDsPitch]>(base_ptr);
-        float (*fa)[kTcDsPitch] = reinterpret_cast<float (*)[kTcDsPitch]>(base_ptr + kTcRows * kTcDsPitch * 4);
-        float (*fb)[kTcFbPitch] =
-            reinterpret_cast<float (*)[kTcFbPitch]>(base_ptr + kTcRows * kTcDsPitch * 4 + r4 * kTcDsPitch * 4);
-        // What the epilogue needs from global memory does not depend on the tile product: the thread's codes and, for
-        // ranks that are multiples of 8 up to 32 (one 16-byte piece of the A slice and two of the B slice per thread),
-        // the factor slices are requested before the wait for the accumulator and parked in registers.
-        const int et = tid;                                       // 0 .. 255
+        // ------------------------------------------------------------------ epilogue: row i0 + q * 32 + lane, 64 columns per thread
+        const int q = warp & 3, ch = warp >> 2, ri = q * 32 + lane, i = i0 + ri;
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         const size_t row_bytes = (size_t)p.b.n * p.b.bits / 8;
-        const int jc = j0 + ch * 32, bits = p.b.bits;
-        // the thread's 32 codes are `bits` consecutive 32-bit words of its row when the group lies
-        // inside the row and the row pitch keeps it word-aligned; otherwise code by code
-        const bool whole_shape = i < p.b.m && jc + 32 <= p.b.n && (row_bytes & 3) == 0;
-        uint32_t cw[5] = {0u, 0u, 0u, 0u, 0u};
-        if (whole_shape) {
-            const uint32_t *src = reinterpret_cast<const uint32_t *>(p.b.q + (size_t)i * row_bytes + (size_t)jc * bits / 8);
+        const int bits = p.b.bits;
+        // the folds of a tile have completed: its columns' contribution to dA leaves TMEM (lane = column, TMEM column = rank)
+        auto store_dA = [&](int t) {
+            if (!mbar_wait_warp(bar_fold, (uint32_t)(t & 1), status, 45)) { failed = true; return; }
+            tc_fence_after_sync();
+            if (!p.part_dA) return;
+            const int j = (t_a + t) * kTcCols + ri;
+            float *out = p.part_dA + (size_t)rb * p.r4 * p.b.n + j;
+            for (int k0 = ch * 16; k0 < p.r4; k0 += 32) {
+                uint32_t v[16];
+                tmem_ld_32x16(lane_addr + C::DA_COL + (uint32_t)k0, v);
+                tmem_wait_ld(v);
+                if (j < p.b.n)
 #pragma unroll
-            for (int w = 0; w < 4; ++w)
-                if (w < bits) cw[w] = __ldg(src + w);
-        }
-        const bool parked = (p.b.r & 7) == 0 && r4 <= 32;
-        uint4 park_a = make_uint4(0u, 0u, 0u, 0u), park_b[2] = {park_a, park_a};
-        if (parked) {
-            const int k = et / (kTcCols / 8), c8 = 8 * (et % (kTcCols / 8));
-            if (k < p.b.r && j0 + c8 < p.b.n) park_a = __ldg(reinterpret_cast<const uint4 *>(p.b.A + (size_t)k * p.b.n + j0 + c8));
-            const int per_row = p.b.r / 8;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int e = et + 256 * h, cidx = e / per_row, k8 = 8 * (e % per_row);
-                if (e < kTcRows * per_row && i0 + cidx < p.b.m)
-                    park_b[h] = __ldg(reinterpret_cast<const uint4 *>(p.b.B + (size_t)(i0 + cidx) * p.b.r + k8));
+                    for (int k = 0; k < 16; ++k)
+                        if (k0 + k < p.r4) __stcg(out + (size_t)(k0 + k) * p.b.n, __uint_as_float(v[k]));
             }
-        }
-        // QAT: the thread's 32 latent weights (64 bytes of its row; n is a multiple of 8, so a group of eight is whole)
-        uint4 wq[QAT ? 4 : 1];
-        if constexpr (QAT) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                wq[v] = make_uint4(0u, 0u, 0u, 0u);
-                if (i < p.b.m && jc + 8 * v < p.b.n) wq[v] = __ldg(reinterpret_cast<const uint4 *>(p.W + (size_t)i * p.b.n + jc + 8 * v));
-            }
-        }
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(bar_acc, 0, status, 43));
-        if (!ok) failed = true;
-        tc_fence_after_sync();
-        uint32_t gacc[32];
-        if (ok) {
-            tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 32), gacc);
-            tmem_wait_ld();
-        }
-        // every MMA has completed (the accumulator barrier), so every stage has been read: the stages'
-        // memory now holds the factor slices and the dS tile
-        auto store_a8 = [&](int k, int c8, const uint4 &v) {
-            *reinterpret_cast<float4 *>(&fa[k][c8]) = make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u),
-                                                                  __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
-            *reinterpret_cast<float4 *>(&fa[k][c8 + 4]) = make_float4(__uint_as_float(v.z << 16), __uint_as_float(v.z & 0xFFFF0000u),
-                                                                      __uint_as_float(v.w << 16), __uint_as_float(v.w & 0xFFFF0000u));
+            tc_fence_before_sync();
         };
-        auto store_b8 = [&](int cidx, int k8, const uint4 &v) {
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        for (int t = 0; t < total; ++t) {
+            const int gb = t % C::NG;
+            // what does not depend on the products is requested first: the thread's codes and latent weights
+            uint32_t cw[2][4];
+            bool whole[2];
+            uint4 wq[QAT ? 2 : 1][4];
 #pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                fb[k8 + 2 * h][cidx] = __uint_as_float(w[h] << 16);
-                fb[k8 + 2 * h + 1][cidx] = __uint_as_float(w[h] & 0xFFFF0000u);
-            }
-        };
-        auto load_slices = [&]() {
-            if (parked) {
-                if (et < r4 * (kTcCols / 8)) store_a8(et / (kTcCols / 8), 8 * (et % (kTcCols / 8)), park_a);
-                const int per_row = p.b.r / 8;
+            for (int c = 0; c < 2; ++c) {
+                const int jc = (t_a + t) * kTcCols + ch * 64 + c * 32;
+                whole[c] = i < p.b.m && jc + 32 <= p.b.n && (row_bytes & 3) == 0;
+                const uint32_t *src = reinterpret_cast<const uint32_t *>(p.b.q + (size_t)(whole[c] ? i : 0) * row_bytes + (whole[c] ? (size_t)jc * bits / 8 : 0));
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int e = et + 256 * h;
-                    if (e < kTcRows * per_row) store_b8(e / per_row, 8 * (e % per_row), park_b[h]);
-                }
-                return;
-            }
-            // A[k][j0 ..]: eight columns (16 bytes) per load -- n is a multiple of 8 on this schedule, so a group
-            // of eight columns is whole and aligned
-            for (int e = et; e < r4 * (kTcCols / 8); e += 256) {
-                const int k = e / (kTcCols / 8), c8 = 8 * (e % (kTcCols / 8));
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (k < p.b.r && j0 + c8 < p.b.n) v = __ldg(reinterpret_cast<const uint4 *>(p.b.A + (size_t)k * p.b.n + j0 + c8));
-                store_a8(k, c8, v);
-            }
-            // B[i0 ..][k] stored [k][i]
-            if ((p.b.r & 7) == 0) {                                   // rows of B are 16-byte multiples: eight ranks per load
-                const int per_row = p.b.r / 8;
-                for (int e = et; e < kTcRows * per_row; e += 256) {
-                    const int cidx = e / per_row, k8 = 8 * (e % per_row);
-                    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                    if (i0 + cidx < p.b.m) v = __ldg(reinterpret_cast<const uint4 *>(p.b.B + (size_t)(i0 + cidx) * p.b.r + k8));
-                    store_b8(cidx, k8, v);
-                }
-            } else {
-                for (int e = et; e < r4 * kTcRows; e += 256) {        // neighbouring threads read one row of B
-                    const int cidx = e / r4, k = e % r4;
-                    fb[k][cidx] = (k < p.b.r && i0 + cidx < p.b.m) ? bf16f(p.b.B[(size_t)(i0 + cidx) * p.b.r + k]) : 0.0f;
+                for (int w = 0; w < 4; ++w) cw[c][w] = whole[c] && w < bits ? __ldg(src + w) : 0u;
+                if constexpr (QAT) {
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        wq[c][v] = make_uint4(0u, 0u, 0u, 0u);
+                        if (i < p.b.m && jc + 8 * v < p.b.n) wq[c][v] = __ldg(reinterpret_cast<const uint4 *>(p.b.W + (size_t)i * p.b.n + jc + 8 * v));
+                    }
                 }
             }
-        };
-        if constexpr (QAT) load_slices();                         // S is rebuilt from them below
-        const bool whole = ok && whole_shape;
-        // QAT: W / S per element (0 where S is 0, and the level is dropped there too: no gradient)
-        float quot[QAT ? 32 : 1];
-        bool live[QAT ? 32 : 1];
-        if constexpr (QAT) {
-            if (p.dW && ok && i < p.b.m) {                        // Eq. 4: dL/dW = dL/dW^
-#pragma unroll
-                for (int c4 = 0; c4 < 32; c4 += 4)
-                    if (jc + c4 < p.b.n)
-                        *reinterpret_cast<float4 *>(p.dW + (size_t)i * p.b.n + jc + c4) =
-                            make_float4(__uint_as_float(gacc[c4]), __uint_as_float(gacc[c4 + 1]), __uint_as_float(gacc[c4 + 2]),
-                                        __uint_as_float(gacc[c4 + 3]));
+            if (!mbar_wait_warp(bar_g + 8 * gb, (uint32_t)((t / C::NG) & 1), status, 43)) { failed = true; break; }
+            if (QAT && !mbar_wait_warp(bar_s, (uint32_t)(t & 1), status, 51)) { failed = true; break; }
+            tc_fence_after_sync();
+            if (t > 0) {
+                store_dA(t - 1);                           // also: the dS buffer is free
+                if (__any_sync(0xffffffffu, failed)) { failed = true; break; }
             }
-            float sv[32];
-            if (scale_mma) {
-                // S of the thread's row and columns from the scale MMA (complete long before the tile product)
-                if (!__all_sync(0xffffffffu, mbar_wait(bar_s_done, 0, status, 45))) failed = true;
-                tc_fence_after_sync();
-                uint32_t sraw[32];
-                tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + kTcTmemCols + (uint32_t)(ch * 32), sraw);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int jc = (t_a + t) * kTcCols + ch * 64 + c * 32;
+                uint32_t gacc[32], sv[QAT ? 32 : 1];
+                tmem_ld_32x32(lane_addr + (uint32_t)(gb * kTcCols + ch * 64 + c * 32), gacc);
+                if constexpr (QAT) tmem_ld_32x32(lane_addr + C::S_COL + (uint32_t)(ch * 64 + c * 32), sv);
                 tmem_wait_ld();
-#pragma unroll
-                for (int cidx = 0; cidx < 32; ++cidx) sv[cidx] = failed ? 0.0f : __uint_as_float(sraw[cidx]);
-            } else {
-                asm volatile("bar.sync 1, 256;" ::: "memory");    // the factor slices are in place
-#pragma unroll
-                for (int cidx = 0; cidx < 32; ++cidx) sv[cidx] = 0.0f;
-                for (int k = 0; k < p.b.r; ++k) {
-                    const float bk = fb[k][ri];
-#pragma unroll
-                    for (int cidx = 0; cidx < 32; ++cidx) sv[cidx] = fmaf(bk, fa[k][ch * 32 + cidx], sv[cidx]);
+                if (c == 1) {
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(bar_g_free + 8 * gb);
+                        if (QAT) mbar_arrive(bar_s_free);
+                    }
                 }
-            }
+                if constexpr (QAT) {
+                    if (p.b.dW && i < p.b.m) {             // Eq. 4: dL/dW = dL/dW^
 #pragma unroll
-            for (int cidx = 0; cidx < 32; ++cidx) {
-                const uint4 &wv = wq[cidx / 8];
-                const uint32_t ww = (cidx % 8) / 2 == 0 ? wv.x : (cidx % 8) / 2 == 1 ? wv.y : (cidx % 8) / 2 == 2 ? wv.z : wv.w;
-                const float w = __uint_as_float((cidx & 1) ? (ww & 0xFFFF0000u) : (ww << 16));
-                live[cidx] = sv[cidx] != 0.0f;
-                // w / S by a reciprocal and one residual correction: exact whenever the quotient is representable
-                // (a weight that its code reproduces exactly gets the factor 0), a rounding error otherwise
-                const float rc = __fdividef(1.0f, sv[cidx]);
-                float qv = w * rc;
-                qv = fmaf(fmaf(-qv, sv[cidx], w), rc, qv);
-                quot[cidx] = live[cidx] ? qv : 0.0f;
-            }
-        }
-        auto factor = [&](int cidx, float level) -> float {
-            if constexpr (QAT) return live[cidx] ? level - quot[cidx] : 0.0f;
-            else return level;
-        };
-        if (whole) {
-            // the positions of the codes inside the words are compile-time constants for each width
-            auto levels_of = [&](auto width) {
-                constexpr int W = decltype(width)::value;
-                float dv[4];
-#pragma unroll
-                for (int cidx = 0; cidx < 32; ++cidx) {
-                    constexpr uint32_t mask = (1u << W) - 1u;
-                    const int bit = cidx * W, w = bit >> 5, sh = bit & 31;
-                    uint32_t code = cw[w] >> sh;
-                    if (sh + W > 32) code |= cw[w + 1] << (32 - sh);
-                    dv[cidx & 3] = __uint_as_float(gacc[cidx]) * factor(cidx, levels_s[code & mask]);
-                    if ((cidx & 3) == 3)
-                        *reinterpret_cast<float4 *>(&ds[ri][ch * 32 + cidx - 3]) = make_float4(dv[0], dv[1], dv[2], dv[3]);
+                        for (int c4 = 0; c4 < 32; c4 += 4)
+                            if (jc + c4 < p.b.n)
+                                *reinterpret_cast<uint4 *>(p.b.dW + (size_t)i * p.b.n + jc + c4) = make_uint4(gacc[c4], gacc[c4 + 1], gacc[c4 + 2], gacc[c4 + 3]);
+                    }
                 }
-            };
-            if (bits == 4) levels_of(std::integral_constant<int, 4>{});
-            else if (bits == 3) levels_of(std::integral_constant<int, 3>{});
-            else levels_of(std::integral_constant<int, 2>{});
-        } else {
+                // the factor of dL/dS: the level, or (QAT, Eq. 5) the level minus W (/) S; 0 where S is 0
+                auto factor = [&](int e, float level) -> float {
+                    if constexpr (QAT) {
+                        const uint4 &wv = wq[c][e / 8];
+                        const uint32_t ww = (e % 8) / 2 == 0 ? wv.x : (e % 8) / 2 == 1 ? wv.y : (e % 8) / 2 == 2 ? wv.z : wv.w;
+                        const float w = __uint_as_float((e & 1) ? (ww & 0xFFFF0000u) : (ww << 16)), s = __uint_as_float(sv[e]);
+                        // w / S by a reciprocal and one residual correction: exact whenever the quotient is representable
+                        // (a weight that its code reproduces exactly gets the factor 0), a rounding error otherwise
+                        const float rc = __fdividef(1.0f, s);
+                        float qv = w * rc;
+                        qv = fmaf(fmaf(-qv, s, w), rc, qv);
+                        return s != 0.0f ? level - qv : 0.0f;
+                    } else {
+                        return level;
+                    }
+                };
+                auto level_at = [&](uint32_t code) { return __uint_as_float(lds_table(levels_s + 4u * code)); };
+                // eight columns at a time: dS, its three terms, one 16-byte store each
+                auto emit = [&](int e8, const float (&d)[8]) {
+                    uint32_t w[3][4];
 #pragma unroll
-            for (int cidx = 0; cidx < 32; ++cidx) {
-                const int j = jc + cidx;
-                float v = 0.0f;
-                if (ok && i < p.b.m && j < p.b.n)
-                    v = __uint_as_float(gacc[cidx]) * factor(cidx, levels_s[read_code(p.b.q, row_bytes, i, j, bits)]);
-                ds[ri][ch * 32 + cidx] = v;
-            }
-        }
-        if constexpr (!QAT) load_slices();
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        // The folds, register-blocked so that a 16-byte word read from shared memory feeds 16 (dB) or 8 (dA)
-        // multiply-adds.  Each output is one thread's sum in index order.
-        if (p.part_dB) {
-            // dB[i][k] = sum_j dS[i][j] A[k][j]: lane = rows lane + 32 a, warp = ranks 4 kg .. 4 kg + 3 (kg = warp, warp + 8, ..)
-            float *out = p.part_dB + ((size_t)jt * p.b.m + i0) * r4;
-            for (int kg = warp; kg < r4 / 4; kg += 8) {
-                const int k0 = 4 * kg;
-                float acc[4][4];
+                    for (int h = 0; h < 4; ++h) {
+                        const float a = d[2 * h], b = d[2 * h + 1];
+                        const float a1 = a - __uint_as_float(__float_as_uint(a) & 0xFFFF0000u), b1 = b - __uint_as_float(__float_as_uint(b) & 0xFFFF0000u);
+                        const float a2 = a1 - __uint_as_float(__float_as_uint(a1) & 0xFFFF0000u), b2 = b1 - __uint_as_float(__float_as_uint(b1) & 0xFFFF0000u);
+                        w[0][h] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+                        w[1][h] = __byte_perm(__float_as_uint(a1), __float_as_uint(b1), 0x7632);
+                        w[2][h] = __byte_perm(__float_as_uint(a2), __float_as_uint(b2), 0x7632);
+                    }
+                    const uint32_t dst = ds0 + (uint32_t)(ch * kTcDsAtom + (ri >> 3) * 1024 + (ri & 7) * 128 + (((c * 4 + e8) ^ (ri & 7)) << 4));
 #pragma unroll
-                for (int a = 0; a < 4; ++a)
+                    for (int k = 0; k < 3; ++k) sts_v4(dst + (uint32_t)(k * kTcDsTerm), make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]));
+                };
+                auto levels_of = [&](auto width) {         // positions of the codes inside the words are constants for each width
+                    constexpr int W = decltype(width)::value;
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
-#pragma unroll 2
-                for (int j4 = 0; j4 < kTcCols / 4; ++j4) {
-                    float4 d[4], w[4];
+                    for (int e8 = 0; e8 < 4; ++e8) {
+                        float d[8];
 #pragma unroll
-                    for (int a = 0; a < 4; ++a) d[a] = *reinterpret_cast<const float4 *>(&ds[lane + 32 * a][4 * j4]);
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) w[b] = *reinterpret_cast<const float4 *>(&fa[k0 + b][4 * j4]);
-#pragma unroll
-                    for (int a = 0; a < 4; ++a)
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            acc[a][b] = fmaf(d[a].x, w[b].x, acc[a][b]);
-                            acc[a][b] = fmaf(d[a].y, w[b].y, acc[a][b]);
-                            acc[a][b] = fmaf(d[a].z, w[b].z, acc[a][b]);
-                            acc[a][b] = fmaf(d[a].w, w[b].w, acc[a][b]);
+                        for (int k = 0; k < 8; ++k) {
+                            const int e = 8 * e8 + k, bit = e * W, w = bit >> 5, sh = bit & 31;
+                            uint32_t code = cw[c][w] >> sh;
+                            if (sh + W > 32) code |= cw[c][w + 1 < 4 ? w + 1 : 3] << (32 - sh);
+                            d[k] = __uint_as_float(gacc[e]) * factor(e, level_at(code & ((1u << W) - 1u)));
                         }
-                }
+                        emit(e8, d);
+                    }
+                };
+                if (__all_sync(0xffffffffu, whole[c])) {
+                    if (bits == 4) levels_of(std::integral_constant<int, 4>{});
+                    else if (bits == 3) levels_of(std::integral_constant<int, 3>{});
+                    else levels_of(std::integral_constant<int, 2>{});
+                } else {
 #pragma unroll
-                for (int a = 0; a < 4; ++a) {
-                    const int ii = lane + 32 * a;
-                    if (i0 + ii < p.b.m)
-                        *reinterpret_cast<float4 *>(&out[(size_t)ii * r4 + k0]) = make_float4(acc[a][0], acc[a][1], acc[a][2], acc[a][3]);
+                    for (int e8 = 0; e8 < 4; ++e8) {
+                        float d[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k) {
+                            const int e = 8 * e8 + k;
+                            d[k] = (i < p.b.m && jc + e < p.b.n) ? __uint_as_float(gacc[e]) * factor(e, level_at(read_code(p.b.q, row_bytes, i, jc + e, bits))) : 0.0f;
+                        }
+                        emit(e8, d);
+                    }
                 }
             }
+            fence_proxy_async_smem();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_ds);
         }
-        if (p.part_dA) {
-            // dA[k][j] = sum_i B[i][k] dS[i][j]: a thread takes 4 ranks x 4 columns over one half of the tile's rows
-            // (warps 0..3: rows 0..63, warps 4..7: rows 64..127); the upper half parks its sums in shared memory
-            // (the A slice's, which the dB fold is done with after the barrier), the lower half adds them to its own.
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-            float *out = p.part_dA + (size_t)it * r4 * p.b.n + j0;
-            float *park = &fa[0][0];                                  // [r4][64] floats
-            const int half = warp >> 2, jq = 4 * (lane & 15), ibase = 64 * half;
-            const int blocks = r4 / 4;
-            for (int kb0 = 0; kb0 < blocks; kb0 += 8) {               // the same trip count for every thread
-                const int kb = kb0 + 2 * (warp & 3) + (lane >> 4);
-                const bool active = kb < blocks;
-                const int k0 = 4 * (active ? kb : 0);
-                float acc[4][4];
+        if (!__any_sync(0xffffffffu, failed) && total > 0) store_dA(total - 1);
+        // dB of the row block over this CTA's tiles: lane = row, TMEM column = rank
+        if (!__any_sync(0xffffffffu, failed) && p.part_dB && total > 0) {
+            float *out = p.part_dB + ((size_t)split * p.b.m + i) * p.r4;
+            for (int k0 = ch * 16; k0 < p.r4; k0 += 32) {
+                uint32_t v[16];
+                tmem_ld_32x16(lane_addr + C::DB_COL + (uint32_t)k0, v);
+                tmem_wait_ld(v);
+                if (i < p.b.m)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[b][0] = acc[b][1] = acc[b][2] = acc[b][3] = 0.0f;
-                if (active) {
-#pragma unroll 4
-                    for (int i2 = 0; i2 < 32; ++i2) {
-                        const int ii = ibase + 2 * i2;
-                        const float4 d0 = *reinterpret_cast<const float4 *>(&ds[ii][jq]);
-                        const float4 d1 = *reinterpret_cast<const float4 *>(&ds[ii + 1][jq]);
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            const float2 bv = *reinterpret_cast<const float2 *>(&fb[k0 + b][ii]);
-                            acc[b][0] = fmaf(bv.x, d0.x, acc[b][0]);
-                            acc[b][1] = fmaf(bv.x, d0.y, acc[b][1]);
-                            acc[b][2] = fmaf(bv.x, d0.z, acc[b][2]);
-                            acc[b][3] = fmaf(bv.x, d0.w, acc[b][3]);
-                            acc[b][0] = fmaf(bv.y, d1.x, acc[b][0]);
-                            acc[b][1] = fmaf(bv.y, d1.y, acc[b][1]);
-                            acc[b][2] = fmaf(bv.y, d1.z, acc[b][2]);
-                            acc[b][3] = fmaf(bv.y, d1.w, acc[b][3]);
-                        }
-                    }
-                    if (half == 1) {
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-                            *reinterpret_cast<float4 *>(&park[(k0 + b) * kTcCols + jq]) = make_float4(acc[b][0], acc[b][1], acc[b][2], acc[b][3]);
-                    }
-                }
-                asm volatile("bar.sync 1, 256;" ::: "memory");
-                if (active && half == 0 && j0 + jq < p.b.n) {        // n is a multiple of 8 on this schedule: a group of four columns is whole
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const float4 u = *reinterpret_cast<const float4 *>(&park[(k0 + b) * kTcCols + jq]);
-                        *reinterpret_cast<float4 *>(&out[(size_t)(k0 + b) * p.b.n + jq]) =
-                            make_float4(acc[b][0] + u.x, acc[b][1] + u.y, acc[b][2] + u.z, acc[b][3] + u.w);
-                    }
-                }
+                    for (int k = 0; k < 16; k += 4)
+                        if (k0 + k < p.r4) __stcg(reinterpret_cast<uint4 *>(out + k0 + k), make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]));
             }
         }
     }
 
-    if (failed) atomicExch(p.status, LORDS_ERR_TIMEOUT);
+    if (failed) {
+        atomicExch(p.status, LORDS_ERR_TIMEOUT);
+        for (int k = 0; k < 100; ++k) __nanosleep(1000);      // copies in flight land before the CTA ends
+    }
     tc_fence_before_sync();
     __syncthreads();
-    if (warp == 8) {
+    if (warp == kTcFoldWarp) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base, kTmemCols);
+        tmem_dealloc(tmem_base, C::TMEM);
     }
 }
 
@@ -852,49 +821,63 @@ int launch_transpose_bf16_pair(const uint16_t *src0, int rows0, int cols0, uint1
     return LORDS_OK;
 }
 
-// The tensor schedule.  W != null: the gradients of quantisation-aware training (dW may be null).
+template <int RA, bool QAT> static int launch_tc_variant(const BwTcParams &k, int ctas, const State &st, cudaStream_t stream)
+{
+    static bool done[kMaxDevices] = {};
+    const int dev = device_slot(st);
+    if (!done[dev]) {
+        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_backward_tc_kernel<RA, QAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwCfg<RA, QAT>::SMEM));
+        done[dev] = true;
+    }
+    lords_backward_tc_kernel<RA, QAT><<<(unsigned)ctas, kTcThreads, BwCfg<RA, QAT>::SMEM, stream>>>(k);
+    LORDS_CUDA_TRY(cudaGetLastError());
+    return LORDS_OK;
+}
+
+// The tensor schedule.  p.W != null: the gradients of quantisation-aware training (dW may be null).
 // LORDS_ERR_UNSUPPORTED when the shapes do not suit it or the workspace cannot hold the contributions.
-static int launch_backward_tc(const BwParams &p, const uint16_t *W, float *dW, State &st, cudaStream_t stream)
+static int launch_backward_tc(const BwParams &p, State &st, cudaStream_t stream)
 {
     const int m = p.m, n = p.n, r = p.r, M = p.M;
-    const int r4 = (r + 3) & ~3;
-    const int it_t = (m + kTcRows - 1) / kTcRows, jt_t = (n + kTcCols - 1) / kTcCols;
-    const size_t nb = p.dB ? (size_t)jt_t * m * r4 * sizeof(float) : 0, na = p.dA ? (size_t)it_t * r4 * n * sizeof(float) : 0;
-    if (m % 8 != 0 || n % 8 != 0 || it_t > 65535 || nb + na + 256 > st.workspace_bytes) return LORDS_ERR_UNSUPPORTED;
     BwTcParams k;
     k.b = p;
+    k.r4 = (r + 3) & ~3;
+    k.r_pad = (r + 15) & ~15;
+    const int row_blocks = (m + kTcRows - 1) / kTcRows;
+    k.col_tiles = (n + kTcCols - 1) / kTcCols;
+    // CTAs per row block: the least rounds of one CTA per SM times (tiles of a CTA + a fixed part worth one)
+    k.splits = 1;
+    double best = 1e30;
+    for (int s = 1; s <= k.col_tiles && s <= 64; ++s) {
+        const double t = (double)(((long long)row_blocks * s + st.sm_count - 1) / st.sm_count) * ((k.col_tiles + s - 1) / s + 1.0);
+        if (t < best) { best = t; k.splits = s; }
+    }
+    const size_t nb = p.dB ? (size_t)k.splits * m * k.r4 * sizeof(float) : 0, na = p.dA ? (size_t)row_blocks * k.r4 * n * sizeof(float) : 0;
+    if (m % 8 != 0 || n % 8 != 0 || nb + na + 256 > st.workspace_bytes || (long long)row_blocks * k.splits > 2147483647LL) return LORDS_ERR_UNSUPPORTED;
     k.part_dB = p.dB ? reinterpret_cast<float *>(st.workspace) : nullptr;
     k.part_dA = p.dA ? reinterpret_cast<float *>(st.workspace + ((nb + 255) & ~(size_t)255)) : nullptr;
     k.status = st.status_word;
-    k.W = W; k.dW = dW;
     if (!make_map_2d(&k.tm_g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.g, (uint64_t)m, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.x, (uint64_t)n, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B))
+        !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.x, (uint64_t)n, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.A, (uint64_t)n, (uint64_t)r, 64, (uint32_t)k.r_pad, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;
-    k.scale_mma = (W && (r & 7) == 0 && r <= 64) ? 1 : 0;
-    k.tm_b = k.tm_g; k.tm_a = k.tm_g;                                      // placeholders when the scale MMA is not used
-    if (k.scale_mma &&
-        (!make_map_2d(&k.tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.B, (uint64_t)r, (uint64_t)m, 64, (uint32_t)kTcRows, CU_TENSOR_MAP_SWIZZLE_128B) ||
-         !make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.A, (uint64_t)n, (uint64_t)r, 64, (uint32_t)((r + 15) & ~15), CU_TENSOR_MAP_SWIZZLE_128B)))
+    k.tm_b = k.tm_a;                                                       // not used where the kernel builds the B tile element by element
+    if ((r & 7) == 0 &&
+        !make_map_2d(&k.tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.B, (uint64_t)r, (uint64_t)m, 64, (uint32_t)kTcRows, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;
-    const int smem = bw_tc_smem(r4, W != nullptr);
-    static bool attr_set[kMaxDevices] = {};
-    const int dev = device_slot(st);
-    if (!attr_set[dev]) {
-        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_backward_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, bw_tc_smem(kRMaxBw, false)));
-        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_backward_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, bw_tc_smem(kRMaxBw, true)));
-        attr_set[dev] = true;
-    }
-    if (W) lords_backward_tc_kernel<true><<<dim3((unsigned)jt_t, (unsigned)it_t), kTcThreads, smem, stream>>>(k);
-    else lords_backward_tc_kernel<false><<<dim3((unsigned)jt_t, (unsigned)it_t), kTcThreads, smem, stream>>>(k);
-    LORDS_CUDA_TRY(cudaGetLastError());
+    const int ctas = row_blocks * k.splits;
+    int rc;
+    if (p.W) rc = r <= 64 ? launch_tc_variant<64, true>(k, ctas, st, stream) : launch_tc_variant<128, true>(k, ctas, st, stream);
+    else rc = r <= 64 ? launch_tc_variant<64, false>(k, ctas, st, stream) : launch_tc_variant<128, false>(k, ctas, st, stream);
+    if (rc != LORDS_OK) return rc;
     int launches = 1;
     if (p.dB || p.dA) {
-        const int rc = launch_reduce(k.part_dB, p.dB, jt_t, k.part_dA, p.dA, it_t, m, n, r, r4, stream);
+        rc = launch_reduce(k.part_dB, p.dB, k.splits, k.part_dA, p.dA, row_blocks, m, n, r, k.r4, stream);
         if (rc != LORDS_OK) return rc;
         ++launches;
     }
     st.last_launches = launches;
-    st.last_path = W ? "backward_qat_tensor" : "backward_tensor";
+    st.last_path = p.W ? "backward_qat_tensor" : "backward_tensor";
     return LORDS_OK;
 }
 
@@ -915,7 +898,7 @@ int launch_backward_factors(const uint16_t *g, const uint16_t *x, const uint8_t 
     const size_t need_b = dB ? (size_t)jt_n * m * r4 * sizeof(float) : 0, need_a = dA ? (size_t)it_n * r4 * n * sizeof(float) : 0;
     // schedule "tensor": the same with 128 x 64 tiles and the tile product on the tensor cores
     if (st.forced_path == 0) {
-        const int rc = launch_backward_tc(p, nullptr, nullptr, st, stream);
+        const int rc = launch_backward_tc(p, st, stream);
         if (rc != LORDS_ERR_UNSUPPORTED) return rc;
     }
     if (it_n <= 65535 && need_b + need_a + 256 <= st.workspace_bytes && st.forced_path != 1) {
@@ -961,12 +944,11 @@ int launch_backward_qat(const uint16_t *g, const uint16_t *x, const uint16_t *W,
     for (int c = 0; c < 16; ++c) p.levels[c] = c < (1 << bits) ? levels[c] : 0.0f;
     p.bits = bits; p.M = M; p.m = m; p.n = n; p.r = r;
     p.dB = dB; p.dA = dA;
-    p.W = nullptr; p.dW = nullptr;                       // the tensor schedule takes them as arguments
+    p.W = W; p.dW = dW;
     if (st.forced_path == 0) {
-        const int rc = launch_backward_tc(p, W, dW, st, stream);
+        const int rc = launch_backward_tc(p, st, stream);
         if (rc != LORDS_ERR_UNSUPPORTED) return rc;
     }
-    p.W = W; p.dW = dW;
     int launches = 0;
     const bool rows_pass = dB || !dA;                    // dL/dW alone is written by the row pass
     if (rows_pass) {
