@@ -58,30 +58,84 @@ __device__ __forceinline__ uint32_t read_code(const uint8_t *__restrict__ q, siz
 }
 
 // ---- transposition of packed codes -----------------------------------------------------------------
-// Thread (j, group): the codes Q[i0 .. i0 + 31][j] become 32 consecutive codes of row j of Q^T.
-// Neighbouring threads take neighbouring j, so the reads of one row of Q are contiguous.
-__global__ void lords_transpose_codes_kernel(const uint8_t *__restrict__ Q, uint8_t *__restrict__ Qt, int m, int n, int bits)
+// A block turns 64 rows x 128 columns around in shared memory, one byte per code: a thread unpacks 32 codes of a row from
+// whole words, another packs 32 codes of a column into whole words (two of them fill a 32-byte sector of a row of
+// Q^T).  Bound: about five instructions per code and one shared-memory byte load; 4096 x 4096, 4 bits: 78 us when every thread
+// collected its column code by code from global memory, 10 us now; 14336 x 4096, 3 bits: 27 (46 with a store of one word per
+// row at a time).
+constexpr int kTrRows = 64, kTrCols = 128, kTrPitch = kTrCols + 4, kTrThreads = 256;
+
+template <int BITS>
+__global__ void __launch_bounds__(kTrThreads) lords_transpose_codes_kernel(const uint8_t *__restrict__ Q, uint8_t *__restrict__ Qt, int m, int n)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    const int i0 = blockIdx.y * 32;
-    if (j >= n) return;
-    const size_t row_bytes = (size_t)n * bits / 8, trow_bytes = (size_t)m * bits / 8;
-    const int count = m - i0 < 32 ? m - i0 : 32;        // a multiple of the pack group, like m
-    unsigned long long lo = 0;                          // up to 128 bits of packed codes
-    unsigned long long hi = 0;
-    for (int ii = 0; ii < count; ++ii) {
-        const unsigned long long c = read_code(Q, row_bytes, i0 + ii, j, bits);
-        const int bit = ii * bits;
-        if (bit < 64) {
-            lo |= c << bit;
-            if (bit + bits > 64) hi |= c >> (64 - bit);
-        } else {
-            hi |= c << (bit - 64);
+    __shared__ __align__(16) uint8_t tile[kTrRows][kTrPitch];
+    __shared__ uint32_t stage[BITS == 4 ? 1 : kTrThreads * BITS];
+    const int tid = threadIdx.x, i0 = (int)blockIdx.y * kTrRows, j0 = (int)blockIdx.x * kTrCols;
+    const size_t row_bytes = (size_t)n * BITS / 8, trow_bytes = (size_t)m * BITS / 8;
+    constexpr uint32_t mask = (1u << BITS) - 1u;
+    {
+        const int row = tid >> 2, seg = tid & 3, i = i0 + row, j = j0 + seg * 32;
+        uint32_t w[BITS + 1];                               // 32 codes are BITS words
+#pragma unroll
+        for (int k = 0; k <= BITS; ++k) w[k] = 0u;
+        if (i < m && j < n) {
+            const uint8_t *src = Q + (size_t)i * row_bytes + (size_t)j * BITS / 8;
+            const int bytes = n - j >= 32 ? 4 * BITS : (n - j) * BITS / 8;
+            if (bytes == 4 * BITS && (row_bytes & 3) == 0) {
+#pragma unroll
+                for (int k = 0; k < BITS; ++k) w[k] = __ldg(reinterpret_cast<const uint32_t *>(src) + k);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4 * BITS; ++k)
+                    if (k < bytes) w[k >> 2] |= (uint32_t)__ldg(src + k) << (8 * (k & 3));
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            uint32_t v = 0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int bit = (4 * q + e) * BITS, wi = bit >> 5, sh = bit & 31;
+                const uint32_t c = (sh + BITS > 32 ? __funnelshift_r(w[wi], w[wi + 1], sh) : w[wi] >> sh) & mask;
+                v |= c << (8 * e);
+            }
+            *reinterpret_cast<uint32_t *>(&tile[row][seg * 32 + 4 * q]) = v;
         }
     }
-    uint8_t *dst = Qt + (size_t)j * trow_bytes + (size_t)i0 * bits / 8;
-    const int bytes = count * bits / 8;
-    for (int b = 0; b < bytes; ++b) dst[b] = (uint8_t)(b < 8 ? lo >> (8 * b) : hi >> (8 * (b - 8)));
+    __syncthreads();
+    {
+        const int col = tid & (kTrCols - 1), half = tid >> 7, j = j0 + col, i = i0 + half * 32;
+        if (j - (tid & 31) < n && i < m) {                  // per warp
+            uint32_t w[BITS + 1];
+#pragma unroll
+            for (int k = 0; k <= BITS; ++k) w[k] = 0u;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                const uint32_t c = tile[half * 32 + e][col];
+                const int bit = e * BITS, wi = bit >> 5, sh = bit & 31;
+                w[wi] |= c << sh;
+                if (sh + BITS > 32) w[wi + 1] |= c >> (32 - sh);
+            }
+            uint8_t *dst = Qt + (size_t)j * trow_bytes + (size_t)i * BITS / 8;
+            const int bytes = m - i >= 32 ? 4 * BITS : (m - i) * BITS / 8;      // m is a multiple of the pack group
+            if (bytes == 4 * BITS && (trow_bytes & 3) == 0) {
+                if constexpr (BITS != 4) {
+                    const int j0w = j - (tid & 31);
+                    store_codes_staged<BITS>(ptx::smem_u32(stage) + (uint32_t)((tid >> 5) * 32 * BITS * 4), Qt + (size_t)j0w * trow_bytes + (size_t)i * BITS / 8,
+                                             trow_bytes, n - j0w, tid & 31, w);
+                } else if (j < n && (trow_bytes & 15) == 0) {
+                    *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                } else if (j < n) {
+#pragma unroll
+                    for (int k = 0; k < BITS; ++k) reinterpret_cast<uint32_t *>(dst)[k] = w[k];
+                }
+            } else if (j < n) {
+#pragma unroll
+                for (int k = 0; k < 4 * BITS; ++k)
+                    if (k < bytes) dst[k] = (uint8_t)(w[k >> 2] >> (8 * (k & 3)));
+            }
+        }
+    }
 }
 
 // Two transpositions in one launch (the factors A and B of a layer): blocks [0, tiles0) take the first matrix,
@@ -374,7 +428,7 @@ __global__ void __launch_bounds__(kBwThreads) lords_backward_tile_kernel(const B
 // K-major for dB and MN-major (transposed) for dA; likewise the A tile and the B tile.  dB stays in TMEM over the CTA's
 // tiles; dA_tile goes to scratch, one contribution per row block.
 // 4096 x 4096, r = 32, 512 tokens: 119 us with the folds on the CUDA cores (bound by shared memory at two multiply-adds per
-// word read), @@US@@ us now; what bounds it is the way of g and x from L2 (32 KB per 64 tokens of a tile) and the
+// word read), 47 us now; what bounds it is the way of g and x from L2 (32 KB per 64 tokens of a tile) and the
 // level multiply with its three-way split (about ten instructions per weight).
 //
 // Warps 0..7: epilogue; 8: TMA of g and x; 9: main MMAs; 10: fold (and scale) MMAs; 11: TMA of the factor tiles.
@@ -804,9 +858,11 @@ int launch_reduce(const float *part_b, float *dB, int tiles_b, const float *part
 
 int launch_transpose_codes(const uint8_t *Q, int m, int n, int bits, uint8_t *Qt, cudaStream_t stream)
 {
-    const dim3 grid((unsigned)((n + 127) / 128), (unsigned)((m + 31) / 32));
+    const dim3 grid((unsigned)((n + kTrCols - 1) / kTrCols), (unsigned)((m + kTrRows - 1) / kTrRows));
     if (grid.y > 65535u) return LORDS_ERR_SHAPE;
-    lords_transpose_codes_kernel<<<grid, 128, 0, stream>>>(Q, Qt, m, n, bits);
+    if (bits == 4) lords_transpose_codes_kernel<4><<<grid, kTrThreads, 0, stream>>>(Q, Qt, m, n);
+    else if (bits == 3) lords_transpose_codes_kernel<3><<<grid, kTrThreads, 0, stream>>>(Q, Qt, m, n);
+    else lords_transpose_codes_kernel<2><<<grid, kTrThreads, 0, stream>>>(Q, Qt, m, n);
     LORDS_CUDA_TRY(cudaGetLastError());
     return LORDS_OK;
 }

@@ -1,5 +1,5 @@
 // Host-side helpers shared by the tensor-core translation units: the tensor-map encoder with a
-// small cache, the output store, and per-device bookkeeping for launch attributes.
+// small cache, the output stores, and per-device bookkeeping for launch attributes.
 #pragma once
 
 #include <cuda.h>
@@ -90,6 +90,25 @@ inline bool make_map_2d(CUtensorMap *map, CUtensorMapDataType dt, int elem_bytes
     e.map = *map;
     e.valid = true;
     return true;
+}
+
+// Packed codes of a warp's 32 rows (32 codes, BITS words each) -> rows of pitch `pitch` at dst0, the first `rows` of them, through shared
+// memory: a store of one word per row touches 32 lines, one of 32 consecutive words 11 (3 bits) or 16 (2 bits).  Quantising
+// 14336 x 4096 to 3 bits spent half of the load/store pipe's time on the former: 72 us a call against 53; transposing it 46 against 27.  (With 4 bits a row's four
+// words go out in one store, which touches as many lines as staged ones would together.)
+template <int BITS> __device__ __forceinline__ void store_codes_staged(uint32_t stage, uint8_t *dst0, size_t pitch, int rows, int lane, const uint32_t *w)
+{
+#pragma unroll
+    for (int k = 0; k < BITS; ++k) asm volatile("st.shared.u32 [%0], %1;" ::"r"(stage + (uint32_t)((lane * BITS + k) * 4)), "r"(w[k]) : "memory");
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < BITS; ++k) {
+        const int e = k * 32 + lane, row = e / BITS;
+        uint32_t v;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(stage + (uint32_t)(e * 4)) : "memory");
+        if (row < rows) reinterpret_cast<uint32_t *>(dst0 + (size_t)row * pitch)[e % BITS] = v;
+    }
+    __syncwarp();
 }
 
 }  // namespace lords
