@@ -5,19 +5,30 @@
 // written out as packed codes in the library's layout.  The paper does not say which level wins a tie:
 // the lowest code does.  S is rebuilt tile by tile on the tensor cores exactly as the forward kernels
 // rebuild it (bf16 operands from shared memory, fp32 in TMEM, never stored in full).  The decision is
-// taken in fp32 with S accumulated in fp32: for a strictly ascending level table by bisection over the
-// midpoints between neighbouring levels (log2 of the level count products and comparisons per weight),
-// for any other table by trying every level in turn (one fused multiply-add and a square per level).
+// taken in fp32 with S accumulated in fp32, in one of three ways (chosen on the host from the level table):
+//   buckets   ascending table whose midpoints lie further apart than a bucket is wide (every NormalFloat table): the
+//             approximate ratio W / S picks a bucket, the bucket gives the one midpoint in it and the code below,
+//             and one exact comparison decides (about thirteen instructions a weight);
+//   bisection any other ascending table: log2 of the level count products and comparisons per weight;
+//   trial     any other table: every level in turn (one fused multiply-add and a square per level).
 //
-// One CTA owns 128 rows of W and a range of 64-column steps.  Warp roles (6 warps):
-//   0..3  search: thread t owns row t; per step it reads its 64 values of S from TMEM (two loads of
-//         32), its 64 weights from global memory, tries the levels, packs the codes and stores them.
-//   4     TMEM allocation and MMA issuer: S[128 x 64] = B_tile (128 x r) * A_tile (r x 64) into one of
-//         two TMEM buffers, as soon as the factor tile has landed and the buffer has been read.
-//   5     TMA producer of the factor tiles A[:, step].
+// A step is a tile of 128 rows and 64 columns.  One CTA per SM takes an equal run of the steps of the whole weight, row tile after row
+// tile (two CTAs per SM, or several rounds of CTAs, paid the set-up of a CTA, worth about three steps, once more: 4096 x 4096 33 us
+// against 20).  Warp roles (18 warps):
+//   0..15 search, two groups of eight on alternating steps (three groups have to make do with 72 registers: 14336 x 4096, 4 bits, 55 us
+//         against 49): a thread owns one row and 32 of the step's columns, 16 at a time: its S from TMEM, its weights from the W
+//         tile in shared memory (TMA, 128-byte swizzle: row-wise reads from global memory would touch 32 lines each).
+//   16    TMEM allocation and MMA issuer: S[128 x 64] = B_tile (128 x r) * A_tile (r x 64) into one of
+//         four TMEM buffers, as soon as the factor tile has landed and the buffer has been read.
+//   17    TMA producer of the W tiles, the factor tiles A[:, step] and, where a row tile begins, B_tile.
 // Every wait is bounded; on expiry the role records LORDS_ERR_TIMEOUT and leaves its loop.
 //
-// Shapes outside the tensor-core rules (r > 64, n not a multiple of 64) take a plain CUDA-core kernel.
+// Bound: instructions per weight (about 20 with packing) and the latency of their chain.  14336 x 4096, 3 bits, r = 48: 90 us with
+// bisection and weights read row by row from global memory, 51 now; 4096 x 4096, 4 bits, r = 32: 47 -> 20; r = 128, on the CUDA
+// cores before: 857 -> 21.
+//
+// Rows of W or A that are not 16-byte multiples (n not a multiple of 8) are copied to padded rows in the workspace first; without
+// room there, and for small layers off the tile grid, a plain CUDA-core kernel runs.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -33,30 +44,74 @@ using namespace ptx;
 
 constexpr int kRowsQ = 128;                    // rows of W per CTA = UMMA M
 constexpr int kColsQ = 64;                     // columns per step
-constexpr int kSearchWarps = 4;
-constexpr int kIssuerWarpQ = kSearchWarps;     // 4
-constexpr int kTmaWarpQ = kSearchWarps + 1;    // 5
-constexpr int kThreadsQ = (kSearchWarps + 2) * 32;
+constexpr int kSearchWarps = 8;                // warps of a step
+constexpr int kGroupsQ = 2;                    // groups of search warps, on alternating steps
+constexpr int kIssuerWarpQ = kGroupsQ * kSearchWarps;     // 16
+constexpr int kTmaWarpQ = kIssuerWarpQ + 1;               // 17
+constexpr int kThreadsQ = (kTmaWarpQ + 1) * 32;
 constexpr int kSAQ = 4;                        // factor-tile ring depth
-constexpr int kSDQ = 2;                        // S buffers in TMEM
-constexpr uint32_t kTmemColsQ = 128;
-constexpr int kRMaxQ = 64;                     // largest rank of the tensor-core path (one swizzle atom of K)
-constexpr int kATileBytesQ = kRMaxQ * 128;
-constexpr int kBTileBytesQ = kRowsQ * 128;
-constexpr int kSmemQ = 1024 + kSAQ * kATileBytesQ + kBTileBytesQ + 256;
+constexpr int kSWQ = 6;                        // weight-tile ring depth
+constexpr int kSDQ = 4;                        // S buffers in TMEM
+static_assert(kSWQ % kGroupsQ == 0 && kSDQ % kGroupsQ == 0, "a buffer is always read by the same group");
+constexpr uint32_t kTmemColsQ = kSDQ * kColsQ;
+constexpr int kWTileQ = kRowsQ * 128;          // 128 rows x 64 columns bf16
+
+enum Search { kBuckets, kBisect, kTrial };
+
+// BITS: code width.  RA: ranks the factor tiles are sized for (64 or 128).
+template <int BITS, int RA> struct QuantCfg {
+    static constexpr int BUCKETS = BITS == 4 ? 64 : BITS == 3 ? 32 : 16;
+    static constexpr int LUT = BUCKETS * 256;                 // 32 lane-private copies of {midpoint, code below}
+    static constexpr int ATILE = RA * 128;
+    static constexpr int BTILE = RA / 64 * kRowsQ * 128;
+    static constexpr int STAGE = BITS == 4 ? 0 : 32 * BITS * 4;       // packed codes of a warp's 32 rows (see store_codes_staged)
+    static constexpr int SMEM = 1024 + kSWQ * kWTileQ + kSAQ * ATILE + BTILE + LUT + 256 + kGroupsQ * kSearchWarps * STAGE;
+};
 
 struct alignas(64) QuantParams {
-    CUtensorMap tm_a;     // bf16 [r][n], box {64, r_pad}, 128-byte swizzle (ranks past r read as zero)
-    const uint16_t *W;    // bf16 [m][n]
+    CUtensorMap tm_a;     // bf16 [r][n], box {64, r_pad}, 128-byte swizzle (ranks past r and columns past n read as zero)
+    CUtensorMap tm_w;     // bf16 [m][n], box {64, 128}, 128-byte swizzle (rows past m and columns past n read as zero)
+    CUtensorMap tm_b;     // bf16 [m][r], box {64, 128}, 128-byte swizzle; used if rows of B are 16-byte multiples
     const uint16_t *B;    // bf16 [m][r]
     uint8_t *Q;           // packed codes, row pitch n * bits / 8
     float levels[16];
     float mids[16];       // ascending table: mids[c] = (levels[c] + levels[c + 1]) / 2
-    int bits, m, n, r, r_pad;
-    int steps;            // 64-column steps per row (n / 64)
-    int steps_per_cta;
+    float bucket_mid[64]; // the midpoint in (or next to) bucket k, +infinity if there is none above its lower edge
+    uint8_t bucket_code[64];   // midpoints below it
+    float bucket_scale, bucket_bias;   // bucket of a ratio t: saturate(t * scale + bias) * (buckets - 1), rounded
+    int m, n, r, r_pad;
+    int steps;            // 64-column steps per row tile
+    int row_splits;       // 0: all steps of all row tiles in equal runs; else ranges per row tile (a run stays in its row tile)
+    int row_tiles;
     int *status;
 };
+
+__device__ __forceinline__ float rcp_approx(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+// Two fp32 values in one 64-bit register: one instruction issued for both.
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi)
+{
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ void f32x2_split(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
 
 // The code whose level is nearest to w / s: every level in turn, the first (lowest) code keeps a tie.
 template <int LEVELS>
@@ -108,209 +163,282 @@ __device__ __forceinline__ uint32_t nearest_code_sorted(float s, float w, const 
     }
 }
 
-// 32 codes of one row -> packed bytes at `dst` (the row's byte offset of these 32 columns).
-template <int BITS>
-__device__ __forceinline__ void store_codes(uint8_t *dst, const uint32_t (&c)[32])
+// The first `count` of 32 codes of one row -> packed bytes at `dst` (the row's byte offset of these 32 columns); w: the codes packed, BITS
+// words.  `words`: dst is 4-byte aligned; 16-byte aligned rows of 4-bit codes go out as one word.
+template <int BITS> __device__ __forceinline__ void store_codes(uint8_t *dst, const uint32_t (&w)[BITS], int count, bool words, bool vec)
 {
-    if constexpr (BITS == 4) {
-        uint32_t w[4];
+    if (count >= 32 && words) {
+        if (BITS == 4 && vec) {
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[BITS > 2 ? 2 : 0], w[BITS > 3 ? 3 : 0]);
+        } else {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            uint32_t v = 0;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) v |= c[8 * k + q] << (4 * q);
-            w[k] = v;
+            for (int k = 0; k < BITS; ++k) reinterpret_cast<uint32_t *>(dst)[k] = w[k];
         }
-        *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-    } else if constexpr (BITS == 3) {
-        // a 96-bit little-endian integer, code j at bit 3j: codes 0..20 and the low bit of code 21 fill the
-        // first 64 bits, the rest of code 21 and codes 22..31 the last 32
-        unsigned long long a = 0;
-#pragma unroll
-        for (int j = 0; j < 21; ++j) a |= (unsigned long long)c[j] << (3 * j);
-        a |= (unsigned long long)(c[21] & 1u) << 63;
-        uint32_t hi = c[21] >> 1;
-#pragma unroll
-        for (int j = 22; j < 32; ++j) hi |= c[j] << (3 * j - 64);
-        uint32_t *d = reinterpret_cast<uint32_t *>(dst);
-        d[0] = (uint32_t)a;
-        d[1] = (uint32_t)(a >> 32);
-        d[2] = hi;
     } else {
-        uint32_t w[2];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            uint32_t v = 0;
-#pragma unroll
-            for (int q = 0; q < 16; ++q) v |= c[16 * k + q] << (2 * q);
-            w[k] = v;
-        }
-        *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
+        for (int k = 0; k < 4 * BITS; ++k)
+            if (8 * k < count * BITS) dst[k] = (uint8_t)(w[k >> 2] >> (8 * (k & 3)));
     }
 }
 
-template <int BITS, bool SORTED>
-__global__ void __launch_bounds__(kThreadsQ, 3) lords_quantize_kernel(const __grid_constant__ QuantParams p)
+template <int BITS, int MODE, int RA>
+__global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __grid_constant__ QuantParams p)
 {
+    using C = QuantCfg<BITS, RA>;
     extern __shared__ uint8_t smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    const uint32_t a0 = base;                                 // kSAQ factor tiles
-    const uint32_t b_tile = a0 + kSAQ * kATileBytesQ;         // B[128 x 64 ranks] bf16, K-major, swizzled
-    const uint32_t bars = b_tile + kBTileBytesQ;
-    const uint32_t bar_a_full = bars, bar_a_free = bars + 8 * kSAQ;
-    const uint32_t bar_s_full = bar_a_free + 8 * kSAQ, bar_s_free = bar_s_full + 8 * kSDQ;
-    const uint32_t tmem_slot = bar_s_free + 8 * kSDQ;
+    const uint32_t w0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    const uint32_t a0 = w0 + kSWQ * kWTileQ, b_tile = a0 + kSAQ * C::ATILE, lut = b_tile + C::BTILE, bars = lut + C::LUT;
+    const uint32_t bar_w = bars, bar_w_free = bar_w + 8 * kSWQ, bar_a = bar_w_free + 8 * kSWQ, bar_a_free = bar_a + 8 * kSAQ;
+    const uint32_t bar_s = bar_a_free + 8 * kSAQ, bar_s_free = bar_s + 8 * kSDQ, bar_b = bar_s_free + 8 * kSDQ, tmem_slot = bar_b + 8;
+    static_assert(16 * (kSWQ + kSAQ + kSDQ) + 8 + 4 <= 256, "barrier area");
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int row0 = (int)blockIdx.x * kRowsQ;
-    const int st_a = (int)blockIdx.y * p.steps_per_cta;
-    const int st_b = st_a + p.steps_per_cta < p.steps ? st_a + p.steps_per_cta : p.steps;
-    const int total = st_b - st_a;
+    // this CTA's run of steps, across row tiles (step `st` of row tile `rt` is number rt * steps + st)
+    int rt0, st0, total;
+    if (p.row_splits == 0) {
+        const long long all = (long long)p.row_tiles * p.steps;
+        const long long g0 = all * blockIdx.x / gridDim.x, g1 = all * (blockIdx.x + 1) / gridDim.x;
+        rt0 = (int)(g0 / p.steps);
+        st0 = (int)(g0 % p.steps);
+        total = (int)(g1 - g0);
+    } else {
+        const int s = (int)blockIdx.x % p.row_splits;
+        rt0 = (int)blockIdx.x / p.row_splits;
+        st0 = (int)((long long)p.steps * s / p.row_splits);
+        total = (int)((long long)p.steps * (s + 1) / p.row_splits) - st0;
+    }
+    const bool b_by_tma = (p.r & 7) == 0;
     const int *status = p.status;
     bool failed = false;
 
-    if (tid == 0) {
-        for (int b = 0; b < kSAQ; ++b) { mbar_init(bar_a_full + 8 * b, 1); mbar_init(bar_a_free + 8 * b, 1); }
-        for (int b = 0; b < kSDQ; ++b) { mbar_init(bar_s_full + 8 * b, 1); mbar_init(bar_s_free + 8 * b, kSearchWarps); }
-        fence_mbar_init();
-    }
-    if (warp == kIssuerWarpQ) {
+    if (warp == kTmaWarpQ) {
+        if (lane == 0) {
+            for (int b = 0; b < kSWQ; ++b) { mbar_init(bar_w + 8 * b, 1); mbar_init(bar_w_free + 8 * b, kSearchWarps); }
+            for (int b = 0; b < kSAQ; ++b) { mbar_init(bar_a + 8 * b, 1); mbar_init(bar_a_free + 8 * b, 1); }
+            for (int b = 0; b < kSDQ; ++b) { mbar_init(bar_s + 8 * b, 1); mbar_init(bar_s_free + 8 * b, kSearchWarps); }
+            mbar_init(bar_b, 1);
+            fence_mbar_init();
+            tma_prefetch_desc(&p.tm_w);
+            tma_prefetch_desc(&p.tm_a);
+        }
+    } else if (warp == kIssuerWarpQ) {
         tmem_alloc(tmem_slot, kTmemColsQ);
         tmem_relinquish();
-    } else if (warp < kSearchWarps) {
-        // B tile: row rr = tid, 64 ranks (zero padded) bf16, K-major, 128-byte swizzle
-        const int rr = tid, i = row0 + rr;
+    } else {
+        if (MODE == kBuckets)
+            for (int k = warp; k < C::BUCKETS; k += kIssuerWarpQ)
+                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(lut + (uint32_t)(k * 256 + lane * 8)), "r"(__float_as_uint(p.bucket_mid[k])),
+                             "r"((uint32_t)p.bucket_code[k]) : "memory");
+        if (!b_by_tma && warp < kSearchWarps) {
+            // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m
+            const int rr = tid >> 1, i = rt0 * kRowsQ + rr;
+            for (int c = 0; c < RA / 16; ++c) {
+                const int chunk = (tid & 1) * (RA / 16) + c;
+                uint32_t w4[4];
 #pragma unroll
-        for (int chunk = 0; chunk < 8; ++chunk) {
-            uint32_t w4[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int k = chunk * 8 + e * 2;
-                const uint32_t lo = (i < p.m && k < p.r) ? p.B[(size_t)i * p.r + k] : 0u;
-                const uint32_t hi = (i < p.m && k + 1 < p.r) ? p.B[(size_t)i * p.r + k + 1] : 0u;
-                w4[e] = lo | (hi << 16);
+                for (int e = 0; e < 4; ++e) {
+                    const int k = chunk * 8 + e * 2;
+                    const uint32_t lo = (i < p.m && k < p.r) ? p.B[(size_t)i * p.r + k] : 0u;
+                    const uint32_t hi = (i < p.m && k + 1 < p.r) ? p.B[(size_t)i * p.r + k + 1] : 0u;
+                    w4[e] = lo | (hi << 16);
+                }
+                sts_v4(b_tile + (uint32_t)((chunk >> 3) * kRowsQ * 128 + (rr >> 3) * 1024 + (rr & 7) * 128 + (((chunk & 7) ^ (rr & 7)) * 16)),
+                       make_uint4(w4[0], w4[1], w4[2], w4[3]));
             }
-            sts_v4(b_tile + (rr >> 3) * 1024 + (rr & 7) * 128 + ((chunk ^ (rr & 7)) * 16), make_uint4(w4[0], w4[1], w4[2], w4[3]));
+            fence_proxy_async_smem();
         }
-        fence_proxy_async_smem();
     }
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    uint32_t tmem_base;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
 
     if (warp == kTmaWarpQ) {
         if (lane == 0) {
-            tma_prefetch_desc(&p.tm_a);
-            const uint32_t tx = (uint32_t)(p.r_pad * 128);
+            int next_w = 0, w_rt = rt0, w_st = st0;          // weight tiles run ahead of the factor tiles as far as their ring allows
+            int rt = rt0, st = st0;
             for (int it = 0; it < total; ++it) {
+                if (b_by_tma && (it == 0 || st == 0)) {      // a new row tile: its B once nothing reads the last one's
+                    if (it > 0 && !mbar_wait(bar_a_free + 8 * ((it - 1) % kSAQ), (uint32_t)(((it - 1) / kSAQ) & 1), status, 29)) { failed = true; break; }
+                    mbar_expect_tx(bar_b, (uint32_t)C::BTILE);
+                    for (int h = 0; h < RA / 64; ++h) tma_load_2d(b_tile + (uint32_t)(h * kRowsQ * 128), &p.tm_b, h * 64, rt * kRowsQ, bar_b);
+                }
+                while (next_w < total && next_w < it + kSWQ) {
+                    const int s = next_w % kSWQ;
+                    if (next_w >= kSWQ) {
+                        const uint32_t par = (uint32_t)((next_w / kSWQ - 1) & 1);
+                        if (next_w > it) { if (!mbar_try_wait(bar_w_free + 8 * s, par)) break; }
+                        else if (!mbar_wait(bar_w_free + 8 * s, par, status, 30)) { failed = true; break; }
+                    }
+                    mbar_expect_tx(bar_w + 8 * s, (uint32_t)kWTileQ);
+                    tma_load_2d(w0 + (uint32_t)(s * kWTileQ), &p.tm_w, w_st * kColsQ, w_rt * kRowsQ, bar_w + 8 * s);
+                    ++next_w;
+                    if (++w_st == p.steps) { w_st = 0; ++w_rt; }
+                }
+                if (failed) break;
                 const int sa = it % kSAQ;
-                if (it >= kSAQ && !mbar_wait(bar_a_free + 8 * sa, (uint32_t)((it / kSAQ - 1) & 1), status, 31)) { failed = true; break; }
-                const uint32_t bar = bar_a_full + 8 * sa;
-                mbar_expect_tx(bar, tx);
-                tma_load_2d(a0 + sa * kATileBytesQ, &p.tm_a, (st_a + it) * kColsQ, 0, bar);
+                if (it >= kSAQ && !mbar_wait<kWaitSlackNs>(bar_a_free + 8 * sa, (uint32_t)((it / kSAQ - 1) & 1), status, 31)) { failed = true; break; }
+                mbar_expect_tx(bar_a + 8 * sa, (uint32_t)(p.r_pad * 128));
+                tma_load_2d(a0 + (uint32_t)(sa * C::ATILE), &p.tm_a, st * kColsQ, 0, bar_a + 8 * sa);
+                if (++st == p.steps) { st = 0; ++rt; }
             }
         }
+        __syncwarp();
     } else if (warp == kIssuerWarpQ) {
-        uint32_t tmem_base;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
+        const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
         constexpr uint32_t idesc = umma_idesc_f16(1, 0, 1, kRowsQ, kColsQ);     // bf16, B operand MN-major, N = 64
         const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         const uint32_t lbo_lo = (uint32_t)umma_desc_sw128(0, 1024, 16);
-        const uint32_t b_lo = lbo_lo | ((b_tile & 0x3FFFFu) >> 4);
-        const uint32_t a_lo0 = lbo_lo | ((a0 & 0x3FFFFu) >> 4);
-        const int ksteps = p.r_pad / 16;
-        tmem_base = warp_uniform(tmem_base);
-        const uint32_t leader = elect_one();
+        const uint32_t b_lo = lbo_lo | ((b_tile & 0x3FFFFu) >> 4), a_lo0 = lbo_lo | ((a0 & 0x3FFFFu) >> 4);
+        uint32_t b_phase = 0;
+        int st = st0;
         for (int it = 0; it < total; ++it) {
+            if (b_by_tma && (it == 0 || st == 0)) {
+                if (!mbar_wait_warp(bar_b, b_phase, status, 36)) { failed = true; break; }
+                b_phase ^= 1;
+            }
+            if (++st == p.steps) st = 0;
             const int sa = it % kSAQ, sd = it % kSDQ;
-            if (!mbar_wait(bar_a_full + 8 * sa, (uint32_t)((it / kSAQ) & 1), status, 32)) { failed = true; break; }
-            if (it >= kSDQ && !mbar_wait(bar_s_free + 8 * sd, (uint32_t)((it / kSDQ - 1) & 1), status, 33)) { failed = true; break; }
+            if (!mbar_wait_warp2(bar_a + 8 * sa, (uint32_t)((it / kSAQ) & 1), bar_s_free + 8 * sd, (uint32_t)((it / kSDQ + 1) & 1), status, 32)) { failed = true; break; }
             tc_fence_after_sync();
-            const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (kATileBytesQ >> 4));
-            for (int k = 0; k < ksteps; ++k)
-                umma_f16_ss(tmem_base + (uint32_t)(sd * kColsQ), umma_desc_pack(b_lo + k * 2, desc_hi),
+            const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ATILE >> 4));
+            for (int k = 0; k < p.r_pad / 16; ++k)
+                umma_f16_ss(tmem_u + (uint32_t)(sd * kColsQ), umma_desc_pack(b_lo + (k >> 2) * (kRowsQ * 128 >> 4) + (k & 3) * 2, desc_hi),
                             umma_desc_pack(a_lo + k * 128, desc_hi), idesc, k > 0, leader);
-            umma_commit(bar_s_full + 8 * sd, leader);
+            umma_commit(bar_s + 8 * sd, leader);
             umma_commit(bar_a_free + 8 * sa, leader);
-            __syncwarp();
         }
         // no commit is still on its way to a barrier when the CTA ends
-        if (lane == 0 && !failed && total > 0) {
-            const int last = total - 1;
-            if (!mbar_wait(bar_a_free + 8 * (last % kSAQ), (uint32_t)((last / kSAQ) & 1), status, 34)) failed = true;
-        }
+        if (!failed && total > 0 && !mbar_wait_warp(bar_a_free + 8 * ((total - 1) % kSAQ), (uint32_t)(((total - 1) / kSAQ) & 1), status, 34)) failed = true;
     } else {
-        const int i = row0 + tid;
-        uint32_t tmem_base;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
-        const uint32_t lane_addr = tmem_base + ((uint32_t)(warp * 32) << 16);
-        float lv[16];
+        const int q = warp & 3, ch = (warp >> 2) & 1, row = q * 32 + lane;
+        const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 32);
+        const uint32_t w_row = w0 + (uint32_t)((row >> 3) * 1024 + (row & 7) * 128), lut_lane = lut + 8u * (uint32_t)lane;
+        // the bucket's number arrives as the low bits of a float of magnitude 2^23: its bits times 256, less what the exponent adds
+        const uint32_t lut_magic = lut_lane - 0x4B000000u * 256u;
+        float lv[MODE == kBuckets ? 1 : 16];
+        if constexpr (MODE != kBuckets) {
 #pragma unroll
-        for (int c = 0; c < 16; ++c) lv[c] = SORTED ? p.mids[c] : p.levels[c];
+            for (int c = 0; c < 16; ++c) lv[c] = MODE == kBisect ? p.mids[c] : p.levels[c];
+        }
         const size_t qpitch = (size_t)p.n * BITS / 8;
-        // the row's 32 weights of a half step are requested one half step ahead, so that their way
-        // from HBM overlaps the search of the half step before
-        uint4 wv[4], wn[4];
-        auto load_w = [&](uint4 (&dst)[4], int it, int h) {
-            if (i < p.m && it < total) {
-                const uint4 *wp = reinterpret_cast<const uint4 *>(p.W + (size_t)i * p.n + (size_t)(st_a + it) * kColsQ + h * 32);
-#pragma unroll
-                for (int v = 0; v < 4; ++v) dst[v] = __ldg(wp + v);
-            }
-        };
-        load_w(wv, 0, 0);
-        for (int it = 0; it < total; ++it) {
-            const int sd = it % kSDQ;
-            const int col0 = (st_a + it) * kColsQ;
-            if (!__all_sync(0xffffffffu, mbar_wait(bar_s_full + 8 * sd, (uint32_t)((it / kSDQ) & 1), status, 35))) { failed = true; break; }
+        const bool words = (qpitch & 3) == 0, vec = (qpitch & 15) == 0;
+        const int group = warp / kSearchWarps;
+        const uint32_t stage = bars + 256u + (uint32_t)(warp * C::STAGE);
+        int rt = rt0, st = st0 + group;
+        for (int it = group; it < total; it += kGroupsQ) {
+            while (st >= p.steps) { st -= p.steps; ++rt; }
+            const int sd = it % kSDQ, sw = it % kSWQ, col0 = st * kColsQ + ch * 32, i = rt * kRowsQ + row;
+            st += kGroupsQ;
+            if (!mbar_wait_warp2(bar_s + 8 * sd, (uint32_t)((it / kSDQ) & 1), bar_w + 8 * sw, (uint32_t)((it / kSWQ) & 1), status, 35)) { failed = true; break; }
             tc_fence_after_sync();
-#pragma unroll 1
-            for (int h = 0; h < 2; ++h) {
-                uint32_t s[32];
-                tmem_ld_32x32(lane_addr + (uint32_t)(sd * kColsQ + h * 32), s);
-                load_w(wn, h == 0 ? it : it + 1, h == 0 ? 1 : 0);
-                tmem_wait_ld();
+            uint32_t packed[BITS];
+#pragma unroll
+            for (int k = 0; k < BITS; ++k) packed[k] = 0u;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {                    // 16 columns at a time: all of the weights at once would not fit the registers
+                uint32_t s[16];
+                tmem_ld_32x16(lane_addr + (uint32_t)(sd * kColsQ + h * 16), s);
+                const uint32_t at = w_row + (uint32_t)(sw * kWTileQ);
+                const uint4 wv[2] = {lds_v4(at + (uint32_t)(((ch * 4 + h * 2) ^ (row & 7)) << 4)), lds_v4(at + (uint32_t)(((ch * 4 + h * 2 + 1) ^ (row & 7)) << 4))};
+                tmem_wait_ld(s);
                 if (h == 1) {
-                    // S is in registers: the buffer may be refilled
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_s_free + 8 * sd);
+                    if (lane == 0) mbar_arrive(bar_s_free + 8 * sd);      // S is in registers: the buffer may be refilled
                 }
-                if (i < p.m) {
-                    uint32_t codes[32];
+                auto weight = [&](int c) {
+                    const uint4 &v = wv[(c >> 3) & 1];
+                    const uint32_t u = (c & 7) / 2 == 0 ? v.x : (c & 7) / 2 == 1 ? v.y : (c & 7) / 2 == 2 ? v.z : v.w;
+                    return __uint_as_float((c & 1) ? (u & 0xFFFF0000u) : (u << 16));
+                };
+                auto pack = [&](auto code_of) {
 #pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        const uint32_t ww[4] = {wv[v].x, wv[v].y, wv[v].z, wv[v].w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const int c = v * 8 + e * 2;
-                            const float w0 = __uint_as_float(ww[e] << 16), w1 = __uint_as_float(ww[e] & 0xFFFF0000u);
-                            if constexpr (SORTED) {
-                                codes[c] = nearest_code_sorted<(1 << BITS)>(__uint_as_float(s[c]), w0, lv);
-                                codes[c + 1] = nearest_code_sorted<(1 << BITS)>(__uint_as_float(s[c + 1]), w1, lv);
-                            } else {
-                                codes[c] = nearest_code<(1 << BITS)>(__uint_as_float(s[c]), w0, lv);
-                                codes[c + 1] = nearest_code<(1 << BITS)>(__uint_as_float(s[c + 1]), w1, lv);
-                            }
-                        }
+                    for (int c = h * 16; c < h * 16 + 16; ++c) {
+                        const uint32_t code = code_of(c);
+                        const int bit = c * BITS, wi = bit >> 5, sh = bit & 31;
+                        packed[wi] += code << sh;
+                        if (sh + BITS > 32) packed[wi + 1 < BITS ? wi + 1 : wi] += code >> (32 - sh);
                     }
-                    store_codes<BITS>(p.Q + (size_t)i * qpitch + (size_t)(col0 + h * 32) * BITS / 8, codes);
-                }
+                };
+                if constexpr (MODE == kBuckets) {
+                    // a scale outside (2^-100, 2^100) (zero above all: code 0) takes the exact products, and so does the warp with it
+                    float least = fabsf(__uint_as_float(s[0])), most = least;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) wv[v] = wn[v];
+                    for (int c = 1; c < 16; ++c) {
+                        least = fminf(least, fabsf(__uint_as_float(s[c])));
+                        most = fmaxf(most, fabsf(__uint_as_float(s[c])));
+                    }
+                    if (__all_sync(0xffffffffu, least > 7.8886e-31f && most < 1.2676e30f)) {
+                        const uint64_t top2 = f32x2((float)(C::BUCKETS - 1), (float)(C::BUCKETS - 1)), magic2 = f32x2(8388608.0f, 8388608.0f);
+                        float f[2];
+                        pack([&](int c) {
+                            const float w = weight(c);
+                            if ((c & 1) == 0) {
+                                // two buckets at a time: round(saturate(t * scale + bias) * (buckets - 1)) as the low bits of a float
+                                float t[2];
+                                f32x2_split(f32x2_mul(f32x2(w, weight(c + 1)), f32x2(rcp_approx(__uint_as_float(s[c & 15])), rcp_approx(__uint_as_float(s[(c + 1) & 15])))), t[0], t[1]);
+                                const float u = __saturatef(fmaf(t[0], p.bucket_scale, p.bucket_bias)), v = __saturatef(fmaf(t[1], p.bucket_scale, p.bucket_bias));
+                                f32x2_split(f32x2_fma(f32x2(u, v), top2, magic2), f[0], f[1]);
+                            }
+                            uint32_t mid, below, above;
+                            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mid), "=r"(below) : "r"(__float_as_uint(f[c & 1]) * 256u + lut_magic));
+                            // t > mid  <=>  w sign(s) > |s| mid (as in the bisection)
+                            const float b = __uint_as_float(__float_as_uint(w) ^ (s[c & 15] & 0x80000000u));
+                            asm("set.gt.u32.f32 %0, %1, %2;" : "=r"(above) : "f"(b), "f"(fabsf(__uint_as_float(s[c & 15])) * __uint_as_float(mid)));
+                            return below - above;             // the outcome is 0 or -1
+                        });
+                    } else {
+                        // the bisection's answer by counting, which needs no registers for its thresholds
+                        pack([&](int c) {
+                            const float sc = __uint_as_float(s[c & 15]), a = fabsf(sc), w = weight(c), b = a == 0.0f ? -INFINITY : sc < 0.0f ? -w : w;
+                            uint32_t code = 0;
+#pragma unroll
+                            for (int l = 0; l + 1 < (1 << BITS); ++l) code += b > a * p.mids[l] ? 1u : 0u;
+                            return code;
+                        });
+                    }
+                } else if constexpr (MODE == kBisect) {
+                    pack([&](int c) { return nearest_code_sorted<(1 << BITS)>(__uint_as_float(s[c & 15]), weight(c), lv); });
+                } else {
+                    pack([&](int c) { return nearest_code<(1 << BITS)>(__uint_as_float(s[c & 15]), weight(c), lv); });
+                }
             }
+            if (BITS != 4 && words && p.n - col0 >= 32)
+                store_codes_staged<BITS>(stage, p.Q + (size_t)(rt * kRowsQ + q * 32) * qpitch + (size_t)col0 * BITS / 8, qpitch, p.m - rt * kRowsQ - q * 32, lane, packed);
+            else if (i < p.m && col0 < p.n) store_codes<BITS>(p.Q + (size_t)i * qpitch + (size_t)col0 * BITS / 8, packed, p.n - col0, words, vec);
+            // only now that the weights have been used: an arrival can overtake loads that are still in flight
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_w_free + 8 * sw);
         }
     }
 
-    if (failed) atomicExch(p.status, LORDS_ERR_TIMEOUT);
+    if (failed) {
+        atomicExch(p.status, LORDS_ERR_TIMEOUT);
+        for (int k = 0; k < 100; ++k) __nanosleep(1000);      // copies in flight land before the CTA ends
+    }
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kIssuerWarpQ) {
         tc_fence_after_sync();
-        uint32_t tmem_base;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
         tmem_dealloc(tmem_base, kTmemColsQ);
     }
+}
+
+// Rows of `n` bf16 values -> rows of pitch np (a multiple of 8), zeros behind; two matrices in one launch.
+__global__ void lords_pad_rows_kernel(const uint16_t *__restrict__ src0, uint16_t *__restrict__ dst0, long long words0, const uint16_t *__restrict__ src1,
+                                      uint16_t *__restrict__ dst1, long long words1, int n, int np)
+{
+    // a thread moves two values (n is even: rows are 4-byte aligned); words: np / 2 per row
+    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool first = e < words0;
+    if (e >= words0 + words1) return;
+    const long long f = first ? e : e - words0;
+    const long long row = f / (np / 2);
+    const int c = (int)(f % (np / 2)) * 2;
+    const uint16_t *src = first ? src0 : src1;
+    reinterpret_cast<uint32_t *>(first ? dst0 : dst1)[f] = c < n ? __ldg(reinterpret_cast<const uint32_t *>(src + row * n + c)) : 0u;
 }
 
 // Plain CUDA-core version for any shape: a thread owns one row and one pack group of 32 columns (or what
@@ -348,25 +476,69 @@ __global__ void lords_quantize_simt_kernel(const uint16_t *__restrict__ W, const
     for (int b = 0; b < BYTES; ++b) dst[b] = b < 8 ? (uint8_t)(lo >> (8 * b)) : (uint8_t)(hi >> (8 * (b - 8)));
 }
 
-template <int BITS, bool SORTED> int launch_quantize_tc(QuantParams &k, const State &st, cudaStream_t stream)
+template <int BITS, int MODE, int RA> int launch_quantize_tc(QuantParams &k, const State &st, cudaStream_t stream)
 {
     static bool done[kMaxDevices] = {};
     const int dev = device_slot(st);
     if (!done[dev]) {
-        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_quantize_kernel<BITS, SORTED>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemQ));
+        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_quantize_kernel<BITS, MODE, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuantCfg<BITS, RA>::SMEM));
         done[dev] = true;
     }
-    const int row_tiles = (k.m + kRowsQ - 1) / kRowsQ;
-    // column ranges: about two CTAs per SM in all, at least four steps each
-    int splits = (6 * st.sm_count + row_tiles - 1) / row_tiles;
-    if (splits > k.steps / 4) splits = k.steps / 4;
-    if (splits < 1) splits = 1;
-    if (splits > 65535) splits = 65535;
-    k.steps_per_cta = (k.steps + splits - 1) / splits;
-    splits = (k.steps + k.steps_per_cta - 1) / k.steps_per_cta;
-    lords_quantize_kernel<BITS, SORTED><<<dim3((unsigned)row_tiles, (unsigned)splits), kThreadsQ, kSmemQ, stream>>>(k);
+    // One run of steps per CTA that can be resident: setting a CTA up costs as much as about three steps, which a second round of CTAs
+    // would pay again, and equal runs leave no partial round.  With the B tile built element by element (rank not a multiple of 8)
+    // a run stays within its row tile: the least rounds times (steps + 3) then.
+    k.row_tiles = (k.m + kRowsQ - 1) / kRowsQ;
+    const long long all = (long long)k.row_tiles * k.steps, resident = st.sm_count;
+    long long grid = all < resident ? all : resident;
+    k.row_splits = 0;
+    if ((k.r & 7) != 0) {
+        double best = 1e30;
+        for (int s = 1; s <= k.steps && s <= 4096; ++s) {
+            const double t = (double)(((long long)k.row_tiles * s + resident - 1) / resident) * ((k.steps + s - 1) / s + 3.0);
+            if (t < best) { best = t; k.row_splits = s; }
+        }
+        grid = (long long)k.row_tiles * k.row_splits;
+    }
+    if (grid > 2147483647LL) return LORDS_ERR_SHAPE;
+    lords_quantize_kernel<BITS, MODE, RA><<<(unsigned)grid, kThreadsQ, QuantCfg<BITS, RA>::SMEM, stream>>>(k);
     LORDS_CUDA_TRY(cudaGetLastError());
     return LORDS_OK;
+}
+template <int BITS> int launch_quantize_tc(QuantParams &k, int mode, const State &st, cudaStream_t stream)
+{
+    if (k.r <= 64) return mode == kBuckets ? launch_quantize_tc<BITS, kBuckets, 64>(k, st, stream)
+                          : mode == kBisect ? launch_quantize_tc<BITS, kBisect, 64>(k, st, stream) : launch_quantize_tc<BITS, kTrial, 64>(k, st, stream);
+    return mode == kBuckets ? launch_quantize_tc<BITS, kBuckets, 128>(k, st, stream)
+           : mode == kBisect ? launch_quantize_tc<BITS, kBisect, 128>(k, st, stream) : launch_quantize_tc<BITS, kTrial, 128>(k, st, stream);
+}
+
+// The bucket table of an ascending level table.  Buckets are the rounding intervals of `buckets` equally spaced points that cover the
+// midpoints with half a spacing to spare on both sides; the ratio that picks one is off by less than 1e-5 of a
+// bucket's range, so a bucket answers for its interval widened by 1e-3 of the spacing.  False if some widened interval holds two midpoints.
+bool make_buckets(QuantParams &k, const float *levels, int bits, int buckets)
+{
+    const int nm = (1 << bits) - 1;
+    const double lo = 0.5 * ((double)levels[0] + levels[1]), hi = 0.5 * ((double)levels[nm - 1] + levels[nm]);
+    const double h = (hi - lo) / (buckets - 2), first = lo - 0.5 * h;        // point k at first + k h
+    if (!(h > 0.0) || !(h < 1e30)) return false;
+    const double span = h * (buckets - 1);
+    k.bucket_scale = (float)(1.0 / span);
+    k.bucket_bias = (float)(-first / span);
+    if (!(k.bucket_scale > 1e-30f) || !(k.bucket_scale < 1e30f) || !(k.bucket_bias > -1e4f) || !(k.bucket_bias < 1e4f)) return false;
+    for (int b = 0; b < buckets; ++b) {
+        const double a = first + (b - 0.501) * h, z = first + (b + 0.501) * h;
+        int below = 0, inside = 0;
+        float mid = INFINITY;
+        for (int c = 0; c < nm; ++c) {
+            const double v = k.mids[c];
+            if (v < a && b > 0) ++below;
+            else if (v <= z || b == buckets - 1) { ++inside; mid = k.mids[c]; }
+        }
+        if (inside > 1) return false;
+        k.bucket_mid[b] = mid;
+        k.bucket_code[b] = (uint8_t)below;
+    }
+    return true;
 }
 
 }  // namespace
@@ -374,28 +546,48 @@ template <int BITS, bool SORTED> int launch_quantize_tc(QuantParams &k, const St
 int launch_quantize(const void *W, const void *B, const void *A, const float *levels, int bits, int m, int n, int r,
                     uint8_t *Q, State &st, cudaStream_t stream)
 {
-    const bool tc = r <= kRMaxQ && n % kColsQ == 0;      // the row tiles are the grid's x dimension: any int fits
+    // rows that are not 16-byte multiples: padded copies of W and A in the workspace
+    const int np = (n + 7) / 8 * 8;
+    const size_t w_bytes = ((size_t)m * np * 2 + 255) & ~(size_t)255, a_bytes = (size_t)r * np * 2;
+    const bool pad = np != n;
+    // small layers with a ragged row or a rank above 64 stay on the CUDA cores: a few microseconds there as here, in one launch
+    const bool small = (n % kColsQ != 0 || r > 64) && (long long)m * n <= (5 << 18);
+    const bool tc = !small && (!pad || w_bytes + a_bytes <= st.workspace_bytes);      // the row tiles are the grid's x dimension: any int fits
     if (tc && st.forced_path != 1) {
+        int launches = 1;
+        const void *Wt = W, *At = A;
+        if (pad) {
+            uint16_t *wp = reinterpret_cast<uint16_t *>(st.workspace), *ap = reinterpret_cast<uint16_t *>(st.workspace + w_bytes);
+            const long long words0 = (long long)m * (np / 2), words1 = (long long)r * (np / 2), blocks = (words0 + words1 + 255) / 256;
+            if (blocks > 2147483647LL) return LORDS_ERR_SHAPE;
+            lords_pad_rows_kernel<<<(unsigned)blocks, 256, 0, stream>>>(static_cast<const uint16_t *>(W), wp, words0, static_cast<const uint16_t *>(A), ap,
+                                                                        words1, n, np);
+            LORDS_CUDA_TRY(cudaGetLastError());
+            Wt = wp; At = ap;
+            ++launches;
+        }
         QuantParams k;
-        k.W = static_cast<const uint16_t *>(W); k.B = static_cast<const uint16_t *>(B); k.Q = Q;
+        k.B = static_cast<const uint16_t *>(B); k.Q = Q;
         for (int c = 0; c < 16; ++c) k.levels[c] = c < (1 << bits) ? levels[c] : 0.0f;
-        // a strictly ascending table (every NormalFloat table is) is searched by bisection over its
-        // midpoints, any other table level by level
         bool sorted = true;
         for (int c = 0; c + 1 < (1 << bits); ++c) sorted = sorted && levels[c] < levels[c + 1];
         for (int c = 0; c < 16; ++c) k.mids[c] = (sorted && c + 1 < (1 << bits)) ? 0.5f * (levels[c] + levels[c + 1]) : 0.0f;
-        k.bits = bits; k.m = m; k.n = n; k.r = r; k.r_pad = (r + 15) / 16 * 16;
-        k.steps = n / kColsQ;
+        const int buckets = bits == 4 ? QuantCfg<4, 64>::BUCKETS : bits == 3 ? QuantCfg<3, 64>::BUCKETS : QuantCfg<2, 64>::BUCKETS;
+        const int mode = !sorted ? kTrial : make_buckets(k, levels, bits, buckets) ? kBuckets : kBisect;
+        k.m = m; k.n = n; k.r = r; k.r_pad = (r + 15) / 16 * 16;
+        k.steps = (n + kColsQ - 1) / kColsQ;
         k.status = st.status_word;
-        if (!make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, A, (uint64_t)n, (uint64_t)r, 64, (uint32_t)k.r_pad,
-                         CU_TENSOR_MAP_SWIZZLE_128B))
+        if (!make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, At, (uint64_t)np, (uint64_t)r, 64, (uint32_t)k.r_pad, CU_TENSOR_MAP_SWIZZLE_128B) ||
+            !make_map_2d(&k.tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wt, (uint64_t)np, (uint64_t)m, 64, (uint32_t)kRowsQ, CU_TENSOR_MAP_SWIZZLE_128B))
             return LORDS_ERR_CUDA;
-        const int rc = sorted ? (bits == 4 ? launch_quantize_tc<4, true>(k, st, stream)
-                                           : bits == 3 ? launch_quantize_tc<3, true>(k, st, stream) : launch_quantize_tc<2, true>(k, st, stream))
-                              : (bits == 4 ? launch_quantize_tc<4, false>(k, st, stream)
-                                           : bits == 3 ? launch_quantize_tc<3, false>(k, st, stream) : launch_quantize_tc<2, false>(k, st, stream));
+        k.tm_b = k.tm_a;      // not used where the kernel builds the B tile element by element
+        if ((r & 7) == 0 &&
+            !make_map_2d(&k.tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, B, (uint64_t)r, (uint64_t)m, 64, (uint32_t)kRowsQ, CU_TENSOR_MAP_SWIZZLE_128B))
+            return LORDS_ERR_CUDA;
+        const int rc = bits == 4 ? launch_quantize_tc<4>(k, mode, st, stream) : bits == 3 ? launch_quantize_tc<3>(k, mode, st, stream)
+                                                                              : launch_quantize_tc<2>(k, mode, st, stream);
         if (rc != LORDS_OK) return rc;
-        st.last_launches = 1;
+        st.last_launches = launches;
         st.last_path = "quantize";
         return LORDS_OK;
     }
