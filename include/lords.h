@@ -316,7 +316,8 @@ int lords_last_cuda_error(void);
 /*
  * Measurement switches.  Keys: "path" = "auto" | "simt" | "decode" (reassociated-form kernel,
  * M <= 2) | "decode16" (scale-MMA form with 128-column k-steps, 3 <= M <= 16) | "umma" (scale-MMA
- * kernel for any M; "prefill" is an alias) | "dense" (weights expanded to fp16 scratch, then a dense product; any shape) | "direct" (weights formed in registers; M <= 128) | "wide" (M <= 16, 64 < r <= 128);
+ * kernel for any M; "prefill" is an alias) | "dense" (weights expanded to fp16 scratch, then a dense product; any shape) | "direct" (weights formed in registers; M <= 128) | "wide" (M <= 16, 64 < r <= 128)
+ * | "pair" (the scale-MMA kernel on CTA pairs, which "umma" and "auto" use for large calls; reports "umma");
  * "splitk" = "0" (auto) or a positive integer (CTAs sharing one tile's k-range); "bn" = "0" (auto)
  * or the token tile 32, 64, 128, 256 of the scale-MMA kernel for M > 16; "inject_status" = "0" or a
  * negative status code: writes that value into the device status word, as a kernel that gave up would

@@ -21,6 +21,7 @@
 #include <cuda_fp16.h>
 
 #include "lords_internal.h"
+#include "lords_pair.cuh"
 #include "lords_ptx.cuh"
 #include "lords_tc_common.cuh"
 #include "lords_warp_mma.cuh"
@@ -263,84 +264,10 @@ struct alignas(64) GemmParams {
     int pairs;            // CTA pairs launched
     int whole;            // tiles [0, whole) run unsplit, one per pair and wave; the k-steps of the rest are dealt out evenly
     float *partial;       // [pair][2][BN][128]: a piece that does not begin its tile
-    int *flags;           // [pair][2]: the piece is in scratch; zero between calls
+    int *flags;           // [pair][2]: warps that have put their part of the piece into scratch; zero between calls
     void *y;
     int y_f32;
     int *status;
-};
-
-__device__ __forceinline__ void tmem_alloc2(uint32_t smem_result, uint32_t cols)
-{
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_result), "r"(cols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t cols)
-{
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
-}
-// D[both CTAs' TMEM] (+)= A * B, operands in both CTAs' shared memory at the same offsets; one thread of the even CTA.
-__device__ __forceinline__ void umma2_f16_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate, uint32_t leader)
-{
-    asm volatile(
-        "{\n"
-        ".reg .pred p, q;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "setp.ne.b32 q, %5, 0;\n"
-        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(leader)
-        : "memory");
-}
-// Arrive once on the barrier at this offset in both CTAs when every MMA issued so far has completed.
-__device__ __forceinline__ void umma2_commit(uint32_t bar, uint32_t leader)
-{
-    asm volatile(
-        "{\n"
-        ".reg .pred q;\n"
-        "setp.ne.b32 q, %2, 0;\n"
-        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n"
-        "}\n" ::"r"(bar), "h"((uint16_t)3), "r"(leader)
-        : "memory");
-}
-// A load into this CTA whose bytes are counted on a barrier of the pair's even CTA.
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const void *tmap, int x, int y, uint32_t cluster_bar)
-{
-    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 ::"r"(dst), "l"(tmap), "r"(cluster_bar), "r"(x), "r"(y) : "memory");
-}
-
-// One piece of work of a pair: k-steps [k0, k1) of a tile.
-struct Piece {
-    int tile, k0, k1;
-};
-
-// The pieces of pair `pair`, in order: its tiles of the whole waves, then its share of the k-steps of the tiles left over.  The
-// share may begin inside a tile (that piece goes to scratch) and end inside one (the pair that begins a
-// tile finishes it: it adds the other pieces, which their pairs do first).
-struct Schedule {
-    int next_whole, pairs, whole, ksteps;
-    long long at, end;
-    __device__ __forceinline__ Schedule(const GemmParams &p, int pair) : next_whole(pair), pairs(p.pairs), whole(p.whole), ksteps(p.ksteps)
-    {
-        const long long left = (long long)(p.tiles - p.whole) * p.ksteps;
-        at = pair * left / pairs;
-        end = (pair + 1) * left / pairs;
-    }
-    __device__ __forceinline__ bool next(Piece &w)
-    {
-        if (next_whole < whole) {
-            w.tile = next_whole; w.k0 = 0; w.k1 = ksteps;
-            next_whole += pairs;
-            return true;
-        }
-        if (at >= end) return false;
-        const int tt = (int)(at / ksteps);
-        w.tile = whole + tt;
-        w.k0 = (int)(at - (long long)tt * ksteps);
-        const long long stop = (long long)(tt + 1) * ksteps < end ? (long long)(tt + 1) * ksteps : end;
-        w.k1 = w.k0 + (int)(stop - at);
-        at = stop;
-        return true;
-    }
 };
 
 template <int BN>
@@ -383,7 +310,7 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
     griddep_launch_dependents();
     griddep_wait();                                                           // W^ and the fp16 activations are the previous launch's
 
-    Schedule sched(p, pair);
+    Schedule sched(p.pairs, p.whole, p.tiles, p.ksteps, pair);
     Piece w;
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA: this CTA's rows and its half of the tokens
@@ -460,7 +387,7 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
                                 for (unsigned tries = 0;; ++tries) {
                                     int v;
                                     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-                                    if (v != 0) return true;
+                                    if (v >= kGEpiWarps) return true;
                                     __nanosleep(kWaitSleepNs);
                                     if ((tries & 63u) == 63u && wait_limit_expired(limit, status, (uint32_t)o, 0, 56)) return false;
                                 }
@@ -512,15 +439,7 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(empty0 + 8 * buf);
-            if (to_scratch) {
-                __threadfence();
-                asm volatile("bar.sync 2, %0;" ::"n"(kGEpiWarps * 32) : "memory");
-                if (tid == kGEpiWarp0 * 32) asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p.flags + 2 * pair + rank), "r"(1) : "memory");
-            } else if (others > 0) {
-                asm volatile("bar.sync 2, %0;" ::"n"(kGEpiWarps * 32) : "memory");       // every warp has read the other pieces
-                if (tid == kGEpiWarp0 * 32)
-                    for (int o = pair + 1; o <= pair + others; ++o) p.flags[2 * o + rank] = 0;
-            }
+            piece_done(p.flags, pair, rank, others, to_scratch, kGEpiWarps, lane);
             ++done;
         }
     }
@@ -620,7 +539,7 @@ template <int BN> int launch_product(GemmParams &k, const void *w16, const void 
     if (pairs > 4LL * k.tiles) pairs = 4LL * k.tiles;
     if (pairs > pairs_max) pairs = pairs_max;
     k.pairs = (int)pairs;
-    k.whole = (int)(k.tiles / k.pairs * k.pairs);
+    k.whole = whole_tiles(k.tiles, k.pairs);
     if (!make_map_2d(&k.tm_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, w16, (uint64_t)np, (uint64_t)k.rows, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, x16, (uint64_t)np, (uint64_t)k.M, 64, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;

@@ -162,6 +162,7 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
         case 5: return launch_dense(p, st, s);
         case 6: return launch_direct(p, st, s);
         case 7: return launch_wide(p, st, s);
+        case 8: return launch_umma_pair(p, st, s);
         default: break;
     }
     const long long weights = (long long)p.m * p.n, grouped = (p.M + 15) / 16 * weights;
@@ -652,6 +653,7 @@ int lords_set_option(const char *key, const char *value)
         else if (std::strcmp(value, "dense") == 0) st.forced_path = 5;
         else if (std::strcmp(value, "direct") == 0) st.forced_path = 6;
         else if (std::strcmp(value, "wide") == 0) st.forced_path = 7;
+        else if (std::strcmp(value, "pair") == 0) st.forced_path = 8;
         else return LORDS_ERR_OPTION;
         return LORDS_OK;
     }

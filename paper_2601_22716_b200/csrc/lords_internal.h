@@ -46,7 +46,7 @@ struct State {
     size_t stage_x_bytes = 0, stage_y_bytes = 0;
     uint8_t *bw_scratch = nullptr;  // transposed factors for the input gradient
     size_t bw_scratch_bytes = 0;
-    int forced_path = 0;            // 0 auto, 1 simt, 2 decode (reassociated form), 3 umma (scale-MMA form), 4 decode16, 5 dense, 6 direct, 7 wide
+    int forced_path = 0;            // 0 auto, 1 simt, 2 decode (reassociated form), 3 umma (scale-MMA form), 4 decode16, 5 dense, 6 direct, 7 wide, 8 pair
     int forced_splitk = 0;          // 0 auto
     int forced_bn = 0;              // 0 auto; else the token tile of the scale-MMA kernel (32, 64, 128, 256)
     int last_cuda_error = 0;
@@ -71,6 +71,10 @@ int launch_simt(const Problem &p, State &st, cudaStream_t stream);
 // Tensor-core path (TMA + tcgen05/TMEM), scale matrix rebuilt per tile by a small MMA.
 // LORDS_ERR_UNSUPPORTED for shapes outside its rules.
 int launch_umma(const Problem &p, State &st, cudaStream_t stream);
+
+// The same on CTA pairs, for large calls, and the pre-pass that both share.
+int launch_umma_pair(const Problem &p, State &st, cudaStream_t stream);
+int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t stream);
 
 // Up to 16 tokens, ranks 65 .. 128: scale MMA on tcgen05, weights formed in registers.  LORDS_ERR_UNSUPPORTED otherwise.
 int launch_wide(const Problem &p, State &st, cudaStream_t stream);

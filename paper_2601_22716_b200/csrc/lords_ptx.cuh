@@ -161,11 +161,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar0, uint32_t par0, con
     if (__all_sync(0xffffffffu, mbar_try_wait(bar0, par0))) return true;
     return __all_sync(0xffffffffu, mbar_wait(bar0, par0, status, tag));
 }
+template <int SLEEP = (int)kWaitSleepNs>
 __device__ __forceinline__ bool mbar_wait_warp2(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, const int *status = nullptr, uint32_t tag = 0)
 {
     const bool a = mbar_try_wait(bar0, par0), b = mbar_try_wait(bar1, par1);
     if (__all_sync(0xffffffffu, a && b)) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar0, par0, status, tag) && mbar_wait(bar1, par1, status, tag + 1));
+    return __all_sync(0xffffffffu, mbar_wait<SLEEP>(bar0, par0, status, tag) && mbar_wait<SLEEP>(bar1, par1, status, tag + 1));
 }
 __device__ __forceinline__ bool mbar_wait_warp3(uint32_t bar0, uint32_t par0, uint32_t bar1, uint32_t par1, uint32_t bar2, uint32_t par2, bool need2,
                                                 const int *status = nullptr, uint32_t tag = 0)
@@ -247,7 +248,7 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&v)[16])
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// The same, tied to the registers that the loads fill, so that nothing computed from them can be scheduled ahead of the wait.
+// The same, tied to the registers that the loads fill (16 or 32), so that nothing computed from them can be scheduled ahead of the wait.
 __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16])
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -255,6 +256,15 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16])
                    "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15])
                  :
                  : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                   "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+                   "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+                   "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+                 ::"memory");
 }
 
 // 32 lanes x 32 consecutive 32-bit columns, registers -> TMEM: thread l writes lane (base_lane + l).
@@ -343,6 +353,12 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
+// The same without release at cluster scope (which costs about a thousand cycles): for what tcgen05 fences and waits
+// order, that is TMEM.
+__device__ __forceinline__ void mbar_arrive_pair(uint32_t cluster_bar)
+{
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
@@ -358,6 +374,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t par
     return ok != 0;
 }
 // Bounded like mbar_wait, with acquire at cluster scope (the arrivals come from other CTAs).
+template <int SLEEP = (int)kWaitSleepNs>
 __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, const int *status = nullptr, uint32_t tag = 0)
 {
     if (mbar_try_wait_cluster(bar, parity)) return true;
@@ -365,7 +382,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity,
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i) {
-            __nanosleep(kWaitSleepNs);
+            if constexpr (SLEEP > 0) __nanosleep(SLEEP);
             if (mbar_try_wait_cluster(bar, parity)) return true;
         }
         if (wait_limit_expired(limit, status, bar, parity, tag)) return false;

@@ -23,6 +23,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "lords_dequant.cuh"
 #include "lords_internal.h"
 #include "lords_ptx.cuh"
 #include "lords_tc_common.cuh"
@@ -90,55 +91,6 @@ struct alignas(64) UmmaParams {
     int y_f32;
     int *status;
 };
-
-// The 32 columns (chunk c of the 128-column code stage) of one row: codes -> level pairs, times the
-// matching pairs of S, as 16 fp16x2 words.
-template <int BITS>
-__device__ __forceinline__ void dequant_chunk(uint32_t qrow, int row, int c, uint32_t lut_lane, const uint32_t (&s)[32],
-                                              uint32_t (&out)[16])
-{
-    uint32_t lv[16];
-    if constexpr (BITS == 4) {
-        // 64-byte rows, 64-byte swizzle: 16-byte chunk c of row i sits at chunk c ^ ((i >> 1) & 3)
-        const uint4 cw = lds_v4(qrow + (((uint32_t)c ^ (uint32_t)((row >> 1) & 3)) << 4));
-        const uint32_t w[4] = {cw.x, cw.y, cw.z, cw.w};
-#pragma unroll
-        for (int wi = 0; wi < 4; ++wi)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                // byte b of the word is the code pair: one byte permute isolates it, one multiply-add makes
-                // the address of its entry (entries are 128 bytes apart)
-                const uint32_t pair = __byte_perm(w[wi], 0u, 0x4440u | (uint32_t)b);
-                lv[wi * 4 + b] = lds_u32(lut_lane + pair * 128u);
-            }
-    } else if constexpr (BITS == 2) {
-        // 32-byte rows: chunk c is the 64-bit group at byte 8c; pair p sits at bit 4p of it
-        const uint32_t w[2] = {lds_u32(qrow + 8 * c), lds_u32(qrow + 8 * c + 4)};
-#pragma unroll
-        for (int pp = 0; pp < 16; ++pp) {
-            const int off = 4 * (pp & 7);
-            const uint32_t sh = off >= 7 ? (w[pp >> 3] >> (off - 7)) : (w[pp >> 3] << (7 - off));
-            lv[pp] = lds_u32(lut_lane + (sh & 0x780u));
-        }
-    } else {
-        // 48-byte rows: chunk c is the 96-bit group at byte 12c; pair p sits at bit 6p of it
-        const uint32_t w[3] = {lds_u32(qrow + 12 * c), lds_u32(qrow + 12 * c + 4), lds_u32(qrow + 12 * c + 8)};
-#pragma unroll
-        for (int pp = 0; pp < 16; ++pp) {
-            const int bit = 6 * pp, wi = bit >> 5, off = bit & 31;
-            uint32_t sh;
-            if (off > 26) sh = __funnelshift_r(w[wi], w[wi + 1 < 3 ? wi + 1 : 2], off - 7);
-            else sh = off >= 7 ? (w[wi] >> (off - 7)) : (w[wi] << (7 - off));
-            lv[pp] = lds_u32(lut_lane + (sh & 0x1F80u));
-        }
-    }
-#pragma unroll
-    for (int pp = 0; pp < 16; ++pp) {
-        const __half2 sv = __floats2half2_rn(__uint_as_float(s[2 * pp]), __uint_as_float(s[2 * pp + 1]));
-        const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv[pp]), sv);
-        out[pp] = *reinterpret_cast<const uint32_t *>(&wv);
-    }
-}
 
 template <int BITS, int BN, int RP>
 __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_constant__ UmmaParams p)
@@ -540,8 +492,10 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
     }
 }
 
-// x bf16 -> fp16 (exact for every bf16 value inside fp16's normal range), 8 elements per thread.
-__global__ void lords_x_to_f16_kernel(const uint4 *__restrict__ x, uint4 *__restrict__ x16, size_t n_vec, int early)
+// x bf16 -> fp16 (exact for every bf16 value inside fp16's normal range), 8 elements per thread.  b_vec > 0: the threads behind
+// copy B into rows of r8 = (r rounded up to 8) ranks, 8 of them per thread, zeros behind rank r.
+__global__ void lords_x_to_f16_kernel(const uint4 *__restrict__ x, uint4 *__restrict__ x16, size_t n_vec, const uint16_t *__restrict__ B,
+                                      uint4 *__restrict__ b_pad, size_t b_vec, int r, int r8, int early)
 {
     // Programmatic dependent launch on both sides (early != 0): the kernel that consumes x16 may begin its
     // set-up (weights only) at once; this kernel itself waits for the previous launch, which may still be
@@ -549,7 +503,20 @@ __global__ void lords_x_to_f16_kernel(const uint4 *__restrict__ x, uint4 *__rest
     if (early) griddep_launch_dependents();
     griddep_wait();
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= n_vec) return;
+    if (e >= n_vec) {
+        e -= n_vec;
+        if (e >= b_vec) return;
+        const size_t row = e / (size_t)(r8 / 8);
+        const int c = (int)(e % (size_t)(r8 / 8)) * 8;
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t lo = c + 2 * k < r ? B[row * r + c + 2 * k] : 0u, hi = c + 2 * k + 1 < r ? B[row * r + c + 2 * k + 1] : 0u;
+            w[k] = lo | (hi << 16);
+        }
+        b_pad[e] = make_uint4(w[0], w[1], w[2], w[3]);
+        return;
+    }
     const uint4 v = x[e];
     const uint32_t in[4] = {v.x, v.y, v.z, v.w};
     uint32_t out[4];
@@ -673,22 +640,8 @@ template <int BITS, int BN, int RP> int launch_variant(UmmaParams &k, const Prob
         const size_t x16_bytes = ((size_t)p.M * p.n * 2 + 255) & ~(size_t)255;
         if (x16_bytes + pair_bytes > st.workspace_bytes) return LORDS_ERR_WORKSPACE;
         k.pair_scratch = reinterpret_cast<float *>(st.workspace + x16_bytes);
-        const size_t n_vec = (size_t)p.M * p.n / 8;
-        // A short pre-pass overlaps the main kernel's set-up (-2 us per call at 512 tokens); next to a long one
-        // (2048 tokens x 14336 columns: 18 us at the HBM rate) the early main kernel's CTAs and weight prefetch
-        // cost more than the overlap gains (+2 us), so there the main kernel starts when the pre-pass is done.
-        const int early = (size_t)p.M * p.n <= ((size_t)8 << 20) ? 1 : 0;
-        cudaLaunchAttribute pre_attr[1];
-        pre_attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        pre_attr[0].val.programmaticStreamSerializationAllowed = early && !p.ordered;
-        cudaLaunchConfig_t pre_cfg = cudaLaunchConfig_t{};
-        pre_cfg.gridDim = dim3((unsigned)((n_vec + 255) / 256));
-        pre_cfg.blockDim = dim3(256);
-        pre_cfg.stream = stream;
-        pre_cfg.attrs = pre_attr;
-        pre_cfg.numAttrs = 1;
-        LORDS_CUDA_TRY(cudaLaunchKernelEx(&pre_cfg, lords_x_to_f16_kernel, reinterpret_cast<const uint4 *>(p.x),
-                                          reinterpret_cast<uint4 *>(st.workspace), n_vec, early));
+        const int prc = launch_umma_prepass(p, st.workspace, nullptr, stream);
+        if (prc != LORDS_OK) return prc;
         xsrc = st.workspace;
     }
     const uint64_t row_bytes = (uint64_t)p.n * BITS / 8;
@@ -705,11 +658,10 @@ template <int BITS, int BN, int RP> int launch_variant(UmmaParams &k, const Prob
     return LORDS_OK;
 }
 
-template <int BITS, int RP> int launch_bits_rank(UmmaParams &k, const Problem &p, State &st, cudaStream_t stream)
+// Token tile: the largest that still gives CTAs for most of the SMs (tiles that fill at most half of the
+// SMs are split over two CTAs each, see launch_variant).
+int token_tile(const Problem &p, const State &st)
 {
-    if (p.M <= 16) return launch_variant<BITS, 16, RP>(k, p, st, stream);
-    // token tile: the largest that still gives CTAs for most of the SMs (tiles that fill at most half of the
-    // SMs are split over two CTAs each, see launch_variant)
     const long long row_tiles = (p.m + BM - 1) / BM;
     auto ctas = [&](int b) {
         const long long t = row_tiles * ((p.M + b - 1) / b);
@@ -717,6 +669,40 @@ template <int BITS, int RP> int launch_bits_rank(UmmaParams &k, const Problem &p
     };
     int bn = 256;
     while (bn > 32 && (p.M <= bn / 2 || 5 * ctas(bn) < 3 * (long long)st.sm_count)) bn /= 2;
+    return bn;
+}
+
+// Whether the kernel on CTA pairs is the faster one: it does a step of 128 columns in about the time that this one needs for a
+// k-step of 64, but divides the work into fewer, larger tiles, and its set-up and its pieces' meeting in scratch cost about
+// 14 us more, so that it takes the large calls (14336 x 4096, 512 tokens: 69 us against 78; 4096 x 14336, 64 tokens: 36
+// against 59; 4096 x 4096, 512 tokens: 35 against 28).  The two estimates below, in microseconds, are least-squares fits to both
+// kernels' times on five layer shapes at 64 to 1536 tokens (within 18 % of every one of them; the faster kernel is chosen to
+// within 2.5 %).
+bool prefer_pair(const Problem &p, const State &st)
+{
+    const double rank = p.r > 32 ? 1.0 : 0.0;
+    const int bn = token_tile(p, st);
+    const long long tiles = (long long)((p.m + BM - 1) / BM) * ((p.M + bn - 1) / bn), sms = st.sm_count;
+    double ksteps = (double)((p.n + BK - 1) / BK), waves = (double)((tiles + sms - 1) / sms);
+    const bool halves = 2 * tiles <= sms;                                        // every tile's k-range over two CTAs
+    if (halves) ksteps *= 0.5;
+    else if (tiles > sms && 2 * ((long long)waves * sms - tiles) >= sms) waves -= 0.5;     // the last wave's are
+    const double single = 2.9 + (halves ? 4.8 : 0.0) + (0.319 + 0.0011 * bn + 0.015 * rank) * ksteps * waves;
+
+    const long long tok_tiles = (p.M + 255) / 256, bn2 = ((p.M + tok_tiles - 1) / tok_tiles + 31) / 32 * 32;
+    const long long tiles2 = (long long)((p.m + 255) / 256) * tok_tiles, steps = (p.n + 127) / 128, total = tiles2 * steps;
+    long long pairs = total / 2 < tiles2 ? tiles2 : total / 2;
+    if (pairs > 4 * tiles2) pairs = 4 * tiles2;
+    if (pairs > sms / 2) pairs = sms / 2;
+    const bool whole = tiles2 % pairs == 0;
+    const double paired = 9.6 + (whole ? 0.0 : 9.6) + (0.0039 * (double)bn2 - 0.077 + 0.163 * rank) * (double)total / (double)pairs;
+    return paired < single;
+}
+
+template <int BITS, int RP> int launch_bits_rank(UmmaParams &k, const Problem &p, State &st, cudaStream_t stream)
+{
+    if (p.M <= 16) return launch_variant<BITS, 16, RP>(k, p, st, stream);
+    int bn = token_tile(p, st);
     if (st.forced_bn > 0) bn = st.forced_bn;   // measurement switch
     switch (bn) {
         case 32: return launch_variant<BITS, 32, RP>(k, p, st, stream);
@@ -733,11 +719,39 @@ template <int BITS> int launch_bits(UmmaParams &k, const Problem &p, State &st, 
 
 }  // namespace
 
+// The activations as fp16 rows at x16 and, where b_pad is not null, B with its rows padded to a multiple of 8 ranks.
+int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t stream)
+{
+    const size_t n_vec = (size_t)p.M * p.n / 8;
+    const int r8 = (p.r + 7) / 8 * 8;
+    const size_t b_vec = b_pad ? (size_t)p.m * r8 / 8 : 0;
+    // A short pre-pass overlaps the main kernel's set-up (-2 us per call at 512 tokens); next to a long one
+    // (2048 tokens x 14336 columns: 18 us at the HBM rate) the early main kernel's CTAs and weight prefetch
+    // cost more than the overlap gains (+2 us), so there the main kernel starts when the pre-pass is done.
+    const int early = (size_t)p.M * p.n <= ((size_t)8 << 20) ? 1 : 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = early && !p.ordered;
+    cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)((n_vec + b_vec + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_x_to_f16_kernel, static_cast<const uint4 *>(static_cast<const void *>(p.x)), static_cast<uint4 *>(x16), n_vec, p.B,
+                                      static_cast<uint4 *>(b_pad), b_vec, p.r, r8, early));
+    return LORDS_OK;
+}
+
 // Rules of this path: r <= 64; n a multiple of 64 (2- and 4-bit codes) or 128 (3-bit), which makes
 // every TMA row pitch a multiple of 16 bytes.  Anything else: LORDS_ERR_UNSUPPORTED.
 int launch_umma(const Problem &p, State &st, cudaStream_t stream)
 {
     if (!umma_takes(p)) return LORDS_ERR_UNSUPPORTED;
+    if (p.M > 32 && st.forced_bn == 0 && prefer_pair(p, st)) {
+        const int prc = launch_umma_pair(p, st, stream);
+        if (prc != LORDS_ERR_UNSUPPORTED && prc != LORDS_ERR_WORKSPACE) return prc;
+    }
 
     UmmaParams k;
     k.B = p.B;
