@@ -23,11 +23,13 @@ constexpr size_t kDirectHostBytes = 1u << 20;   // above this the copy engines w
 constexpr int kFetchBlocks = 64, kFetchThreads = 256;
 constexpr int kFetchPerThread = (int)(kDirectHostBytes / 16 / (kFetchBlocks * kFetchThreads));   // 4
 
-__global__ void __launch_bounds__(kFetchThreads) lords_fetch_host_kernel(const uint4 *__restrict__ src, uint4 *__restrict__ dst, size_t n16)
+__global__ void __launch_bounds__(kFetchThreads) lords_fetch_host_kernel(const uint4 *__restrict__ src, uint4 *__restrict__ dst, size_t n16, int tail)
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
     uint4 v[kFetchPerThread];
+    uint16_t e = 0;                         // `tail` bf16 values behind the last whole word, one per thread
+    if (t < (size_t)tail) e = reinterpret_cast<const uint16_t *>(src + n16)[t];
 #pragma unroll
     for (int k = 0; k < kFetchPerThread; ++k)
         if (t + k * stride < n16) v[k] = src[t + k * stride];
@@ -35,6 +37,7 @@ __global__ void __launch_bounds__(kFetchThreads) lords_fetch_host_kernel(const u
 #pragma unroll
     for (int k = 0; k < kFetchPerThread; ++k)
         if (t + k * stride < n16) dst[t + k * stride] = v[k];
+    if (t < (size_t)tail) reinterpret_cast<uint16_t *>(dst + n16)[t] = e;
 }
 
 // A still smaller x travels inside the launch itself: the call copies it from the (page-locked) host buffer into the
@@ -58,12 +61,13 @@ __global__ void __launch_bounds__(256) lords_stage_params_kernel(const __grid_co
 template <int BYTES> static int stage_params(const void *src, void *dst, size_t bytes, cudaStream_t s)
 {
     HostBlob<BYTES> x;
+    x.v[(bytes - 1) / 16] = make_uint4(0u, 0u, 0u, 0u);
     memcpy(&x, src, bytes);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
-    const int n16 = (int)(bytes / 16);
+    const int n16 = (int)((bytes + 15) / 16);        // the staging buffer has room for the last word's rest
     cfg.gridDim = dim3((unsigned)((n16 + 255) / 256));
     cfg.blockDim = dim3(256);
     cfg.stream = s;
@@ -99,7 +103,7 @@ static int fetch_host(const void *src, void *dst, size_t bytes, cudaStream_t s)
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_fetch_host_kernel, static_cast<const uint4 *>(src), static_cast<uint4 *>(dst), n16));
+    LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_fetch_host_kernel, static_cast<const uint4 *>(src), static_cast<uint4 *>(dst), n16, (int)(bytes % 16 / 2)));
     return LORDS_OK;
 }
 
@@ -408,7 +412,7 @@ int lords_linear_forward_host(const void *x_host, const uint8_t *Qpacked, const 
     if (xb > st.stage_x_bytes) {
         if (st.stage_x) cudaFree(st.stage_x);
         st.stage_x = nullptr; st.stage_x_bytes = 0;
-        LORDS_CUDA_TRY(cudaMalloc(&st.stage_x, xb));
+        LORDS_CUDA_TRY(cudaMalloc(&st.stage_x, (xb + 15) / 16 * 16));
         st.stage_x_bytes = xb;
     }
     if (yb > st.stage_y_bytes) {
@@ -419,7 +423,9 @@ int lords_linear_forward_host(const void *x_host, const uint8_t *Qpacked, const 
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     void *x_map = nullptr, *y_map = nullptr;
-    const bool aligned = xb % 16 == 0 && yb % 16 == 0 && (reinterpret_cast<uintptr_t>(x_host) | reinterpret_cast<uintptr_t>(y_host)) % 16 == 0;
+    // the buffers' addresses, not their lengths: a layer with 3050 rows went through the copy engines for its length (25 us a call at
+    // 1024 columns, one token; 9 now)
+    const bool aligned = (reinterpret_cast<uintptr_t>(x_host) | reinterpret_cast<uintptr_t>(y_host)) % 16 == 0;
     const bool direct = aligned && xb <= kDirectHostBytes && yb <= kDirectHostBytes && mapped_device_pointer(x_host, &x_map) &&
                         mapped_device_pointer(y_host, &y_map);
     int rc;

@@ -40,3 +40,19 @@ def test_x_by_parameters_by_fetch_and_in_a_graph(lords, M):
     torch.cuda.synchronize()
     assert np.array_equal(yh.numpy().view(np.uint16), want)
     assert lords.lords_poll_status() == 0
+
+
+@pytest.mark.parametrize("m,n,M", [(193, 258, 1), (195, 514, 3), (250, 5122, 3), (97, 6002, 7)])       # rows that are no 16-byte multiples; the last two: by fetch
+def test_ragged_lengths(lords, m, n, M):
+    import torch
+    lay = gen.make_layer(m, n, 8, M, bits=4, seed=m)
+    dl = DeviceLayer(lay)
+    _, want = dl.forward()
+    xh = torch.from_numpy(lay.x.view(np.int16)).pin_memory()
+    room = torch.full((M * m + 8,), 0x7FC0, dtype=torch.int16).pin_memory()
+    yh = room[:M * m].view(M, m)
+    lords.lords_linear_forward_host(xh, dl.q, dl.B, dl.A, lay.codebook, 4, M, lay.m, lay.n, lay.r, yh)
+    torch.cuda.synchronize()
+    assert np.array_equal(yh.numpy().view(np.uint16), want)
+    assert bool((room[M * m:] == 0x7FC0).all())
+    assert lords.lords_poll_status() == 0
