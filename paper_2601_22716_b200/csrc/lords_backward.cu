@@ -84,6 +84,8 @@ __global__ void __launch_bounds__(kTrThreads) lords_transpose_codes_kernel(const
             if (bytes == 4 * BITS && (row_bytes & 3) == 0) {
 #pragma unroll
                 for (int k = 0; k < BITS; ++k) w[k] = __ldg(reinterpret_cast<const uint32_t *>(src) + k);
+            } else if (bytes == 4 * BITS) {
+                load_words_anywhere<BITS>(src, Q + (size_t)m * row_bytes, w);
             } else {
 #pragma unroll
                 for (int k = 0; k < 4 * BITS; ++k)
@@ -129,6 +131,8 @@ __global__ void __launch_bounds__(kTrThreads) lords_transpose_codes_kernel(const
 #pragma unroll
                     for (int k = 0; k < BITS; ++k) reinterpret_cast<uint32_t *>(dst)[k] = w[k];
                 }
+            } else if (j < n && bytes == 4 * BITS) {
+                store_words_anywhere<BITS>(dst, w);
             } else if (j < n) {
 #pragma unroll
                 for (int k = 0; k < 4 * BITS; ++k)
@@ -415,8 +419,8 @@ __global__ void __launch_bounds__(kBwThreads) lords_backward_tile_kernel(const B
     }
 }
 
-// Schedule "tensor": both products on the tensor cores.  A CTA owns 128 rows of W and walks over its share of the 128-column
-// tiles.  Per tile:
+// Schedule "tensor": both products on the tensor cores.  A CTA takes a run of 128 x 128 tiles of W, row block after row block.  Per
+// tile:
 //   G[128 x 128] = sum_t g[t][i] x[t][j]   operands as they lie in memory (MN-major: a shared-memory row is one token), 64 tokens
 //                                          per stage, accumulators in TMEM (two of them: the next tile's product
 //                                          runs while this one is worked on)
@@ -426,16 +430,18 @@ __global__ void __launch_bounds__(kBwThreads) lords_backward_tile_kernel(const B
 // and the factors are bf16 as given, so every product is exact and the sums are fp32: the precision of the fp32
 // folds on the CUDA cores that this replaces, at the tensor cores' rate.  One shared-memory tile serves both folds,
 // K-major for dB and MN-major (transposed) for dA; likewise the A tile and the B tile.  dB stays in TMEM over the CTA's
-// tiles; dA_tile goes to scratch, one contribution per row block.
-// 4096 x 4096, r = 32, 512 tokens: 119 us with the folds on the CUDA cores (bound by shared memory at two multiply-adds per
-// word read), 47 us now; what bounds it is the way of g and x from L2 (32 KB per 64 tokens of a tile) and the
-// level multiply with its three-way split (about ten instructions per weight).
+// tiles of a row block; dA_tile goes to scratch, one contribution per row block.
+// 4096 x 4096, r = 32: 512 tokens 119 us with the folds on the CUDA cores (bound by shared memory at two multiply-adds per word
+// read), 43 now; QAT (with 67 MB of dW) 176 -> 74, at 1024 tokens 83.  What bounds it: with many tokens the way of g and x
+// from L2 into shared memory (32 KB per 64 tokens of a tile, about 50 bytes a clock and SM), with few the epilogue (7 thousand cycles a
+// tile; QAT 14, of which 5 for dW's stores and 3 for the quotients) and the first tile, which nothing overlaps.
 //
-// Warps 0..7: epilogue; 8: TMA of g and x; 9: main MMAs; 10: fold (and scale) MMAs; 11: TMA of the factor tiles.
+// Warps 0..15: epilogue (eight of them: 47 and 94 us); 16: TMA of g and x; 17: main MMAs; 18: fold (and scale) MMAs; 19: TMA of the factor
+// tiles.
 constexpr int kTcRows = 128, kTcCols = 128, kTcTok = 64;
-constexpr int kTcEpiWarps = 8;
-constexpr int kTcTmaWarp = 8, kTcMainWarp = 9, kTcFoldWarp = 10, kTcFactorWarp = 11;
-constexpr int kTcThreads = 12 * 32;
+constexpr int kTcEpiWarps = 16;
+constexpr int kTcTmaWarp = 16, kTcMainWarp = 17, kTcFoldWarp = 18, kTcFactorWarp = 19;
+constexpr int kTcThreads = 20 * 32;
 constexpr int kTcGAtom = kTcTok * 128;                        // 64 tokens x 64 rows (or columns) of W, bf16
 constexpr int kTcStage = 4 * kTcGAtom;                        // g: two atoms, x: two
 constexpr int kTcDsAtom = kTcRows * 128;                      // 128 rows x 64 columns of one term of dS
@@ -449,10 +455,31 @@ template <int RA, bool QAT> struct BwCfg {
     static constexpr int AATOM = RA * 128;                    // RA ranks x 64 columns
     static constexpr int ATILE = 2 * AATOM;
     static constexpr int BTILE = RA / 64 * kTcRows * 128;     // 128 rows x RA ranks, 64 ranks per atom
-    static constexpr int SMEM = 1024 + STAGES * kTcStage + 3 * kTcDsTerm + NA * ATILE + BTILE + 512;
+    static constexpr int WSTAGE = QAT && RA == 64 ? kTcEpiWarps * 1024 : 0;       // dW on its way out (with RA = 128 there is no room for it)
+    static constexpr int SMEM = 1024 + STAGES * kTcStage + 3 * kTcDsTerm + NA * ATILE + BTILE + WSTAGE + 512;
     static constexpr uint32_t S_COL = NG * kTcCols, DB_COL = S_COL + (QAT ? kTcCols : 0), DA_COL = DB_COL + RA;
     static constexpr uint32_t TMEM = 512;
     static_assert(SMEM <= 232448 && DA_COL + RA <= 512, "shared memory and TMEM");
+};
+
+// The division of all 128 x 128 tiles, row block after row block, into one run per CTA.  row_splits 0: equal runs, which may cross from a row
+// block into the next (no CTA idles: 1024 tiles over 148 SMs are 7 rounds, four CTAs per row block 8); else that many runs per row
+// block (the element-wise B tile is built once per CTA).
+struct Runs {
+    int row_blocks, col_tiles, ctas, row_splits;
+    __host__ __device__ long long begin(int c) const
+    {
+        if (row_splits == 0) return (long long)row_blocks * col_tiles * c / ctas;
+        return (long long)(c / row_splits) * col_tiles + (long long)col_tiles * (c % row_splits) / row_splits;
+    }
+    // the CTA whose run holds tile t
+    __host__ __device__ int owner(long long t) const
+    {
+        const long long all = (long long)row_blocks * col_tiles;
+        return (int)(((t + 1) * ctas + all - 1) / all - 1);
+    }
+    __host__ __device__ int first(int rb) const { return row_splits == 0 ? owner((long long)rb * col_tiles) : rb * row_splits; }
+    __host__ __device__ int parts(int rb) const { return row_splits == 0 ? owner((long long)(rb + 1) * col_tiles - 1) - first(rb) + 1 : row_splits; }
 };
 
 struct alignas(64) BwTcParams {
@@ -462,27 +489,38 @@ struct alignas(64) BwTcParams {
     CUtensorMap tm_b;     // bf16 [m][r], box {64 ranks, 128 rows}, 128-byte swizzle; used if rows of B are 16-byte multiples
     BwParams b;
     int r4, r_pad;
-    int col_tiles, splits;   // 128-column tiles; CTAs that share a row block
-    float *part_dB;       // [splits][m][r4] or null
+    Runs runs;            // which tiles a CTA takes
+    int da_bufs;          // TMEM has room for one or two accumulators of dA
+    float *part_dB;       // [contribution][m][r4] or null
     float *part_dA;       // [row blocks][r4][n] or null
     int *status;
 };
 
-template <int RA, bool QAT>
+// RAGGED: g, x or A are padded copies, and rows of W, dW and the codes may begin anywhere (checks that would cost the others 5 %).
+template <int RA, bool QAT, bool RAGGED>
 __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const __grid_constant__ BwTcParams p)
 {
     using C = BwCfg<RA, QAT>;
     extern __shared__ uint8_t tc_smem_raw[];
     const uint32_t base = (smem_u32(tc_smem_raw) + 1023u) & ~1023u;
-    const uint32_t ds0 = base + C::STAGES * kTcStage, a_s = ds0 + 3 * kTcDsTerm, b_s = a_s + C::NA * C::ATILE, bars = b_s + C::BTILE;
+    const uint32_t ds0 = base + C::STAGES * kTcStage, a_s = ds0 + 3 * kTcDsTerm, b_s = a_s + C::NA * C::ATILE, w_stage = b_s + C::BTILE, bars = w_stage + C::WSTAGE;
     const uint32_t bar_full = bars, bar_empty = bar_full + 8 * C::STAGES, bar_g = bar_empty + 8 * C::STAGES, bar_g_free = bar_g + 16;
-    const uint32_t bar_a = bar_g_free + 16, bar_ds = bar_a + 16, bar_fold = bar_ds + 8, bar_b = bar_fold + 8, bar_s = bar_b + 8, bar_s_free = bar_s + 8;
+    const uint32_t bar_a = bar_g_free + 16, bar_ds = bar_a + 16, bar_fold = bar_ds + 8, bar_b = bar_fold + 16, bar_s = bar_b + 8, bar_s_free = bar_s + 8;
     const uint32_t tmem_slot = bar_s_free + 8, levels_s = bars + 256;      // sixteen floats
-    static_assert(16 * C::STAGES + 16 * 3 + 8 * 5 + 4 <= 256, "barrier area");
+    static_assert(16 * C::STAGES + 16 * 4 + 8 * 4 + 4 <= 256, "barrier area");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rb = (int)blockIdx.x / p.splits, split = (int)blockIdx.x % p.splits;
-    const int i0 = rb * kTcRows;
-    const int t_a = (int)((long long)split * p.col_tiles / p.splits), total = (int)((long long)(split + 1) * p.col_tiles / p.splits) - t_a;
+    const int cta = (int)blockIdx.x, col_tiles = p.runs.col_tiles;
+    const long long t_a = p.runs.begin(cta);
+    const int total = (int)(p.runs.begin(cta + 1) - t_a);
+    const int rb_a = (int)(t_a / col_tiles), ct_a = (int)(t_a % col_tiles);
+    // tile t of the run: its column tile and row block; true where a row block begins
+    auto col_of = [&](int t) { return (ct_a + t) % col_tiles; };
+    auto row_of = [&](int t) { return rb_a + (ct_a + t) / col_tiles; };
+    auto new_rows = [&](int t) { return t == 0 || col_of(t) == 0; };
+    // "the folds of tile t have completed": two barriers, by turns, because the folds may run two tiles ahead of the factor tiles' lane
+    // where a row block begins (a phase's parity is also that of the one two before)
+    auto fold_bar = [&](int t) { return bar_fold + 8u * (uint32_t)(t & 1); };
+    auto fold_phase = [&](int t) { return (uint32_t)((t >> 1) & 1); };
     const int chunks = (p.b.M + kTcTok - 1) / kTcTok;
     const bool b_by_tma = (p.b.r & 7) == 0;
     const int *status = p.status;
@@ -494,6 +532,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
             for (int s = 0; s < 2; ++s) { mbar_init(bar_g + 8 * s, 1); mbar_init(bar_g_free + 8 * s, kTcEpiWarps); mbar_init(bar_a + 8 * s, 1); }
             mbar_init(bar_ds, kTcEpiWarps);
             mbar_init(bar_fold, 1);
+            mbar_init(bar_fold + 8, 1);
             mbar_init(bar_b, 1);
             mbar_init(bar_s, 1);
             mbar_init(bar_s_free, kTcEpiWarps);
@@ -509,9 +548,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
         if (tid < 16) sts_u32(levels_s + 4 * tid, __float_as_uint(p.b.levels[tid]));
         if (!b_by_tma) {
             // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m
-            const int rr = tid >> 1, i = i0 + rr;
-            for (int c = 0; c < RA / 16; ++c) {
-                const int chunk = (tid & 1) * (RA / 16) + c;
+            const int rr = tid >> 2, i = rb_a * kTcRows + rr;
+            for (int c = 0; c < RA / 32; ++c) {
+                const int chunk = (tid & 3) * (RA / 32) + c;
                 uint32_t w4[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -537,7 +576,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
         if (lane == 0) {
             int it = 0;
             for (int t = 0; t < total && !failed; ++t) {
-                const int j0 = (t_a + t) * kTcCols;
+                const int j0 = col_of(t) * kTcCols, i0 = row_of(t) * kTcRows;
                 for (int c = 0; c < chunks; ++c, ++it) {
                     const int s = it % C::STAGES;
                     if (it >= C::STAGES && !mbar_wait(bar_empty + 8 * s, (uint32_t)((it / C::STAGES - 1) & 1), status, 41)) { failed = true; break; }
@@ -552,18 +591,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
         }
         __syncwarp();
     } else if (warp == kTcFactorWarp) {
-        // ------------------------------------------------------------------ the B tile once, an A tile per column tile
+        // ------------------------------------------------------------------ the B tile per row block, an A tile per column tile
         if (lane == 0) {
-            if (b_by_tma) {
-                mbar_expect_tx(bar_b, (uint32_t)C::BTILE);
-                for (int h = 0; h < RA / 64; ++h) tma_load_2d(b_s + (uint32_t)(h * kTcRows * 128), &p.tm_b, h * 64, i0, bar_b);
-            }
             for (int t = 0; t < total; ++t) {
-                // its buffer is free when the folds of the tile NA before it have completed (with two buffers the folds cannot
-                // run a phase ahead of this wait: the scale MMA issued before them needs the tile loaded here)
-                if (t >= C::NA && !mbar_wait(bar_fold, (uint32_t)((t - C::NA) & 1), status, 46)) { failed = true; break; }
+                // an A buffer is free when the folds of the tile NA before have completed, the B tile when those of the tile right before have
+                if (t >= C::NA && !mbar_wait(fold_bar(t - C::NA), fold_phase(t - C::NA), status, 46)) { failed = true; break; }
+                if (b_by_tma && new_rows(t)) {
+                    if (t > 0 && !mbar_wait(fold_bar(t - 1), fold_phase(t - 1), status, 46)) { failed = true; break; }
+                    mbar_expect_tx(bar_b, (uint32_t)C::BTILE);
+                    for (int h = 0; h < RA / 64; ++h) tma_load_2d(b_s + (uint32_t)(h * kTcRows * 128), &p.tm_b, h * 64, row_of(t) * kTcRows, bar_b);
+                }
                 const uint32_t bar = bar_a + 8 * (t % C::NA), dst = a_s + (uint32_t)((t % C::NA) * C::ATILE);
-                const int j0 = (t_a + t) * kTcCols;
+                const int j0 = col_of(t) * kTcCols;
                 mbar_expect_tx(bar, (uint32_t)(2 * p.r_pad * 128));
                 tma_load_2d(dst, &p.tm_a, j0, 0, bar);
                 tma_load_2d(dst + C::AATOM, &p.tm_a, j0 + 64, 0, bar);
@@ -602,8 +641,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
         const uint32_t hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         auto desc_lo = [&](uint32_t addr, uint32_t lbo) { return (uint32_t)umma_desc_sw128(0, 1024, lbo) | ((addr & 0x3FFFFu) >> 4); };
         const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
-        if (b_by_tma && !mbar_wait_warp(bar_b, 0, status, 44)) failed = true;
+        uint32_t b_phase = 0;
+        // B of a row block, before its first use
+        auto wait_b = [&](int t) {
+            if (!b_by_tma || !new_rows(t)) return;
+            if (!mbar_wait_warp(bar_b, b_phase, status, 44)) failed = true;
+            b_phase ^= 1u;
+        };
         auto scale = [&](int t) {
+            wait_b(t);
+            if (failed) return;
             if (!mbar_wait_warp(bar_a + 8 * (t % C::NA), (uint32_t)((t / C::NA) & 1), status, 48) ||
                 (t > 0 && !mbar_wait_warp(bar_s_free, (uint32_t)((t - 1) & 1), status, 49))) { failed = true; return; }
             tc_fence_after_sync();
@@ -616,11 +663,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
         if (QAT && total > 0 && !failed) scale(0);
         for (int t = 0; t < total && !failed; ++t) {
             const int an = t % C::NA;
-            if (QAT && C::NA == 2 && t + 1 < total) scale(t + 1);
+            const bool ahead = C::NA == 2 && t + 1 < total && !new_rows(t + 1);       // (a new row block's B replaces the one that this tile's folds read)
+            if (QAT && ahead) scale(t + 1);
+            if (!QAT) wait_b(t);
             if (failed) break;
             if (!mbar_wait_warp2(bar_a + 8 * an, (uint32_t)((t / C::NA) & 1), bar_ds, (uint32_t)(t & 1), status, 50)) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_tile = a_s + (uint32_t)(an * C::ATILE);
+            const bool first = new_rows(t);
+            const uint32_t da_col = tmem_u + C::DA_COL + (uint32_t)(p.da_bufs == 2 && (t & 1) ? p.r_pad : 0);
             if (p.part_dB) {
                 const uint32_t db = desc_lo(a_tile, 16);
 #pragma unroll 1
@@ -629,7 +680,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
 #pragma unroll
                     for (int k = 0; k < kTcCols / 16; ++k)
                         umma_f16_ss(tmem_u + C::DB_COL, umma_desc_pack(da + (k >> 2) * (kTcDsAtom >> 4) + (k & 3) * 2, hi),
-                                    umma_desc_pack(db + (k >> 2) * (C::AATOM >> 4) + (k & 3) * 2, hi), idesc_b, (t > 0 || e > 0 || k > 0) ? 1u : 0u, leader);
+                                    umma_desc_pack(db + (k >> 2) * (C::AATOM >> 4) + (k & 3) * 2, hi), idesc_b, (!first || e > 0 || k > 0) ? 1u : 0u, leader);
                 }
             }
             if (p.part_dA) {
@@ -639,163 +690,46 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
                     const uint32_t da = desc_lo(ds0 + (uint32_t)(e * kTcDsTerm), (uint32_t)kTcDsAtom);
 #pragma unroll
                     for (int k = 0; k < kTcRows / 16; ++k)
-                        umma_f16_ss(tmem_u + C::DA_COL, umma_desc_pack(da + k * 128, hi), umma_desc_pack(db + k * 128, hi), idesc_a,
+                        umma_f16_ss(da_col, umma_desc_pack(da + k * 128, hi), umma_desc_pack(db + k * 128, hi), idesc_a,
                                     (e > 0 || k > 0) ? 1u : 0u, leader);
                 }
             }
-            umma_commit(bar_fold, leader);
-            if (QAT && C::NA == 1 && t + 1 < total) scale(t + 1);
+            umma_commit(fold_bar(t), leader);
+            if (QAT && !ahead && t + 1 < total) scale(t + 1);
         }
     } else {
-        // ------------------------------------------------------------------ epilogue: row i0 + q * 32 + lane, 64 columns per thread
-        const int q = warp & 3, ch = warp >> 2, ri = q * 32 + lane, i = i0 + ri;
+        // ------------------------------------------------------------------ epilogue: one row of the tile and 32 columns per thread
+        const int q = warp & 3, ch = warp >> 2, ri = q * 32 + lane;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
         const size_t row_bytes = (size_t)p.b.n * p.b.bits / 8;
         const int bits = p.b.bits;
-        // the folds of a tile have completed: its columns' contribution to dA leaves TMEM (lane = column, TMEM column = rank)
+        const uint8_t *q_end = p.b.q + (size_t)p.b.m * row_bytes;
+        // where 8 columns (16 bytes) of one term of dS go: row `row` of the tile, position pos (0 .. 3) of the warp's 32 columns
+        auto ds_at = [&](int row, int term, int pos) {
+            return ds0 + (uint32_t)(term * kTcDsTerm + (ch >> 1) * kTcDsAtom + (row >> 3) * 1024 + (row & 7) * 128 + ((((ch & 1) * 4 + pos) ^ (row & 7)) << 4));
+        };
+        // a tile's contribution to dA leaves TMEM once its folds have completed (lane = column, TMEM column = rank)
         auto store_dA = [&](int t) {
-            if (!mbar_wait_warp(bar_fold, (uint32_t)(t & 1), status, 45)) { failed = true; return; }
-            tc_fence_after_sync();
             if (!p.part_dA) return;
-            const int j = (t_a + t) * kTcCols + ri;
-            float *out = p.part_dA + (size_t)rb * p.r4 * p.b.n + j;
-            for (int k0 = ch * 16; k0 < p.r4; k0 += 32) {
-                uint32_t v[16];
-                tmem_ld_32x16(lane_addr + C::DA_COL + (uint32_t)k0, v);
-                tmem_wait_ld(v);
+            const int j = col_of(t) * kTcCols + ri;
+            float *out = p.part_dA + (size_t)row_of(t) * p.r4 * p.b.n + j;
+            const uint32_t col = C::DA_COL + (uint32_t)(p.da_bufs == 2 && (t & 1) ? p.r_pad : 0);
+            for (int k0 = ch * 8; k0 < p.r4; k0 += 32) {          // eight ranks each: all sixteen warps have a part up to rank 32
+                uint32_t v[8];
+                tmem_ld_32x8(lane_addr + col + (uint32_t)k0, v);
                 if (j < p.b.n)
 #pragma unroll
-                    for (int k = 0; k < 16; ++k)
+                    for (int k = 0; k < 8; ++k)
                         if (k0 + k < p.r4) __stcg(out + (size_t)(k0 + k) * p.b.n, __uint_as_float(v[k]));
             }
             tc_fence_before_sync();
         };
-        for (int t = 0; t < total; ++t) {
-            const int gb = t % C::NG;
-            // what does not depend on the products is requested first: the thread's codes and latent weights
-            uint32_t cw[2][4];
-            bool whole[2];
-            uint4 wq[QAT ? 2 : 1][4];
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int jc = (t_a + t) * kTcCols + ch * 64 + c * 32;
-                whole[c] = i < p.b.m && jc + 32 <= p.b.n && (row_bytes & 3) == 0;
-                const uint32_t *src = reinterpret_cast<const uint32_t *>(p.b.q + (size_t)(whole[c] ? i : 0) * row_bytes + (whole[c] ? (size_t)jc * bits / 8 : 0));
-#pragma unroll
-                for (int w = 0; w < 4; ++w) cw[c][w] = whole[c] && w < bits ? __ldg(src + w) : 0u;
-                if constexpr (QAT) {
-#pragma unroll
-                    for (int v = 0; v < 4; ++v) {
-                        wq[c][v] = make_uint4(0u, 0u, 0u, 0u);
-                        if (i < p.b.m && jc + 8 * v < p.b.n) wq[c][v] = __ldg(reinterpret_cast<const uint4 *>(p.b.W + (size_t)i * p.b.n + jc + 8 * v));
-                    }
-                }
-            }
-            if (!mbar_wait_warp(bar_g + 8 * gb, (uint32_t)((t / C::NG) & 1), status, 43)) { failed = true; break; }
-            if (QAT && !mbar_wait_warp(bar_s, (uint32_t)(t & 1), status, 51)) { failed = true; break; }
-            tc_fence_after_sync();
-            if (t > 0) {
-                store_dA(t - 1);                           // also: the dS buffer is free
-                if (__any_sync(0xffffffffu, failed)) { failed = true; break; }
-            }
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int jc = (t_a + t) * kTcCols + ch * 64 + c * 32;
-                uint32_t gacc[32], sv[QAT ? 32 : 1];
-                tmem_ld_32x32(lane_addr + (uint32_t)(gb * kTcCols + ch * 64 + c * 32), gacc);
-                if constexpr (QAT) tmem_ld_32x32(lane_addr + C::S_COL + (uint32_t)(ch * 64 + c * 32), sv);
-                tmem_wait_ld();
-                if (c == 1) {
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(bar_g_free + 8 * gb);
-                        if (QAT) mbar_arrive(bar_s_free);
-                    }
-                }
-                if constexpr (QAT) {
-                    if (p.b.dW && i < p.b.m) {             // Eq. 4: dL/dW = dL/dW^
-#pragma unroll
-                        for (int c4 = 0; c4 < 32; c4 += 4)
-                            if (jc + c4 < p.b.n)
-                                *reinterpret_cast<uint4 *>(p.b.dW + (size_t)i * p.b.n + jc + c4) = make_uint4(gacc[c4], gacc[c4 + 1], gacc[c4 + 2], gacc[c4 + 3]);
-                    }
-                }
-                // the factor of dL/dS: the level, or (QAT, Eq. 5) the level minus W (/) S; 0 where S is 0
-                auto factor = [&](int e, float level) -> float {
-                    if constexpr (QAT) {
-                        const uint4 &wv = wq[c][e / 8];
-                        const uint32_t ww = (e % 8) / 2 == 0 ? wv.x : (e % 8) / 2 == 1 ? wv.y : (e % 8) / 2 == 2 ? wv.z : wv.w;
-                        const float w = __uint_as_float((e & 1) ? (ww & 0xFFFF0000u) : (ww << 16)), s = __uint_as_float(sv[e]);
-                        // w / S by a reciprocal and one residual correction: exact whenever the quotient is representable
-                        // (a weight that its code reproduces exactly gets the factor 0), a rounding error otherwise
-                        const float rc = __fdividef(1.0f, s);
-                        float qv = w * rc;
-                        qv = fmaf(fmaf(-qv, s, w), rc, qv);
-                        return s != 0.0f ? level - qv : 0.0f;
-                    } else {
-                        return level;
-                    }
-                };
-                auto level_at = [&](uint32_t code) { return __uint_as_float(lds_table(levels_s + 4u * code)); };
-                // eight columns at a time: dS, its three terms, one 16-byte store each
-                auto emit = [&](int e8, const float (&d)[8]) {
-                    uint32_t w[3][4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        const float a = d[2 * h], b = d[2 * h + 1];
-                        const float a1 = a - __uint_as_float(__float_as_uint(a) & 0xFFFF0000u), b1 = b - __uint_as_float(__float_as_uint(b) & 0xFFFF0000u);
-                        const float a2 = a1 - __uint_as_float(__float_as_uint(a1) & 0xFFFF0000u), b2 = b1 - __uint_as_float(__float_as_uint(b1) & 0xFFFF0000u);
-                        w[0][h] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
-                        w[1][h] = __byte_perm(__float_as_uint(a1), __float_as_uint(b1), 0x7632);
-                        w[2][h] = __byte_perm(__float_as_uint(a2), __float_as_uint(b2), 0x7632);
-                    }
-                    const uint32_t dst = ds0 + (uint32_t)(ch * kTcDsAtom + (ri >> 3) * 1024 + (ri & 7) * 128 + (((c * 4 + e8) ^ (ri & 7)) << 4));
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) sts_v4(dst + (uint32_t)(k * kTcDsTerm), make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]));
-                };
-                auto levels_of = [&](auto width) {         // positions of the codes inside the words are constants for each width
-                    constexpr int W = decltype(width)::value;
-#pragma unroll
-                    for (int e8 = 0; e8 < 4; ++e8) {
-                        float d[8];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int e = 8 * e8 + k, bit = e * W, w = bit >> 5, sh = bit & 31;
-                            uint32_t code = cw[c][w] >> sh;
-                            if (sh + W > 32) code |= cw[c][w + 1 < 4 ? w + 1 : 3] << (32 - sh);
-                            d[k] = __uint_as_float(gacc[e]) * factor(e, level_at(code & ((1u << W) - 1u)));
-                        }
-                        emit(e8, d);
-                    }
-                };
-                if (__all_sync(0xffffffffu, whole[c])) {
-                    if (bits == 4) levels_of(std::integral_constant<int, 4>{});
-                    else if (bits == 3) levels_of(std::integral_constant<int, 3>{});
-                    else levels_of(std::integral_constant<int, 2>{});
-                } else {
-#pragma unroll
-                    for (int e8 = 0; e8 < 4; ++e8) {
-                        float d[8];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) {
-                            const int e = 8 * e8 + k;
-                            d[k] = (i < p.b.m && jc + e < p.b.n) ? __uint_as_float(gacc[e]) * factor(e, level_at(read_code(p.b.q, row_bytes, i, jc + e, bits))) : 0.0f;
-                        }
-                        emit(e8, d);
-                    }
-                }
-            }
-            fence_proxy_async_smem();
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_ds);
-        }
-        if (!__any_sync(0xffffffffu, failed) && total > 0) store_dA(total - 1);
-        // dB of the row block over this CTA's tiles: lane = row, TMEM column = rank
-        if (!__any_sync(0xffffffffu, failed) && p.part_dB && total > 0) {
-            float *out = p.part_dB + ((size_t)split * p.b.m + i) * p.r4;
-            for (int k0 = ch * 16; k0 < p.r4; k0 += 32) {
+        // dB of a row block over this CTA's tiles of it (the last one is t): lane = row, TMEM column = rank
+        auto store_dB = [&](int t) {
+            if (!p.part_dB) return;
+            const int rb = row_of(t), i = rb * kTcRows + ri;
+            float *out = p.part_dB + ((size_t)(cta - p.runs.first(rb)) * p.b.m + i) * p.r4;
+            for (int k0 = ch * 16; k0 < p.r4; k0 += 64) {
                 uint32_t v[16];
                 tmem_ld_32x16(lane_addr + C::DB_COL + (uint32_t)k0, v);
                 tmem_wait_ld(v);
@@ -804,13 +738,185 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
                     for (int k = 0; k < 16; k += 4)
                         if (k0 + k < p.r4) __stcg(reinterpret_cast<uint4 *>(out + k0 + k), make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]));
             }
+            tc_fence_before_sync();
+        };
+        for (int t = 0; t < total; ++t) {
+            const int gb = t % C::NG, i = row_of(t) * kTcRows + ri, jc = col_of(t) * kTcCols + ch * 32;
+            // what does not depend on the products is requested first: the thread's codes and latent weights
+            // (the last condition holds for every launch without RAGGED; left out, the loads below are scheduled worse: QAT 74 -> 80 us)
+            const bool whole = i < p.b.m && jc + 32 <= p.b.n && (RAGGED || (row_bytes & 3) == 0);
+            uint32_t cw[4];
+            {
+                const uint8_t *src = p.b.q + (whole ? (size_t)i * row_bytes + (size_t)jc * bits / 8 : 0);
+                if constexpr (!RAGGED) {
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) cw[w] = whole && w < bits ? __ldg(reinterpret_cast<const uint32_t *>(src) + w) : 0u;
+                } else {
+#pragma unroll
+                    for (int w = 0; w < 4; ++w) cw[w] = 0u;
+                    if (whole && bits == 4) load_words_anywhere<4>(src, q_end, cw);
+                    else if (whole && bits == 3) load_words_anywhere<3>(src, q_end, cw);
+                    else if (whole) load_words_anywhere<2>(src, q_end, cw);
+                }
+            }
+            uint4 wq[QAT ? 4 : 1];
+            if constexpr (QAT) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    wq[v] = make_uint4(0u, 0u, 0u, 0u);
+                    if constexpr (!RAGGED) {
+                        if (i < p.b.m && jc + 8 * v < p.b.n) wq[v] = __ldg(reinterpret_cast<const uint4 *>(p.b.W + (size_t)i * p.b.n + jc + 8 * v));
+                    } else if (i < p.b.m && jc + 8 * v < p.b.n) {                  // n is even: 4-byte aligned
+                        const uint32_t *two = reinterpret_cast<const uint32_t *>(p.b.W + (size_t)i * p.b.n + jc + 8 * v);
+                        const int left = p.b.n - jc - 8 * v;
+                        wq[v] = make_uint4(__ldg(two), left > 2 ? __ldg(two + 1) : 0u, left > 4 ? __ldg(two + 2) : 0u, left > 6 ? __ldg(two + 3) : 0u);
+                    }
+                }
+            }
+            if (!mbar_wait_warp(bar_g + 8 * gb, (uint32_t)((t / C::NG) & 1), status, 43)) { failed = true; break; }
+            tc_fence_after_sync();
+            if constexpr (QAT) {
+                // Eq. 4: dL/dW = dL/dW^.  Eight rows at a time through the warp's own kilobyte of shared memory, so that a store covers
+                // four rows' 128 bytes: a store takes the load/store unit as many cycles as it touches lines (4096 x 4096, 512 tokens: 4.5
+                // thousand of a tile's 15 thousand cycles with eight rows x 32 bytes per store)
+                if (p.b.dW) {
+                    const uint32_t own = w_stage + (uint32_t)(warp * 1024);
+                    const int ir = i - ri + q * 32, lr = lane >> 2, rr = lane >> 3, rc = lane & 7;
+#pragma unroll
+                    for (int hh = 0; hh < 2; ++hh) {
+                        uint32_t g[16];
+                        tmem_ld_16x32_frag(lane_addr + ((uint32_t)(hh * 16) << 16) + (uint32_t)(gb * kTcCols + ch * 32), g);
+                        tmem_wait_ld(g);
+                        if constexpr (C::WSTAGE == 0) {
+#pragma unroll
+                            for (int k = 0; k < 8; ++k) {
+                                const int row = ir + hh * 16 + (k & 1) * 8 + lr, col = jc + 2 * (lane & 3) + (k >> 1) * 8;
+                                if (row < p.b.m && col < p.b.n) *reinterpret_cast<uint2 *>(p.b.dW + (size_t)row * p.b.n + col) = make_uint2(g[2 * k], g[2 * k + 1]);
+                            }
+                            continue;
+                        }
+#pragma unroll
+                        for (int v = 0; v < 2; ++v) {
+                            __syncwarp();
+                            // 16-byte chunk c of row l at chunk c ^ l: neither the 8-byte writes nor the 16-byte reads meet in a bank
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(own + (uint32_t)(lr * 128 + (((2 * u + ((lane >> 1) & 1)) ^ lr) << 4) + (lane & 1) * 8)),
+                                             "r"(g[4 * u + 2 * v]), "r"(g[4 * u + 2 * v + 1]) : "memory");
+                            __syncwarp();
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                const int l = k * 4 + rr, row = ir + hh * 16 + v * 8 + l;
+                                const uint4 o = lds_v4(own + (uint32_t)(l * 128 + ((rc ^ l) << 4)));
+                                const int col = jc + 4 * rc;
+                                if constexpr (!RAGGED) {
+                                    if (row < p.b.m && col < p.b.n) __stcs(reinterpret_cast<uint4 *>(p.b.dW + (size_t)row * p.b.n + col), o);
+                                } else if (row < p.b.m && col < p.b.n) {          // n is even: 8-byte aligned
+                                    float *dst = p.b.dW + (size_t)row * p.b.n + col;
+                                    *reinterpret_cast<uint2 *>(dst) = make_uint2(o.x, o.y);
+                                    if (col + 2 < p.b.n) *reinterpret_cast<uint2 *>(dst + 2) = make_uint2(o.z, o.w);
+                                }
+                            }
+                        }
+                    }
+                }
+            }
+            if (QAT && !mbar_wait_warp(bar_s, (uint32_t)(t & 1), status, 51)) { failed = true; break; }
+            tc_fence_after_sync();
+            // dS in registers: all that does not need the buffer that the folds of the tile before still read
+            float d[32];
+            auto level_at = [&](uint32_t code) { return __uint_as_float(lds_table(levels_s + 4u * code)); };
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint32_t gacc[16], sv[QAT ? 16 : 1];
+                tmem_ld_32x16(lane_addr + (uint32_t)(gb * kTcCols + ch * 32 + h * 16), gacc);
+                if constexpr (QAT) tmem_ld_32x16(lane_addr + C::S_COL + (uint32_t)(ch * 32 + h * 16), sv);
+                tmem_wait_ld(gacc);
+                if constexpr (QAT) tmem_wait_ld(sv);
+                if (h == 1) {
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(bar_g_free + 8 * gb);
+                        if (QAT) mbar_arrive(bar_s_free);
+                    }
+                }
+                // the factor of dL/dS: the level, or (QAT, Eq. 5) the level minus W (/) S; 0 where S is 0
+                auto factor = [&](int e, float level) -> float {
+                    if constexpr (QAT) {
+                        const uint4 &wv = wq[e / 8];
+                        const uint32_t ww = (e % 8) / 2 == 0 ? wv.x : (e % 8) / 2 == 1 ? wv.y : (e % 8) / 2 == 2 ? wv.z : wv.w;
+                        const float w = __uint_as_float((e & 1) ? (ww & 0xFFFF0000u) : (ww << 16)), sc = __uint_as_float(sv[e & 15]);
+                        // w / S by a reciprocal and one residual correction: exact whenever the quotient is representable
+                        // (a weight that its code reproduces exactly gets the factor 0), a rounding error otherwise
+                        const float rc = rcp_approx(sc);
+                        float qv = w * rc;
+                        qv = fmaf(fmaf(-qv, sc, w), rc, qv);
+                        return fabsf(sc) >= 1.17549435e-38f ? level - qv : 0.0f;      // (the reciprocal takes subnormal numbers for zero)
+                    } else {
+                        return level;
+                    }
+                };
+                auto levels_of = [&](auto width) {         // positions of the codes inside the words are constants for each width
+                    constexpr int W = decltype(width)::value;
+#pragma unroll
+                    for (int e = 16 * h; e < 16 * h + 16; ++e) {
+                        const int bit = e * W, w = bit >> 5, sh = bit & 31;
+                        uint32_t code = cw[w] >> sh;
+                        if (sh + W > 32) code |= cw[w + 1 < 4 ? w + 1 : 3] << (32 - sh);
+                        d[e] = __uint_as_float(gacc[e & 15]) * factor(e, level_at(code & ((1u << W) - 1u)));
+                    }
+                };
+                if (__all_sync(0xffffffffu, whole)) {
+                    if (bits == 4) levels_of(std::integral_constant<int, 4>{});
+                    else if (bits == 3) levels_of(std::integral_constant<int, 3>{});
+                    else levels_of(std::integral_constant<int, 2>{});
+                } else {
+#pragma unroll
+                    for (int e = 16 * h; e < 16 * h + 16; ++e)
+                        d[e] = (i < p.b.m && jc + e < p.b.n) ? __uint_as_float(gacc[e & 15]) * factor(e, level_at(read_code(p.b.q, row_bytes, i, jc + e, bits))) : 0.0f;
+                }
+            }
+            // the folds of the tile before have completed: the dS buffer is free, dB and dA of it are in TMEM
+            if (t > 0 && !mbar_wait_warp(fold_bar(t - 1), fold_phase(t - 1), status, 45)) { failed = true; break; }
+            tc_fence_after_sync();
+            if (t > 0 && new_rows(t)) store_dB(t - 1);
+            // the three terms, eight columns (one 16-byte store each) at a time
+#pragma unroll
+            for (int e8 = 0; e8 < 4; ++e8) {
+                uint32_t w[3][4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const float a = d[8 * e8 + 2 * k], b = d[8 * e8 + 2 * k + 1];
+                    const float a1 = a - __uint_as_float(__float_as_uint(a) & 0xFFFF0000u), b1 = b - __uint_as_float(__float_as_uint(b) & 0xFFFF0000u);
+                    const float a2 = a1 - __uint_as_float(__float_as_uint(a1) & 0xFFFF0000u), b2 = b1 - __uint_as_float(__float_as_uint(b1) & 0xFFFF0000u);
+                    w[0][k] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+                    w[1][k] = __byte_perm(__float_as_uint(a1), __float_as_uint(b1), 0x7632);
+                    w[2][k] = __byte_perm(__float_as_uint(a2), __float_as_uint(b2), 0x7632);
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) sts_v4(ds_at(ri, k, e8), make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]));
+            }
+            // dA of the tile before: with one accumulator it has to leave before this tile's folds begin
+            if (t > 0 && p.da_bufs == 1) store_dA(t - 1);
+            fence_proxy_async_smem();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_ds);
+            if (t > 0 && p.da_bufs == 2) store_dA(t - 1);
+        }
+        if (!__any_sync(0xffffffffu, failed) && total > 0) {
+            if (!mbar_wait_warp(fold_bar(total - 1), fold_phase(total - 1), status, 45)) {
+                failed = true;
+            } else {
+                tc_fence_after_sync();
+                store_dA(total - 1);
+                store_dB(total - 1);
+            }
         }
     }
 
-    if (failed) {
-        atomicExch(p.status, LORDS_ERR_TIMEOUT);
-        for (int k = 0; k < 100; ++k) __nanosleep(1000);      // copies in flight land before the CTA ends
-    }
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kTcFoldWarp) {
@@ -819,42 +925,96 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
     }
 }
 
-// out[e] = sum over tiles t (in order) of part[t * stride + pos(e)], for dB (rows = m, inner = r, inner4 = r4:
-// blocks below blocks_b) and for dA (rows = r, inner = inner4 = n: the other blocks) in one launch.
+// A thread moves eight values, two at a time where rows are 4-byte aligned.
+__global__ void lords_pad_rows_kernel(const PadJobs jobs)
+{
+    long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    int k = 0;
+    while (k < jobs.count && e >= jobs.job[k].words) e -= jobs.job[k++].words;
+    if (k == jobs.count) return;
+    const PadJob &j = jobs.job[k];
+    const long long row = e / (j.pitch / 8);
+    const int c = (int)(e % (j.pitch / 8)) * 8;
+    const uint16_t *src = j.src + row * j.cols + c;
+    uint32_t w[4];
+    if ((j.cols & 1) == 0) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) w[v] = c + 2 * v < j.cols ? __ldg(reinterpret_cast<const uint32_t *>(src) + v) : 0u;
+    } else {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const uint32_t lo = c + 2 * v < j.cols ? __ldg(src + 2 * v) : 0u, hi = c + 2 * v + 1 < j.cols ? __ldg(src + 2 * v + 1) : 0u;
+            w[v] = lo | (hi << 16);
+        }
+    }
+    reinterpret_cast<uint4 *>(j.dst)[e] = make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// out[e] = sum over contributions t (in order) of part[t * stride + pos(e)], for dB (rows = m, inner = r, inner4 = r4:
+// blocks below blocks_b) and for dA (rows = r, inner = inner4 = n: the other blocks) in one launch.  A thread has sixteen contributions on
+// their way at a time (four neighbours per thread leave too few threads: 13 us instead of 10 for 4096 x 4096, r = 32, cold).
 struct ReduceJob {
     const float *part;
     float *out;
     int tiles, rows, inner, inner4;
     size_t stride;
+    Runs runs;            // tiles < 0: the number of contributions depends on the row block
 };
 
-__global__ void lords_backward_reduce_kernel(const ReduceJob jb, const ReduceJob ja, int blocks_b)
+__global__ void __launch_bounds__(256) lords_backward_reduce_kernel(const ReduceJob jb, const ReduceJob ja, int blocks_b)
 {
     const bool isb = (int)blockIdx.x < blocks_b;
     const ReduceJob &j = isb ? jb : ja;
     const size_t e = (size_t)(isb ? blockIdx.x : blockIdx.x - blocks_b) * blockDim.x + threadIdx.x;
+    griddep_wait();
     if (e >= (size_t)j.rows * j.inner) return;
     const size_t row = e / j.inner, col = e % j.inner;
+    const int tiles = j.tiles >= 0 ? j.tiles : j.runs.parts((int)(row / kTcRows));
+    const float *src = j.part + row * j.inner4 + col;
     float s = 0.0f;
-    for (int t = 0; t < j.tiles; ++t) s += j.part[(size_t)t * j.stride + row * j.inner4 + col];
+    for (int t0 = 0; t0 < tiles; t0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = t0 + k < tiles ? __ldcg(src + (size_t)(t0 + k) * j.stride) : 0.0f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) s += v[k];
+    }
     j.out[e] = s;
 }
 
-// The sums of the tiles' contributions to dB ([tiles_b][m][r4]) and dA ([tiles_a][r4][n]); either may be absent.
-int launch_reduce(const float *part_b, float *dB, int tiles_b, const float *part_a, float *dA, int tiles_a, int m, int n, int r, int r4,
+// The sums of the contributions to dB ([tiles_b][m][r4]; tiles_b < 0: see runs) and dA ([tiles_a][r4][n]); either may be absent.
+int launch_reduce(const float *part_b, float *dB, int tiles_b, const Runs &runs, const float *part_a, float *dA, int tiles_a, int m, int n, int r, int r4,
                   cudaStream_t stream)
 {
-    ReduceJob jb = {part_b, dB, tiles_b, dB ? m : 0, r, r4, (size_t)m * r4};
-    ReduceJob ja = {part_a, dA, tiles_a, dA ? r : 0, n, n, (size_t)r4 * n};
+    ReduceJob jb = {part_b, dB, tiles_b, dB ? m : 0, r, r4, (size_t)m * r4, runs};
+    ReduceJob ja = {part_a, dA, tiles_a, dA ? r : 0, n, n, (size_t)r4 * n, runs};
     const size_t nb = ((size_t)jb.rows * r + 255) / 256, na = ((size_t)ja.rows * n + 255) / 256;
     if (nb + na == 0) return LORDS_OK;
     if (nb + na > 2147483647u) return LORDS_ERR_SHAPE;
-    lords_backward_reduce_kernel<<<(unsigned)(nb + na), 256, 0, stream>>>(jb, ja, (int)nb);
-    LORDS_CUDA_TRY(cudaGetLastError());
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)(nb + na));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_backward_reduce_kernel, jb, ja, (int)nb));
     return LORDS_OK;
 }
 
 }  // namespace
+
+int launch_pad_rows(const PadJobs &jobs, cudaStream_t stream)
+{
+    long long words = 0;
+    for (int c = 0; c < jobs.count; ++c) words += jobs.job[c].words;
+    if ((words + 255) / 256 > 2147483647LL) return LORDS_ERR_SHAPE;
+    lords_pad_rows_kernel<<<(unsigned)((words + 255) / 256), 256, 0, stream>>>(jobs);
+    LORDS_CUDA_TRY(cudaGetLastError());
+    return LORDS_OK;
+}
 
 int launch_transpose_codes(const uint8_t *Q, int m, int n, int bits, uint8_t *Qt, cudaStream_t stream)
 {
@@ -877,15 +1037,16 @@ int launch_transpose_bf16_pair(const uint16_t *src0, int rows0, int cols0, uint1
     return LORDS_OK;
 }
 
-template <int RA, bool QAT> static int launch_tc_variant(const BwTcParams &k, int ctas, const State &st, cudaStream_t stream)
+template <int RA, bool QAT, bool RAGGED> static int launch_tc_variant(BwTcParams &k, const State &st, cudaStream_t stream)
 {
     static bool done[kMaxDevices] = {};
     const int dev = device_slot(st);
     if (!done[dev]) {
-        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_backward_tc_kernel<RA, QAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwCfg<RA, QAT>::SMEM));
+        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_backward_tc_kernel<RA, QAT, RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwCfg<RA, QAT>::SMEM));
         done[dev] = true;
     }
-    lords_backward_tc_kernel<RA, QAT><<<(unsigned)ctas, kTcThreads, BwCfg<RA, QAT>::SMEM, stream>>>(k);
+    k.da_bufs = BwCfg<RA, QAT>::DA_COL + 2 * (uint32_t)k.r_pad <= 512 ? 2 : 1;
+    lords_backward_tc_kernel<RA, QAT, RAGGED><<<(unsigned)k.runs.ctas, kTcThreads, BwCfg<RA, QAT>::SMEM, stream>>>(k);
     LORDS_CUDA_TRY(cudaGetLastError());
     return LORDS_OK;
 }
@@ -899,36 +1060,79 @@ static int launch_backward_tc(const BwParams &p, State &st, cudaStream_t stream)
     k.b = p;
     k.r4 = (r + 3) & ~3;
     k.r_pad = (r + 15) & ~15;
-    const int row_blocks = (m + kTcRows - 1) / kTcRows;
-    k.col_tiles = (n + kTcCols - 1) / kTcCols;
-    // CTAs per row block: the least rounds of one CTA per SM times (tiles of a CTA + a fixed part worth one)
-    k.splits = 1;
-    double best = 1e30;
-    for (int s = 1; s <= k.col_tiles && s <= 64; ++s) {
-        const double t = (double)(((long long)row_blocks * s + st.sm_count - 1) / st.sm_count) * ((k.col_tiles + s - 1) / s + 1.0);
-        if (t < best) { best = t; k.splits = s; }
+    Runs &runs = k.runs;
+    runs.row_blocks = (m + kTcRows - 1) / kTcRows;
+    runs.col_tiles = (n + kTcCols - 1) / kTcCols;
+    const long long tiles = (long long)runs.row_blocks * runs.col_tiles;
+    runs.row_splits = 0;
+    int parts = 1;
+    if ((r & 7) == 0) {
+        runs.ctas = (int)(tiles < st.sm_count ? tiles : st.sm_count);
+        for (int rb = 0; rb < runs.row_blocks; ++rb) parts = runs.parts(rb) > parts ? runs.parts(rb) : parts;
+    } else {
+        // the least rounds of one CTA per SM times (tiles of a CTA + a fixed part worth one)
+        double best = 1e30;
+        for (int s = 1; s <= runs.col_tiles && s <= 64; ++s) {
+            const double t = (double)(((long long)runs.row_blocks * s + st.sm_count - 1) / st.sm_count) * ((runs.col_tiles + s - 1) / s + 1.0);
+            if (t < best) { best = t; runs.row_splits = s; }
+        }
+        parts = runs.row_splits;
+        if ((long long)runs.row_blocks * parts > 2147483647LL) return LORDS_ERR_UNSUPPORTED;
+        runs.ctas = runs.row_blocks * parts;
     }
-    const size_t nb = p.dB ? (size_t)k.splits * m * k.r4 * sizeof(float) : 0, na = p.dA ? (size_t)row_blocks * k.r4 * n * sizeof(float) : 0;
-    if (m % 8 != 0 || n % 8 != 0 || nb + na + 256 > st.workspace_bytes || (long long)row_blocks * k.splits > 2147483647LL) return LORDS_ERR_UNSUPPORTED;
+    // rows of g, x or A that are not 16-byte multiples: padded copies, except where the call is so small that the CUDA cores' tiles are as
+    // good (1024 x 300, two tokens)
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const int m8 = (m + 7) & ~7, n8 = (n + 7) & ~7;
+    const bool pad = m8 != m || n8 != n;
+    if (pad && (long long)M * m * n <= (1 << 22)) return LORDS_ERR_UNSUPPORTED;
+    const size_t nb = up(p.dB ? (size_t)parts * m * k.r4 * sizeof(float) : 0), na = up(p.dA ? (size_t)runs.row_blocks * k.r4 * n * sizeof(float) : 0);
+    const size_t ng = up(m8 != m ? (size_t)M * m8 * 2 : 0), nx = up(n8 != n ? (size_t)M * n8 * 2 : 0), nf = up(n8 != n ? (size_t)r * n8 * 2 : 0);
+    if (nb + na + ng + nx + nf > st.workspace_bytes) return LORDS_ERR_UNSUPPORTED;
     k.part_dB = p.dB ? reinterpret_cast<float *>(st.workspace) : nullptr;
-    k.part_dA = p.dA ? reinterpret_cast<float *>(st.workspace + ((nb + 255) & ~(size_t)255)) : nullptr;
+    k.part_dA = p.dA ? reinterpret_cast<float *>(st.workspace + nb) : nullptr;
     k.status = st.status_word;
-    if (!make_map_2d(&k.tm_g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.g, (uint64_t)m, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.x, (uint64_t)n, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.A, (uint64_t)n, (uint64_t)r, 64, (uint32_t)k.r_pad, CU_TENSOR_MAP_SWIZZLE_128B))
+    const uint16_t *g = p.g, *x = p.x, *A = p.A;
+    int launches = 1;
+    if (pad) {
+        uint16_t *at = reinterpret_cast<uint16_t *>(st.workspace + nb + na);
+        PadJobs jobs;
+        jobs.count = 0;
+        auto copy = [&](const uint16_t *&src, int rows, int cols, int pitch, size_t bytes) {
+            if (bytes == 0) return;
+            jobs.job[jobs.count++] = {src, at, cols, pitch, (long long)rows * (pitch / 8)};
+            src = at;
+            at += bytes / 2;
+        };
+        copy(g, M, m, m8, ng);
+        copy(x, M, n, n8, nx);
+        copy(A, r, n, n8, nf);
+        const int prc = launch_pad_rows(jobs, stream);
+        if (prc != LORDS_OK) return prc;
+        ++launches;
+    }
+    if (!make_map_2d(&k.tm_g, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, g, (uint64_t)m8, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x, (uint64_t)n8, (uint64_t)M, 64, 64, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, A, (uint64_t)n8, (uint64_t)r, 64, (uint32_t)k.r_pad, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;
     k.tm_b = k.tm_a;                                                       // not used where the kernel builds the B tile element by element
     if ((r & 7) == 0 &&
         !make_map_2d(&k.tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, p.B, (uint64_t)r, (uint64_t)m, 64, (uint32_t)kTcRows, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;
-    const int ctas = row_blocks * k.splits;
     int rc;
-    if (p.W) rc = r <= 64 ? launch_tc_variant<64, true>(k, ctas, st, stream) : launch_tc_variant<128, true>(k, ctas, st, stream);
-    else rc = r <= 64 ? launch_tc_variant<64, false>(k, ctas, st, stream) : launch_tc_variant<128, false>(k, ctas, st, stream);
+    const bool ragged = pad || (size_t)n * p.bits / 8 % 4 != 0;       // (2-bit codes: rows of 8 columns are 2 bytes)
+    auto variant = [&](auto ra, auto qat) {
+        constexpr int RA = decltype(ra)::value;
+        constexpr bool QAT = decltype(qat)::value;
+        return ragged ? launch_tc_variant<RA, QAT, true>(k, st, stream) : launch_tc_variant<RA, QAT, false>(k, st, stream);
+    };
+    using Small = std::integral_constant<int, 64>;
+    using Large = std::integral_constant<int, 128>;
+    if (p.W) rc = r <= 64 ? variant(Small{}, std::true_type{}) : variant(Large{}, std::true_type{});
+    else rc = r <= 64 ? variant(Small{}, std::false_type{}) : variant(Large{}, std::false_type{});
     if (rc != LORDS_OK) return rc;
-    int launches = 1;
     if (p.dB || p.dA) {
-        rc = launch_reduce(k.part_dB, p.dB, k.splits, k.part_dA, p.dA, row_blocks, m, n, r, k.r4, stream);
+        rc = launch_reduce(k.part_dB, p.dB, -1, runs, k.part_dA, p.dA, runs.row_blocks, m, n, r, k.r4, stream);
         if (rc != LORDS_OK) return rc;
         ++launches;
     }
@@ -964,7 +1168,7 @@ int launch_backward_factors(const uint16_t *g, const uint16_t *x, const uint8_t 
         LORDS_CUDA_TRY(cudaGetLastError());
         ++launches;
         {
-            const int rc = launch_reduce(part_b, dB, jt_n, part_a, dA, it_n, m, n, r, r4, stream);
+            const int rc = launch_reduce(part_b, dB, jt_n, Runs{}, part_a, dA, it_n, m, n, r, r4, stream);
             if (rc != LORDS_OK) return rc;
             ++launches;
         }

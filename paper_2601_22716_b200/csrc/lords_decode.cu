@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
         }
     }
 
-    if (failed) atomicExch(p.status, LORDS_ERR_TIMEOUT);
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kIssuerWarp0) {

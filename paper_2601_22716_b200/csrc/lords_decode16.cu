@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         }
     }
 
-    if (failed) atomicExch(p.status, LORDS_ERR_TIMEOUT);
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kIssuerWarp0) {

@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
                 }
             }
     }
-    if (failed) atomicExch(p.status, LORDS_ERR_TIMEOUT);
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     // no CTA leaves while stores of its own may be on their way to another
     asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");

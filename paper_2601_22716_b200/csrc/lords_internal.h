@@ -94,6 +94,19 @@ int launch_decode(const Problem &p, State &st, cudaStream_t stream);
 // LORDS_ERR_UNSUPPORTED for shapes outside its rules.
 int launch_decode16(const Problem &p, State &st, cudaStream_t stream);
 
+// Up to three matrices of 16-bit values copied to rows of `pitch` (a multiple of 8) values, zeros behind.
+struct PadJob {
+    const uint16_t *src;  // 4-byte aligned
+    uint16_t *dst;
+    int cols, pitch;
+    long long words;      // rows * pitch / 8
+};
+struct PadJobs {
+    PadJob job[3];
+    int count;
+};
+int launch_pad_rows(const PadJobs &jobs, cudaStream_t stream);
+
 // Quantisation step (codes from W, B, A): tensor-core kernel where its rules hold, CUDA cores otherwise.
 int launch_quantize(const void *W, const void *B, const void *A, const float *levels, int bits, int m, int n, int r,
                     uint8_t *Q, State &st, cudaStream_t stream);

@@ -92,6 +92,15 @@ __device__ __forceinline__ bool wait_limit_expired(WaitLimit &w, const int *stat
     return false;
 }
 
+// A thread that gave up a wait records it and stays about 100 us: copies and MMAs that other roles of its CTA have issued end in that
+// time, before the CTA's final barrier lets its shared memory and TMEM go.
+__device__ __forceinline__ void record_give_up(int *status, int code)
+{
+    atomicExch(status, code);
+    const unsigned long long t0 = global_ns();
+    for (int k = 0; k < 1000 && global_ns() - t0 < 100000ull; ++k) __nanosleep(1000);
+}
+
 // Up to 64 tries, SLEEP nanoseconds apart (0: as fast as the tries return).  Written out because a waiting warp takes issue slots
 // from the warps it waits for: four instructions a try, where the compiler's version of this loop took about fourteen
 // (in a decode kernel with ten waiting warps that was more than half of everything the SM issued).
@@ -222,6 +231,13 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols) : "memory");
 }
 
+__device__ __forceinline__ float rcp_approx(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 // 32 lanes x 32 consecutive 32-bit columns: thread l of the warp receives lane (base_lane + l).
 __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&v)[32])
 {
@@ -246,8 +262,31 @@ __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&v)[16])
         : "r"(taddr)
         : "memory");
 }
+// 16 lanes x 32 consecutive fp32 columns in the accumulator layout of m16n8: for column group u of eight, v[4u], v[4u + 1] are row
+// lane / 4, columns 2 (lane % 4) and + 1, v[4u + 2], v[4u + 3] the same of row lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld_16x32_frag(uint32_t taddr, uint32_t (&v)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr)
+        : "memory");
+}
+
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// Eight columns, complete on return.
+__device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t (&v)[8])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+        "tcgen05.wait::ld.sync.aligned;"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "r"(taddr)
+        : "memory");
+}
 // The same, tied to the registers that the loads fill (16 or 32), so that nothing computed from them can be scheduled ahead of the wait.
 __device__ __forceinline__ void tmem_wait_ld(uint32_t (&v)[16])
 {

@@ -86,12 +86,6 @@ struct alignas(64) QuantParams {
     int *status;
 };
 
-__device__ __forceinline__ float rcp_approx(float v)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
-}
 // Two fp32 values in one 64-bit register: one instruction issued for both.
 __device__ __forceinline__ uint64_t f32x2(float lo, float hi)
 {
@@ -174,6 +168,8 @@ template <int BITS> __device__ __forceinline__ void store_codes(uint8_t *dst, co
 #pragma unroll
             for (int k = 0; k < BITS; ++k) reinterpret_cast<uint32_t *>(dst)[k] = w[k];
         }
+    } else if (count >= 32) {
+        store_words_anywhere<BITS>(dst, w);
     } else {
 #pragma unroll
         for (int k = 0; k < 4 * BITS; ++k)
@@ -414,31 +410,13 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
         }
     }
 
-    if (failed) {
-        atomicExch(p.status, LORDS_ERR_TIMEOUT);
-        for (int k = 0; k < 100; ++k) __nanosleep(1000);      // copies in flight land before the CTA ends
-    }
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kIssuerWarpQ) {
         tc_fence_after_sync();
         tmem_dealloc(tmem_base, kTmemColsQ);
     }
-}
-
-// Rows of `n` bf16 values -> rows of pitch np (a multiple of 8), zeros behind; two matrices in one launch.
-__global__ void lords_pad_rows_kernel(const uint16_t *__restrict__ src0, uint16_t *__restrict__ dst0, long long words0, const uint16_t *__restrict__ src1,
-                                      uint16_t *__restrict__ dst1, long long words1, int n, int np)
-{
-    // a thread moves two values (n is even: rows are 4-byte aligned); words: np / 2 per row
-    const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool first = e < words0;
-    if (e >= words0 + words1) return;
-    const long long f = first ? e : e - words0;
-    const long long row = f / (np / 2);
-    const int c = (int)(f % (np / 2)) * 2;
-    const uint16_t *src = first ? src0 : src1;
-    reinterpret_cast<uint32_t *>(first ? dst0 : dst1)[f] = c < n ? __ldg(reinterpret_cast<const uint32_t *>(src + row * n + c)) : 0u;
 }
 
 // Plain CUDA-core version for any shape: a thread owns one row and one pack group of 32 columns (or what
@@ -558,11 +536,12 @@ int launch_quantize(const void *W, const void *B, const void *A, const float *le
         const void *Wt = W, *At = A;
         if (pad) {
             uint16_t *wp = reinterpret_cast<uint16_t *>(st.workspace), *ap = reinterpret_cast<uint16_t *>(st.workspace + w_bytes);
-            const long long words0 = (long long)m * (np / 2), words1 = (long long)r * (np / 2), blocks = (words0 + words1 + 255) / 256;
-            if (blocks > 2147483647LL) return LORDS_ERR_SHAPE;
-            lords_pad_rows_kernel<<<(unsigned)blocks, 256, 0, stream>>>(static_cast<const uint16_t *>(W), wp, words0, static_cast<const uint16_t *>(A), ap,
-                                                                        words1, n, np);
-            LORDS_CUDA_TRY(cudaGetLastError());
+            PadJobs jobs;
+            jobs.count = 2;
+            jobs.job[0] = {static_cast<const uint16_t *>(W), wp, n, np, (long long)m * (np / 8)};
+            jobs.job[1] = {static_cast<const uint16_t *>(A), ap, n, np, (long long)r * (np / 8)};
+            const int rc = launch_pad_rows(jobs, stream);
+            if (rc != LORDS_OK) return rc;
             Wt = wp; At = ap;
             ++launches;
         }

@@ -370,10 +370,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
         }
     }
 
-    if (failed) {
-        atomicExch(p.status, LORDS_ERR_TIMEOUT);
-        for (int k = 0; k < 100; ++k) __nanosleep(1000);      // copies in flight land before the CTA ends
-    }
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     tc_fence_before_sync();
     __syncthreads();
     // neither CTA leaves while the other may still signal its barriers or read its operands

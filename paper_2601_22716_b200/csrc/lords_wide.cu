@@ -87,19 +87,6 @@ __device__ __forceinline__ void st_async_cluster_2f32(uint32_t addr, float a, fl
                  ::"r"(addr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(bar) : "memory");
 }
 
-// 16 lanes x 32 consecutive fp32 columns in the accumulator layout of m16n8: for column group u of eight, v[4u], v[4u + 1] are row
-// lane / 4, columns 2 (lane % 4) and + 1, v[4u + 2], v[4u + 3] the same of row lane / 4 + 8.
-__device__ __forceinline__ void tmem_ld_16x32_frag(uint32_t taddr, uint32_t (&v)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr)
-        : "memory");
-}
-
 // Byte offset of 32-column group c (0..3) of row `row` in a code tile as the tensor-map copy lays it out: 4-bit rows are 64
 // bytes with 16-byte chunks swizzled over four, 2-bit rows 32 bytes (a group is 8 bytes) with chunks swapped
 // every four rows, 3-bit rows 48 bytes as they are; eight consecutive rows fall into different banks.
@@ -395,10 +382,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
                 }
         }
     }
-    if (failed) {
-        atomicExch(p.status, LORDS_ERR_TIMEOUT);
-        for (int k = 0; k < 100; ++k) __nanosleep(1000);      // copies in flight land before the CTA ends
-    }
+    if (failed) ptx::record_give_up(p.status, LORDS_ERR_TIMEOUT);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == kScaleWarp) {
