@@ -36,6 +36,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <cstring>
 #include <type_traits>
 
 #include "lords_internal.h"
@@ -179,9 +180,24 @@ __device__ __forceinline__ void dequant_row_to_tmem(uint32_t qrow, int row, int 
     }
 }
 
-template <int BITS, int NTOK, int H>
-__global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_constant__ DecodeParams p)
+// What a launch carries.  XB > 0: also the activations themselves (a host buffer's, at most XB bytes).  Such a launch depends on no
+// earlier one but for the order of the results: it waits for the previous launch just before it stores y.  (With x staged by a
+// kernel of its own, every call paid for that launch and began only when it had ended: 4096 x 4096, host to host, calls back
+// to back 12.1 us, 7.2 so.)
+template <int XB> struct DecodeArgs {
+    DecodeParams p;
+    uint4 x[XB / 16];
+};
+template <> struct DecodeArgs<0> {
+    DecodeParams p;
+};
+constexpr int kInlineBytes = 8192;             // XB of the one such variant
+constexpr int kInlineSlice = 10240;            // room for a CTA's slice of x
+
+template <int BITS, int NTOK, int H, int XB>
+__global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_constant__ DecodeArgs<XB> args)
 {
+    const DecodeParams &p = args.p;
     using C = DCfg<BITS, H>;
     constexpr int S = C::S, SQ = C::SQ, kTileRows = C::TILE_ROWS, kGroups = C::GROUPS, kGroupWarps = C::GROUP_WARPS;
     extern __shared__ uint8_t smem_raw[];
@@ -196,7 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
     if constexpr (BITS == 4) {
         ax_lo = (raw + 1023u) & ~1023u;
         xs0 = ax_lo + kAxLow * C::AXSTAGE;
-        red0 = xs0 + ((S * C::XSTAGE + 1023) & ~1023);
+        red0 = xs0 + (XB ? kInlineSlice : (S * C::XSTAGE + 1023) & ~1023);
         bars = red0 + C::RED_BYTES;
         q0 = lut + C::LUT_BYTES;
         ax_hi = q0 + SQ * C::QSTAGE;
@@ -206,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
         ax_lo = q0 + SQ * C::QSTAGE;
         ax_hi = ax_lo;
         xs0 = ax_lo + S * C::AXSTAGE;
-        red0 = xs0 + S * C::XSTAGE;
+        red0 = xs0 + (XB ? kInlineSlice : S * C::XSTAGE);
         bars = red0 + C::RED_BYTES;
     }
     auto ax_stage = [&](int s) -> uint32_t {
@@ -289,7 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
                 if (it >= SQ) {
                     // a stage is freed by work that stands behind the dependency point: pass it first, so that
                     // the bounded wait does not run while the previous launch (however long) still works
-                    if (it == SQ) griddep_wait();
+                    if (!XB && it == SQ) griddep_wait();
                     if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1), status, 1)) { failed = true; break; }
                 }
                 const uint32_t bar = bar_q_full + 8 * sq;
@@ -329,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
     // Everything except the two streams of weights (packed codes, first factor tiles) waits here for
     // the previous launch to finish: a CTA that starts early sets up, prefetches and then stands still,
     // so every bounded wait below begins behind the dependency point.
-    if (warp != kTmaQWarp && warp != kTmaAWarp) griddep_wait();
+    if (!XB && warp != kTmaQWarp && warp != kTmaAWarp) griddep_wait();
 
     if (warp == kTmaQWarp) {
         // all done above
@@ -341,19 +357,20 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
             auto load_a = [&](int it) {
                 const int s = it % S, j0 = (ks_a + it) * kStep;
                 const uint32_t bar = bar_a_full + 8 * (it % kAF);
-                mbar_expect_tx(bar, tx_a + (uint32_t)(NTOK * kStep * 2));
+                mbar_expect_tx(bar, tx_a + (uint32_t)(XB ? 0 : NTOK * kStep * 2));
 #pragma unroll
                 for (int at = 0; at < kAtoms; ++at)
                     tma_load_2d(ax_stage(s) + at * kAtomBytes, &p.tm_a, j0 + at * 64, 0, bar);
             };
             auto load_x = [&](int it) {
+                if constexpr (XB > 0) return;
                 const int s = it % S;
                 tma_load_2d(xs0 + s * C::XSTAGE, &p.tm_x, (ks_a + it) * kStep, 0, bar_a_full + 8 * (it % kAF));
             };
             // the factors are weights: the first stages are filled before the dependency point
             const int pre = total < S ? total : S;
             for (int it = 0; it < pre; ++it) load_a(it);
-            griddep_wait();   // x may be the previous launch's output
+            if (!XB) griddep_wait();   // x may be the previous launch's output
             for (int it = 0; it < pre; ++it) load_x(it);
             for (int it = S; it < total; ++it) {
                 if (!mbar_wait<kWaitSlackNs>(bar_mma_done + 8 * ((it - S) % kAF), (uint32_t)(((it - S) / kAF) & 1), status, 2)) { failed = true; break; }
@@ -402,6 +419,15 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
         const int c16 = lane & 7, rsub = cw * 4 + (lane >> 3);
         constexpr int kRowStep = 4 * kConvGroupWarps;          // 16
         constexpr int kRowIters = kNMax / kRowStep;            // 4
+        if constexpr (XB > 0) {
+            // this CTA's slice of x, [k-step][token][128] bf16, zeros past column n
+            for (int c = tid - kConvWarp0 * 32; c < total * NTOK * 16; c += kConvGroups * kConvGroupWarps * 32) {
+                const int t = (c >> 4) % NTOK, col = (ks_a + (c >> 4) / NTOK) * kStep + (c & 15) * 8;
+                const uint4 v = args.x[col < p.n ? (t * p.n + col) >> 3 : 0];
+                sts_v4(xs0 + (uint32_t)(c * 16), col < p.n ? v : make_uint4(0u, 0u, 0u, 0u));
+            }
+            asm volatile("bar.sync 3, %0;" ::"n"(kConvGroups * kConvGroupWarps * 32) : "memory");
+        }
         for (int it = cgp; it < total; it += kConvGroups) {
             const int s = it % S;
             if (!__all_sync(0xffffffffu, mbar_wait(bar_a_full + 8 * (it % kAF), (uint32_t)((it / kAF) & 1), status, 5))) { failed = true; break; }
@@ -418,7 +444,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
 #pragma unroll
                 for (int t = 0; t < NTOK; ++t) {
                     // columns past n were filled with zeros by the tensor-map copy
-                    const uint4 xv = lds_v4(xs0 + s * C::XSTAGE + t * (kStep * 2) + at * 128 + c16 * 16);
+                    const uint4 xv = lds_v4(xs0 + (XB ? it * NTOK * kStep * 2 : s * C::XSTAGE) + t * (kStep * 2) + at * 128 + c16 * 16);
                     const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
@@ -552,6 +578,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
                 }
             }
             if (!ok) failed = true;
+            if (XB && rank == 0) griddep_wait();            // the previous launch's results come first
             if (csize == 1) {
                 if (ok && i < p.m)
 #pragma unroll
@@ -607,13 +634,14 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
 
 // One (code width, tokens, halves) instantiation: its launch attributes, how many clusters of each
 // size the device can hold at once, and the launch itself.
-template <int BITS, int NTOK, int H> struct DecodeVariant {
+template <int BITS, int NTOK, int H, int XB = 0> struct DecodeVariant {
+    static constexpr int SMEM = DCfg<BITS, H>::SMEM + (XB && BITS != 4 ? kInlineSlice : 0);
     static int prepare(int dev)
     {
         static bool done[kMaxDevices] = {};
         if (!done[dev]) {
-            auto kernel = lords_decode_kernel<BITS, NTOK, H>;
-            LORDS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DCfg<BITS, H>::SMEM));
+            auto kernel = lords_decode_kernel<BITS, NTOK, H, XB>;
+            LORDS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
             // cluster sizes above 8 are outside the portable range; they are used only where the
             // occupancy query below says such a cluster fits
             LORDS_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -634,7 +662,7 @@ template <int BITS, int NTOK, int H> struct DecodeVariant {
         cfg = cudaLaunchConfig_t{};
         cfg.gridDim = dim3((unsigned)(clusters * cs));
         cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = DCfg<BITS, H>::SMEM;
+        cfg.dynamicSmemBytes = SMEM;
         cfg.stream = stream;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
@@ -648,19 +676,19 @@ template <int BITS, int NTOK, int H> struct DecodeVariant {
             cudaLaunchAttribute attr[2];
             fill(cfg, attr, cs, 1, nullptr);
             int n = 0;
-            const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, lords_decode_kernel<BITS, NTOK, H>, &cfg);
+            const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, lords_decode_kernel<BITS, NTOK, H, XB>, &cfg);
             if (e != cudaSuccess) (void)cudaGetLastError();
             cache[dev][cs] = (e == cudaSuccess && n >= 1) ? n : -1;
         }
         return cache[dev][cs] > 0 ? cache[dev][cs] : 0;
     }
-    static int launch(const DecodeParams &k, int tiles, int cs, bool ordered, cudaStream_t stream)
+    static int launch(const DecodeArgs<XB> &k, int tiles, int cs, bool ordered, cudaStream_t stream)
     {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
         fill(cfg, attr, cs, tiles, stream);
         if (ordered) attr[1].val.programmaticStreamSerializationAllowed = 0;
-        LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_decode_kernel<BITS, NTOK, H>, k));
+        LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_decode_kernel<BITS, NTOK, H, XB>, k));
         return LORDS_OK;
     }
 };
@@ -689,7 +717,9 @@ template <int BITS, int NTOK, int H> int choose_cluster(int dev, int tiles, int 
     return cs;
 }
 
-template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem &p, const State &st, cudaStream_t stream)
+// x_host: null, or the activations to be carried by the launch (at most kInlineBytes); LORDS_ERR_UNSUPPORTED when a CTA's slice of them
+// is too large.
+template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem &p, const void *x_host, const State &st, cudaStream_t stream)
 {
     const int dev = device_slot(st), forced_cs = st.forced_splitk;
     const int qrow = DCfg<BITS, 1>::QROW;
@@ -703,6 +733,11 @@ template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem
     const int cs1 = choose_cluster<BITS, NTOK, 1>(dev, tiles1, k.ksteps, forced_cs, cost1);
     const int cs2 = choose_cluster<BITS, NTOK, 2>(dev, tiles2, k.ksteps, forced_cs, cost2);
     const bool two = cost2 < cost1;
+    if (x_host) {
+        if ((k.ksteps + (two ? cs2 : cs1) - 1) / (two ? cs2 : cs1) * NTOK * kStep * 2 > kInlineSlice) return LORDS_ERR_UNSUPPORTED;
+        rc = two ? DecodeVariant<BITS, NTOK, 2, kInlineBytes>::prepare(dev) : DecodeVariant<BITS, NTOK, 1, kInlineBytes>::prepare(dev);
+        if (rc != LORDS_OK) return rc;
+    }
     const uint64_t row_bytes = (uint64_t)p.n * BITS / 8;
     if (!make_map_2d(&k.tm_q, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, p.q, row_bytes, (uint64_t)p.m, (uint32_t)qrow,
                      two ? 256u : 128u, BITS == 4 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE) ||
@@ -712,15 +747,24 @@ template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem
                      CU_TENSOR_MAP_SWIZZLE_NONE))
         return LORDS_ERR_CUDA;
     k.tiles = two ? tiles2 : tiles1;
-    return two ? DecodeVariant<BITS, NTOK, 2>::launch(k, tiles2, cs2, p.ordered, stream)
-               : DecodeVariant<BITS, NTOK, 1>::launch(k, tiles1, cs1, p.ordered, stream);
+    if (x_host) {
+        DecodeArgs<kInlineBytes> args;
+        args.p = k;
+        memcpy(args.x, x_host, (size_t)p.M * p.n * 2);
+        return two ? DecodeVariant<BITS, NTOK, 2, kInlineBytes>::launch(args, tiles2, cs2, false, stream)
+                   : DecodeVariant<BITS, NTOK, 1, kInlineBytes>::launch(args, tiles1, cs1, false, stream);
+    }
+    DecodeArgs<0> args;
+    args.p = k;
+    return two ? DecodeVariant<BITS, NTOK, 2>::launch(args, tiles2, cs2, p.ordered, stream)
+               : DecodeVariant<BITS, NTOK, 1>::launch(args, tiles1, cs1, p.ordered, stream);
 }
 
 }  // namespace
 
 // Rules of this path: M <= 2 with M * ceil16(r) <= 64; n a multiple of 32 (4-bit), 64 (2-bit) or 128
 // (3-bit), which makes every TMA row pitch a multiple of 16 bytes.  Anything else: LORDS_ERR_UNSUPPORTED.
-int launch_decode(const Problem &p, State &st, cudaStream_t stream)
+static int run_decode(const Problem &p, const void *x_host, State &st, cudaStream_t stream)
 {
     if (!decode_takes(p)) return LORDS_ERR_UNSUPPORTED;
     const int r_pad = (p.r + 15) / 16 * 16;
@@ -731,13 +775,20 @@ int launch_decode(const Problem &p, State &st, cudaStream_t stream)
     k.y = p.y; k.y_f32 = p.y_f32;
     k.status = st.status_word;
     int rc;
-    if (p.bits == 4) rc = p.M == 1 ? launch_bits_tok<4, 1>(k, p, st, stream) : launch_bits_tok<4, 2>(k, p, st, stream);
-    else if (p.bits == 3) rc = p.M == 1 ? launch_bits_tok<3, 1>(k, p, st, stream) : launch_bits_tok<3, 2>(k, p, st, stream);
-    else rc = p.M == 1 ? launch_bits_tok<2, 1>(k, p, st, stream) : launch_bits_tok<2, 2>(k, p, st, stream);
+    if (p.bits == 4) rc = p.M == 1 ? launch_bits_tok<4, 1>(k, p, x_host, st, stream) : launch_bits_tok<4, 2>(k, p, x_host, st, stream);
+    else if (p.bits == 3) rc = p.M == 1 ? launch_bits_tok<3, 1>(k, p, x_host, st, stream) : launch_bits_tok<3, 2>(k, p, x_host, st, stream);
+    else rc = p.M == 1 ? launch_bits_tok<2, 1>(k, p, x_host, st, stream) : launch_bits_tok<2, 2>(k, p, x_host, st, stream);
     if (rc != LORDS_OK) return rc;
     st.last_launches = 1;
     st.last_path = "decode";
     return LORDS_OK;
+}
+
+int launch_decode(const Problem &p, State &st, cudaStream_t stream) { return run_decode(p, nullptr, st, stream); }
+
+int launch_decode_inline(const Problem &p, const void *x_host, State &st, cudaStream_t stream)
+{
+    return (size_t)p.M * p.n * 2 <= (size_t)kInlineBytes ? run_decode(p, x_host, st, stream) : LORDS_ERR_UNSUPPORTED;
 }
 
 }  // namespace lords

@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kFetchThreads) lords_fetch_host_kernel(const u
     if (t < (size_t)tail) reinterpret_cast<uint16_t *>(dst + n16)[t] = e;
 }
 
+// (Up to 8 KiB for the decode kernel: inside that kernel's own launch, lords_decode.cu; no staging at all.)
 // A still smaller x travels inside the launch itself: the call copies it from the (page-locked) host buffer into the
 // kernel's parameters, and the kernel stores it to the staging buffer.  No thread waits for a read across the bus,
 // which the fetch kernel above does once per call (4096 columns, one token, calls back to back: 14.2 us a call with the fetch kernel,
@@ -156,6 +157,8 @@ static int validate(const void *x, const uint8_t *q, const void *B, const void *
 //   - ranks above 64 with up to 16 tokens: the wide-rank kernel, or for small layers the direct kernel;
 //   - everything else: the direct kernel while token groups x weights stay under 32 M (4096 x 4094, 32 tokens: 28 us
 //     against 30; 37 tokens: 46 against 33), then the two-phase path; the CUDA cores for a handful of weights.
+static bool small_for_decode(const Problem &p) { return (long long)p.m * p.n <= (1 << 19); }
+
 static int dispatch(const Problem &p, State &st, cudaStream_t s)
 {
     switch (st.forced_path) {
@@ -172,7 +175,7 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
     const long long weights = (long long)p.m * p.n, grouped = (p.M + 15) / 16 * weights;
     int rc = LORDS_ERR_UNSUPPORTED;
     if (decode_takes(p)) {
-        if (weights <= (1 << 19)) {
+        if (small_for_decode(p)) {
             rc = launch_direct(p, st, s);
             if (rc == LORDS_OK) st.last_path = "decode";
         } else {
@@ -216,7 +219,7 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
 }
 
 static int forward_common(const void *x, const uint8_t *q, const void *B, const void *A, const float *cb,
-                          int bits, int M, int m, int n, int r, void *y, int y_f32, void *stream, int ordered = 0)
+                          int bits, int M, int m, int n, int r, void *y, int y_f32, void *stream, int ordered = 0, const void *x_host = nullptr)
 {
     int rc = validate(x, q, B, A, cb, bits, M, m, n, r, y);
     if (rc != LORDS_OK) return rc;
@@ -233,6 +236,11 @@ static int forward_common(const void *x, const uint8_t *q, const void *B, const 
     st.last_launches = 0;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
 
+    if (x_host) {
+        // x is in host memory: only the decode kernel can take it with the launch
+        const bool decode = decode_takes(p) && (st.forced_path == 2 || (st.forced_path == 0 && !small_for_decode(p)));
+        return decode ? launch_decode_inline(p, x_host, st, s) : LORDS_ERR_UNSUPPORTED;
+    }
     return dispatch(p, st, s);
 }
 
@@ -432,6 +440,10 @@ int lords_linear_forward_host(const void *x_host, const uint8_t *Qpacked, const 
     if (direct) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         const bool by_params = xb <= kParamHostBytes && cudaStreamIsCapturing(s, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+        if (by_params) {
+            rc = forward_common(st.stage_x, Qpacked, B, A, codebook, bits, M, m, n, r, y_map, 0, stream, 0, x_host);
+            if (rc != LORDS_ERR_UNSUPPORTED) return rc;
+        }
         if (!by_params) rc = fetch_host(x_map, st.stage_x, xb, s);
         else if (xb <= 2048) rc = stage_params<2048>(x_host, st.stage_x, xb, s);
         else if (xb <= 8192) rc = stage_params<8192>(x_host, st.stage_x, xb, s);

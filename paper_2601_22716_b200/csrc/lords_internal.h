@@ -89,6 +89,8 @@ int launch_dense(const Problem &p, State &st, cudaStream_t stream);
 // Tensor-core decode path (M <= 2), reassociated form with the scale factors folded into the
 // activation operand.  LORDS_ERR_UNSUPPORTED for shapes outside its rules.
 int launch_decode(const Problem &p, State &st, cudaStream_t stream);
+// The same with small activations carried by the launch itself (p.x is not read); LORDS_ERR_UNSUPPORTED when they do not fit.
+int launch_decode_inline(const Problem &p, const void *x_host, State &st, cudaStream_t stream);
 
 // Tensor-core decode path for 3 .. 16 tokens, scale-MMA form with 128-column k-steps.
 // LORDS_ERR_UNSUPPORTED for shapes outside its rules.

@@ -56,3 +56,24 @@ def test_ragged_lengths(lords, m, n, M):
     assert np.array_equal(yh.numpy().view(np.uint16), want)
     assert bool((room[M * m:] == 0x7FC0).all())
     assert lords.lords_poll_status() == 0
+
+
+@pytest.mark.parametrize("bits,m,n,r,M", [(4, 1024, 4096, 32, 1), (4, 4096, 2048, 20, 2), (3, 1300, 1152, 48, 1), (2, 3000, 1088, 16, 2), (4, 16500, 32, 8, 1),
+                                          (4, 140, 4064, 64, 1)])
+def test_x_carried_by_the_decode_launch(lords, bits, m, n, r, M):
+    """One or two tokens, up to 8 KiB: x travels with the decode launch, back to back calls keep their order."""
+    import torch
+    lay = gen.make_layer(m, n, r, M, bits=bits, seed=m + n)
+    dl = DeviceLayer(lay)
+    _, want = dl.forward()
+    args = (dl.q, dl.B, dl.A, lay.codebook, bits, M, lay.m, lay.n, lay.r)
+    xh = torch.from_numpy(lay.x.view(np.int16)).pin_memory()
+    zero = torch.zeros_like(xh).pin_memory()
+    yh = torch.full((M, lay.m), 0x7FC0, dtype=torch.int16).pin_memory()
+    for _ in range(20):                                   # the last call's y stays
+        lords.lords_linear_forward_host(zero, *args, yh)
+        lords.lords_linear_forward_host(xh, *args, yh)
+    assert lords.lords_last_path() == "decode" and lords.lords_last_launch_count() == 1
+    torch.cuda.synchronize()
+    assert np.array_equal(yh.numpy().view(np.uint16), want)
+    assert lords.lords_poll_status() == 0
