@@ -342,10 +342,11 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
     }
     // let a dependent launch (the next layer) begin its own weight prefetch as SMs become free
     griddep_launch_dependents();
-    // Everything except the two streams of weights (packed codes, first factor tiles) waits here for
-    // the previous launch to finish: a CTA that starts early sets up, prefetches and then stands still,
-    // so every bounded wait below begins behind the dependency point.
-    if (!XB && warp != kTmaQWarp && warp != kTmaAWarp) griddep_wait();
+    // What works on x waits here for the previous launch to finish.  What works on weights alone runs on: the streams of packed codes and
+    // factor tiles as far as their rings go, and the workers until the W ring is full (with the 16-token kernel: a block at one token 76.1 -> 75.0 us, at eight 89.6 -> 85.6).  Each passes the dependency point before its
+    // first wait for something that x is needed for, so that no bounded wait runs while the previous launch (however
+    // long) still works.
+    if (!XB && warp >= kConvWarp0 && warp < kTmaQWarp) griddep_wait();
 
     if (warp == kTmaQWarp) {
         // all done above
@@ -491,6 +492,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
 
         for (int it = g; it < total; it += kGroups) {
             const int sq = it % SQ, s = it % S;
+            if (!XB && it >= S && it < S + kGroups) griddep_wait();
             // the W slot is free once the MMAs of step it - S have completed
             if (it >= S && !__all_sync(0xffffffffu, mbar_wait(bar_mma_done + 8 * ((it - S) % kAF), (uint32_t)(((it - S) / kAF) & 1), status, 6))) { failed = true; break; }
             tc_fence_after_sync();
@@ -508,6 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
             }
         }
 
+        if (!XB) griddep_wait();
         // Epilogue (group 0): z (TMEM) . B row -> this CTA's partial y, parked in the cluster
         // leader's shared memory; the leader adds the cluster's partials in rank order.
         if (g == 0 && ch == 0) {

@@ -312,10 +312,10 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
     }
     // let a dependent launch (the next layer) begin its own weight prefetch as SMs become free
     griddep_launch_dependents();
-    // Everything except the stream of packed codes waits here for the previous launch to finish: a CTA
-    // that starts early sets up, prefetches its codes and then stands still, so that every bounded
-    // wait below begins behind the dependency point.
-    if (warp != kTmaQWarp) griddep_wait();
+    // What works on x waits here for the previous launch to finish.  What works on weights alone (codes, factor tiles, scale MMAs, workers)
+    // runs on until the W ring is full (a block at eight tokens 89.6 -> 85.6 us); each passes the dependency point before its first wait for something that x is needed
+    // for, so that no bounded wait runs while the previous launch (however long) still works.
+    if (warp == kTmaXWarp || (warp >= kConvWarp0 && warp < kScaleWarp0)) griddep_wait();
 
     if (warp == kTmaQWarp) {
         // all done above
@@ -329,6 +329,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             const uint32_t tx = (uint32_t)(2 * p.r_pad * 128);
             for (int it = 0; it < total; ++it) {
                 const int sa = it % C::SA;
+                if (it == (C::SA > WS ? C::SA : WS)) griddep_wait();
                 if (it >= C::SA && !mbar_wait<kWaitSlackNs>(bar_a_done + 8 * sa, (uint32_t)((it / C::SA - 1) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_a_full + 8 * sa;
                 mbar_expect_tx(bar, tx);
@@ -372,6 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         if (b_by_tma && sj < total && !mbar_wait(bar_b_full, 0)) failed = true;
         for (int it = sj; !BLOCK && it < total && !failed; it += 2) {
             const int sa = it % C::SA, sd = it % SD;
+            if (it >= WS && it < WS + 2) griddep_wait();
             if (!mbar_wait<kWaitSpin>(bar_a_full + 8 * sa, (uint32_t)((it / C::SA) & 1))) { failed = true; break; }
             if (it >= SD && !mbar_wait<kWaitSpin>(bar_s_empty + 8 * sd, (uint32_t)((it / SD - 1) & 1))) { failed = true; break; }
             tc_fence_after_sync();
@@ -448,6 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
 
         for (int it = g; it < total; it += 2) {
             const int sq = it % SQ, sd = it % SD, ws = it % WS;
+            if (it >= WS && it < WS + 2) griddep_wait();
             // S and the codes have landed, and the W slot is free: the MMAs of step it - WS have completed
             const uint32_t bar_first = BLOCK ? bar_q_full + 8 * sq : bar_s_full + 8 * sd, par_q = (uint32_t)((it / SQ) & 1);
             if (!mbar_wait_warp3(bar_first, BLOCK ? par_q : (uint32_t)((it / SD) & 1), bar_q_full + 8 * sq, par_q,
@@ -501,6 +504,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             }
         }
 
+        griddep_wait();
         // Epilogue (group 0, column half 0: one thread per row): the two accumulators -> this CTA's
         // partial y, parked in the cluster leader's shared memory; the leader adds in rank order.
         if (g == 0 && ch == 0 && !failed) {
