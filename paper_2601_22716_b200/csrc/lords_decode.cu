@@ -714,9 +714,9 @@ template <int BITS, int NTOK, int H> int choose_cluster(int dev, int tiles, int 
     const int resident = V::max_clusters(dev, cs) > 0 ? V::max_clusters(dev, cs) : 1;
     const int waves = (tiles + resident - 1) / resident;
     const int steps = (ksteps + cs - 1) / cs;
-    // a two-half step covers twice the rows in about 1.7 times the time of a one-half step, and every
-    // launch pays a fixed prologue + reduction worth a few steps
-    cost = (double)waves * ((double)steps * (H == 2 ? 1.7 : 1.0) + 2.0);
+    // a two-half step covers twice the rows in about 1.4 times the time of a one-half step (1400 cycles against 1000: converting the
+    // factor tile costs both the same), and every launch pays a fixed prologue + reduction worth a few steps
+    cost = (double)waves * ((double)steps * (H == 2 ? 1.4 : 1.0) + 2.0);
     return cs;
 }
 
