@@ -149,6 +149,9 @@ __global__ void lords_transpose_bf16_pair_kernel(const uint16_t *__restrict__ sr
                                                  int tiles0)
 {
     __shared__ uint16_t tile[32][33];
+    // A dependent launch on both sides: the next one (the pre-pass over the activations) may begin when all before this one has ended.
+    griddep_wait();
+    griddep_launch_dependents();
     const bool first = (int)blockIdx.x < tiles0;
     const uint16_t *src = first ? src0 : src1;
     uint16_t *dst = first ? dst0 : dst1;
@@ -1032,8 +1035,16 @@ int launch_transpose_bf16_pair(const uint16_t *src0, int rows0, int cols0, uint1
 {
     const long long t0 = (long long)((cols0 + 31) / 32) * ((rows0 + 31) / 32), t1 = (long long)((cols1 + 31) / 32) * ((rows1 + 31) / 32);
     if (t0 + t1 > 2147483647LL) return LORDS_ERR_SHAPE;
-    lords_transpose_bf16_pair_kernel<<<(unsigned)(t0 + t1), dim3(32, 8), 0, stream>>>(src0, dst0, rows0, cols0, src1, dst1, rows1, cols1, (int)t0);
-    LORDS_CUDA_TRY(cudaGetLastError());
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3((unsigned)(t0 + t1));
+    cfg.blockDim = dim3(32, 8);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_transpose_bf16_pair_kernel, src0, dst0, rows0, cols0, src1, dst1, rows1, cols1, (int)t0));
     return LORDS_OK;
 }
 

@@ -20,7 +20,7 @@ struct Problem {
     int bits, M, m, n, r;
     void *y;             // bf16 [M][m] or float [M][m]
     int y_f32;           // 1: store the fp32 accumulator
-    int ordered = 0;     // 1: the weights come from the launch just before: the first kernel must not begin ahead of its end
+    int ordered = 0;     // 1: the weights come from the launch just before (which lets a dependent launch begin when all before it has ended): nothing may read them ahead of its end
 };
 
 // Which calls the aligned tensor-core kernels take: TMA wants row pitches that are multiples of 16 bytes.

@@ -497,15 +497,18 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
 __global__ void lords_x_to_f16_kernel(const uint4 *__restrict__ x, uint4 *__restrict__ x16, size_t n_vec, const uint16_t *__restrict__ B,
                                       uint4 *__restrict__ b_pad, size_t b_vec, int r, int r8, int early)
 {
-    // Programmatic dependent launch on both sides (early != 0): the kernel that consumes x16 may begin its
+    // Programmatic dependent launch on both sides (early 1): the kernel that consumes x16 may begin its
     // set-up (weights only) at once; this kernel itself waits for the previous launch, which may still be
     // writing x or reading the scratch that x16 overwrites.  (Without the launch attribute both are no-ops.)
-    if (early) griddep_launch_dependents();
-    griddep_wait();
+    // early 2: the previous launch writes the factors, and let this one begin only when all before it had ended: x is converted beside it,
+    // and the consumer begins when both are done.
+    if (early == 1) griddep_launch_dependents();
+    if (early != 2) griddep_wait();
     size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= n_vec) {
         e -= n_vec;
         if (e >= b_vec) return;
+        if (early == 2) griddep_wait();
         const size_t row = e / (size_t)(r8 / 8);
         const int c = (int)(e % (size_t)(r8 / 8)) * 8;
         uint32_t w[4];
@@ -528,6 +531,10 @@ __global__ void lords_x_to_f16_kernel(const uint4 *__restrict__ x, uint4 *__rest
         out[q] = *reinterpret_cast<const uint32_t *>(&h);
     }
     x16[e] = make_uint4(out[0], out[1], out[2], out[3]);
+    if (early == 2) {
+        griddep_wait();
+        griddep_launch_dependents();
+    }
 }
 
 template <int BITS, int BN, int RP> struct UmmaVariant {
@@ -728,10 +735,10 @@ int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t s
     // A short pre-pass overlaps the main kernel's set-up (-2 us per call at 512 tokens); next to a long one
     // (2048 tokens x 14336 columns: 18 us at the HBM rate) the early main kernel's CTAs and weight prefetch
     // cost more than the overlap gains (+2 us), so there the main kernel starts when the pre-pass is done.
-    const int early = (size_t)p.M * p.n <= ((size_t)8 << 20) ? 1 : 0;
+    const int early = p.ordered ? 2 : (size_t)p.M * p.n <= ((size_t)8 << 20) ? 1 : 0;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = early && !p.ordered;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     cudaLaunchConfig_t cfg = cudaLaunchConfig_t{};
     cfg.gridDim = dim3((unsigned)((n_vec + b_vec + 255) / 256));
     cfg.blockDim = dim3(256);
