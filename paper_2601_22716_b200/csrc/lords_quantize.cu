@@ -32,6 +32,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "lords_internal.h"
 #include "lords_ptx.cuh"
 #include "lords_tc_common.cuh"
@@ -177,7 +179,8 @@ template <int BITS> __device__ __forceinline__ void store_codes(uint8_t *dst, co
     }
 }
 
-template <int BITS, int MODE, int RA>
+// EDGE: some tile reaches past the matrix (a variant of its own: the check costs the others 3 %).
+template <int BITS, int MODE, int RA, bool EDGE>
 __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __grid_constant__ QuantParams p)
 {
     using C = QuantCfg<BITS, RA>;
@@ -329,6 +332,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
             st += kGroupsQ;
             if (!mbar_wait_warp2(bar_s + 8 * sd, (uint32_t)((it / kSDQ) & 1), bar_w + 8 * sw, (uint32_t)((it / kSWQ) & 1), status, 35)) { failed = true; break; }
             tc_fence_after_sync();
+            const float past = EDGE && (i >= p.m || col0 >= p.n) ? 1.0f : 0.0f;
             uint32_t packed[BITS];
 #pragma unroll
             for (int k = 0; k < BITS; ++k) packed[k] = 0u;
@@ -359,14 +363,16 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                     }
                 };
                 if constexpr (MODE == kBuckets) {
-                    // a scale outside (2^-100, 2^100) (zero above all: code 0) takes the exact products, and so does the warp with it
+                    // a scale outside (2^-100, 2^100) (zero above all: code 0) takes the exact products, and so does the warp with it; rows and
+                    // columns past the matrix have scale zero and are not stored, so they have no say (6001 x 2048: the warps of the
+                    // last row tile were the whole call's tail, 35 us against 16)
                     float least = fabsf(__uint_as_float(s[0])), most = least;
 #pragma unroll
                     for (int c = 1; c < 16; ++c) {
                         least = fminf(least, fabsf(__uint_as_float(s[c])));
                         most = fmaxf(most, fabsf(__uint_as_float(s[c])));
                     }
-                    if (__all_sync(0xffffffffu, least > 7.8886e-31f && most < 1.2676e30f)) {
+                    if (__all_sync(0xffffffffu, (EDGE ? fmaxf(least, past) : least) > 7.8886e-31f && most < 1.2676e30f)) {
                         const uint64_t top2 = f32x2((float)(C::BUCKETS - 1), (float)(C::BUCKETS - 1)), magic2 = f32x2(8388608.0f, 8388608.0f);
                         float f[2];
                         pack([&](int c) {
@@ -454,12 +460,12 @@ __global__ void lords_quantize_simt_kernel(const uint16_t *__restrict__ W, const
     for (int b = 0; b < BYTES; ++b) dst[b] = b < 8 ? (uint8_t)(lo >> (8 * b)) : (uint8_t)(hi >> (8 * (b - 8)));
 }
 
-template <int BITS, int MODE, int RA> int launch_quantize_tc(QuantParams &k, const State &st, cudaStream_t stream)
+template <int BITS, int MODE, int RA, bool EDGE> int launch_quantize_tc(QuantParams &k, const State &st, cudaStream_t stream)
 {
     static bool done[kMaxDevices] = {};
     const int dev = device_slot(st);
     if (!done[dev]) {
-        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_quantize_kernel<BITS, MODE, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuantCfg<BITS, RA>::SMEM));
+        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_quantize_kernel<BITS, MODE, RA, EDGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuantCfg<BITS, RA>::SMEM));
         done[dev] = true;
     }
     // One run of steps per CTA that can be resident: setting a CTA up costs as much as about three steps, which a second round of CTAs
@@ -478,16 +484,20 @@ template <int BITS, int MODE, int RA> int launch_quantize_tc(QuantParams &k, con
         grid = (long long)k.row_tiles * k.row_splits;
     }
     if (grid > 2147483647LL) return LORDS_ERR_SHAPE;
-    lords_quantize_kernel<BITS, MODE, RA><<<(unsigned)grid, kThreadsQ, QuantCfg<BITS, RA>::SMEM, stream>>>(k);
+    lords_quantize_kernel<BITS, MODE, RA, EDGE><<<(unsigned)grid, kThreadsQ, QuantCfg<BITS, RA>::SMEM, stream>>>(k);
     LORDS_CUDA_TRY(cudaGetLastError());
     return LORDS_OK;
 }
 template <int BITS> int launch_quantize_tc(QuantParams &k, int mode, const State &st, cudaStream_t stream)
 {
-    if (k.r <= 64) return mode == kBuckets ? launch_quantize_tc<BITS, kBuckets, 64>(k, st, stream)
-                          : mode == kBisect ? launch_quantize_tc<BITS, kBisect, 64>(k, st, stream) : launch_quantize_tc<BITS, kTrial, 64>(k, st, stream);
-    return mode == kBuckets ? launch_quantize_tc<BITS, kBuckets, 128>(k, st, stream)
-           : mode == kBisect ? launch_quantize_tc<BITS, kBisect, 128>(k, st, stream) : launch_quantize_tc<BITS, kTrial, 128>(k, st, stream);
+    auto run = [&](auto ra) {
+        constexpr int RA = decltype(ra)::value;
+        if (mode == kBisect) return launch_quantize_tc<BITS, kBisect, RA, false>(k, st, stream);
+        if (mode == kTrial) return launch_quantize_tc<BITS, kTrial, RA, false>(k, st, stream);
+        return k.m % kRowsQ != 0 || k.n % kColsQ != 0 ? launch_quantize_tc<BITS, kBuckets, RA, true>(k, st, stream)
+                                                      : launch_quantize_tc<BITS, kBuckets, RA, false>(k, st, stream);
+    };
+    return k.r <= 64 ? run(std::integral_constant<int, 64>{}) : run(std::integral_constant<int, 128>{});
 }
 
 // The bucket table of an ascending level table.  Buckets are the rounding intervals of `buckets` equally spaced points that cover the
