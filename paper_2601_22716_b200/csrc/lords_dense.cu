@@ -529,14 +529,10 @@ template <int BN> int launch_product(GemmParams &k, const void *w16, const void 
     k.tok_tiles = (k.M + BN - 1) / BN;
     k.tiles = ((k.rows + kGRows - 1) / kGRows) * k.tok_tiles;
     k.ksteps = np / kGK;
-    // pairs: all that can be resident, but at least four k-steps each and about four pieces to a tile (a piece costs a trip
-    // through scratch, and the owner of the tile adds them up)
-    const long long total = (long long)k.tiles * k.ksteps;
-    long long pairs = total / 4 < k.tiles ? k.tiles : total / 4;
-    if (pairs > 4LL * k.tiles) pairs = 4LL * k.tiles;
-    if (pairs > pairs_max) pairs = pairs_max;
-    k.pairs = (int)pairs;
-    k.whole = whole_tiles(k.tiles, k.pairs);
+    // (a k-step is half a step of the pair kernel; 2816 x 3072, rank 100, 1024 tokens: 56 us a call with cut tiles, 45 with whole ones)
+    const Division division = divide_tiles(k.tiles, k.ksteps, pairs_max, 4, 2 * kMeetSteps);
+    k.pairs = division.pairs;
+    k.whole = division.whole;
     if (!make_map_2d(&k.tm_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, w16, (uint64_t)np, (uint64_t)k.rows, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, x16, (uint64_t)np, (uint64_t)k.M, 64, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;

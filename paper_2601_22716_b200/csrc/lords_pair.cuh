@@ -95,13 +95,41 @@ struct Schedule {
     }
 };
 
-// Tiles that run unsplit: whole waves, less one where the tiles left over are few.  Cut into a share for every pair, a few tiles
-// would be many pieces each, which their owners add up one after the other (two tiles over 74 pairs, 37 pieces each: 209 us a call
-// at 14336 x 4096, 1024 tokens, where two thirds of that are due); with a wave more to cut, a tile is two or three pieces.
-inline int whole_tiles(int tiles, int pairs)
+// The division of `tiles` tiles of `steps` steps among at most `pairs_max` CTA pairs: how many pairs, and how many tiles run unsplit,
+// one per pair and wave; the steps of the others are dealt out evenly.  The pieces of a tile meet in scratch, so tiles are cut only
+// where that takes more than `meet` steps off the busiest pair (4096 x 4096, 2048 tokens, 128 tiles over 74 pairs: 77 us cut, 67 in
+// two waves).  Few tiles left over are cut together with a whole wave: by themselves they would be many pieces each, which their
+// owners add up one after the other (two tiles over 74 pairs, 37 pieces each: 209 us a call at 14336 x 4096, 1024 tokens, where
+// two thirds of that are due).
+// 20: on four layer shapes at 64 to 2048 tokens, two waves against cut tiles, uncut was the faster or level where cutting saved 4 to
+// 21.6 steps (by 1 to 20 %; 14336 x 4096 at 384 tokens lost 2 %), and the slower where it saved 22.5 and more.
+constexpr double kMeetSteps = 20.0;      // steps of 128 columns
+struct Division {
+    int pairs, whole;
+    double per_pair;      // steps that the busiest pair does
+};
+inline Division divide_tiles(int tiles, int steps, int pairs_max, int least_steps, double meet)
 {
-    const int whole = tiles / pairs * pairs, left = tiles - whole;
-    return left > 0 && whole > 0 && 3 * left < pairs ? whole - pairs : whole;
+    Division d;
+    const long long total = (long long)tiles * steps;
+    const double uncut = (double)((tiles + pairs_max - 1) / pairs_max) * steps;
+    // cut: all pairs that can be resident, but at least `least_steps` each and about four pieces to a tile
+    long long pairs = total / least_steps < tiles ? tiles : total / least_steps;
+    if (pairs > 4LL * tiles) pairs = 4LL * tiles;
+    if (pairs > pairs_max) pairs = pairs_max;
+    const double cut = (double)total / (double)pairs;
+    if (uncut <= cut + meet) {
+        d.pairs = tiles < pairs_max ? tiles : pairs_max;
+        d.whole = tiles;
+        d.per_pair = uncut;
+        return d;
+    }
+    d.pairs = (int)pairs;
+    d.whole = tiles / d.pairs * d.pairs;
+    const int left = tiles - d.whole;
+    if (left > 0 && d.whole > 0 && 3 * left < d.pairs) d.whole -= d.pairs;
+    d.per_pair = cut;
+    return d;
 }
 
 // A warp's last act on a piece.  A piece that went to scratch: one count on its flag, which is complete at `warps`.  A tile's owner:

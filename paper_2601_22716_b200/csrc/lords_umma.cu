@@ -25,6 +25,7 @@
 
 #include "lords_dequant.cuh"
 #include "lords_internal.h"
+#include "lords_pair.cuh"
 #include "lords_ptx.cuh"
 #include "lords_tc_common.cuh"
 
@@ -680,11 +681,11 @@ int token_tile(const Problem &p, const State &st)
 }
 
 // Whether the kernel on CTA pairs is the faster one: it does a step of 128 columns in about the time that this one needs for a
-// k-step of 64, but divides the work into fewer, larger tiles, and its set-up and its pieces' meeting in scratch cost about
-// 14 us more, so that it takes the large calls (14336 x 4096, 512 tokens: 69 us against 78; 4096 x 14336, 64 tokens: 36
-// against 59; 4096 x 4096, 512 tokens: 35 against 28).  The two estimates below, in microseconds, are least-squares fits to both
-// kernels' times on five layer shapes at 64 to 1536 tokens (within 18 % of every one of them; the faster kernel is chosen to
-// within 2.5 %).
+// k-step of 64, but divides the work into fewer, larger tiles, and where it cuts them, the meeting of the pieces costs about 15 us,
+// so that it takes the large calls (14336 x 4096, 512 tokens: 68 us against 78; 4096 x 14336, 64 tokens: 38 against 59;
+// 4096 x 4096: 32 against 28 at 512 tokens, 34 against 40 at 1024).  The two estimates below, in microseconds, are least-squares fits to
+// the kernels' times on four layer shapes at 64 to 2048 tokens.  The one for pairs is off by up to 25 %, most where both are short,
+// but on those shapes no call gets a kernel more than 2 % slower than the other.
 bool prefer_pair(const Problem &p, const State &st)
 {
     const double rank = p.r > 32 ? 1.0 : 0.0;
@@ -697,12 +698,10 @@ bool prefer_pair(const Problem &p, const State &st)
     const double single = 2.9 + (halves ? 4.8 : 0.0) + (0.319 + 0.0011 * bn + 0.015 * rank) * ksteps * waves;
 
     const long long tok_tiles = (p.M + 255) / 256, bn2 = ((p.M + tok_tiles - 1) / tok_tiles + 31) / 32 * 32;
-    const long long tiles2 = (long long)((p.m + 255) / 256) * tok_tiles, steps = (p.n + 127) / 128, total = tiles2 * steps;
-    long long pairs = total / 2 < tiles2 ? tiles2 : total / 2;
-    if (pairs > 4 * tiles2) pairs = 4 * tiles2;
-    if (pairs > sms / 2) pairs = sms / 2;
-    const bool whole = tiles2 % pairs == 0;
-    const double paired = 9.6 + (whole ? 0.0 : 9.6) + (0.0039 * (double)bn2 - 0.077 + 0.163 * rank) * (double)total / (double)pairs;
+    const long long tiles2 = (long long)((p.m + 255) / 256) * tok_tiles;
+    if (tiles2 > 0x3fffffffLL) return false;
+    const Division d = divide_tiles((int)tiles2, (p.n + 127) / 128, (int)(sms / 2), 2, kMeetSteps);
+    const double paired = 2.4 + (d.whole < (int)tiles2 ? 15.0 : 0.0) + (0.436 + 0.0021 * (double)bn2 + 0.097 * rank) * d.per_pair;
     return paired < single;
 }
 

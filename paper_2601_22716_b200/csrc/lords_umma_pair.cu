@@ -437,19 +437,14 @@ template <int BITS, int RP> int launch_pair_variant(const Problem &p, State &st,
     const long long row_tiles = (p.m + kPRows - 1) / kPRows, tiles = row_tiles * k.tok_tiles;
     if (tiles > 0x3fffffffLL) return LORDS_ERR_UNSUPPORTED;
     k.tiles = (int)tiles;
-    // pairs: all that can be resident, but at least two steps each and about four pieces to a tile (a piece costs a trip through
-    // scratch, and the owner of the tile adds them up)
-    const long long total = tiles * k.steps;
-    long long pairs = total / 2 < tiles ? tiles : total / 2;
-    if (pairs > 4 * tiles) pairs = 4 * tiles;
-    if (pairs > pairs_max) pairs = pairs_max;
-    k.pairs = (int)pairs;
-    k.whole = whole_tiles(k.tiles, k.pairs);
+    const Division division = divide_tiles(k.tiles, k.steps, pairs_max, 2, kMeetSteps);
+    k.pairs = division.pairs;
+    k.whole = division.whole;
     auto up = [](size_t b) { return (b + 1023) & ~(size_t)1023; };
     const int r8 = (p.r + 7) / 8 * 8;
     const bool pad_b = r8 != p.r;
     const size_t x_bytes = up((size_t)p.M * p.n * 2), b_bytes = pad_b ? up((size_t)p.m * r8 * 2) : 0;
-    const size_t part_bytes = (size_t)pairs * 2 * k.bn * 128 * sizeof(float);
+    const size_t part_bytes = (size_t)k.pairs * 2 * k.bn * 128 * sizeof(float);
     if (x_bytes + b_bytes + part_bytes > st.workspace_bytes) return LORDS_ERR_WORKSPACE;
     void *const b_pad = pad_b ? st.workspace + x_bytes : nullptr;
     int rc = launch_umma_prepass(p, st.workspace, b_pad, stream);

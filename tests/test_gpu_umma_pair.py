@@ -53,3 +53,21 @@ def test_pair_kernel_shapes(lords, bits, m, n, r, M, mixed):
     assert np.array_equal(y32, again[0]) and np.array_equal(ybf, again[1])
     assert lords.lords_poll_status() == 0
     check_against_oracle(y32, ybf, oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits))
+
+
+@pytest.mark.parametrize("path", ["pair", "dense"])
+@pytest.mark.parametrize("bits,m,n,r,M", [
+    (4, 5000, 512, 32, 1100),       # two waves of whole tiles, the last one partial
+    (3, 5000, 4224, 8, 1100),       # a whole wave, the tiles left over cut
+    (4, 4700, 2880, 16, 1000),      # few tiles more than a wave: all of them cut
+])
+def test_division_of_tiles(lords, path, bits, m, n, r, M):
+    lay = gen.make_layer(m, n, r, M, bits=bits, seed=m + n + r + M)
+    lords.lords_set_option("path", path)
+    try:
+        dl = DeviceLayer(lay)
+        y32, ybf = dl.forward()
+    finally:
+        lords.lords_set_option("path", "auto")
+    assert lords.lords_poll_status() == 0
+    check_against_oracle(y32, ybf, oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits))
