@@ -29,8 +29,9 @@
 //
 // Rows of W or A that are not 16-byte multiples (n not a multiple of 8) are copied to padded rows in the workspace first; without
 // room there, and for small layers off the tile grid, a plain CUDA-core kernel runs.
-// That kernel compares squared errors, this one midpoints: both round in fp32, and a weight whose two nearest levels are equally far to
-// within that rounding (2e-7 of |W|; 10 bytes in 28.8 M at most, 5472 x 10524) can get the other of the two.
+// That kernel sums S on the CUDA cores and compares squared errors, this one midpoints: both round in fp32, and a weight whose two nearest
+// levels are equally far to within that rounding can get the other of the two (5472 x 10524, r = 6: 10 bytes in 28.8 M at most, the
+// two errors 2e-7 of |W| apart).
 #include <cuda.h>
 #include <cuda_bf16.h>
 
