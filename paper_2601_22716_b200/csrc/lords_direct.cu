@@ -1,17 +1,25 @@
 // Direct path for few tokens: W^ = L[Q] (.) (BA) is formed in registers and multiplied there.
 //
 // A warp owns 16 rows of W^.  Per 32 columns it forms S = B A with warp-level MMAs (Eq. 3; bf16 operands, fp32 sums),
-// turns the sums into fp16 pairs, multiplies them by the level pairs of the codes (lane-private table) and
-// feeds the products straight to the next MMA as its left operand: the accumulator layout of one MMA is the
-// operand layout of the other, so nothing of W^ leaves the register file, and there is no hand-over between
-// warps but one barrier per 64-column strip.  Rows need no alignment and any rank goes.
+// multiplies them by the levels of the codes (lane-private table) and feeds the products straight to the next MMA as its
+// left operand: the accumulator layout of one MMA is the operand layout of the other, so nothing of W^ leaves the
+// register file, and there is no hand-over between warps but one barrier per 64-column strip.  Rows need no
+// alignment and any rank goes.
+//
+// Two forms.  Layers that the 16-token and the scale-MMA kernel take as well have the operands of those kernels: S, the levels, W^ and x
+// in fp16.  All others (EXACT: ragged rows, ranks above 64; and one or two tokens) hold S, the levels and W^ in fp32, as the CUDA-core
+// path does: W^ enters the product as three bf16 parts, x as it is.  Tensor cores cut sums off instead of rounding
+// them, so S of every 16 ranks and the first parts' products of every 16 columns start from zero and are added on the
+// CUDA cores; the lower parts' products, 2^-8 of the sum, keep to the tensor cores.  Error of the fp32 sums
+// against 64 bits, norms, normal activations, 256 x 256 to 1024 x 14336, ranks 4 to 128: 6e-8 to 1.7e-7 (CUDA cores 8e-8 to 1.6e-7; the
+// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 16.0 us a call (fp16 form 10.7, CUDA cores 67.6).
 //
 // A cluster shares one tile of 128 rows and splits its columns; every CTA sends its partial sums to the CTA that owns
 // the row (asynchronous stores counted on that CTA's barrier), which adds them in rank order: deterministic,
 // no atomics, no trip through global memory.  Tokens beyond sixteen are further groups of CTAs (grid y).
 //
-// Bound: warp instructions -- four per code pair for the table and the product, the MMAs (2 RK + M / 8 per 16 x 16
-// weights at the warp-level rate) and the loads around them; codes, factors and activations come by
+// Bound: warp instructions -- four per code pair for the table and the product (EXACT: about twenty), the MMAs (2 RK + M / 8, or
+// 3 M / 8, per 16 x 16 weights at the warp-level rate) and the loads around them; codes, factors and activations come by
 // asynchronous copies several strips ahead.  CTAs are small (eight warps, under 110 KB), so that two or more share an SM
 // and the next call's CTAs load their weights while this call computes (programmatic dependent launch).
 #include <cuda.h>
@@ -38,13 +46,14 @@ constexpr int kAPitch = kCols * 2 + 16;             // bytes per rank (or token)
 constexpr int kQPitch = 48;                         // bytes per code row: eight rows in eight different 16-byte bank groups
 
 // BITS: code width.  RK: rank in steps of 16 (zero padded).  MT: tokens (8 or 16, zero padded).
-template <int BITS, int RK, int MT> struct DirCfg {
-    static constexpr int ENTRIES = BITS == 4 ? 256 : BITS == 3 ? 64 : 16;     // level pairs
-    static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair
+template <int BITS, int RK, int MT, bool EXACT> struct DirCfg {
+    static constexpr int ENTRIES = EXACT ? 1 << BITS : 1 << 2 * BITS;         // levels, or level pairs
+    static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every entry
     static constexpr int SA = RK <= 4 ? 3 : 2;                                // strips of A and x in flight
     static constexpr int SQ = 4;                                              // strips of codes in flight
     static constexpr int ASTAGE = RK * 16 * kAPitch;
-    static constexpr int XSTAGE = MT * kAPitch;
+    static constexpr int XPART = MT * kAPitch;
+    static constexpr int XSTAGE = EXACT ? 2 * XPART : XPART;                  // EXACT: x, and x without infinities and NaNs
     static constexpr int QSTAGE = kRows * kQPitch;
     static constexpr int RED = (kRows + kClusterMax) * MT * 4;                // partial sums received: cluster x rows owned x tokens
     static constexpr int SMEM = LUT + SA * ASTAGE + 3 * XSTAGE + SQ * QSTAGE + RED + 16;
@@ -71,10 +80,10 @@ __device__ __forceinline__ void st_async_cluster_2f32(uint32_t addr, float a, fl
                  ::"r"(addr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(bar) : "memory");
 }
 
-template <int BITS, int RK, int MT, bool ALIGNED>
-__global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel(const DirectParams p)
+template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT>
+__global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direct_kernel(const DirectParams p)
 {
-    using C = DirCfg<BITS, RK, MT>;
+    using C = DirCfg<BITS, RK, MT, EXACT>;
     constexpr int TG = MT / 8;                      // groups of eight tokens
     extern __shared__ __align__(1024) uint8_t dir_smem[];
     const uint32_t lut = smem_u32(dir_smem);
@@ -177,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
             }
         }
     };
-    // activations: eight columns of one token per thread, bf16 -> fp16 on the way (registers one strip ahead)
+    // activations: eight columns of one token per thread, converted on the way (registers one strip ahead)
     constexpr int XT = MT * (kCols / 8);             // threads that take part (64 or 128)
     const int xt = tid / (kCols / 8), xc = tid % (kCols / 8) * 8;
     auto load_x = [&](int it, uint32_t (&v)[4]) {
@@ -199,13 +208,19 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
     };
     auto store_x = [&](int it, const uint32_t (&v)[4]) {
         if (tid < XT) {
+            const uint32_t dst = x_s + (uint32_t)((it % 3) * C::XSTAGE + xt * kAPitch + xc * 2);
             uint32_t o[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const __half2 h = __floats2half2_rn(__uint_as_float(v[k] << 16), __uint_as_float(v[k] & 0xFFFF0000u));
-                o[k] = *reinterpret_cast<const uint32_t *>(&h);
+                if constexpr (EXACT) {
+                    o[k] = finite_pair(v[k]);
+                } else {
+                    const __half2 h = __floats2half2_rn(__uint_as_float(v[k] << 16), __uint_as_float(v[k] & 0xFFFF0000u));
+                    o[k] = *reinterpret_cast<const uint32_t *>(&h);
+                }
             }
-            sts_v4(x_s + (uint32_t)((it % 3) * C::XSTAGE + xt * kAPitch + xc * 2), make_uint4(o[0], o[1], o[2], o[3]));
+            if constexpr (EXACT) sts_v4(dst, make_uint4(v[0], v[1], v[2], v[3]));
+            sts_v4(dst + (EXACT ? C::XPART : 0), make_uint4(o[0], o[1], o[2], o[3]));
         }
     };
 
@@ -221,10 +236,15 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
     stage_a(1); commit();
     if constexpr (ALIGNED) stage_q(2);
     commit();
-    // level pairs: one entry per thread, its 32 copies as eight 16-byte stores that rotate over the banks
+    // levels or level pairs: one entry per thread, its 32 copies as eight 16-byte stores that rotate over the banks
     if (tid < C::ENTRIES) {
-        const __half2 h = __floats2half2_rn(p.levels[tid & ((1 << BITS) - 1)], p.levels[tid >> BITS]);
-        const uint32_t v = *reinterpret_cast<const uint32_t *>(&h);
+        uint32_t v;
+        if constexpr (EXACT) {
+            v = __float_as_uint(p.levels[tid]);
+        } else {
+            const __half2 h = __floats2half2_rn(p.levels[tid & ((1 << BITS) - 1)], p.levels[tid >> BITS]);
+            v = *reinterpret_cast<const uint32_t *>(&h);
+        }
 #pragma unroll
         for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(v, v, v, v));
     }
@@ -244,9 +264,11 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
     store_x(0, xv);
     load_x(1, xv);
 
-    float acc[TG][4];
+    float acc[TG][4], low[EXACT ? TG : 1][4];        // low: the sums of the weights' lower parts
 #pragma unroll
     for (int k = 0; k < TG; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.0f;
+#pragma unroll
+    for (int k = 0; k < (EXACT ? TG : 1); ++k) low[k][0] = low[k][1] = low[k][2] = low[k][3] = 0.0f;
     const uint32_t lut_lane = lut + 4u * (uint32_t)lane;
 
     for (int it = 0; it < total; ++it) {
@@ -273,6 +295,9 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
                     if (k == 0) {
                         mma_bf16_first(s[2 * h], bf[k], v[0], v[1]);
                         mma_bf16_first(s[2 * h + 1], bf[k], v[2], v[3]);
+                    } else if constexpr (EXACT) {
+                        add_mma_bf16(s[2 * h], bf[k], v[0], v[1]);
+                        add_mma_bf16(s[2 * h + 1], bf[k], v[2], v[3]);
                     } else {
                         mma_bf16(s[2 * h], bf[k], v[0], v[1]);
                         mma_bf16(s[2 * h + 1], bf[k], v[2], v[3]);
@@ -281,18 +306,38 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
             CodeWords<BITS> w0, w1;
             w0.read(q_row + (uint32_t)(c * 4 * BITS));
             w1.read(q_row + (uint32_t)(8 * kQPitch + c * 4 * BITS));
-            uint32_t xb[TG][4];
+            uint32_t xb[TG][4], xf[EXACT ? TG : 1][4];
+            const uint32_t x_lane = x_tile + (uint32_t)((lane & 7) * kAPitch + c * 64 + (lane >> 3) * 16);
 #pragma unroll
-            for (int k = 0; k < TG; ++k) ldmatrix_x4(x_tile + (uint32_t)((k * 8 + (lane & 7)) * kAPitch + c * 64 + (lane >> 3) * 16), xb[k]);
+            for (int k = 0; k < TG; ++k) {
+                ldmatrix_x4(x_lane + (uint32_t)(k * 8 * kAPitch), xb[k]);
+                if constexpr (EXACT) ldmatrix_x4(x_lane + (uint32_t)(C::XPART + k * 8 * kAPitch), xf[k]);
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                uint32_t wa[4];
-                wa[0] = scaled_pair(lds_table(w0.address(2 * h, t, lut_lane)), s[2 * h][0], s[2 * h][1]);
-                wa[1] = scaled_pair(lds_table(w1.address(2 * h, t, lut_lane)), s[2 * h][2], s[2 * h][3]);
-                wa[2] = scaled_pair(lds_table(w0.address(2 * h + 1, t, lut_lane)), s[2 * h + 1][0], s[2 * h + 1][1]);
-                wa[3] = scaled_pair(lds_table(w1.address(2 * h + 1, t, lut_lane)), s[2 * h + 1][2], s[2 * h + 1][3]);
+                if constexpr (EXACT) {
+                    float w[8];
+                    w0.weights(2 * h, t, lut_lane, s[2 * h][0], s[2 * h][1], w[0], w[1]);
+                    w1.weights(2 * h, t, lut_lane, s[2 * h][2], s[2 * h][3], w[2], w[3]);
+                    w0.weights(2 * h + 1, t, lut_lane, s[2 * h + 1][0], s[2 * h + 1][1], w[4], w[5]);
+                    w1.weights(2 * h + 1, t, lut_lane, s[2 * h + 1][2], s[2 * h + 1][3], w[6], w[7]);
+                    uint32_t hi[4], mid[4], lo[4];
+                    split_weights(w, hi, mid, lo);
 #pragma unroll
-                for (int k = 0; k < TG; ++k) mma_f16(acc[k], wa, xb[k][2 * h], xb[k][2 * h + 1]);
+                    for (int k = 0; k < TG; ++k) {
+                        add_mma_bf16(acc[k], hi, xb[k][2 * h], xb[k][2 * h + 1]);
+                        mma_bf16(low[k], mid, xf[k][2 * h], xf[k][2 * h + 1]);
+                        mma_bf16(low[k], lo, xf[k][2 * h], xf[k][2 * h + 1]);
+                    }
+                } else {
+                    uint32_t wa[4];
+                    wa[0] = scaled_pair(lds_table(w0.address(2 * h, t, lut_lane)), s[2 * h][0], s[2 * h][1]);
+                    wa[1] = scaled_pair(lds_table(w1.address(2 * h, t, lut_lane)), s[2 * h][2], s[2 * h][3]);
+                    wa[2] = scaled_pair(lds_table(w0.address(2 * h + 1, t, lut_lane)), s[2 * h + 1][0], s[2 * h + 1][1]);
+                    wa[3] = scaled_pair(lds_table(w1.address(2 * h + 1, t, lut_lane)), s[2 * h + 1][2], s[2 * h + 1][3]);
+#pragma unroll
+                    for (int k = 0; k < TG; ++k) mma_f16(acc[k], wa, xb[k][2 * h], xb[k][2 * h + 1]);
+                }
             }
         }
         if constexpr (C::SA == 2) {
@@ -302,6 +347,12 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
+    if constexpr (EXACT) {
+#pragma unroll
+        for (int k = 0; k < TG; ++k)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[k][e] += low[k][e];
+    }
 
     // ---- partial sums: lane holds rows g, g + 8 of the warp's tile, tokens 2t, 2t + 1 of each group
     bool failed = false;
@@ -343,8 +394,8 @@ __global__ void __launch_bounds__(kThreads, RK <= 4 ? 3 : 2) lords_direct_kernel
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
-template <int BITS, int RK, int MT, bool ALIGNED> struct DirectVariant {
-    using C = DirCfg<BITS, RK, MT>;
+template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirectVariant {
+    using C = DirCfg<BITS, RK, MT, EXACT>;
     static void fill(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int cs, int tiles, int groups, cudaStream_t stream)
     {
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -366,7 +417,7 @@ template <int BITS, int RK, int MT, bool ALIGNED> struct DirectVariant {
     {
         static int cache[kMaxDevices][kClusterMax + 1];   // 0 = not asked yet, -1 = cannot run
         if (cache[dev][cs] == 0) {
-            auto kernel = lords_direct_kernel<BITS, RK, MT, ALIGNED>;
+            auto kernel = lords_direct_kernel<BITS, RK, MT, ALIGNED, EXACT>;
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute attr[2];
             fill(cfg, attr, cs, 1, 1, nullptr);
@@ -404,26 +455,32 @@ template <int BITS, int RK, int MT, bool ALIGNED> struct DirectVariant {
         cudaLaunchAttribute attr[2];
         fill(cfg, attr, cs, tiles, groups, stream);
         if (ordered) attr[1].val.programmaticStreamSerializationAllowed = 0;
-        LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_direct_kernel<BITS, RK, MT, ALIGNED>, k));
+        LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_direct_kernel<BITS, RK, MT, ALIGNED, EXACT>, k));
         return LORDS_OK;
     }
 };
 
-template <int BITS, int RK, int MT> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
+template <int BITS, int RK, int MT, bool EXACT> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
     const size_t row_bytes = (size_t)p.n * BITS / 8;
     const bool aligned = row_bytes % (BITS == 3 ? 8 : 16) == 0 && p.n % 8 == 0;
     const int tiles = (p.m + kRows - 1) / kRows;
-    return aligned ? DirectVariant<BITS, RK, MT, true>::launch(k, tiles, p.ordered, st.forced_splitk, st, stream)
-                   : DirectVariant<BITS, RK, MT, false>::launch(k, tiles, p.ordered, st.forced_splitk, st, stream);
+    if constexpr (EXACT)
+        if (!aligned) return DirectVariant<BITS, RK, MT, false, true>::launch(k, tiles, p.ordered, st.forced_splitk, st, stream);
+    // the fp16 form: n is a multiple of 64 (128 for 3 bits), so its rows are aligned
+    return DirectVariant<BITS, RK, MT, true, EXACT>::launch(k, tiles, p.ordered, st.forced_splitk, st, stream);
 }
-template <int BITS, int RK> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
+template <int BITS, int RK, bool EXACT> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
-    return p.M <= 8 ? launch_direct<BITS, RK, 8>(k, p, st, stream) : launch_direct<BITS, RK, 16>(k, p, st, stream);
+    return p.M <= 8 ? launch_direct<BITS, RK, 8, EXACT>(k, p, st, stream) : launch_direct<BITS, RK, 16, EXACT>(k, p, st, stream);
 }
 template <int BITS> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
-    return p.r <= 32 ? launch_direct<BITS, 2>(k, p, st, stream) : p.r <= 64 ? launch_direct<BITS, 4>(k, p, st, stream) : launch_direct<BITS, 8>(k, p, st, stream);
+    // fp16 operands only where the kernel this one stands in for has them (decode16, umma): what else ran on the CUDA cores in fp32, or,
+    // with one or two tokens, on the reassociated form, keeps that range and precision
+    if (umma_takes(p) && !decode_takes(p)) return p.r <= 32 ? launch_direct<BITS, 2, false>(k, p, st, stream) : launch_direct<BITS, 4, false>(k, p, st, stream);
+    return p.r <= 32 ? launch_direct<BITS, 2, true>(k, p, st, stream)
+                     : p.r <= 64 ? launch_direct<BITS, 4, true>(k, p, st, stream) : launch_direct<BITS, 8, true>(k, p, st, stream);
 }
 
 }  // namespace
