@@ -12,13 +12,13 @@
 // them, so S of every 16 ranks and the first parts' products of every 16 columns start from zero and are added on the
 // CUDA cores; the lower parts' products, 2^-8 of the sum, keep to the tensor cores.  Error of the fp32 sums
 // against 64 bits, norms, normal activations, 256 x 256 to 1024 x 14336, ranks 4 to 128: 6e-8 to 1.7e-7 (CUDA cores 8e-8 to 1.6e-7; the
-// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 16.0 us a call (fp16 form 10.7, CUDA cores 67.6).
+// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 17.0 us a call (fp16 form 10.7, CUDA cores 67.6).
 //
 // A cluster shares one tile of 128 rows and splits its columns; every CTA sends its partial sums to the CTA that owns
 // the row (asynchronous stores counted on that CTA's barrier), which adds them in rank order: deterministic,
 // no atomics, no trip through global memory.  Tokens beyond sixteen are further groups of CTAs (grid y).
 //
-// Bound: warp instructions -- four per code pair for the table and the product (EXACT: about twenty), the MMAs (2 RK + M / 8, or
+// Bound: warp instructions -- four per code pair for the table and the product (EXACT: some twenty), the MMAs (2 RK + M / 8, or
 // 3 M / 8, per 16 x 16 weights at the warp-level rate) and the loads around them; codes, factors and activations come by
 // asynchronous copies several strips ahead.  CTAs are small (eight warps, under 110 KB), so that two or more share an SM
 // and the next call's CTAs load their weights while this call computes (programmatic dependent launch).
@@ -47,8 +47,8 @@ constexpr int kQPitch = 48;                         // bytes per code row: eight
 
 // BITS: code width.  RK: rank in steps of 16 (zero padded).  MT: tokens (8 or 16, zero padded).
 template <int BITS, int RK, int MT, bool EXACT> struct DirCfg {
-    static constexpr int ENTRIES = EXACT ? 1 << BITS : 1 << 2 * BITS;         // levels, or level pairs
-    static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every entry
+    static constexpr int ENTRIES = 1 << 2 * BITS;                             // level pairs
+    static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair (EXACT: 16 of 8 bytes)
     static constexpr int SA = RK <= 4 ? 3 : 2;                                // strips of A and x in flight
     static constexpr int SQ = 4;                                              // strips of codes in flight
     static constexpr int ASTAGE = RK * 16 * kAPitch;
@@ -56,7 +56,7 @@ template <int BITS, int RK, int MT, bool EXACT> struct DirCfg {
     static constexpr int XSTAGE = EXACT ? 2 * XPART : XPART;                  // EXACT: x, and x without infinities and NaNs
     static constexpr int QSTAGE = kRows * kQPitch;
     static constexpr int RED = (kRows + kClusterMax) * MT * 4;                // partial sums received: cluster x rows owned x tokens
-    static constexpr int SMEM = LUT + SA * ASTAGE + 3 * XSTAGE + SQ * QSTAGE + RED + 16;
+    static constexpr int SMEM = LUT + SA * ASTAGE + 2 * XSTAGE + SQ * QSTAGE + RED + 16;
 };
 
 struct DirectParams {
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     constexpr int TG = MT / 8;                      // groups of eight tokens
     extern __shared__ __align__(1024) uint8_t dir_smem[];
     const uint32_t lut = smem_u32(dir_smem);
-    const uint32_t a_s = lut + C::LUT, x_s = a_s + C::SA * C::ASTAGE, q_s = x_s + 3 * C::XSTAGE;
+    const uint32_t a_s = lut + C::LUT, x_s = a_s + C::SA * C::ASTAGE, q_s = x_s + 2 * C::XSTAGE;
     const uint32_t red = q_s + C::SQ * C::QSTAGE, bar = red + C::RED;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
 
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     };
     auto store_x = [&](int it, const uint32_t (&v)[4]) {
         if (tid < XT) {
-            const uint32_t dst = x_s + (uint32_t)((it % 3) * C::XSTAGE + xt * kAPitch + xc * 2);
+            const uint32_t dst = x_s + (uint32_t)((it & 1) * C::XSTAGE + xt * kAPitch + xc * 2);
             uint32_t o[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -236,17 +236,16 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     stage_a(1); commit();
     if constexpr (ALIGNED) stage_q(2);
     commit();
-    // levels or level pairs: one entry per thread, its 32 copies as eight 16-byte stores that rotate over the banks
+    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
     if (tid < C::ENTRIES) {
-        uint32_t v;
-        if constexpr (EXACT) {
-            v = __float_as_uint(p.levels[tid]);
-        } else {
-            const __half2 h = __floats2half2_rn(p.levels[tid & ((1 << BITS) - 1)], p.levels[tid >> BITS]);
-            v = *reinterpret_cast<const uint32_t *>(&h);
+        const float l0 = p.levels[tid & ((1 << BITS) - 1)], l1 = p.levels[tid >> BITS];
+        uint32_t v0 = __float_as_uint(l0), v1 = __float_as_uint(l1);
+        if constexpr (!EXACT) {
+            const __half2 h = __floats2half2_rn(l0, l1);
+            v0 = v1 = *reinterpret_cast<const uint32_t *>(&h);
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(v, v, v, v));
+        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(v0, v1, v0, v1));
     }
     // B fragments of the warp's rows
     const int i0 = row0 + warp * 16 + g, i1 = i0 + 8;
@@ -269,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     for (int k = 0; k < TG; ++k) acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.0f;
 #pragma unroll
     for (int k = 0; k < (EXACT ? TG : 1); ++k) low[k][0] = low[k][1] = low[k][2] = low[k][3] = 0.0f;
-    const uint32_t lut_lane = lut + 4u * (uint32_t)lane;
+    const uint32_t lut_lane = lut + (EXACT ? 8u * (uint32_t)(lane & 15) : 4u * (uint32_t)lane);
 
     for (int it = 0; it < total; ++it) {
         asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
@@ -280,7 +279,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
         commit();
         store_x(it + 1, xv);
         load_x(it + 2, xv);
-        const uint32_t a_tile = a_s + (uint32_t)((it % C::SA) * C::ASTAGE), x_tile = x_s + (uint32_t)((it % 3) * C::XSTAGE);
+        const uint32_t a_tile = a_s + (uint32_t)((it % C::SA) * C::ASTAGE), x_tile = x_s + (uint32_t)((it & 1) * C::XSTAGE);
         const uint32_t q_row = q_s + (uint32_t)((it % C::SQ) * C::QSTAGE + (warp * 16 + g) * kQPitch);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
@@ -306,28 +305,36 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
             CodeWords<BITS> w0, w1;
             w0.read(q_row + (uint32_t)(c * 4 * BITS));
             w1.read(q_row + (uint32_t)(8 * kQPitch + c * 4 * BITS));
-            uint32_t xb[TG][4], xf[EXACT ? TG : 1][4];
-            const uint32_t x_lane = x_tile + (uint32_t)((lane & 7) * kAPitch + c * 64 + (lane >> 3) * 16);
+            // x of 32 columns: token row lane & 7, 16-byte chunk lane >> 3.  EXACT, which is short of registers, takes it 16 columns at
+            // a time: chunk lane >> 3 & 1, and with two groups of tokens group lane >> 4
+            const uint32_t x_lane = x_tile + (uint32_t)((lane & 7) * kAPitch + c * 64 +
+                                                        (EXACT ? (TG == 2 ? (lane >> 4) * 8 * kAPitch : 0) + ((lane >> 3) & 1) * 16 : (lane >> 3) * 16));
+            uint32_t xb[EXACT ? 1 : TG][4];
+            if constexpr (!EXACT) {
 #pragma unroll
-            for (int k = 0; k < TG; ++k) {
-                ldmatrix_x4(x_lane + (uint32_t)(k * 8 * kAPitch), xb[k]);
-                if constexpr (EXACT) ldmatrix_x4(x_lane + (uint32_t)(C::XPART + k * 8 * kAPitch), xf[k]);
+                for (int k = 0; k < TG; ++k) ldmatrix_x4(x_lane + (uint32_t)(k * 8 * kAPitch), xb[k]);
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if constexpr (EXACT) {
-                    float w[8];
-                    w0.weights(2 * h, t, lut_lane, s[2 * h][0], s[2 * h][1], w[0], w[1]);
-                    w1.weights(2 * h, t, lut_lane, s[2 * h][2], s[2 * h][3], w[2], w[3]);
-                    w0.weights(2 * h + 1, t, lut_lane, s[2 * h + 1][0], s[2 * h + 1][1], w[4], w[5]);
-                    w1.weights(2 * h + 1, t, lut_lane, s[2 * h + 1][2], s[2 * h + 1][3], w[6], w[7]);
+                    auto scales = [&](int u, int e) { return f32x2(s[u][e], s[u][e + 1]); };
+                    const uint64_t w[4] = {w0.weights(2 * h, t, lut_lane, scales(2 * h, 0)), w1.weights(2 * h, t, lut_lane, scales(2 * h, 2)),
+                                           w0.weights(2 * h + 1, t, lut_lane, scales(2 * h + 1, 0)), w1.weights(2 * h + 1, t, lut_lane, scales(2 * h + 1, 2))};
                     uint32_t hi[4], mid[4], lo[4];
                     split_weights(w, hi, mid, lo);
+                    uint32_t xa[2 * TG], xf[2 * TG];
+                    if constexpr (TG == 2) {
+                        ldmatrix_x4(x_lane + (uint32_t)(h * 32), xa);
+                        ldmatrix_x4(x_lane + (uint32_t)(h * 32 + C::XPART), xf);
+                    } else {
+                        ldmatrix_x2(x_lane + (uint32_t)(h * 32), xa);
+                        ldmatrix_x2(x_lane + (uint32_t)(h * 32 + C::XPART), xf);
+                    }
 #pragma unroll
                     for (int k = 0; k < TG; ++k) {
-                        add_mma_bf16(acc[k], hi, xb[k][2 * h], xb[k][2 * h + 1]);
-                        mma_bf16(low[k], mid, xf[k][2 * h], xf[k][2 * h + 1]);
-                        mma_bf16(low[k], lo, xf[k][2 * h], xf[k][2 * h + 1]);
+                        add_mma_bf16(acc[k], hi, xa[2 * k], xa[2 * k + 1]);
+                        mma_bf16(low[k], mid, xf[2 * k], xf[2 * k + 1]);
+                        mma_bf16(low[k], lo, xf[2 * k], xf[2 * k + 1]);
                     }
                 } else {
                     uint32_t wa[4];
@@ -349,9 +356,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     asm volatile("cp.async.wait_all;" ::: "memory");
     if constexpr (EXACT) {
 #pragma unroll
-        for (int k = 0; k < TG; ++k)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[k][e] += low[k][e];
+        for (int k = 0; k < TG; ++k) add_low(acc[k], low[k]);
     }
 
     // ---- partial sums: lane holds rows g, g + 8 of the warp's tile, tokens 2t, 2t + 1 of each group

@@ -91,27 +91,6 @@ struct alignas(64) QuantParams {
     int *status;
 };
 
-// Two fp32 values in one 64-bit register: one instruction issued for both.
-__device__ __forceinline__ uint64_t f32x2(float lo, float hi)
-{
-    uint64_t v;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
-    return v;
-}
-__device__ __forceinline__ void f32x2_split(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t f32x2_mul(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
 // The code whose level is nearest to w / s: every level in turn, the first (lowest) code keeps a tie.
 template <int LEVELS>
 __device__ __forceinline__ uint32_t nearest_code(float s, float w, const float (&lv)[16])

@@ -28,6 +28,10 @@ __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&v)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
 }
+__device__ __forceinline__ void ldmatrix_x2(uint32_t addr, uint32_t (&v)[2])
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(v[0]), "=r"(v[1]) : "r"(addr) : "memory");
+}
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&v)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -49,8 +53,8 @@ __device__ __forceinline__ void add_mma_bf16(float (&d)[4], const uint32_t (&a)[
 {
     float v[4];
     mma_bf16_first(v, a, b0, b1);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) d[e] += v[e];
+    f32x2_split(f32x2_add(f32x2(d[0], d[1]), f32x2(v[0], v[1])), d[0], d[1]);
+    f32x2_split(f32x2_add(f32x2(d[2], d[3]), f32x2(v[2], v[3])), d[2], d[3]);
 }
 __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
@@ -77,29 +81,34 @@ __device__ __forceinline__ uint32_t scaled_pair(uint32_t level, float s0, float 
 
 // Weights held in 32 bits, multiplied by the tensor cores.  A weight is the sum of three bf16 values (8 bits of its significand
 // each, exactly: the parts are cut off, not rounded), so its product with a bf16 activation is the sum of three exact
-// products, over the whole range of a float.  The parts of eight weights in the MMA's operand layout: words of two, w[2k] the lower half.
-// Only the first part of an infinity is one (the others would be NaN); the lower parts of a float below 2^-110 reach bf16's last bit.
+// products, over the whole range of a float.  The parts of eight weights (pairs w[k]) in the MMA's operand layout.  An infinity's lower
+// parts are NaN (see add_low); the lower parts of a float below 2^-110 reach bf16's last bit.
 __device__ __forceinline__ float cut_bf16(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFF0000u); }
-__device__ __forceinline__ uint32_t high_halves(float lo, float hi) { return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632u); }
-__device__ __forceinline__ void split_weights(const float (&w)[8], uint32_t (&hi)[4], uint32_t (&mid)[4], uint32_t (&lo)[4])
+__device__ __forceinline__ uint32_t cut_pair(uint64_t w, uint64_t &rest)
 {
-    float rest[8], most = 0.0f;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        most = fmaxf(most, fabsf(w[e]));
-        rest[e] = w[e] - cut_bf16(w[e]);
-    }
-    if (most > 3.402823466e38f) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            if (fabsf(w[e]) > 3.402823466e38f) rest[e] = 0.0f;
-    }
+    float a, b;
+    f32x2_split(w, a, b);
+    rest = f32x2_fma(f32x2(cut_bf16(a), cut_bf16(b)), f32x2(-1.0f, -1.0f), w);
+    return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632u);
+}
+__device__ __forceinline__ void split_weights(const uint64_t (&w)[4], uint32_t (&hi)[4], uint32_t (&mid)[4], uint32_t (&lo)[4])
+{
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        hi[k] = high_halves(w[2 * k], w[2 * k + 1]);
-        mid[k] = high_halves(rest[2 * k], rest[2 * k + 1]);
-        lo[k] = high_halves(rest[2 * k] - cut_bf16(rest[2 * k]), rest[2 * k + 1] - cut_bf16(rest[2 * k + 1]));
+        uint64_t rest, last;
+        hi[k] = cut_pair(w[k], rest);
+        mid[k] = cut_pair(rest, last);
+        float a, b;
+        f32x2_split(last, a, b);
+        lo[k] = __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632u);
     }
+}
+// The sum of the lower parts' products added to that of the first parts'.  It is a NaN only where a weight is infinite or a NaN, and
+// there the first parts' products have made the sum what it is.
+__device__ __forceinline__ void add_low(float (&sum)[4], const float (&low)[4])
+{
+#pragma unroll
+    for (int e = 0; e < 4; ++e) sum[e] += low[e] == low[e] ? low[e] : 0.0f;
 }
 
 // Two bf16 activations with infinities and NaNs replaced by zero: what the lower parts of a weight are multiplied by (a part that is
@@ -110,8 +119,7 @@ __device__ __forceinline__ uint32_t finite_pair(uint32_t v)
 }
 
 // The 32 codes of one row's 32-column group; a lane's pair in 8-column tile u are columns 8u + 2t, 8u + 2t + 1, i.e. pair 4u + t.
-// address: of that pair in a table of level pairs, entries 128 bytes apart.  pair_bits: the pair from bit 7 up (what stands above
-// it is other codes), which are the offsets of its two levels in a table of levels, entries 128 bytes apart as well.
+// address: of that pair in a table of level pairs, entries 128 bytes apart.
 template <int BITS> struct CodeWords {
     uint32_t w[BITS];
     __device__ __forceinline__ void read(uint32_t addr)
@@ -124,31 +132,23 @@ template <int BITS> struct CodeWords {
             for (int k = 0; k < BITS; ++k) w[k] = lds_u32(addr + 4 * k);
         }
     }
-    __device__ __forceinline__ uint32_t pair_bits(int u, int t) const
+    __device__ __forceinline__ uint32_t address(int u, int t, uint32_t lut_lane) const
     {
         if constexpr (BITS == 4) {
-            return __byte_perm(w[u], 0u, 0x4440u | (uint32_t)t) << 7;                         // byte t of word u
+            return __byte_perm(w[u], 0u, 0x4440u | (uint32_t)t) * 128u + lut_lane;            // byte t of word u
         } else if constexpr (BITS == 3) {
             // the tile's four pairs are bits 24u .. 24u + 23 of the 96; moved to bits 7 .. 30, then by 6t
             const uint32_t v = u == 0 ? w[0] << 7 : u == 1 ? __funnelshift_r(w[0], w[1], 17) : u == 2 ? __funnelshift_r(w[1], w[2], 9) : w[2] >> 1;
-            return v >> (6 * t);
+            return ((v >> (6 * t)) & 0x1F80u) + lut_lane;
         } else {
             const uint32_t v = (u & 1) ? w[u >> 1] >> 9 : w[u >> 1] << 7;                     // half-word u at bits 7 .. 22
-            return v >> (4 * t);
+            return ((v >> (4 * t)) & 0x780u) + lut_lane;
         }
     }
-    __device__ __forceinline__ uint32_t address(int u, int t, uint32_t lut_lane) const
+    // the pair's weights in fp32: levels (a table of fp32 pairs) times scales
+    __device__ __forceinline__ uint64_t weights(int u, int t, uint32_t lut_lane, uint64_t scales) const
     {
-        if constexpr (BITS == 4) return __byte_perm(w[u], 0u, 0x4440u | (uint32_t)t) * 128u + lut_lane;
-        else return (pair_bits(u, t) & (((1u << 2 * BITS) - 1u) << 7)) + lut_lane;
-    }
-    // the pair's weights: level times scale, in fp32
-    __device__ __forceinline__ void weights(int u, int t, uint32_t lut_lane, float s0, float s1, float &w0, float &w1) const
-    {
-        constexpr uint32_t mask = ((1u << BITS) - 1u) << 7;
-        const uint32_t v = pair_bits(u, t);
-        w0 = __uint_as_float(lds_table((v & mask) + lut_lane)) * s0;
-        w1 = __uint_as_float(lds_table(((v >> BITS) & mask) + lut_lane)) * s1;
+        return f32x2_mul(lds_table64(address(u, t, lut_lane)), scales);
     }
 };
 

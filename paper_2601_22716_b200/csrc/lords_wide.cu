@@ -1,24 +1,31 @@
 // Wide-rank path (65 <= r <= 128) for up to 16 tokens: the scale tile comes from tcgen05, W^ = L[Q] (.) (BA) is formed in the
 // registers of the warp that multiplies it.
 //
-// Per strip of 128 columns one thread issues the scale MMA  S[128 x 128] = B_tile * A[:, strip]  (Eq. 3; bf16 operands from
+// Per strip of 128 columns one thread issues the scale MMAs  S[128 x 128] = B_tile * A[:, strip]  (Eq. 3; bf16 operands from
 // shared memory, fp32 in TMEM).  A consumer warp reads its part of S from TMEM in the accumulator layout of the
-// warp-level MMA, rounds it to fp16 pairs, multiplies by the level pairs of the codes (lane-private table) and feeds
-// the products straight to mma.sync as the left operand against the activations: that layout is the operand
-// layout, so nothing of W^ is written anywhere.  TMEM holds nothing but a ring of two S strips.
+// warp-level MMA, multiplies by the levels of the codes (lane-private table) and feeds the products straight to
+// mma.sync as the left operand against the activations: that layout is the operand layout, so nothing of W^ is
+// written anywhere.  TMEM holds nothing but a ring of two S strips.
+//
+// Layers of these ranks are computed in 32 bits, as on the CUDA cores: S, the levels and W^ are fp32, W^ enters the product as three
+// bf16 parts, x as it is (see split_weights).  Tensor cores cut sums off instead of rounding them, so S of either 64 ranks and the
+// first parts' products of every 16 columns start from zero and are added on the CUDA cores; the lower parts' products, 2^-8 of the
+// sum, keep to the tensor cores.  Error of the fp32 sums against 64 bits, norms, normal activations, 4096 columns and
+// more: 9e-8 to 1.4e-7 (CUDA cores 1.2e-7 to 1.6e-7; W^ and x rounded to fp16 3e-4).
 //
 // Why a kernel of its own: the factor strip of 128 ranks is 32 KB, which the level table and the rings of the 16-token
 // decode kernel leave no room for, and at 128 ranks the scale product outweighs everything else, so it belongs on
 // tcgen05: with S by warp-level MMAs (the direct kernel) every warp reads the whole factor strip from shared memory
-// again.  4096 x 4096, r = 128, 16 tokens: CUDA cores 585 us, direct kernel 22.5 us, this kernel 10.7 us.
+// again.  4096 x 4096, r = 128, 16 tokens: CUDA cores 585 us, direct kernel 31.7 us, this kernel 19.4 us (10.4 with W^ in fp16).
 //
-// CTA: 128 rows; sixteen consumer warps (32 rows and 32 columns of the strip each), a TMA producer, a converter of the
-// activations (bf16 -> fp16) and a scale issuer.  A cluster shares one row tile and splits its strips; every warp
+// CTA: 128 rows; sixteen consumer warps (32 rows and 32 columns of the strip each), a TMA producer, a warp that makes the copy of the
+// activations without infinities and NaNs, and a scale issuer.  A cluster shares one row tile and splits its strips; every warp
 // sends its partial sums to the CTA that owns the row (asynchronous stores counted on that CTA's barrier), which
 // adds them in a fixed order: deterministic, no atomics, no trip through global memory.
 //
-// Bound: shared memory -- operands of the scale MMAs (8 KB per 16 ranks), the factor strip's arrival (32 KB) and the
-// look-ups (2 bytes a weight), per strip of 16384 weights.
+// Bound: the consumers' instructions (about sixteen a weight: look-up, product, cutting into parts, MMAs) and the latency of their chain, four
+// warps to a scheduler: 1.6 us a strip of 16384 weights (the call above with twice the columns: 31.9 us), of which the strip's
+// arrival (44 KB from L2) and its scale MMAs (8 KB of operands per 16 ranks) are about a third each and overlap.
 //
 // Every wait is bounded; on expiry the role records LORDS_ERR_TIMEOUT and leaves its loop.
 #include <cuda.h>
@@ -44,22 +51,22 @@ constexpr int kTmaWarp = kConsumers, kConvWarp = kConsumers + 1, kScaleWarp = kC
 constexpr int kThreads = (kConsumers + 3) * 32;
 constexpr int kClusterMax = 16;
 constexpr int DS = 2;                               // S strips in TMEM
-constexpr uint32_t kTmemCols = DS * kStrip;
+constexpr uint32_t kTmemCols = DS * 2 * kStrip;     // S of ranks 0 .. 63 and of the others, apart
 constexpr int kRankMax = 128;
 constexpr int kAAtom = kRankMax * 128;              // 64 columns of the factor strip, 128-byte swizzle
 constexpr int kBAtom = kRows * 128;                 // B[128 x 64 ranks], K-major, 128-byte swizzle; two of them
 
 // BITS: code width.  TG: tokens in groups of eight (zero padded).
 template <int BITS, int TG> struct WideCfg {
-    static constexpr int ENTRIES = BITS == 4 ? 256 : BITS == 3 ? 64 : 16;     // level pairs
-    static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair
+    static constexpr int ENTRIES = 1 << 2 * BITS;                             // level pairs
+    static constexpr int LUT = ENTRIES * 128;                                 // 16 copies of every pair in fp32, one for a lane of each half warp
     static constexpr int QROW = kStrip * BITS / 8;                            // 64 / 48 / 32 bytes
     static constexpr int QTILE = kRows * QROW;
     static constexpr int XATOM = TG * 8 * 128;                                // 64 columns of the activations, 128-byte swizzle
-    static constexpr int XTILE = 2 * XATOM;                                   // arrives as bf16, converted in place
+    static constexpr int XTILE = 2 * XATOM;
     static constexpr int RED = (kRows + kClusterMax) * TG * 8 * 4;            // partial sums received: cluster x rows owned x tokens
     static constexpr int FIXED = 1024 + 2 * kBAtom + LUT + RED + 512;
-    static constexpr int STAGE = 2 * kAAtom + QTILE + XTILE;
+    static constexpr int STAGE = 2 * kAAtom + QTILE + 2 * XTILE;              // the activations as they are and without infinities and NaNs
     static constexpr int D = (232448 - FIXED) / STAGE < 4 ? (232448 - FIXED) / STAGE : 4;    // strips in flight
     static constexpr int SMEM = FIXED + D * STAGE;
     static_assert(D >= 2 && QTILE % 1024 == 0 && XATOM % 1024 == 0, "swizzled tiles start on their pattern's boundary");
@@ -97,6 +104,8 @@ template <int BITS> __device__ __forceinline__ uint32_t code_offset(int row, int
     else return (uint32_t)(row * 32 + (((c >> 1) ^ ((row >> 2) & 1)) << 4) + (c & 1) * 8);
 }
 
+__device__ __forceinline__ uint64_t pair_at(const uint32_t (&v)[16], int e) { return f32x2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])); }
+
 template <int BITS, int TG>
 __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_constant__ WideParams p)
 {
@@ -104,12 +113,12 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
     constexpr int D = C::D, MT = TG * 8;
     extern __shared__ uint8_t wide_smem[];
     const uint32_t b_tile = (smem_u32(wide_smem) + 1023u) & ~1023u;
-    const uint32_t a_s = b_tile + 2 * kBAtom, q_s = a_s + D * 2 * kAAtom, x_s = q_s + D * C::QTILE, lut = x_s + D * C::XTILE;
+    const uint32_t a_s = b_tile + 2 * kBAtom, q_s = a_s + D * 2 * kAAtom, x_s = q_s + D * C::QTILE, lut = x_s + D * 2 * C::XTILE;
     const uint32_t red = lut + C::LUT, bars = red + C::RED;
-    const uint32_t bar_q = bars, bar_raw = bar_q + 8 * D, bar_x = bar_raw + 8 * D, bar_free = bar_x + 8 * D;
+    const uint32_t bar_q = bars, bar_x = bar_q + 8 * D, bar_free = bar_x + 8 * D;              // bar_q: codes and activations have landed
     const uint32_t bar_a = bar_free + 8 * D, bar_a_free = bar_a + 8 * D, bar_s = bar_a_free + 8 * D, bar_s_free = bar_s + 8 * DS;
     const uint32_t bar_b = bar_s_free + 8 * DS, bar_red = bar_b + 8, tmem_slot = bar_red + 8;
-    static_assert(8 * (6 * D + 2 * DS + 2) + 4 <= 512, "barrier area");
+    static_assert(8 * (5 * D + 2 * DS + 2) + 4 <= 512, "barrier area");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     const int csize = (int)cluster_nctarank(), rank = (int)cluster_ctarank();
@@ -125,8 +134,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         if (lane == 0) {
 #pragma unroll
             for (int k = 0; k < D; ++k) {
-                mbar_init(bar_q + 8 * k, 1);
-                mbar_init(bar_raw + 8 * k, 1);
+                mbar_init(bar_q + 8 * k, 2);
                 mbar_init(bar_x + 8 * k, 1);
                 mbar_init(bar_free + 8 * k, kConsumers);
                 mbar_init(bar_a + 8 * k, 1);
@@ -153,8 +161,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
             tma_load_2d(q_s + (uint32_t)((it % D) * C::QTILE), &p.tm_q, (s_a + it) * C::QROW, row0, bar);
         };
         auto activations = [&](int it) {
-            const uint32_t bar = bar_raw + 8 * (it % D);
-            const uint32_t dst = x_s + (uint32_t)((it % D) * C::XTILE);
+            const uint32_t bar = bar_q + 8 * (it % D);
+            const uint32_t dst = x_s + (uint32_t)((it % D) * 2 * C::XTILE);
             mbar_expect_tx(bar, (uint32_t)C::XTILE);
             tma_load_2d(dst, &p.tm_x, (s_a + it) * kStrip, 0, bar);
             tma_load_2d(dst + C::XATOM, &p.tm_x, (s_a + it) * kStrip + 64, 0, bar);
@@ -186,31 +194,22 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         }
         __syncwarp();
     } else if (warp == kConvWarp) {
-        // ------------------------------------------------------------------ converter: in place, eight columns per 16-byte word wherever the swizzle put it
+        // ------------------------------------------------------------------ the second copy of the activations, word by word wherever the swizzle put it
         asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
         asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
         griddep_launch_dependents();
         griddep_wait();
         for (int it = 0; it < total; ++it) {
             const int st = it % D;
-            if (!mbar_wait_warp(bar_raw + 8 * st, (uint32_t)((it / D) & 1), status, 75)) { failed = true; break; }
+            if (!mbar_wait_warp(bar_q + 8 * st, (uint32_t)((it / D) & 1), status, 75)) { failed = true; break; }
             // all loads first: one after the other's store, each would wait for the way through shared memory
-            const uint32_t base = x_s + (uint32_t)(st * C::XTILE + lane * 16);
+            const uint32_t base = x_s + (uint32_t)(st * 2 * C::XTILE + lane * 16);
             uint4 v[MT / 2];
 #pragma unroll
             for (int k = 0; k < MT / 2; ++k) v[k] = lds_v4(base + (uint32_t)(k * 512));
 #pragma unroll
-            for (int k = 0; k < MT / 2; ++k) {
-                const uint32_t in[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-                uint32_t o[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const __half2 h = __floats2half2_rn(__uint_as_float(in[e] << 16), __uint_as_float(in[e] & 0xFFFF0000u));
-                    o[e] = *reinterpret_cast<const uint32_t *>(&h);
-                }
-                sts_v4(base + (uint32_t)(k * 512), make_uint4(o[0], o[1], o[2], o[3]));
-            }
-            fence_proxy_async_smem();        // the next TMA copy into this stage comes after these stores
+            for (int k = 0; k < MT / 2; ++k)
+                sts_v4(base + (uint32_t)(C::XTILE + k * 512), make_uint4(finite_pair(v[k].x), finite_pair(v[k].y), finite_pair(v[k].z), finite_pair(v[k].w)));
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_x + 8 * st);
         }
@@ -239,9 +238,9 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
             if (!mbar_wait_warp2(bar_a + 8 * sa, (uint32_t)((it / D) & 1), bar_s_free + 8 * sd, (uint32_t)((it / DS + 1) & 1), status, 78)) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_lo = a_lo0 + (uint32_t)(sa * ((2 * kAAtom) >> 4));
-            for (int k = 0; k < rsteps; ++k)                                   // 64 ranks per atom of the B tile
-                umma_f16_ss(tmem_base + (uint32_t)(sd * kStrip), umma_desc_pack(b_lo + (k >> 2) * (kBAtom >> 4) + (k & 3) * 2, desc_hi),
-                            umma_desc_pack(a_lo + k * 128, desc_hi), idesc, k > 0, leader);
+            for (int k = 0; k < rsteps; ++k)                                   // 64 ranks per atom of the B tile, and per sum
+                umma_f16_ss(tmem_base + (uint32_t)((2 * sd + (k >> 2)) * kStrip), umma_desc_pack(b_lo + (k >> 2) * (kBAtom >> 4) + (k & 3) * 2, desc_hi),
+                            umma_desc_pack(a_lo + k * 128, desc_hi), idesc, (k & 3) > 0, leader);
             umma_commit(bar_s + 8 * sd, leader);
             umma_commit(bar_a_free + 8 * sa, leader);
         }
@@ -251,12 +250,11 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         // ------------------------------------------------------------------ consumers
         // row group rw (its TMEM quadrant), column quarter ch
         const int g = lane >> 2, t = lane & 3, rw = warp & 3, ch = warp >> 2;
-        // level pairs: one entry per thread, its 32 copies as eight 16-byte stores that rotate over the banks
+        // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
         if (tid < C::ENTRIES) {
-            const __half2 h = __floats2half2_rn(p.levels[tid & ((1 << BITS) - 1)], p.levels[tid >> BITS]);
-            const uint32_t v = *reinterpret_cast<const uint32_t *>(&h);
+            const uint32_t l0 = __float_as_uint(p.levels[tid & ((1 << BITS) - 1)]), l1 = __float_as_uint(p.levels[tid >> BITS]);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(v, v, v, v));
+            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(l0, l1, l0, l1));
         }
         if (!b_by_tma) {
             // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m
@@ -280,14 +278,19 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         uint32_t tmem_base;
         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
 
-        float acc[2][TG][4];
+        float acc[2][TG][4], low[2][TG][4];                                    // low: the sums of the weights' lower parts
 #pragma unroll
         for (int rg = 0; rg < 2; ++rg)
 #pragma unroll
-            for (int k = 0; k < TG; ++k) acc[rg][k][0] = acc[rg][k][1] = acc[rg][k][2] = acc[rg][k][3] = 0.0f;
-        const uint32_t lut_lane = lut + 4u * (uint32_t)lane;
-        // x: token row lane & 7, 16-byte chunk lane >> 3 of the 32-column group, chunks swizzled by the row
-        const uint32_t x_lane = x_s + (uint32_t)((ch >> 1) * C::XATOM + (lane & 7) * 128 + (((((ch & 1) * 4) + (lane >> 3)) ^ (lane & 7)) << 4));
+            for (int k = 0; k < TG; ++k) {
+                acc[rg][k][0] = acc[rg][k][1] = acc[rg][k][2] = acc[rg][k][3] = 0.0f;
+                low[rg][k][0] = low[rg][k][1] = low[rg][k][2] = low[rg][k][3] = 0.0f;
+            }
+        const uint32_t lut_lane = lut + 8u * (uint32_t)(lane & 15);
+        // x, 16 columns at a time: token row lane & 7 of group lane >> 4, 16-byte chunk lane >> 3 & 1 (the next 16 columns are two chunks
+        // on, bit 5 of the address), chunks swizzled by the row
+        const uint32_t x_lane = x_s + (uint32_t)((ch >> 1) * C::XATOM + (TG == 2 ? (lane >> 4) * 1024 : 0) + (lane & 7) * 128 +
+                                                 (((((ch & 1) * 4) + ((lane >> 3) & 1)) ^ (lane & 7)) << 4));
         const uint32_t s_lane = tmem_base + ((uint32_t)(rw * 32) << 16) + (uint32_t)(ch * 32);
 
         for (int it = 0; it < total; ++it) {
@@ -295,41 +298,54 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
             if (!mbar_wait_warp3(bar_s + 8 * sd, (uint32_t)((it / DS) & 1), bar_q + 8 * st, (uint32_t)((it / D) & 1),
                                  bar_x + 8 * st, (uint32_t)((it / D) & 1), true, status, 72)) { failed = true; break; }
             tc_fence_after_sync();
-            const uint32_t q_tile = q_s + (uint32_t)(st * C::QTILE), x_tile = x_lane + (uint32_t)(st * C::XTILE);
-            const uint32_t s_tile = s_lane + (uint32_t)(sd * kStrip);
-            // both units of 16 rows x 32 columns come from TMEM while the codes and activations are read
-            uint32_t s[2][16];
-            tmem_ld_16x32_frag(s_tile, s[0]);
-            tmem_ld_16x32_frag(s_tile + (16u << 16), s[1]);
-            uint32_t xb[TG][4];
+            const uint32_t q_tile = q_s + (uint32_t)(st * C::QTILE), x_tile = x_lane + (uint32_t)(st * 2 * C::XTILE);
 #pragma unroll
-            for (int k = 0; k < TG; ++k) ldmatrix_x4(x_tile + (uint32_t)(k * 1024), xb[k]);
-            CodeWords<BITS> w[2][2];
+            for (int rg = 0; rg < 2; ++rg) {                                   // units of 16 rows x 32 columns
+                uint32_t u[16], v[16];
+                const uint32_t at = s_lane + ((uint32_t)(rg * 16) << 16) + (uint32_t)(2 * sd * kStrip);
+                tmem_ld_16x32_frag(at, u);
+                tmem_ld_16x32_frag(at + kStrip, v);
+                CodeWords<BITS> w0, w1;
+                w0.read(q_tile + code_offset<BITS>(rw * 32 + rg * 16 + g, ch));
+                w1.read(q_tile + code_offset<BITS>(rw * 32 + rg * 16 + g + 8, ch));
+                tmem_wait_ld(u);
+                tmem_wait_ld(v);
+                uint64_t s[8];
 #pragma unroll
-            for (int rg = 0; rg < 2; ++rg)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) w[rg][h].read(q_tile + code_offset<BITS>(rw * 32 + rg * 16 + g + 8 * h, ch));
-            tmem_wait_ld(s[0]);
-            tmem_wait_ld(s[1]);
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_s_free + 8 * sd);                   // S is in registers: the next one may be written
-#pragma unroll
-            for (int rg = 0; rg < 2; ++rg) {
-                const uint32_t (&v)[16] = s[rg];
-                auto pair = [&](const CodeWords<BITS> &cw, int tile, int e) {
-                    return scaled_pair(lds_table(cw.address(tile, t, lut_lane)), __uint_as_float(v[4 * tile + e]), __uint_as_float(v[4 * tile + e + 1]));
-                };
+                for (int e = 0; e < 8; ++e) s[e] = f32x2_add(pair_at(u, e), pair_at(v, e));
+                if (rg == 1) {
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_s_free + 8 * sd);         // S is in registers: the next one may be written
+                }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const uint32_t wa[4] = {pair(w[rg][0], 2 * h, 0), pair(w[rg][1], 2 * h, 2), pair(w[rg][0], 2 * h + 1, 0), pair(w[rg][1], 2 * h + 1, 2)};
+                    const uint64_t w[4] = {w0.weights(2 * h, t, lut_lane, s[4 * h]), w1.weights(2 * h, t, lut_lane, s[4 * h + 1]),
+                                           w0.weights(2 * h + 1, t, lut_lane, s[4 * h + 2]), w1.weights(2 * h + 1, t, lut_lane, s[4 * h + 3])};
+                    uint32_t hi[4], mid[4], lo[4];
+                    split_weights(w, hi, mid, lo);
+                    uint32_t xb[2 * TG], xf[2 * TG];
+                    if constexpr (TG == 2) {
+                        ldmatrix_x4(x_tile ^ (uint32_t)(h * 32), xb);
+                        ldmatrix_x4((x_tile ^ (uint32_t)(h * 32)) + C::XTILE, xf);
+                    } else {
+                        ldmatrix_x2(x_tile ^ (uint32_t)(h * 32), xb);
+                        ldmatrix_x2((x_tile ^ (uint32_t)(h * 32)) + C::XTILE, xf);
+                    }
 #pragma unroll
-                    for (int k = 0; k < TG; ++k) mma_f16(acc[rg][k], wa, xb[k][2 * h], xb[k][2 * h + 1]);
+                    for (int k = 0; k < TG; ++k) {
+                        add_mma_bf16(acc[rg][k], hi, xb[2 * k], xb[2 * k + 1]);
+                        mma_bf16(low[rg][k], mid, xf[2 * k], xf[2 * k + 1]);
+                        mma_bf16(low[rg][k], lo, xf[2 * k], xf[2 * k + 1]);
+                    }
                 }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_free + 8 * st);
         }
+
+#pragma unroll
+        for (int k = 0; k < 2 * TG; ++k) add_low(acc[k / TG][k % TG], low[k / TG][k % TG]);
 
         // The four column quarters of a row group meet first, in the factor ring (every copy into it and every MMA on it has
         // completed: the last strip's S has been waited for), so that one partial sum per row and token goes out.
