@@ -40,13 +40,16 @@
  *     read only the weights (Qpacked, B, A); x is read, and y written, after it.  So the weights must
  *     not be produced by work that is still in flight on `stream` when a forward call is made
  *     (synchronise the stream once after loading or updating weights); activations may be.
- *   - precision and range: products are accumulated in fp32.  The tensor-core kernels hold their
- *     operands in fp16, each rounded once: the dequantised weight L[Q_ij] * (BA)_ij (M > 2), or the bare
- *     level L[Q_ij] and the product A_kj * x_tj (M <= 2), and x itself (M > 2).  These values must lie
- *     within fp16's range: magnitudes above 65504 overflow to infinity, magnitudes below 6.1e-5 are
- *     rounded to multiples of 6e-8 (which matters only where such terms dominate a sum).  Layer
- *     weights and activations of the usual scales (|x| up to a few thousand, factors around 1e-2 to 1)
- *     are far inside; the CUDA-core path ("path" = "simt") is fp32 throughout and has no such limit.
+ *   - precision and range: sums are fp32.  Layers on the tensor cores' grid (n a multiple of 64, or of 128
+ *     for 3-bit codes, and r <= 64) hold their operands in fp16, each rounded once:
+ *         the dequantised weight L[Q_ij] * (BA)_ij and x itself; or,
+ *         with M <= 2, M * (r rounded up to 16) <= 64 and m * n > 2^19 (for such calls n need only be a multiple
+ *         of 32 with 4-bit codes), the bare level L[Q_ij] and the product A_kj * x_tj.
+ *     These values must lie within fp16's range: magnitudes above 65504 overflow to infinity, magnitudes
+ *     below 6.1e-5 are rounded to multiples of 6e-8 (which matters only where such terms dominate a sum).
+ *     Layer weights and activations of the usual scales (|x| up to a few thousand, factors around 1e-2 to 1)
+ *     are far inside.  All other calls (rows off that grid, ranks above 64, the smaller layers with M <= 2) and
+ *     the CUDA-core path ("path" = "simt") are computed in fp32 throughout and have no such limit.
  *   - forward calls validate on the host, enqueue work on `stream` and return
  *     without synchronising.  They use library-owned scratch memory, so two forward
  *     calls may only overlap on the GPU if they are ordered on the same stream.

@@ -1,19 +1,27 @@
-// Two-phase path for any shape: W^ = L[Q] (.) (BA) is expanded once into fp16 scratch, then one dense fp16 product
+// Two-phase path for any shape: W^ = L[Q] (.) (BA) is expanded once into scratch, then one dense product
 // y = x W^T runs on the tensor cores.
 //
-//   expand:  S = B A by warp-level MMAs (Eq. 3; bf16 operands, fp32 sums in registers), the level of every code from a
-//            lane-private pair table, the product rounded once to fp16 -- the same operand the scale-MMA kernel
-//            forms -- and stored row-major with the row padded to a multiple of 64 columns.  The same launch
-//            converts the activations to fp16 rows of that pitch.  No tensor map touches the caller's
-//            tensors, so rows need no alignment and any rank goes.
-//   product: tcgen05 on CTA pairs (cta_group::2, 256 rows of W^ x BN tokens per pair), both operands by TMA.  The tiles
-//            of whole waves run one per pair; the k-steps of the tiles left over are dealt out evenly
-//            over all pairs, and the pieces of a tile meet in scratch in a fixed order (no atomics on data).
+// The layers that come here (ragged rows, ranks above 64) are computed in 32 bits, as on the CUDA cores: S, the levels and W^ are
+// fp32, W^ enters the product as three bf16 parts, x as it is (see split_weights).
 //
-// When it pays: the scale-MMA kernel rebuilds W^ for every token tile and puts its k-steps through a chain of
-// scale MMA -> registers -> main MMA; this path pays 2 m n bytes of scratch traffic once and then runs at the rate
-// of a plain product.  It also takes what the tensor maps of the other kernels cannot express (row pitches
-// that are not multiples of 16 bytes, ranks above 64), which only the CUDA cores took before.
+//   expand:  S = B A by warp-level MMAs (Eq. 3; bf16 operands, fp32 sums in registers, every 16 ranks from zero), the level of every
+//            code from a table of fp32 pairs, their product cut into its parts, which are stored row-major, one after the
+//            other, each padded to a multiple of 64 columns.  The same launch copies the activations to rows of that
+//            pitch, and once more without infinities and NaNs, which is what the lower parts are multiplied by.  No tensor map
+//            touches the caller's tensors, so rows need no alignment and any rank goes.
+//   product: tcgen05 on CTA pairs (cta_group::2, 256 rows of W^ x BN tokens per pair), both operands by TMA, three MMAs where one
+//            would do in 16 bits.  Tensor cores cut sums off instead of rounding them, so the first parts' products of every 64
+//            columns start from zero in one accumulator and the epilogue adds them up in registers, while the MMAs of the lower
+//            parts, whose sum is 2^-8 of the other, run in a second accumulator.  The tiles of whole waves run one per pair; the
+//            k-steps of the tiles left over are dealt out evenly over all pairs, and the pieces of a tile meet in scratch in a
+//            fixed order (no atomics on data).
+//
+// Error of the fp32 sums against 64 bits, norms, normal activations, 200 to 1024 tokens: 1.0e-7 to 1.9e-7 (CUDA cores 1.7e-7 to 3.8e-7,
+// W^ and x rounded to fp16 3e-4).
+//
+// When it pays: W^ is formed once for all tokens, where the CUDA cores (the only other path for most of these shapes) need r + M
+// multiply-adds a weight: 5952 x 7008, r = 11, 578 tokens: 9160 us there, 255 here (97 with W^ in fp16, a third of the MMAs
+// and of the scratch).
 //
 // Every wait is bounded; on expiry the role records LORDS_ERR_TIMEOUT and leaves its loop.
 #include <cuda.h>
@@ -42,7 +50,7 @@ constexpr int kExPitch = kExCols * 2 + 16;          // bytes per rank row of a s
 
 template <int BITS, int RK> struct ExCfg {
     static constexpr int ENTRIES = BITS == 4 ? 256 : BITS == 3 ? 64 : 16;     // level pairs
-    static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair
+    static constexpr int LUT = ENTRIES * 128;                                 // 16 copies of every pair in fp32, one for a lane of each half warp
     static constexpr int STAGE = RK * 16 * kExPitch;
     static constexpr int SMEM = LUT + kExStages * STAGE;
 };
@@ -53,8 +61,8 @@ struct ExpandParams {
     const uint16_t *B;     // first row of this chunk
     const uint16_t *A;
     const uint16_t *x;
-    uint16_t *w16;         // [rows][np]
-    uint16_t *x16;         // [M][np]
+    uint16_t *w16;         // [rows][3][np]: the parts of W^
+    uint16_t *x16;         // [M][2][np]: the activations, and without infinities and NaNs
     float levels[16];
     int rows, n, np, r, M;
     int strips, splits;    // strips of 64 columns; CTAs that share a row tile's strips
@@ -87,7 +95,7 @@ __device__ __forceinline__ uint32_t load_codes8(const uint8_t *row, int c, const
     }
 }
 
-// Bound: at m n fp16 stores the write stream to L2 / HBM (2 bytes a weight against bits / 8 read); up to rank 64 the
+// Bound: the write stream to L2 / HBM (6 bytes a weight against bits / 8 read); up to rank 64 the
 // MMAs (rank / 8 per 16 x 8 tile at the warp-level rate) and the four instructions per code pair stay below it.
 // RK: the rank in steps of 16 that the B fragments hold (zero padded).
 template <int BITS, int RK, bool ALIGNED>
@@ -118,12 +126,9 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
                         if (c + 2 * k < p.n) w[k] = __ldg(src + k);
                 }
             }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const __half2 h = __floats2half2_rn(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xFFFF0000u));
-                w[k] = *reinterpret_cast<const uint32_t *>(&h);
-            }
-            *reinterpret_cast<uint4 *>(p.x16 + t * p.np + c) = make_uint4(w[0], w[1], w[2], w[3]);
+            uint16_t *dst = p.x16 + 2 * t * p.np + c;
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4 *>(dst + p.np) = make_uint4(finite_pair(w[0]), finite_pair(w[1]), finite_pair(w[2]), finite_pair(w[3]));
         }
         return;
     }
@@ -155,14 +160,13 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
         else asm volatile("cp.async.commit_group;" ::: "memory");
     }
 
-    // level pairs: one entry per thread, its 32 lane-private copies as eight 16-byte stores that rotate over the banks
+    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
+    const uint4 v = level_pair<BITS>(p.levels, tid);
     if (tid < C::ENTRIES) {
-        const __half2 h = __floats2half2_rn(p.levels[tid & ((1 << BITS) - 1)], p.levels[tid >> BITS]);
-        const uint32_t v = *reinterpret_cast<const uint32_t *>(&h);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(v, v, v, v));
+        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
     }
-    const uint32_t lut_lane = lut + 4u * (uint32_t)lane;
+    const uint32_t lut_lane = lut + 8u * (uint32_t)(lane & 15);
 
     // B fragments of the warp's 16 rows, kept for every strip
     uint32_t bf[RK][4];
@@ -209,28 +213,31 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
                         mma_bf16_first(acc[2 * h], bf[k], v[0], v[1]);
                         mma_bf16_first(acc[2 * h + 1], bf[k], v[2], v[3]);
                     } else {
-                        mma_bf16(acc[2 * h], bf[k], v[0], v[1]);
-                        mma_bf16(acc[2 * h + 1], bf[k], v[2], v[3]);
+                        add_mma_bf16(acc[2 * h], bf[k], v[0], v[1]);
+                        add_mma_bf16(acc[2 * h + 1], bf[k], v[2], v[3]);
                     }
                 }
 #pragma unroll
             for (int rr = 0; rr < 2; ++rr) {
                 const uint32_t w = cur[c][rr];
-                uint32_t out[4];
+                uint64_t v[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     // pair u of the lane's eight columns, at bit 2 BITS u
                     constexpr uint32_t mask = (uint32_t)(C::ENTRIES - 1) << 7;
                     const int off = 2 * BITS * u;
                     const uint32_t sh = off >= 7 ? w >> (off - 7) : w << (7 - off);
-                    const uint32_t lv = lds_table(lut_lane + (sh & mask));
-                    const __half2 sv = __floats2half2_rn(acc[u][2 * rr], acc[u][2 * rr + 1]);
-                    const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), sv);
-                    out[u] = *reinterpret_cast<const uint32_t *>(&wv);
+                    v[u] = f32x2_mul(lds_table64(lut_lane + (sh & mask)), f32x2(acc[u][2 * rr], acc[u][2 * rr + 1]));
                 }
+                uint32_t hi[4], mid[4], lo[4];
+                split_weights(v, hi, mid, lo);
                 const int i = rr ? i1 : i0;
-                if (i < p.rows)
-                    *reinterpret_cast<uint4 *>(p.w16 + (size_t)i * p.np + s * kExCols + c * 32 + 8 * t) = make_uint4(out[0], out[1], out[2], out[3]);
+                if (i < p.rows) {
+                    uint16_t *dst = p.w16 + 3 * (size_t)i * p.np + s * kExCols + c * 32 + 8 * t;
+                    *reinterpret_cast<uint4 *>(dst) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                    *reinterpret_cast<uint4 *>(dst + p.np) = make_uint4(mid[0], mid[1], mid[2], mid[3]);
+                    *reinterpret_cast<uint4 *>(dst + 2 * p.np) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                }
             }
         }
 #pragma unroll
@@ -242,25 +249,26 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
 // ------------------------------------------------------------------------------------------------ product
 constexpr int kGRows = 256;                         // rows of W^ per CTA pair
 constexpr int kGK = 64;                             // columns per k-step
-constexpr int kGEpiWarp0 = 4, kGEpiWarps = 8;       // warps 4..11: epilogue; 0: TMA, 1: MMA issuer, 2: TMEM
-constexpr int kGThreads = (kGEpiWarp0 + kGEpiWarps) * 32;
+constexpr int kGEpiWarp0 = 4;                       // warps from 4 on: epilogue; 0: TMA, 1: MMA issuer, 2: TMEM
 constexpr uint32_t kGTmemCols = 512;
 
 template <int BN> struct GCfg {
-    static constexpr int ATILE = 128 * 128;                      // this CTA's 128 rows, 64 columns fp16
+    static constexpr int EPI = BN >= 256 ? 16 : 8;               // epilogue warps (a k-step's first parts have to be read while the MMAs of its lower parts run: 2816 x 3072, 1024 tokens, 95 us with eight, 85 with sixteen)
+    static constexpr int THREADS = (kGEpiWarp0 + EPI) * 32;
+    static constexpr int ATILE = 128 * 128;                      // this CTA's 128 rows, 64 columns of one part
     static constexpr int BTILE = (BN / 2) * 128;                 // this CTA's half of the tokens
     static constexpr int STAGE = ATILE + BTILE;
     static constexpr int STAGES = BN >= 256 ? 6 : BN >= 128 ? 8 : 10;
     static constexpr int SMEM = 1024 + STAGES * STAGE + 256;
-    static constexpr uint32_t ACC = BN < 32 ? 32 : BN;           // columns of one accumulator; two of them
+    static constexpr uint32_t ACC = BN < 32 ? 32 : BN;           // columns of one accumulator: first parts, lower parts
 };
 
 struct alignas(64) GemmParams {
-    CUtensorMap tm_w;     // fp16 [rows][np], box {64, 128}, 128-byte swizzle (rows past the end read as zero)
-    CUtensorMap tm_x;     // fp16 [M][np], box {64, BN / 2}
+    CUtensorMap tm_w;     // bf16 [rows][3 np], box {64, 128}, 128-byte swizzle (rows past the end read as zero)
+    CUtensorMap tm_x;     // bf16 [M][2 np], box {64, BN / 2}
     int M, rows;          // rows of this chunk
     int row0, ldy;        // first row of the chunk inside y, row length of y
-    int tok_tiles, tiles, ksteps;
+    int tok_tiles, tiles, ksteps, np;
     int pairs;            // CTA pairs launched
     int whole;            // tiles [0, whole) run unsplit, one per pair and wave; the k-steps of the rest are dealt out evenly
     float *partial;       // [pair][2][BN][128]: a piece that does not begin its tile
@@ -271,7 +279,7 @@ struct alignas(64) GemmParams {
 };
 
 template <int BN>
-__global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_constant__ GemmParams p)
+__global__ void __launch_bounds__(GCfg<BN>::THREADS, 1) lords_dense_kernel(const __grid_constant__ GemmParams p)
 {
     using C = GCfg<BN>;
     constexpr int STAGES = C::STAGES;
@@ -294,7 +302,7 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
     if (warp == 0) {
         if (lane < 2 * STAGES) mbar_init(bars + 8 * lane, 1);
         if (lane >= 2 * STAGES && lane < 2 * STAGES + 2) mbar_init(bars + 8 * lane, 1);                        // accumulator full: one commit
-        if (lane >= 2 * STAGES + 2 && lane < 2 * STAGES + 4) mbar_init(bars + 8 * lane, 2 * kGEpiWarps);       // read by both CTAs' epilogue
+        if (lane >= 2 * STAGES + 2 && lane < 2 * STAGES + 4) mbar_init(bars + 8 * lane, 2 * C::EPI);           // read by both CTAs' epilogue
         fence_mbar_init();
         if (lane == 0) { tma_prefetch_desc(&p.tm_w); tma_prefetch_desc(&p.tm_x); }
     } else if (warp == 2) {
@@ -319,13 +327,13 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
             int it = 0;
             while (!failed && sched.next(w)) {
                 const int rt = w.tile / p.tok_tiles, tt = w.tile - rt * p.tok_tiles;
-                for (int k = w.k0; k < w.k1; ++k, ++it) {
-                    const int s = it % STAGES;
+                for (int j = 3 * w.k0; j < 3 * w.k1; ++j, ++it) {              // part j % 3 of k-step j / 3
+                    const int s = it % STAGES, k = j / 3, part = j - 3 * k;
                     if (it >= STAGES && !mbar_wait(bar_empty + 8 * s, (uint32_t)((it / STAGES - 1) & 1), status, 51)) { failed = true; break; }
                     if (rank == 0) mbar_expect_tx(bar_full + 8 * s, 2u * C::STAGE);
                     const uint32_t dst = base + (uint32_t)(s * C::STAGE);
-                    tma_load_2d_pair(dst, &p.tm_w, k * kGK, rt * kGRows + rank * 128, full0 + 8 * s);
-                    tma_load_2d_pair(dst + C::ATILE, &p.tm_x, k * kGK, tt * BN + rank * (BN / 2), full0 + 8 * s);
+                    tma_load_2d_pair(dst, &p.tm_w, part * p.np + k * kGK, rt * kGRows + rank * 128, full0 + 8 * s);
+                    tma_load_2d_pair(dst + C::ATILE, &p.tm_x, (part > 0 ? p.np : 0) + k * kGK, tt * BN + rank * (BN / 2), full0 + 8 * s);
                 }
             }
             // nothing of this CTA is in flight when it ends: the last round of stages has been read
@@ -335,43 +343,71 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
         __syncwarp();
     } else if (warp == 1 && rank == 0) {
         // ------------------------------------------------------------------ MMA issuer (the pair's even CTA)
-        constexpr uint32_t idesc = umma_idesc_f16(0, 0, 0, kGRows, BN);
+        constexpr uint32_t idesc = umma_idesc_f16(1, 0, 0, kGRows, BN);
         const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
         const uint32_t lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((base & 0x3FFFFu) >> 4);
         const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
-        int it = 0, done = 0;
+        int it = 0, steps = 0, pieces = 0;
         while (!failed && sched.next(w)) {
-            const int buf = done & 1;
-            const uint32_t acc = tmem_u + (uint32_t)buf * C::ACC;
-            if (done >= 2 && !mbar_wait_cluster(bar_acc_empty + 8 * buf, (uint32_t)((done / 2 - 1) & 1), status, 53)) { failed = true; break; }
-            tc_fence_after_sync();
-            for (int k = w.k0; k < w.k1; ++k, ++it) {
-                const int s = it % STAGES;
-                if (!mbar_wait_cluster(bar_full + 8 * s, (uint32_t)((it / STAGES) & 1), status, 54)) { failed = true; break; }
-                tc_fence_after_sync();
-                const uint32_t a_lo = lo0 + (uint32_t)((s * C::STAGE) >> 4), b_lo = a_lo + (C::ATILE >> 4);
+            for (int k = w.k0; k < w.k1 && !failed; ++k, ++steps) {
+                if (steps > 0 && !mbar_wait_cluster(bar_acc_empty, (uint32_t)((steps - 1) & 1), status, 53)) { failed = true; break; }
+                for (int part = 0; part < 3; ++part, ++it) {
+                    if (part == 1 && k == w.k0 && pieces > 0 && !mbar_wait_cluster(bar_acc_empty + 8, (uint32_t)((pieces - 1) & 1), status, 57)) { failed = true; break; }
+                    const int s = it % STAGES;
+                    if (!mbar_wait_cluster(bar_full + 8 * s, (uint32_t)((it / STAGES) & 1), status, 54)) { failed = true; break; }
+                    tc_fence_after_sync();
+                    const uint32_t a_lo = lo0 + (uint32_t)((s * C::STAGE) >> 4), b_lo = a_lo + (C::ATILE >> 4);
+                    const uint32_t acc = tmem_u + (part > 0 ? C::ACC : 0u);
+                    const bool onto = part == 2 || (part == 1 && k > w.k0);   // first parts start from zero every k-step, lower ones every piece
 #pragma unroll
-                for (int kk = 0; kk < kGK / 16; ++kk)
-                    umma2_f16_ss(acc, umma_desc_pack(a_lo + kk * 2, desc_hi), umma_desc_pack(b_lo + kk * 2, desc_hi), idesc,
-                                 (k > w.k0 || kk > 0) ? 1u : 0u, leader);
-                umma2_commit(bar_empty + 8 * s, leader);
-                if (k == w.k1 - 1) umma2_commit(bar_acc_full + 8 * buf, leader);
-                __syncwarp();
+                    for (int kk = 0; kk < kGK / 16; ++kk)
+                        umma2_f16_ss(acc, umma_desc_pack(a_lo + kk * 2, desc_hi), umma_desc_pack(b_lo + kk * 2, desc_hi), idesc,
+                                     (onto || kk > 0) ? 1u : 0u, leader);
+                    umma2_commit(bar_empty + 8 * s, leader);
+                    if (part == 0) umma2_commit(bar_acc_full, leader);
+                    if (part == 2 && k == w.k1 - 1) umma2_commit(bar_acc_full + 8, leader);
+                    __syncwarp();
+                }
             }
-            ++done;
+            ++pieces;
         }
     } else if (warp >= kGEpiWarp0) {
         // ------------------------------------------------------------------ epilogue: lane = row, columns = tokens
-        const int q = warp & 3, ch = (warp - kGEpiWarp0) >> 2;                // row quadrant, half of the columns
+        const int q = warp & 3, ch = (warp - kGEpiWarp0) >> 2;                // row quadrant, share of the columns
         const int row = q * 32 + lane;
-        constexpr int CW = BN / 2 < 16 ? 16 : BN / 2;                         // columns of one half
+        constexpr int CW = BN / (C::EPI / 4);
+        static_assert(CW % 16 == 0, "columns are read sixteen at a time");
         const uint32_t empty0 = map_to_rank(bar_acc_empty, 0);
-        int done = 0;
+        const uint32_t acc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * CW);
+        int steps = 0, pieces = 0;
         while (!failed && sched.next(w)) {
-            const int buf = done & 1;
-            if (!__all_sync(0xffffffffu, mbar_wait_cluster(bar_acc_full + 8 * buf, (uint32_t)((done / 2) & 1), status, 55))) { failed = true; break; }
-            tc_fence_after_sync();
-            const uint32_t acc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)buf * C::ACC;
+            float sum[CW];
+#pragma unroll
+            for (int c = 0; c < CW; ++c) sum[c] = 0.0f;
+            for (int k = w.k0; k <= w.k1; ++k) {
+                // the first parts of a k-step, and after the last one the lower parts of the piece
+                const bool lower = k == w.k1;
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(bar_acc_full + (lower ? 8 : 0), (uint32_t)((lower ? pieces : steps) & 1), status, 55))) { failed = true; break; }
+                tc_fence_after_sync();
+#pragma unroll
+                for (int c0 = 0; c0 < CW; c0 += 16) {
+                    uint32_t v[16];
+                    tmem_ld_32x16(acc + (lower ? C::ACC : 0u) + (uint32_t)c0, v);
+                    tmem_wait_ld(v);
+#pragma unroll
+                    for (int c = 0; c < 16; c += 2) {
+                        float a = __uint_as_float(v[c]), b = __uint_as_float(v[c + 1]);
+                        if (lower) { a = a == a ? a : 0.0f; b = b == b ? b : 0.0f; }          // as add_low
+                        f32x2_split(f32x2_add(f32x2(sum[c0 + c], sum[c0 + c + 1]), f32x2(a, b)), sum[c0 + c], sum[c0 + c + 1]);
+                    }
+                }
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_pair(empty0 + (lower ? 8 : 0));
+                if (!lower) ++steps;
+            }
+            ++pieces;
+            if (failed) break;
             const int rt = w.tile / p.tok_tiles, tt = w.tile - rt * p.tok_tiles;
             const int i = rt * kGRows + rank * 128 + row;                     // row of the chunk
             const bool to_scratch = w.k0 > 0;
@@ -387,7 +423,7 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
                                 for (unsigned tries = 0;; ++tries) {
                                     int v;
                                     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-                                    if (v >= kGEpiWarps) return true;
+                                    if (v >= C::EPI) return true;
                                     __nanosleep(kWaitSleepNs);
                                     if ((tries & 63u) == 63u && wait_limit_expired(limit, status, (uint32_t)o, 0, 56)) return false;
                                 }
@@ -396,51 +432,33 @@ __global__ void __launch_bounds__(kGThreads, 1) lords_dense_kernel(const __grid_
                 for (int o = pair + 1; o < p.pairs && o * left / p.pairs < tile_end; ++o) others = o - pair;
             }
             if (failed) break;
-#pragma unroll 1
-            for (int c0 = ch * CW; c0 < (ch + 1) * CW && c0 < BN; c0 += 16) {
-                uint32_t v[16];
-                tmem_ld_32x16(acc + (uint32_t)c0, v);
-                tmem_wait_ld();
+#pragma unroll
+            for (int c0 = 0; c0 < CW; c0 += 16) {
+                const int col = ch * CW + c0;
                 if (to_scratch) {
-                    float *part = p.partial + ((size_t)(2 * pair + rank) * BN + c0) * 128 + row;
+                    float *part = p.partial + ((size_t)(2 * pair + rank) * BN + col) * 128 + row;
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) __stcg(part + (size_t)c * 128, __uint_as_float(v[c]));
+                    for (int c = 0; c < 16; ++c) __stcg(part + (size_t)c * 128, sum[c0 + c]);
                 } else {
-                    float sum[16];
+                    // the other pieces, added in a fixed order: along k
+                    for (int o = pair + 1; o <= pair + others; ++o) {
+                        const float *part = p.partial + ((size_t)(2 * o + rank) * BN + col) * 128 + row;
+                        float pv[16];
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) sum[c] = __uint_as_float(v[c]);
-                    const long long left = (long long)(p.tiles - p.whole) * p.ksteps;
-                    // the other pieces, four at a time in flight (one trip to L2 each would be paid in turn otherwise), added in a
-                    // fixed order: along k
-                    for (int o0 = pair + 1; o0 <= pair + others; o0 += 4) {
-                        float pv[4][16];
+                        for (int c = 0; c < 16; ++c) pv[c] = __ldcg(part + (size_t)c * 128);
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int o = o0 + j;
-                            const bool has = o <= pair + others && (o + 1) * left / p.pairs != o * left / p.pairs;
-                            const float *part = p.partial + ((size_t)(2 * (has ? o : pair) + rank) * BN + c0) * 128 + row;
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) pv[j][c] = has ? __ldcg(part + (size_t)c * 128) : 0.0f;
-                        }
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) sum[c] += pv[j][c];
+                        for (int c = 0; c < 16; ++c) sum[c0 + c] += pv[c];
                     }
                     if (i < p.rows) {
 #pragma unroll
                         for (int c = 0; c < 16; ++c) {
-                            const int tok = tt * BN + c0 + c;
-                            if (tok < p.M) store_out(p.y, p.y_f32, (size_t)tok * p.ldy + p.row0 + i, sum[c]);
+                            const int tok = tt * BN + col + c;
+                            if (tok < p.M) store_out(p.y, p.y_f32, (size_t)tok * p.ldy + p.row0 + i, sum[c0 + c]);
                         }
                     }
                 }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(empty0 + 8 * buf);
-            piece_done(p.flags, pair, rank, others, to_scratch, kGEpiWarps, lane);
-            ++done;
+            piece_done(p.flags, pair, rank, others, to_scratch, C::EPI, lane);
         }
     }
 
@@ -499,7 +517,7 @@ template <int BN> struct DenseVariant {
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg = cudaLaunchConfig_t{};
         cfg.gridDim = dim3((unsigned)(2 * pairs));
-        cfg.blockDim = dim3(kGThreads);
+        cfg.blockDim = dim3(GCfg<BN>::THREADS);
         cfg.dynamicSmemBytes = GCfg<BN>::SMEM;
         cfg.stream = stream;
         cfg.attrs = attr;
@@ -529,12 +547,13 @@ template <int BN> int launch_product(GemmParams &k, const void *w16, const void 
     k.tok_tiles = (k.M + BN - 1) / BN;
     k.tiles = ((k.rows + kGRows - 1) / kGRows) * k.tok_tiles;
     k.ksteps = np / kGK;
-    // (a k-step is half a step of the pair kernel; 2816 x 3072, rank 100, 1024 tokens: 56 us a call with cut tiles, 45 with whole ones)
-    const Division division = divide_tiles(k.tiles, k.ksteps, pairs_max, 4, 2 * kMeetSteps);
+    k.np = np;
+    // (a k-step, twelve MMAs, is one and a half steps of the pair kernel)
+    const Division division = divide_tiles(k.tiles, k.ksteps, pairs_max, 4, kMeetSteps / 1.5);
     k.pairs = division.pairs;
     k.whole = division.whole;
-    if (!make_map_2d(&k.tm_w, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, w16, (uint64_t)np, (uint64_t)k.rows, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, x16, (uint64_t)np, (uint64_t)k.M, 64, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B))
+    if (!make_map_2d(&k.tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, w16, (uint64_t)np * 3, (uint64_t)k.rows, 64, 128, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_2d(&k.tm_x, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, x16, (uint64_t)np * 2, (uint64_t)k.M, 64, BN / 2, CU_TENSOR_MAP_SWIZZLE_128B))
         return LORDS_ERR_CUDA;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
@@ -549,12 +568,19 @@ template <int BN> int run_dense(const Problem &p, State &st, cudaStream_t stream
     if (pairs < 1 || 2 * pairs > st.counter_slots) return LORDS_ERR_UNSUPPORTED;
     const int np = (p.n + 63) / 64 * 64;
     auto up = [](size_t b) { return (b + 1023) & ~(size_t)1023; };
-    const size_t x_bytes = up((size_t)p.M * np * 2), part_bytes = up(DenseVariant<BN>::partial_bytes(pairs));
+    const size_t x_bytes = up((size_t)p.M * np * 4), part_bytes = up(DenseVariant<BN>::partial_bytes(pairs));
     if (x_bytes + part_bytes >= st.workspace_bytes) return LORDS_ERR_WORKSPACE;
     // rows per chunk: what the rest of the workspace holds (all rows, usually)
-    long long chunk = (long long)((st.workspace_bytes - x_bytes - part_bytes) / ((size_t)np * 2));
-    if (chunk >= p.m) chunk = p.m;
-    else chunk = chunk / kGRows * kGRows;
+    long long chunk = (long long)((st.workspace_bytes - x_bytes - part_bytes) / ((size_t)np * 6));
+    if (chunk >= p.m) {
+        chunk = p.m;
+    } else {
+        // chunks of about equal size: a small last one would leave most pairs idle (5952 x 7008, 578 tokens: 308 us, 255 so)
+        chunk /= kGRows;
+        if (chunk < 1) return LORDS_ERR_WORKSPACE;
+        const long long row_tiles = (p.m + kGRows - 1) / kGRows, chunks = (row_tiles + chunk - 1) / chunk;
+        chunk = (row_tiles + chunks - 1) / chunks * kGRows;
+    }
     if (chunk < 1) return LORDS_ERR_WORKSPACE;
 
     ExpandParams e;

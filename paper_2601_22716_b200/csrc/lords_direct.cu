@@ -12,7 +12,7 @@
 // them, so S of every 16 ranks and the first parts' products of every 16 columns start from zero and are added on the
 // CUDA cores; the lower parts' products, 2^-8 of the sum, keep to the tensor cores.  Error of the fp32 sums
 // against 64 bits, norms, normal activations, 256 x 256 to 1024 x 14336, ranks 4 to 128: 6e-8 to 1.7e-7 (CUDA cores 8e-8 to 1.6e-7; the
-// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 17.0 us a call (fp16 form 10.7, CUDA cores 67.6).
+// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 13.7 us a call (fp16 form 10.7, CUDA cores 67.6).
 //
 // A cluster shares one tile of 128 rows and splits its columns; every CTA sends its partial sums to the CTA that owns
 // the row (asynchronous stores counted on that CTA's barrier), which adds them in rank order: deterministic,
@@ -237,15 +237,14 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     if constexpr (ALIGNED) stage_q(2);
     commit();
     // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
+    uint4 v = level_pair<BITS>(p.levels, tid);
+    if constexpr (!EXACT) {
+        const __half2 h = __floats2half2_rn(__uint_as_float(v.x), __uint_as_float(v.y));
+        v.x = v.y = v.z = v.w = *reinterpret_cast<const uint32_t *>(&h);
+    }
     if (tid < C::ENTRIES) {
-        const float l0 = p.levels[tid & ((1 << BITS) - 1)], l1 = p.levels[tid >> BITS];
-        uint32_t v0 = __float_as_uint(l0), v1 = __float_as_uint(l1);
-        if constexpr (!EXACT) {
-            const __half2 h = __floats2half2_rn(l0, l1);
-            v0 = v1 = *reinterpret_cast<const uint32_t *>(&h);
-        }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(v0, v1, v0, v1));
+        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
     }
     // B fragments of the warp's rows
     const int i0 = row0 + warp * 16 + g, i1 = i0 + 8;

@@ -154,10 +154,22 @@ static int validate(const void *x, const uint8_t *q, const void *B, const void *
 //     TMEM) is most of the call: there the direct kernel stands in for them, under their name (256 x 256: 4.6 -> 3.2 us,
 //     1024 x 2048: 6.1 -> 4.6; level at 2048 x 2048 with rank 32; the two-token kernel sets up less: level at 1024 x 1024;
 //     beyond 16 tokens while token groups x weights stay under 8 M: 1024 x 1024, 64 tokens 7.0 -> 5.9, 128 tokens 8.0 -> 7.5);
-//   - ranks above 64 with up to 16 tokens: the wide-rank kernel, or for small layers the direct kernel;
-//   - everything else: the direct kernel while token groups x weights stay under 32 M (4096 x 4094, 32 tokens: 28 us
-//     against 30; 37 tokens: 46 against 33), then the two-phase path; the CUDA cores for a handful of weights.
+//   - ranks above 64 with up to 16 tokens: the wide-rank kernel, or for small layers the direct kernel (r = 128, 16 tokens: 512 x 512 4.8
+//     against 5.2 us, 768 x 768 5.8 against 5.3);
+//   - everything else: the direct kernel or the two-phase path, whichever an estimate puts first; the CUDA cores for a handful of
+//     weights.
 static bool small_for_decode(const Problem &p) { return (long long)p.m * p.n <= (1 << 19); }
+
+// The direct kernel rebuilds W^ for every group of 16 tokens; the two-phase path does it once, at the price of 6 bytes of scratch a weight
+// (which beyond L2's size go to memory and back) and of two launches.  Microseconds, fitted to eight shapes of 0.7 to 58 M weights at 16 to
+// 128 tokens (direct against two-phase: 4096 x 4094, r = 32: 32 tokens 38 : 53, 48 63 : 57; 1000 x 2730, 128 tokens 27 : 40; 2816 x
+// 3072, r = 100: 32 tokens 29 : 37, 64 52 : 41; 5472 x 10524, 48 tokens 170 : 212): the line misses by at most 4 % of a call there.
+static bool direct_first(const Problem &p)
+{
+    if (p.M > 128) return false;
+    const double w = (double)p.m * p.n / 1048576.0, groups = (p.M + 15) / 16;
+    return 4.0 + (p.r <= 64 ? 1.15 : 1.55) * groups * w <= 25.0 + (w <= 24.0 ? 1.9 : 3.2) * w;
+}
 
 static int dispatch(const Problem &p, State &st, cudaStream_t s)
 {
@@ -202,11 +214,11 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
         if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
     }
     if (weights > (1 << 13)) {
-        if (weights > (1 << 20)) {
+        if (weights > (1 << 19)) {
             rc = launch_wide(p, st, s);
             if (rc != LORDS_ERR_UNSUPPORTED) return rc;
         }
-        if (grouped <= (32 << 20)) {
+        if (direct_first(p)) {
             rc = launch_direct(p, st, s);
             if (rc != LORDS_ERR_UNSUPPORTED) return rc;
         }

@@ -79,7 +79,7 @@ int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t s
 // Up to 16 tokens, ranks 65 .. 128: scale MMA on tcgen05, weights formed in registers.  LORDS_ERR_UNSUPPORTED otherwise.
 int launch_wide(const Problem &p, State &st, cudaStream_t stream);
 
-// Up to 16 tokens, any shape: weights formed in registers and multiplied there (warp-level MMAs).
+// Up to 128 tokens, any shape: weights formed in registers and multiplied there (warp-level MMAs).
 int launch_direct(const Problem &p, State &st, cudaStream_t stream);
 
 // Two-phase tensor-core path for any shape: W^ expanded once into scratch, then a dense product.

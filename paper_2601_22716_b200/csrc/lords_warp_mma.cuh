@@ -62,6 +62,17 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// A level pair's two fp32 words, twice, for the table of pairs; called by whole warps.  (One level a lane and two shuffles: indexed by
+// the pair, the parameters were read again for every copy that is stored, sixteen addresses to a warp: 128 x 128, one token, 3.9 us
+// a call against 2.4.)
+template <int BITS> __device__ __forceinline__ uint4 level_pair(const float (&levels)[16], int pair)
+{
+    const float mine = levels[threadIdx.x & 15];
+    const uint32_t l0 = __float_as_uint(__shfl_sync(0xffffffffu, mine, pair & ((1 << BITS) - 1)));
+    const uint32_t l1 = __float_as_uint(__shfl_sync(0xffffffffu, mine, (pair >> BITS) & ((1 << BITS) - 1)));
+    return make_uint4(l0, l1, l0, l1);
+}
+
 // B[i][k], B[i][k + 1] (k even) as one word, zeros outside the matrix
 __device__ __forceinline__ uint32_t load_b_pair(const uint16_t *B, int i, int k, int rows, int r)
 {

@@ -16,7 +16,7 @@
 // Why a kernel of its own: the factor strip of 128 ranks is 32 KB, which the level table and the rings of the 16-token
 // decode kernel leave no room for, and at 128 ranks the scale product outweighs everything else, so it belongs on
 // tcgen05: with S by warp-level MMAs (the direct kernel) every warp reads the whole factor strip from shared memory
-// again.  4096 x 4096, r = 128, 16 tokens: CUDA cores 585 us, direct kernel 31.7 us, this kernel 19.4 us (10.4 with W^ in fp16).
+// again.  4096 x 4096, r = 128, 16 tokens: CUDA cores 585 us, direct kernel 29 us, this kernel 17.5 us (10.4 with W^ in fp16).
 //
 // CTA: 128 rows; sixteen consumer warps (32 rows and 32 columns of the strip each), a TMA producer, a warp that makes the copy of the
 // activations without infinities and NaNs, and a scale issuer.  A cluster shares one row tile and splits its strips; every warp
@@ -24,7 +24,7 @@
 // adds them in a fixed order: deterministic, no atomics, no trip through global memory.
 //
 // Bound: the consumers' instructions (about sixteen a weight: look-up, product, cutting into parts, MMAs) and the latency of their chain, four
-// warps to a scheduler: 1.6 us a strip of 16384 weights (the call above with twice the columns: 31.9 us), of which the strip's
+// warps to a scheduler: 1.6 us a strip of 16384 weights (8192 columns, eight more strips a CTA, take 12.6 us more), of which the strip's
 // arrival (44 KB from L2) and its scale MMAs (8 KB of operands per 16 ranks) are about a third each and overlap.
 //
 // Every wait is bounded; on expiry the role records LORDS_ERR_TIMEOUT and leaves its loop.
@@ -251,10 +251,10 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         // row group rw (its TMEM quadrant), column quarter ch
         const int g = lane >> 2, t = lane & 3, rw = warp & 3, ch = warp >> 2;
         // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
+        const uint4 v = level_pair<BITS>(p.levels, tid);
         if (tid < C::ENTRIES) {
-            const uint32_t l0 = __float_as_uint(p.levels[tid & ((1 << BITS) - 1)]), l1 = __float_as_uint(p.levels[tid >> BITS]);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), make_uint4(l0, l1, l0, l1));
+            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
         }
         if (!b_by_tma) {
             // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m

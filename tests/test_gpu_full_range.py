@@ -20,7 +20,8 @@ DIRECT = [
     (4, 1000, 2730, 10, 37),     # ragged, several token groups
     (2, 333, 1028, 64, 9),
     (3, 130, 352, 33, 16),
-    (4, 640, 1024, 128, 5),      # wide, small
+    (4, 500, 1000, 128, 16),     # wide and ragged
+    (4, 512, 640, 128, 5),       # wide, small
 ]
 WIDE = [
     # ranks above 64: more than a million weights, up to 16 tokens; three and four sums of 32 ranks, with and without a rest
@@ -29,6 +30,13 @@ WIDE = [
     (2, 530, 2112, 97, 16),
     (4, 300, 4096, 128, 8),
 ]
+DENSE = [
+    # more than 128 tokens: every part of W^ through scratch; one and several token tiles, cut and whole tiles
+    (4, 300, 1030, 9, 130),
+    (3, 270, 2080, 100, 257),
+    (2, 700, 516, 40, 300),
+]
+SHAPES = DIRECT + WIDE + DENSE
 
 
 @pytest.fixture(scope="module")
@@ -45,7 +53,7 @@ def _scaled(bits, words, factor):
     return gen.bf16_bits(torch.from_numpy(gen.bf16_to_f32(words) * np.float32(factor)))
 
 
-@pytest.mark.parametrize("bits,m,n,r,M", DIRECT + WIDE)
+@pytest.mark.parametrize("bits,m,n,r,M", SHAPES)
 @pytest.mark.parametrize("xs,bs", [(1.0, 1.0), (2.0**30, 2.0**-20), (2.0**-30, 2.0**-30), (2.0**-20, 2.0**40)])
 def test_precision_and_range(lords, bits, m, n, r, M, xs, bs):
     """x to 2^30 and factors from 2^-30 to 2^40: far outside fp16, with the precision of fp32."""
@@ -53,12 +61,13 @@ def test_precision_and_range(lords, bits, m, n, r, M, xs, bs):
     lay.x, lay.B = _scaled(bits, lay.x, xs), _scaled(bits, lay.B, bs)
     dl = DeviceLayer(lay)
     y32, _ = dl.forward()
-    assert (lords.lords_last_path() == "wide") == ((bits, m, n, r, M) in WIDE)
+    shape = (bits, m, n, r, M)
+    assert (lords.lords_last_path() == "wide", lords.lords_last_path() == "dense") == (shape in WIDE, shape in DENSE)
     normwise, _ = error_metrics(y32, oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits))
     assert normwise <= FP32_TOL
 
 
-@pytest.mark.parametrize("bits,m,n,r,M", DIRECT + WIDE)
+@pytest.mark.parametrize("bits,m,n,r,M", SHAPES)
 def test_infinities_and_nans_as_on_the_cuda_cores(lords, bits, m, n, r, M):
     """One infinite, one NaN activation, a row of infinite weights and one of NaNs.  Integer data: most weights have lower parts that
     are exactly zero, which must not meet an infinity.  Products that overflow a float are infinite as well."""
