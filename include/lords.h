@@ -180,9 +180,10 @@ int lords_linear_forward_host(const void *x_host, const uint8_t *Qpacked, const 
  * Quantisation step of the alternating refinement (Alg. 1, step 2.1; Sec. 3.3): with the factors fixed,
  *     Q_ij = argmin over the codes c of (S_ij * L[c] - W_ij)^2,   S = B A (Eq. 3),
  * written as packed codes in the layout above (ready for the forward calls).  The paper does not say
- * which level wins a tie: the lowest code does.  S is accumulated in fp32 and every level is tried in
+ * which level wins a tie: the lowest code does.  S is accumulated in fp32 and the decision is taken in
  * fp32, so a weight within rounding distance of the midpoint between two levels' products may get
- * either neighbour.
+ * either neighbour.  (Layers with n no multiple of 64 or r > 64 whose S comes from the tensor cores have
+ * such decisions taken in 64 bits.)
  *   W        : device, bf16 [m][n], the weight to quantise (out-features x in-features)
  *   B, A     : device, bf16 [m][r] and [r][n]
  *   codebook : HOST, 2^bits floats (ascending or not: codes index it as given)

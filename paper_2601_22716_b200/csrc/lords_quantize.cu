@@ -25,17 +25,19 @@
 //
 // Bound: instructions per weight (about 20 with packing) and the latency of their chain.  14336 x 4096, 3 bits, r = 48: 90 us with
 // bisection and weights read row by row from global memory, 51 now; 4096 x 4096, 4 bits, r = 32: 47 -> 20; r = 128, on the CUDA
-// cores before: 857 -> 21.
+// cores before: 834 -> 60.
 //
 // Rows of W or A that are not 16-byte multiples (n not a multiple of 8) are copied to padded rows in the workspace first; without
 // room there, and for small layers off the tile grid, a plain CUDA-core kernel runs.
-// That kernel sums S on the CUDA cores and compares squared errors, this one midpoints: both round in fp32, and a weight whose two nearest
-// levels are equally far to within that rounding can get the other of the two (5472 x 10524, r = 6: 10 bytes in 28.8 M at most, the
-// two errors 2e-7 of |W| apart).
+//
+// Layers with a ragged row (n not a multiple of 64) or a rank above 64 ran on the CUDA cores before, whose sums (rounded to nearest) and
+// comparison of errors (one rounding of a small difference) are nearer to the exact decision than the tensor cores' S, which is cut off,
+// and a rounded product.  For them (SURE) a weight that lies nearer to a midpoint than S and the midpoint may be off is decided in
+// 64 bits: their codes are the exact ones (of 1.2e9 weights none differs from the decision in 64 bits; on the CUDA cores 1 to 7 of 16.8 M at
+// r = 128 did).  4096 x 4096, r = 128: 60 us a call, 180 with factors of mixed sign, whose S cancels (CUDA cores 834; 19 with the tensor cores'
+// S for every decision); 5472 x 10524, r = 6: 227 (437; 199).
 #include <cuda.h>
 #include <cuda_bf16.h>
-
-#include <type_traits>
 
 #include "lords_internal.h"
 #include "lords_ptx.cuh"
@@ -78,11 +80,15 @@ struct alignas(64) QuantParams {
     CUtensorMap tm_w;     // bf16 [m][n], box {64, 128}, 128-byte swizzle (rows past m and columns past n read as zero)
     CUtensorMap tm_b;     // bf16 [m][r], box {64, 128}, 128-byte swizzle; used if rows of B are 16-byte multiples
     const uint16_t *B;    // bf16 [m][r]
+    const uint16_t *A;    // bf16 [r][n]
+    const float *a_norm;  // SURE: per step, how far S of a row of norm 1 may put a weight from its midpoint
+    const float *b_norm;  // SURE: per row, the norm of its B
     uint8_t *Q;           // packed codes, row pitch n * bits / 8
     float levels[16];
     float mids[16];       // ascending table: mids[c] = (levels[c] + levels[c + 1]) / 2
     float bucket_mid[64]; // the midpoint in (or next to) bucket k, +infinity if there is none above its lower edge
     uint8_t bucket_code[64];   // midpoints below it
+    float least_scale;    // SURE: |S| has to be more than this times what it may be off for the bucket to be the right one
     float bucket_scale, bucket_bias;   // bucket of a ratio t: saturate(t * scale + bias) * (buckets - 1), rounded
     int m, n, r, r_pad;
     int steps;            // 64-column steps per row tile
@@ -141,6 +147,34 @@ __device__ __forceinline__ uint32_t nearest_code_sorted(float s, float w, const 
     }
 }
 
+// The exact decision: S in 64 bits (products of bf16 are exact there), every level in turn.
+template <int LEVELS>
+__device__ __noinline__ uint32_t exact_code(const QuantParams &p, int i, int j, float w)
+{
+    const uint16_t *b = p.B + (size_t)i * p.r, *a = p.A + j;
+    double s = 0.0;
+    for (int k = 0; k < p.r; ++k)         // (unrolled sixteen times it is slower: r = 128, mixed signs, 409 us against 260)
+        s = fma((double)__uint_as_float((uint32_t)b[k] << 16), (double)__uint_as_float((uint32_t)a[(size_t)k * p.n] << 16), s);
+    uint32_t best = 0;
+    double e_best = 0.0;
+    for (int c = 0; c < LEVELS; ++c) {
+        const double d = fma(s, (double)p.levels[c], -(double)w), e = d * d;
+        if (c == 0 || e < e_best) { e_best = e; best = (uint32_t)c; }
+    }
+    return best;
+}
+// Code c of the 32 in `packed` replaced.
+template <int BITS> __device__ __forceinline__ void replace_code(uint32_t (&packed)[BITS], int c, uint32_t code)
+{
+    constexpr uint32_t mask = (1u << BITS) - 1u;
+    const int at = c * BITS >> 5, sh = c * BITS & 31;
+#pragma unroll
+    for (int k = 0; k < BITS; ++k) {
+        if (k == at) packed[k] = (packed[k] & ~(mask << sh)) | code << sh;
+        if (k == at + 1 && sh + BITS > 32) packed[k] = (packed[k] & ~(mask >> (32 - sh))) | code >> (32 - sh);
+    }
+}
+
 // The first `count` of 32 codes of one row -> packed bytes at `dst` (the row's byte offset of these 32 columns); w: the codes packed, BITS
 // words.  `words`: dst is 4-byte aligned; 16-byte aligned rows of 4-bit codes go out as one word.
 template <int BITS> __device__ __forceinline__ void store_codes(uint8_t *dst, const uint32_t (&w)[BITS], int count, bool words, bool vec)
@@ -161,8 +195,8 @@ template <int BITS> __device__ __forceinline__ void store_codes(uint8_t *dst, co
     }
 }
 
-// EDGE: some tile reaches past the matrix (a variant of its own: the check costs the others 3 %).
-template <int BITS, int MODE, int RA, bool EDGE>
+// EDGE: some tile reaches past the matrix (a variant of its own: the check costs the others 3 %).  SURE: close decisions in 64 bits.
+template <int BITS, int MODE, int RA, bool EDGE, bool SURE>
 __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __grid_constant__ QuantParams p)
 {
     using C = QuantCfg<BITS, RA>;
@@ -307,10 +341,17 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
         const bool words = (qpitch & 3) == 0, vec = (qpitch & 15) == 0;
         const int group = warp / kSearchWarps;
         const uint32_t stage = bars + 256u + (uint32_t)(warp * C::STAGE);
-        int rt = rt0, st = st0 + group;
+        int rt = rt0, st = st0 + group, b_row = -1;
+        float b_norm = 0.0f;
         for (int it = group; it < total; it += kGroupsQ) {
             while (st >= p.steps) { st -= p.steps; ++rt; }
             const int sd = it % kSDQ, sw = it % kSWQ, col0 = st * kColsQ + ch * 32, i = rt * kRowsQ + row;
+            float off = 0.0f, least_s = 0.0f;                // SURE: a product of S and a midpoint is off by no more than this
+            if constexpr (SURE) {
+                if (i != b_row) { b_row = i; b_norm = i < p.m ? __ldg(p.b_norm + i) : 0.0f; }
+                off = b_norm * __ldg(p.a_norm + st);
+                least_s = off * p.least_scale;
+            }
             st += kGroupsQ;
             if (!mbar_wait_warp2(bar_s + 8 * sd, (uint32_t)((it / kSDQ) & 1), bar_w + 8 * sw, (uint32_t)((it / kSWQ) & 1), status, 35)) { failed = true; break; }
             tc_fence_after_sync();
@@ -323,6 +364,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                 uint32_t s[16];
                 tmem_ld_32x16(lane_addr + (uint32_t)(sd * kColsQ + h * 16), s);
                 const uint32_t at = w_row + (uint32_t)(sw * kWTileQ);
+                uint32_t unsure = 0;                         // SURE: a bit per column
                 const uint4 wv[2] = {lds_v4(at + (uint32_t)(((ch * 4 + h * 2) ^ (row & 7)) << 4)), lds_v4(at + (uint32_t)(((ch * 4 + h * 2 + 1) ^ (row & 7)) << 4))};
                 tmem_wait_ld(s);
                 if (h == 1) {
@@ -370,9 +412,18 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                             asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(mid), "=r"(below) : "r"(__float_as_uint(f[c & 1]) * 256u + lut_magic));
                             // t > mid  <=>  w sign(s) > |s| mid (as in the bisection)
                             const float b = __uint_as_float(__float_as_uint(w) ^ (s[c & 15] & 0x80000000u));
+                            if constexpr (SURE) {
+                                const float d = fmaf(-fabsf(__uint_as_float(s[c & 15])), __uint_as_float(mid), b);
+                                asm("set.gt.u32.f32 %0, %1, %2;" : "=r"(above) : "f"(d), "f"(0.0f));
+                                if (!(fabsf(d) > off && fabsf(__uint_as_float(s[c & 15])) > least_s && fabsf(w) < INFINITY)) unsure |= 1u << (c & 15);
+                                return below - above;
+                            }
                             asm("set.gt.u32.f32 %0, %1, %2;" : "=r"(above) : "f"(b), "f"(fabsf(__uint_as_float(s[c & 15])) * __uint_as_float(mid)));
                             return below - above;             // the outcome is 0 or -1
                         });
+                    } else if constexpr (SURE) {
+                        pack([](int) { return 0u; });
+                        unsure = 0xFFFFu;
                     } else {
                         // the bisection's answer by counting, which needs no registers for its thresholds
                         pack([&](int c) {
@@ -382,6 +433,20 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                             for (int l = 0; l + 1 < (1 << BITS); ++l) code += b > a * p.mids[l] ? 1u : 0u;
                             return code;
                         });
+                    }
+                    if constexpr (SURE) {
+                        const int left = i < p.m ? p.n - col0 - h * 16 : 0;          // columns of the sixteen that exist
+                        unsure &= left >= 16 ? 0xFFFFu : left > 0 ? (1u << left) - 1u : 0u;
+                        if (__any_sync(0xffffffffu, unsure != 0u)) {
+                            for (; unsure != 0u; unsure &= unsure - 1u) {
+                                const int c = h * 16 + __ffs((int)unsure) - 1;
+                                float w = 0.0f;
+#pragma unroll
+                                for (int e = h * 16; e < h * 16 + 16; ++e) w = e == c ? weight(e) : w;
+                                replace_code<BITS>(packed, c, exact_code<(1 << BITS)>(p, i, col0 + c, w));
+                            }
+                            __syncwarp();
+                        }
                     }
                 } else if constexpr (MODE == kBisect) {
                     pack([&](int c) { return nearest_code_sorted<(1 << BITS)>(__uint_as_float(s[c & 15]), weight(c), lv); });
@@ -442,12 +507,50 @@ __global__ void lords_quantize_simt_kernel(const uint16_t *__restrict__ W, const
     for (int b = 0; b < BYTES; ++b) dst[b] = b < 8 ? (uint8_t)(lo >> (8 * b)) : (uint8_t)(hi >> (8 * (b - 8)));
 }
 
-template <int BITS, int MODE, int RA, bool EDGE> int launch_quantize_tc(QuantParams &k, const State &st, cudaStream_t stream)
+// Blocks below `steps`: how far S of a row of norm 1 may put a weight from a midpoint, over the 64 columns of a step, i.e. `scale` times the
+// largest norm of a column of A.  The others: norms of eight rows of B each.
+__global__ void __launch_bounds__(256) lords_quantize_norms_kernel(const uint16_t *__restrict__ B, const uint16_t *__restrict__ A, int m, int n, int r,
+                                                                   int steps, float scale, float *__restrict__ a_norm, float *__restrict__ b_norm)
+{
+    __shared__ float part[256];
+    const int tid = threadIdx.x, lane = tid & 31;
+    float sum = 0.0f;
+    if ((int)blockIdx.x < steps) {
+        const int j = (int)blockIdx.x * kColsQ + (tid & 63);
+        if (j < n)
+            for (int k = tid >> 6; k < r; k += 4) {
+                const float v = __uint_as_float((uint32_t)A[(size_t)k * n + j] << 16);
+                sum = fmaf(v, v, sum);
+            }
+        part[tid] = sum;
+        __syncthreads();
+        if (tid < 32) {
+            float most = 0.0f;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) most = fmaxf(most, part[tid + 32 * h] + part[tid + 32 * h + 64] + part[tid + 32 * h + 128] + part[tid + 32 * h + 192]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
+            if (tid == 0) a_norm[blockIdx.x] = scale * sqrtf(most);
+        }
+    } else {
+        const int i = ((int)blockIdx.x - steps) * 8 + (tid >> 5);
+        if (i >= m) return;
+        for (int k = lane; k < r; k += 32) {
+            const float v = __uint_as_float((uint32_t)B[(size_t)i * r + k] << 16);
+            sum = fmaf(v, v, sum);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0) b_norm[i] = sqrtf(sum);
+    }
+}
+
+template <int BITS, int MODE, int RA, bool EDGE, bool SURE> int launch_quantize_tc(QuantParams &k, const State &st, cudaStream_t stream)
 {
     static bool done[kMaxDevices] = {};
     const int dev = device_slot(st);
     if (!done[dev]) {
-        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_quantize_kernel<BITS, MODE, RA, EDGE>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuantCfg<BITS, RA>::SMEM));
+        LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_quantize_kernel<BITS, MODE, RA, EDGE, SURE>, cudaFuncAttributeMaxDynamicSharedMemorySize, QuantCfg<BITS, RA>::SMEM));
         done[dev] = true;
     }
     // One run of steps per CTA that can be resident: setting a CTA up costs as much as about three steps, which a second round of CTAs
@@ -466,37 +569,35 @@ template <int BITS, int MODE, int RA, bool EDGE> int launch_quantize_tc(QuantPar
         grid = (long long)k.row_tiles * k.row_splits;
     }
     if (grid > 2147483647LL) return LORDS_ERR_SHAPE;
-    lords_quantize_kernel<BITS, MODE, RA, EDGE><<<(unsigned)grid, kThreadsQ, QuantCfg<BITS, RA>::SMEM, stream>>>(k);
+    lords_quantize_kernel<BITS, MODE, RA, EDGE, SURE><<<(unsigned)grid, kThreadsQ, QuantCfg<BITS, RA>::SMEM, stream>>>(k);
     LORDS_CUDA_TRY(cudaGetLastError());
     return LORDS_OK;
 }
-template <int BITS> int launch_quantize_tc(QuantParams &k, int mode, const State &st, cudaStream_t stream)
+template <int BITS> int launch_quantize_tc(QuantParams &k, int mode, bool sure, const State &st, cudaStream_t stream)
 {
-    auto run = [&](auto ra) {
-        constexpr int RA = decltype(ra)::value;
-        if (mode == kBisect) return launch_quantize_tc<BITS, kBisect, RA, false>(k, st, stream);
-        if (mode == kTrial) return launch_quantize_tc<BITS, kTrial, RA, false>(k, st, stream);
-        return k.m % kRowsQ != 0 || k.n % kColsQ != 0 ? launch_quantize_tc<BITS, kBuckets, RA, true>(k, st, stream)
-                                                      : launch_quantize_tc<BITS, kBuckets, RA, false>(k, st, stream);
-    };
-    return k.r <= 64 ? run(std::integral_constant<int, 64>{}) : run(std::integral_constant<int, 128>{});
+    if (sure) return k.r <= 64 ? launch_quantize_tc<BITS, kBuckets, 64, true, true>(k, st, stream) : launch_quantize_tc<BITS, kBuckets, 128, true, true>(k, st, stream);
+    if (mode == kBisect) return launch_quantize_tc<BITS, kBisect, 64, false, false>(k, st, stream);
+    if (mode == kTrial) return launch_quantize_tc<BITS, kTrial, 64, false, false>(k, st, stream);
+    return k.m % kRowsQ != 0 ? launch_quantize_tc<BITS, kBuckets, 64, true, false>(k, st, stream) : launch_quantize_tc<BITS, kBuckets, 64, false, false>(k, st, stream);
 }
 
 // The bucket table of an ascending level table.  Buckets are the rounding intervals of `buckets` equally spaced points that cover the
 // midpoints with half a spacing to spare on both sides; the ratio that picks one is off by less than 1e-5 of a
-// bucket's range, so a bucket answers for its interval widened by 1e-3 of the spacing.  False if some widened interval holds two midpoints.
-bool make_buckets(QuantParams &k, const float *levels, int bits, int buckets)
+// bucket's range (what S is off by comes on top: SURE), so a bucket answers for its interval widened by 1e-3 of the spacing, or with SURE
+// by a quarter of it.  False if some widened interval holds two midpoints.
+bool make_buckets(QuantParams &k, const float *levels, int bits, int buckets, bool sure)
 {
     const int nm = (1 << bits) - 1;
     const double lo = 0.5 * ((double)levels[0] + levels[1]), hi = 0.5 * ((double)levels[nm - 1] + levels[nm]);
     const double h = (hi - lo) / (buckets - 2), first = lo - 0.5 * h;        // point k at first + k h
     if (!(h > 0.0) || !(h < 1e30)) return false;
-    const double span = h * (buckets - 1);
+    const double span = h * (buckets - 1), widened = 0.5 + (sure ? 0.25 : 1e-3);
+    k.least_scale = (float)(1.0 / (0.2 * h));        // a ratio inside the table's range is then off by less than a fifth of a spacing
     k.bucket_scale = (float)(1.0 / span);
     k.bucket_bias = (float)(-first / span);
     if (!(k.bucket_scale > 1e-30f) || !(k.bucket_scale < 1e30f) || !(k.bucket_bias > -1e4f) || !(k.bucket_bias < 1e4f)) return false;
     for (int b = 0; b < buckets; ++b) {
-        const double a = first + (b - 0.501) * h, z = first + (b + 0.501) * h;
+        const double a = first + (b - widened) * h, z = first + (b + widened) * h;
         int below = 0, inside = 0;
         float mid = INFINITY;
         for (int c = 0; c < nm; ++c) {
@@ -516,13 +617,24 @@ bool make_buckets(QuantParams &k, const float *levels, int bits, int buckets)
 int launch_quantize(const void *W, const void *B, const void *A, const float *levels, int bits, int m, int n, int r,
                     uint8_t *Q, State &st, cudaStream_t stream)
 {
-    // rows that are not 16-byte multiples: padded copies of W and A in the workspace
+    QuantParams k;
+    for (int c = 0; c < 16; ++c) k.levels[c] = c < (1 << bits) ? levels[c] : 0.0f;
+    bool sorted = true;
+    for (int c = 0; c + 1 < (1 << bits); ++c) sorted = sorted && levels[c] < levels[c + 1];
+    for (int c = 0; c < 16; ++c) k.mids[c] = (sorted && c + 1 < (1 << bits)) ? 0.5f * (levels[c] + levels[c + 1]) : 0.0f;
+    const int buckets = bits == 4 ? QuantCfg<4, 64>::BUCKETS : bits == 3 ? QuantCfg<3, 64>::BUCKETS : QuantCfg<2, 64>::BUCKETS;
     const int np = (n + 7) / 8 * 8;
-    const size_t w_bytes = ((size_t)m * np * 2 + 255) & ~(size_t)255, a_bytes = (size_t)r * np * 2;
-    const bool pad = np != n;
-    // small layers with a ragged row or a rank above 64 stay on the CUDA cores: a few microseconds there as here, in one launch
-    const bool small = (n % kColsQ != 0 || r > 64) && (long long)m * n <= (5 << 18);
-    const bool tc = !small && (!pad || w_bytes + a_bytes <= st.workspace_bytes);      // the row tiles are the grid's x dimension: any int fits
+    const bool pad = np != n, sure = n % kColsQ != 0 || r > 64;
+    const int mode = !sorted ? kTrial : make_buckets(k, levels, bits, buckets, sure) ? kBuckets : kBisect;
+    // rows that are not 16-byte multiples: padded copies of W and A in the workspace; behind them the norms that close decisions need
+    k.steps = (n + kColsQ - 1) / kColsQ;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t w_bytes = pad ? up((size_t)m * np * 2) : 0, a_bytes = pad ? up((size_t)r * np * 2) : 0;
+    const size_t norm_bytes = sure ? ((size_t)k.steps + (size_t)m) * sizeof(float) : 0;
+    // Layers with a ragged row or a rank above 64 stay on the CUDA cores where they are small (a few microseconds there as here, in one
+    // launch) and with level tables that have no buckets.
+    const bool simt = sure && ((long long)m * n <= (5 << 18) || mode != kBuckets);
+    const bool tc = !simt && w_bytes + a_bytes + norm_bytes <= st.workspace_bytes && k.steps + ((long long)m + 7) / 8 <= 2147483647LL;
     if (tc && st.forced_path != 1) {
         int launches = 1;
         const void *Wt = W, *At = A;
@@ -537,17 +649,23 @@ int launch_quantize(const void *W, const void *B, const void *A, const float *le
             Wt = wp; At = ap;
             ++launches;
         }
-        QuantParams k;
-        k.B = static_cast<const uint16_t *>(B); k.Q = Q;
-        for (int c = 0; c < 16; ++c) k.levels[c] = c < (1 << bits) ? levels[c] : 0.0f;
-        bool sorted = true;
-        for (int c = 0; c + 1 < (1 << bits); ++c) sorted = sorted && levels[c] < levels[c + 1];
-        for (int c = 0; c < 16; ++c) k.mids[c] = (sorted && c + 1 < (1 << bits)) ? 0.5f * (levels[c] + levels[c + 1]) : 0.0f;
-        const int buckets = bits == 4 ? QuantCfg<4, 64>::BUCKETS : bits == 3 ? QuantCfg<3, 64>::BUCKETS : QuantCfg<2, 64>::BUCKETS;
-        const int mode = !sorted ? kTrial : make_buckets(k, levels, bits, buckets) ? kBuckets : kBisect;
+        k.B = static_cast<const uint16_t *>(B); k.A = static_cast<const uint16_t *>(A); k.Q = Q;
         k.m = m; k.n = n; k.r = r; k.r_pad = (r + 15) / 16 * 16;
-        k.steps = (n + kColsQ - 1) / kColsQ;
         k.status = st.status_word;
+        k.a_norm = k.b_norm = nullptr;
+        if (sure) {
+            // How far S is off, relative to the sum of absolute products, which the product of norms bounds: an MMA over 16 ranks cuts its
+            // sum off below 2^-23 of what has been summed so far, so K of them by (K + 1) 2^-24; 2^-24 more for the midpoint's own rounding.
+            // (With a quarter of this no code of 1.2e9 was wrong either, with a sixteenth one in 2e8.)
+            float most = 0.0f;
+            for (int c = 0; c + 1 < (1 << bits); ++c) most = k.mids[c] > most ? k.mids[c] : -k.mids[c] > most ? -k.mids[c] : most;
+            float *a_norm = reinterpret_cast<float *>(st.workspace + w_bytes + a_bytes), *b_norm = a_norm + k.steps;
+            lords_quantize_norms_kernel<<<(unsigned)(k.steps + (m + 7) / 8), 256, 0, stream>>>(k.B, k.A, m, n, r, k.steps, most * (float)(k.r_pad / 16 + 2) * 5.960464478e-8f,
+                                                                                              a_norm, b_norm);
+            LORDS_CUDA_TRY(cudaGetLastError());
+            k.a_norm = a_norm; k.b_norm = b_norm;
+            ++launches;
+        }
         if (!make_map_2d(&k.tm_a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, At, (uint64_t)np, (uint64_t)r, 64, (uint32_t)k.r_pad, CU_TENSOR_MAP_SWIZZLE_128B) ||
             !make_map_2d(&k.tm_w, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Wt, (uint64_t)np, (uint64_t)m, 64, (uint32_t)kRowsQ, CU_TENSOR_MAP_SWIZZLE_128B))
             return LORDS_ERR_CUDA;
@@ -555,8 +673,8 @@ int launch_quantize(const void *W, const void *B, const void *A, const float *le
         if ((r & 7) == 0 &&
             !make_map_2d(&k.tm_b, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, B, (uint64_t)r, (uint64_t)m, 64, (uint32_t)kRowsQ, CU_TENSOR_MAP_SWIZZLE_128B))
             return LORDS_ERR_CUDA;
-        const int rc = bits == 4 ? launch_quantize_tc<4>(k, mode, st, stream) : bits == 3 ? launch_quantize_tc<3>(k, mode, st, stream)
-                                                                              : launch_quantize_tc<2>(k, mode, st, stream);
+        const int rc = bits == 4 ? launch_quantize_tc<4>(k, mode, sure, st, stream) : bits == 3 ? launch_quantize_tc<3>(k, mode, sure, st, stream)
+                                                                                    : launch_quantize_tc<2>(k, mode, sure, st, stream);
         if (rc != LORDS_OK) return rc;
         st.last_launches = launches;
         st.last_path = "quantize";
