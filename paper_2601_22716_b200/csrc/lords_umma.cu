@@ -266,6 +266,12 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
     }
     // let a dependent launch begin its own weight prefetch as SMs become free
     griddep_launch_dependents();
+    // Every role passes the end of the previous launch before its first bounded wait for something that needs the activations, itself or
+    // by way of another role that waits there; what comes before that (SD k-steps) runs ahead on weights alone.
+    bool passed = false;
+    auto previous_launch = [&] {
+        if (!passed) { griddep_wait(); passed = true; }
+    };
 
     if (warp == kTmaWarp) {
         // all done above
@@ -280,6 +286,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                 // commit the workers wait for as well (this lane looks at every phase of those barriers
                 // in turn, and no slot barrier can run a phase ahead of it: the scale MMA of k-step
                 // j - SA + SD needs a factor tile that this lane has not loaded yet)
+                if (j >= SA + SD) previous_launch();
                 if (j >= SA && !mbar_wait<kWaitSlackNs>(bar_s_full + 8 * ((j - SA) % SD), (uint32_t)(((j - SA) / SD) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_a_full + 8 * sa;
                 mbar_expect_tx(bar, tx);
@@ -302,6 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
         const uint32_t leader = elect_one();
         for (int j = 0; j < total; ++j) {
             const int sa = j % SA, sd = j % SD;
+            if (j >= SD) previous_launch();
             if (!mbar_wait<kWaitSpin>(bar_a_full + 8 * sa, (uint32_t)((j / SA) & 1))) { failed = true; break; }
             // the slot is free once the main MMAs of k-step j - SD have read their operand out of it
             if (j >= SD && !mbar_wait<kWaitSpin>(bar_done + 8 * ((j - SD) % DR), (uint32_t)(((j - SD) / DR) & 1))) { failed = true; break; }
@@ -322,6 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
         const uint32_t x_lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((x0 & 0x3FFFFu) >> 4);
         tmem_base = warp_uniform(tmem_base);
         const uint32_t leader = elect_one();
+        previous_launch();
         for (int it = 0; it < total; ++it) {
             const int sx = it % SX, ws = it % SD;
             // W^ of the k-step is in TMEM and its activation tile has landed
@@ -350,6 +359,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
 
         for (int it = g; it < total; it += 2) {
             const int sx = it % SX, sd = it % SD, pr = it >> 1, sq = pr % SQ;
+            if (it >= SD || C::kConvertInKernel) previous_launch();
             if (!__all_sync(0xffffffffu, mbar_wait(bar_s_full + 8 * sd, (uint32_t)((it / SD) & 1)))) { failed = true; break; }
             tc_fence_after_sync();
             uint32_t s[32];
@@ -400,6 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                 asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
                 cluster_waited = true;
             }
+            previous_launch();
             if (total > 0) ok = __all_sync(0xffffffffu, mbar_wait(bar_acc_full, 0));
             tc_fence_after_sync();
             const int i = row0 + row;

@@ -140,11 +140,16 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
     Schedule sched(p.pairs, p.whole, p.tiles, p.steps, pair);
     Piece w;
     int st = 0;                                   // steps so far, over all pieces: ring positions and phases
+    // Every role passes the end of the previous launch before its first bounded wait for something that needs the activations, itself or
+    // by way of another role that waits there; what comes before that runs ahead on weights alone.
+    bool passed = false;
+    auto previous_launch = [&] {
+        if (!passed) { griddep_wait(); passed = true; }
+    };
     if (warp == kPTmaX) {
         // ------------------------------------------------------------------ activations (this CTA's half of the tokens) and codes
         if (lane == 0) {
             const uint32_t x_pair0 = map_to_rank(bar_x, 0);
-            bool waited = false;
             const uint32_t x_tx = (uint32_t)(p.bn * 128);
             while (!failed && sched.next(w)) {
                 const int rt = w.tile / p.tok_tiles, tt = w.tile - rt * p.tok_tiles;
@@ -153,7 +158,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
                     if (st >= kPSQ && !mbar_wait<kWaitSlackNs>(bar_q_free + 8 * sq, (uint32_t)((st / kPSQ - 1) & 1), status, 61)) { failed = true; break; }
                     mbar_expect_tx(bar_q + 8 * sq, (uint32_t)C::QSTAGE);
                     tma_load_2d(q0 + (uint32_t)(sq * C::QSTAGE), &p.tm_q, k * C::QROW, rt * kPRows + rank * 128, bar_q + 8 * sq);
-                    if (!waited) { griddep_wait(); waited = true; }           // the activations are the pre-pass's
+                    previous_launch();                                        // the activations are the pre-pass's
                     for (int h = 0; h < 2; ++h) {
                         const int ks = 2 * st + h, sx = ks % C::SX, prev = ks - C::SX;
                         if (prev >= 0 && !mbar_wait(bar_done + 8 * (prev % kPDone), (uint32_t)((prev / kPDone) & 1), status, 62)) { failed = true; break; }
@@ -173,15 +178,17 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             const uint32_t a_pair0 = map_to_rank(bar_a, 0), b_pair0 = map_to_rank(bar_b, 0);
             tma_prefetch_desc(&p.tm_a);
             tma_prefetch_desc(&p.tm_b);
-            if (!p.b_early) griddep_wait();
+            if (!p.b_early) previous_launch();
             while (!failed && sched.next(w)) {
                 const int rt = w.tile / p.tok_tiles;
+                if (st > 0) previous_launch();
                 // the scale MMAs of the piece before have read its B
                 if (st > 0 && !mbar_wait(bar_a_free + 8 * ((st - 1) % kPSA), (uint32_t)(((st - 1) / kPSA) & 1), status, 64)) { failed = true; break; }
                 if (rank == 0) mbar_expect_tx(bar_b, 2u * C::BTILE);
                 tma_load_2d_pair(b_tile, &p.tm_b, 0, rt * kPRows + rank * 128, b_pair0);
                 for (int k = w.k0; k < w.k1; ++k, ++st) {
                     const int sa = st % kPSA;
+                    if (st >= kPSA) previous_launch();
                     if (st >= kPSA && !mbar_wait<kWaitSlackNs>(bar_a_free + 8 * sa, (uint32_t)((st / kPSA - 1) & 1), status, 65)) { failed = true; break; }
                     if (rank == 0) mbar_expect_tx(bar_a + 8 * sa, (uint32_t)(2 * p.r_pad * 128));
                     tma_load_2d_pair(a0 + (uint32_t)(sa * C::ATILE), &p.tm_a, (2 * k + rank) * 64, 0, a_pair0 + 8 * sa);
@@ -201,9 +208,11 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
             const int ranks16 = p.r_pad / 16;
             for (int piece = 0; !failed && sched.next(w); ++piece) {
+                if (piece > 0 || !p.b_early) previous_launch();
                 if (!mbar_wait_warp(bar_b, (uint32_t)(piece & 1), status, 69)) { failed = true; break; }
                 for (int k = w.k0; k < w.k1; ++k, ++st) {
                     const int sa = st % kPSA;
+                    if (st >= kPW / 2) previous_launch();                  // the workers stop there, and with them the steps behind
                     if (!mbar_wait_warp2<kWaitSpin>(bar_a + 8 * sa, (uint32_t)((st / kPSA) & 1), bar_s_free, (uint32_t)((st + 1) & 1), status, 67)) { failed = true; break; }
                     tc_fence_after_sync();
                     const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ATILE >> 4));
@@ -224,6 +233,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             const uint32_t desc_hi = (uint32_t)(umma_desc_sw128(0, 1024, 16) >> 32);
             const uint32_t x_lo0 = (uint32_t)umma_desc_sw128(0, 1024, 16) | ((x0 & 0x3FFFFu) >> 4);
             const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
+            previous_launch();
             for (int piece = 0; !failed && sched.next(w); ++piece) {
                 if (piece > 0 && !mbar_wait_warp(bar_acc_free, (uint32_t)((piece - 1) & 1), status, 70)) { failed = true; break; }
                 for (int k = w.k0; k < w.k1 && !failed; ++k, ++st) {
@@ -251,6 +261,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
         while (!failed && sched.next(w)) {
             for (int k = w.k0; k < w.k1; ++k, ++st) {
                 const int sq = st % kPSQ, ks = 2 * st + g, ws = ks % kPW;
+                if (!p.b_early || 2 * st >= kPW) previous_launch();
                 if (!mbar_wait_warp2(bar_s, (uint32_t)(st & 1), bar_q + 8 * sq, (uint32_t)((st / kPSQ) & 1), status, 73)) { failed = true; break; }
                 tc_fence_after_sync();
                 uint32_t s[32];
@@ -276,6 +287,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             }
             if (failed) break;
             // ---------------------------------------------------------------- epilogue: lane = row, columns = tokens
+            previous_launch();
             if (!mbar_wait_warp(bar_acc, (uint32_t)(piece & 1), status, 76)) { failed = true; break; }
             tc_fence_after_sync();
             const int rt = w.tile / p.tok_tiles, tt = w.tile - rt * p.tok_tiles;
