@@ -36,15 +36,17 @@
  *   - the caller owns every buffer it passes for the whole asynchronous lifetime of
  *     the call; the library neither retains nor frees them.  x/y aliasing is undefined.
  *   - the tensor-core kernels are launched with programmatic dependent launch: they may begin while
- *     the previous kernel on `stream` is still draining, and until that kernel has finished they
- *     read only the weights (Qpacked, B, A); x is read, and y written, after it.  So the weights must
- *     not be produced by work that is still in flight on `stream` when a forward call is made
- *     (synchronise the stream once after loading or updating weights); activations may be.
+ *     the previous kernel on `stream` is still draining.  Until that kernel has finished, layers on the tensor
+ *     cores' grid (next item) read only their weights (Qpacked, B, A); x is read, and y written, after it.  So the
+ *     weights of these must not be produced by work that is still in flight on `stream` when a forward call is
+ *     made (synchronise the stream once after loading or updating weights); activations may be.  All other calls
+ *     (rows off that grid, ranks above 64) read and write everything in the stream's order.
  *   - precision and range: sums are fp32.  Layers on the tensor cores' grid (n a multiple of 64, or of 128
- *     for 3-bit codes, and r <= 64) hold their operands in fp16, each rounded once:
+ *     for 3-bit codes, and r <= 64; with M * (r rounded up to 16) <= 64 and M <= 2 also n a multiple of 32 for
+ *     4-bit codes) hold their operands in fp16, each rounded once:
  *         the dequantised weight L[Q_ij] * (BA)_ij and x itself; or,
- *         with M <= 2, M * (r rounded up to 16) <= 64 and m * n > 2^19 (for such calls n need only be a multiple
- *         of 32 with 4-bit codes), the bare level L[Q_ij] and the product A_kj * x_tj.
+ *         with M <= 2, M * (r rounded up to 16) <= 64 and m * n > 2^19, the bare level L[Q_ij] and the product
+ *         A_kj * x_tj.
  *     These values must lie within fp16's range: magnitudes above 65504 overflow to infinity, magnitudes
  *     below 6.1e-5 are rounded to multiples of 6e-8 (which matters only where such terms dominate a sum).
  *     Layer weights and activations of the usual scales (|x| up to a few thousand, factors around 1e-2 to 1)

@@ -67,6 +67,7 @@ struct ExpandParams {
     int rows, n, np, r, M;
     int strips, splits;    // strips of 64 columns; CTAs that share a row tile's strips
     int w_blocks;          // blocks below this index expand, the others convert activations
+    int late;              // nothing is read before the previous launch has ended (stream_ordered)
 };
 
 // The 8 codes at column c of a row (8 * BITS bits, c a multiple of 8), low code first.  ALIGNED: the row starts on a
@@ -140,6 +141,18 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
     const int g = lane >> 2, t = lane & 3;
     const int i0 = row0 + g, i1 = row0 + g + 8;
 
+    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
+    const uint4 v = level_pair<BITS>(p.levels, tid);
+    if (tid < C::ENTRIES) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
+    }
+    const uint32_t lut_lane = lut + 8u * (uint32_t)(lane & 15);
+    if (p.late) {
+        griddep_launch_dependents();
+        griddep_wait();
+    }
+
     // A strip: RK * 16 ranks x 64 columns by 4-byte asynchronous copies (rows of A are 4-byte aligned, n being even),
     // zeros past rank r and past column n.  A thread moves column pairs; the pair (4 tt + u) of each group of 32
     // columns goes to position (4 u + tt), which hands a lane of the MMA eight consecutive columns over four tiles.
@@ -159,14 +172,6 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
         if (s_a + k < s_b) stage_a(s_a + k, k);
         else asm volatile("cp.async.commit_group;" ::: "memory");
     }
-
-    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
-    const uint4 v = level_pair<BITS>(p.levels, tid);
-    if (tid < C::ENTRIES) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
-    }
-    const uint32_t lut_lane = lut + 8u * (uint32_t)(lane & 15);
 
     // B fragments of the warp's 16 rows, kept for every strip
     uint32_t bf[RK][4];
@@ -589,6 +594,7 @@ template <int BN> int run_dense(const Problem &p, State &st, cudaStream_t stream
     e.w16 = reinterpret_cast<uint16_t *>(st.workspace + x_bytes + part_bytes);
     for (int c = 0; c < 16; ++c) e.levels[c] = p.levels[c];
     e.n = p.n; e.np = np; e.r = p.r; e.M = p.M;
+    e.late = stream_ordered(p);
     e.strips = np / kExCols;
     const size_t row_bytes = (size_t)p.n * p.bits / 8;
     e.q_end = p.q + (size_t)p.m * row_bytes;

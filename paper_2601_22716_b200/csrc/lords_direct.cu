@@ -12,7 +12,7 @@
 // them, so S of every 16 ranks and the first parts' products of every 16 columns start from zero and are added on the
 // CUDA cores; the lower parts' products, 2^-8 of the sum, keep to the tensor cores.  Error of the fp32 sums
 // against 64 bits, norms, normal activations, 256 x 256 to 1024 x 14336, ranks 4 to 128: 6e-8 to 1.7e-7 (CUDA cores 8e-8 to 1.6e-7; the
-// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 13.7 us a call (fp16 form 10.7, CUDA cores 67.6).
+// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 14.9 us a call (fp16 form 10.7, CUDA cores 67.6).
 //
 // A cluster shares one tile of 128 rows and splits its columns; every CTA sends its partial sums to the CTA that owns
 // the row (asynchronous stores counted on that CTA's barrier), which adds them in rank order: deterministic,
@@ -21,7 +21,8 @@
 // Bound: warp instructions -- four per code pair for the table and the product (EXACT: some twenty), the MMAs (2 RK + M / 8, or
 // 3 M / 8, per 16 x 16 weights at the warp-level rate) and the loads around them; codes, factors and activations come by
 // asynchronous copies several strips ahead.  CTAs are small (eight warps, under 110 KB), so that two or more share an SM
-// and the next call's CTAs load their weights while this call computes (programmatic dependent launch).
+// and the next call's CTAs set up (and, where that call is not `late`, load their weights) while this call computes (programmatic
+// dependent launch).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -67,6 +68,7 @@ struct DirectParams {
     float levels[16];
     int M, m, n, r;
     int strips;            // 64-column strips per row
+    int late;              // nothing is read before the previous launch has ended (stream_ordered)
     int per_rank;          // rows of the tile that one CTA of the cluster adds up: ceil(128 / cluster)
     uint32_t per_rank_inv; // ceil(65536 / per_rank): row / per_rank by a multiplication
     void *y;
@@ -224,7 +226,27 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
         }
     };
 
-    // ---- weights first: they do not depend on the previous launch.  Copies are committed in the order
+    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
+    auto fill_table = [&] {
+        uint4 v = level_pair<BITS>(p.levels, tid);
+        if constexpr (!EXACT) {
+            const __half2 h = __floats2half2_rn(__uint_as_float(v.x), __uint_as_float(v.y));
+            v.x = v.y = v.z = v.w = *reinterpret_cast<const uint32_t *>(&h);
+        }
+        if (tid < C::ENTRIES) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
+        }
+    };
+    if constexpr (EXACT) {
+        fill_table();
+        if (p.late) {
+            griddep_launch_dependents();
+            griddep_wait();
+        }
+    }
+
+    // ---- weights first: where the call is not `late` they do not depend on the previous launch.  Copies are committed in the order
     // q0, a0, q1, a1, q2, then per strip a + 2 and q + 3 (or, with two stages of A, q + 3 and a + 2 at its end).
     constexpr int kPending = C::SA == 3 ? 3 : 2;     // youngest copies that strip `it` does not need
     if constexpr (ALIGNED) stage_q(0);
@@ -236,16 +258,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     stage_a(1); commit();
     if constexpr (ALIGNED) stage_q(2);
     commit();
-    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
-    uint4 v = level_pair<BITS>(p.levels, tid);
-    if constexpr (!EXACT) {
-        const __half2 h = __floats2half2_rn(__uint_as_float(v.x), __uint_as_float(v.y));
-        v.x = v.y = v.z = v.w = *reinterpret_cast<const uint32_t *>(&h);
-    }
-    if (tid < C::ENTRIES) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
-    }
+    if constexpr (!EXACT) fill_table();
     // B fragments of the warp's rows
     const int i0 = row0 + warp * 16 + g, i1 = i0 + 8;
     uint32_t bf[RK][4];
@@ -498,6 +511,7 @@ int launch_direct(const Problem &p, State &st, cudaStream_t stream)
     for (int c = 0; c < 16; ++c) k.levels[c] = p.levels[c];
     k.M = p.M; k.m = p.m; k.n = p.n; k.r = p.r;
     k.strips = (p.n + kCols - 1) / kCols;
+    k.late = stream_ordered(p);
     k.y = p.y; k.y_f32 = p.y_f32;
     k.status = st.status_word;
     const int rc = p.bits == 4 ? launch_direct<4>(k, p, st, stream) : p.bits == 3 ? launch_direct<3>(k, p, st, stream) : launch_direct<2>(k, p, st, stream);

@@ -30,6 +30,9 @@ inline bool decode_takes(const Problem &p)      // reassociated form: M * ceil16
 }
 inline bool decode16_takes(const Problem &p) { return p.M <= 16 && p.r <= 64 && p.n % (p.bits == 3 ? 128 : 64) == 0; }
 inline bool umma_takes(const Problem &p) { return p.r <= 64 && p.n % (p.bits == 3 ? 128 : 64) == 0; }
+// Calls that none of them takes read nothing, weights included, before the work ahead of them on the stream has ended: the interface
+// asks no more of their callers than the stream's order.
+inline bool stream_ordered(const Problem &p) { return !decode_takes(p) && !decode16_takes(p) && !umma_takes(p); }
 
 // Library-owned device memory and switches (one instance per process).
 struct State {

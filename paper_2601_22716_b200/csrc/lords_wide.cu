@@ -149,6 +149,11 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
             mbar_expect_tx(bar_red, (uint32_t)(csize * own_n * ((p.M + 1) / 2) * 8));
         }
         __syncwarp();
+        // these ranks are stream-ordered calls: no weight is read before the previous launch has ended
+        asm volatile("bar.arrive 1, %0;" ::"n"(kThreads) : "memory");          // the barriers exist
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // waited for before the first remote store
+        griddep_launch_dependents();
+        griddep_wait();
         auto factors = [&](int it) {
             const uint32_t bar = bar_a + 8 * (it % D), dst = a_s + (uint32_t)((it % D) * 2 * kAAtom);
             mbar_expect_tx(bar, (uint32_t)(2 * p.r_pad * 128));
@@ -176,14 +181,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
             for (int it = 0; it < D && it < total; ++it) {
                 factors(it);
                 codes(it);
+                activations(it);
             }
-        }
-        asm volatile("bar.arrive 1, %0;" ::"n"(kThreads) : "memory");          // the barriers exist
-        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // waited for before the first remote store
-        griddep_launch_dependents();
-        griddep_wait();                                                        // x may be the previous launch's output
-        if (lane == 0) {
-            for (int it = 0; it < D && it < total; ++it) activations(it);
             for (int it = D; it < total; ++it) {
                 if (!mbar_wait(bar_a_free + 8 * (it % D), (uint32_t)((it / D - 1) & 1), status, 76)) { failed = true; break; }
                 factors(it);
@@ -258,6 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         }
         if (!b_by_tma) {
             // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m
+            griddep_wait();
             const int rr = tid >> 2, i = row0 + rr;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
