@@ -420,21 +420,10 @@ __global__ void __launch_bounds__(GCfg<BN>::THREADS, 1) lords_dense_kernel(const
             int others = 0;
             if (w.k0 == 0 && w.k1 < p.ksteps) {
                 const long long left = (long long)(p.tiles - p.whole) * p.ksteps, tile_end = (long long)(w.tile - p.whole + 1) * p.ksteps;
-                for (int o = pair + 1; o < p.pairs && o * left / p.pairs < tile_end; ++o)
-                    if ((o + 1) * left / p.pairs > o * left / p.pairs) {
-                        if (!__all_sync(0xffffffffu, [&] {
-                                WaitLimit limit = wait_limit_start();
-                                const int *flag = p.flags + 2 * o + rank;
-                                for (unsigned tries = 0;; ++tries) {
-                                    int v;
-                                    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-                                    if (v >= C::EPI) return true;
-                                    __nanosleep(kWaitSleepNs);
-                                    if ((tries & 63u) == 63u && wait_limit_expired(limit, status, (uint32_t)o, 0, 56)) return false;
-                                }
-                            }())) { failed = true; break; }
-                    }
-                for (int o = pair + 1; o < p.pairs && o * left / p.pairs < tile_end; ++o) others = o - pair;
+                for (int o = pair + 1; o < p.pairs && o * left / p.pairs < tile_end; ++o) {
+                    others = o - pair;
+                    if (!__all_sync(0xffffffffu, piece_ready(p.flags + 2 * o + rank, C::EPI, status, (uint32_t)o, 56))) { failed = true; break; }
+                }
             }
             if (failed) break;
 #pragma unroll

@@ -65,6 +65,8 @@ struct Piece {
     int tile, k0, k1;
 };
 
+// (divide_tiles cuts tiles only where every pair gets steps of them: cutting has to save more than `meet` steps, so a tile has more steps than
+// that, and at least a third as many tiles as pairs are cut.)
 // The pieces of pair `pair`, in order: its tiles of the whole waves, then its share of the k-steps of the tiles left over.  The
 // share may begin inside a tile (that piece goes to scratch) and end inside one (the pair that begins a
 // tile finishes it: it adds the other pieces, which their pairs do first).
@@ -130,6 +132,19 @@ inline Division divide_tiles(int tiles, int steps, int pairs_max, int least_step
     if (left > 0 && d.whole > 0 && 3 * left < d.pairs) d.whole -= d.pairs;
     d.per_pair = cut;
     return d;
+}
+
+// A piece in scratch is complete: all `warps` warps of its CTA have counted on its flag.  Bounded; false if that does not come about.
+__device__ __forceinline__ bool piece_ready(const int *flag, int warps, const int *status, uint32_t who, uint32_t tag)
+{
+    WaitLimit limit = wait_limit_start();
+    for (unsigned tries = 0;; ++tries) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+        if (v >= warps) return true;
+        __nanosleep(kWaitSleepNs);
+        if ((tries & 63u) == 63u && wait_limit_expired(limit, status, who, 0, tag)) return false;
+    }
 }
 
 // A warp's last act on a piece.  A piece that went to scratch: one count on its flag, which is complete at `warps`.  A tile's owner:

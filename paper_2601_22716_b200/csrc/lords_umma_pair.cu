@@ -299,19 +299,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             if (w.k0 == 0 && w.k1 < p.steps) {
                 for (int o = pair + 1; o < p.pairs && o * left / p.pairs < tile_end; ++o) {
                     others = o - pair;
-                    if ((o + 1) * left / p.pairs > o * left / p.pairs) {
-                        if (!__all_sync(0xffffffffu, [&] {
-                                WaitLimit limit = wait_limit_start();
-                                const int *flag = p.flags + 2 * o + rank;
-                                for (unsigned tries = 0;; ++tries) {
-                                    int v;
-                                    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
-                                    if (v >= kPWorkers) return true;
-                                    __nanosleep(kWaitSleepNs);
-                                    if ((tries & 63u) == 63u && wait_limit_expired(limit, status, (uint32_t)o, 0, 77)) return false;
-                                }
-                            }())) { failed = true; break; }
-                    }
+                    if (!__all_sync(0xffffffffu, piece_ready(p.flags + 2 * o + rank, kPWorkers, status, (uint32_t)o, 77))) { failed = true; break; }
                 }
             }
             if (failed) break;
@@ -340,7 +328,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         const int o = o0 + j;
-                        const bool has = o <= pair + others && (o + 1) * left / p.pairs != o * left / p.pairs;
+                        const bool has = o <= pair + others;
                         const float4 *part = reinterpret_cast<const float4 *>(p.partial + ((size_t)(2 * (has ? o : pair) + rank) * p.bn + c0) * 128) + row;
 #pragma unroll
                         for (int c = 0; c < 4; ++c) pv[j][c] = has ? __ldcg(part + c * 128) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
