@@ -8,13 +8,14 @@ missing or a call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import sysconfig
 from pathlib import Path
 
 import numpy as np
 
 _PKG = Path(__file__).resolve().parent
 _LIBPATH = _PKG / "liblords.so"
-_NATIVEPATH = _PKG / "_native.so"
+_NATIVEPATH = _PKG / f"_native.{sysconfig.get_config_var('SOABI')}.so"      # this interpreter's
 _lib = None
 
 

@@ -12,7 +12,8 @@ PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 LIB = PKG / "liblords.so"
-NATIVE = PKG / "_native.so"      # the CPython module over it
+# the CPython module over it; the tag (cpython-312-x86_64-linux-gnu) keeps an interpreter from loading another's
+NATIVE = PKG / f"_native.{sysconfig.get_config_var('SOABI')}.so"
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -74,7 +75,7 @@ def _run(cmd, verbose: bool = False):
 
 
 def build_module() -> Path:
-    tmp = NATIVE.with_name(f"_native.tmp{os.getpid()}.so")
+    tmp = NATIVE.with_name(f"_native_tmp{os.getpid()}.so")
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-I{INCLUDE}", f"-I{sysconfig.get_paths()['include']}",
            str(CSRC / "lords_module.cc"), f"-L{PKG}", "-l:liblords.so", "-Wl,-rpath,$ORIGIN", "-o", str(tmp)]
     _run(cmd)

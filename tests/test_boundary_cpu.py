@@ -149,3 +149,12 @@ def test_concat_layers_is_the_concatenation_of_the_layers_outputs():
         packing.concat_layers([lays[0].codes, lays[1].codes[:, :64]], [lays[0].B, lays[1].B], [lays[0].A, lays[1].A[:, :64]])
     with pytest.raises(ValueError):
         packing.concat_layers([lays[0].codes], [lays[1].B], [lays[0].A])
+
+
+def test_native_module_is_this_interpreters():
+    """The module over the library carries the interpreter's tag, so that one built under another Python is neither loaded nor kept."""
+    import sysconfig
+    from paper_2601_22716_b200 import build
+    tag = sysconfig.get_config_var("EXT_SUFFIX")
+    assert lords._native().__file__.endswith("_native" + tag) and build.NATIVE.name == "_native" + tag
+    assert build.NATIVE == lords._NATIVEPATH
