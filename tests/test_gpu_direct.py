@@ -31,6 +31,12 @@ SHAPES = [
     (3, 130, 352, 48, 40, False),
     (4, 1000, 2730, 10, 37, False),
     (2, 140, 260, 70, 128, True),
+    # the form with fp16 operands (n a multiple of 64 or 128, ranks up to 64, three tokens and more; the others are computed in fp32)
+    (4, 130, 128, 33, 9, True),
+    (4, 129, 64, 5, 17, False),
+    (3, 127, 128, 16, 3, True),
+    (3, 300, 1024, 64, 16, False),
+    (2, 300, 192, 48, 8, True),
 ]
 
 

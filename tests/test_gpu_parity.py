@@ -326,14 +326,17 @@ def test_linearity_on_gpu(lords):
 def test_operand_range_edges(lords, M, xscale, what):
     """The tensor-core paths keep x (or A*x) and the dequantised weight in fp16.  Inside the documented
     range -- |x| up to a few thousand with factors of the order 1e-2, and activations as small as 1e-2 --
-    the tolerances still hold on every path (M = 1: reassociated form, 8: 128-column form A, 40: form A)."""
+    the tolerances still hold on every path (M = 1: reassociated form, 8: 128-column form A, 40: form A;
+    "auto" takes the direct kernel for a layer of this size, under their names, so they are forced too)."""
     import torch
     lay = gen.make_layer(384, 1024, 32, M, bits=4, seed=91 + M, scale_gain=0.005, scale_shift=0.01)
     x = gen.bf16_to_f32(lay.x) * np.float32(xscale)
     lay.x = gen.bf16_bits(torch.from_numpy(x))
-    dl, y32, ybf = _run(lords, lay, "auto")
-    assert lords.lords_last_path() in ("decode", "decode16", "umma")
-    check_against_oracle(y32, ybf, _oracle(lay, dl.packed_host))
+    named = {1: "decode", 8: "decode16", 40: "umma"}[M]
+    for path in ("auto", named):
+        dl, y32, ybf = _run(lords, lay, path)
+        assert lords.lords_last_path() == named
+        check_against_oracle(y32, ybf, _oracle(lay, dl.packed_host), label=f"operand range x {xscale} M={M} {path}")
 
 
 def _sampled_rows(m, count, seed):
@@ -455,7 +458,8 @@ def test_many_back_to_back_launches_leave_no_status(lords, m, n, r, bits, M, pat
         assert torch.equal(y, f)
 
 
-@pytest.mark.parametrize("M,path", [(1, "auto"), (4, "auto"), (40, "auto"), (3, "simt"), (300, "auto")])
+@pytest.mark.parametrize("M,path", [(1, "auto"), (4, "auto"), (40, "auto"), (3, "simt"), (300, "auto"),
+                                    (1, "decode"), (4, "decode16"), (40, "umma"), (4, "direct"), (40, "dense")])
 def test_host_buffer_entry_point_matches_device_entry(lords, M, path):
     """x from and y into pinned host memory (small buffers: y is stored by the kernels straight into the
     mapped host buffer; 300 tokens: staged copies), on every kind of kernel: bit-identical to the device entry."""
