@@ -51,7 +51,8 @@
  *     below 6.1e-5 are rounded to multiples of 6e-8 (which matters only where such terms dominate a sum).
  *     Layer weights and activations of the usual scales (|x| up to a few thousand, factors around 1e-2 to 1)
  *     are far inside.  All other calls (rows off that grid, ranks above 64, the smaller layers with M <= 2) and
- *     the CUDA-core path ("path" = "simt") are computed in fp32 throughout and have no such limit.
+ *     the CUDA-core path ("path" = "simt") are computed in fp32 throughout and have no such limit (off the
+ *     CUDA cores, weights below 1e-33 lose low bits).
  *   - forward calls validate on the host, enqueue work on `stream` and return
  *     without synchronising.  They use library-owned scratch memory, so two forward
  *     calls may only overlap on the GPU if they are ordered on the same stream.

@@ -512,36 +512,41 @@ __global__ void lords_quantize_simt_kernel(const uint16_t *__restrict__ W, const
 __global__ void __launch_bounds__(256) lords_quantize_norms_kernel(const uint16_t *__restrict__ B, const uint16_t *__restrict__ A, int m, int n, int r,
                                                                    int steps, float scale, float *__restrict__ a_norm, float *__restrict__ b_norm)
 {
-    __shared__ float part[256];
+    __shared__ float part[256];                     // (squares in 64 bits: those of factors below 1e-19 or above 1e19 leave the range of a float)
     const int tid = threadIdx.x, lane = tid & 31;
-    float sum = 0.0f;
+    double sum = 0.0;
     if ((int)blockIdx.x < steps) {
         const int j = (int)blockIdx.x * kColsQ + (tid & 63);
         if (j < n)
             for (int k = tid >> 6; k < r; k += 4) {
-                const float v = __uint_as_float((uint32_t)A[(size_t)k * n + j] << 16);
-                sum = fmaf(v, v, sum);
+                const double v = __uint_as_float((uint32_t)A[(size_t)k * n + j] << 16);
+                sum = fma(v, v, sum);
             }
-        part[tid] = sum;
+        part[tid] = (float)sqrt(sum);
         __syncthreads();
         if (tid < 32) {
             float most = 0.0f;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) most = fmaxf(most, part[tid + 32 * h] + part[tid + 32 * h + 64] + part[tid + 32 * h + 128] + part[tid + 32 * h + 192]);
+            for (int h = 0; h < 2; ++h) {
+                double four = 0.0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) four = fma((double)part[tid + 32 * h + 64 * q], (double)part[tid + 32 * h + 64 * q], four);
+                most = fmaxf(most, (float)sqrt(four));
+            }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) most = fmaxf(most, __shfl_xor_sync(0xffffffffu, most, o));
-            if (tid == 0) a_norm[blockIdx.x] = scale * sqrtf(most);
+            if (tid == 0) a_norm[blockIdx.x] = scale * most;
         }
     } else {
         const int i = ((int)blockIdx.x - steps) * 8 + (tid >> 5);
         if (i >= m) return;
         for (int k = lane; k < r; k += 32) {
-            const float v = __uint_as_float((uint32_t)B[(size_t)i * r + k] << 16);
-            sum = fmaf(v, v, sum);
+            const double v = __uint_as_float((uint32_t)B[(size_t)i * r + k] << 16);
+            sum = fma(v, v, sum);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0) b_norm[i] = sqrtf(sum);
+        if (lane == 0) b_norm[i] = (float)sqrt(sum);
     }
 }
 

@@ -54,9 +54,9 @@ def _scaled(bits, words, factor):
 
 
 @pytest.mark.parametrize("bits,m,n,r,M", SHAPES)
-@pytest.mark.parametrize("xs,bs", [(1.0, 1.0), (2.0**30, 2.0**-20), (2.0**-30, 2.0**-30), (2.0**-20, 2.0**40)])
+@pytest.mark.parametrize("xs,bs", [(1.0, 1.0), (2.0**30, 2.0**-20), (2.0**-30, 2.0**-30), (2.0**-20, 2.0**40), (2.0**-129, 2.0**60)])
 def test_precision_and_range(lords, bits, m, n, r, M, xs, bs):
-    """x to 2^30 and factors from 2^-30 to 2^40: far outside fp16, with the precision of fp32."""
+    """x to 2^30 and factors from 2^-30 to 2^60, subnormal x: far outside fp16, with the precision of fp32."""
     lay = gen.make_layer(m, n, r, M, bits=bits, seed=m + n + r + M, mixed_sign=True)
     lay.x, lay.B = _scaled(bits, lay.x, xs), _scaled(bits, lay.B, bs)
     dl = DeviceLayer(lay)
