@@ -141,12 +141,7 @@ __global__ void __launch_bounds__(kExThreads, RK <= 4 ? 2 : 1) lords_expand_kern
     const int g = lane >> 2, t = lane & 3;
     const int i0 = row0 + g, i1 = row0 + g + 8;
 
-    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
-    const uint4 v = level_pair<BITS>(p.levels, tid);
-    if (tid < C::ENTRIES) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
-    }
+    fill_pair_table<BITS, false>(lut, p.levels, tid);
     const uint32_t lut_lane = lut + 8u * (uint32_t)(lane & 15);
     if (p.late) {
         griddep_launch_dependents();

@@ -76,12 +76,6 @@ struct DirectParams {
     int *status;
 };
 
-__device__ __forceinline__ void st_async_cluster_2f32(uint32_t addr, float a, float b, uint32_t bar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
-                 ::"r"(addr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(bar) : "memory");
-}
-
 template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT>
 __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direct_kernel(const DirectParams p)
 {
@@ -226,20 +220,8 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
         }
     };
 
-    // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
-    auto fill_table = [&] {
-        uint4 v = level_pair<BITS>(p.levels, tid);
-        if constexpr (!EXACT) {
-            const __half2 h = __floats2half2_rn(__uint_as_float(v.x), __uint_as_float(v.y));
-            v.x = v.y = v.z = v.w = *reinterpret_cast<const uint32_t *>(&h);
-        }
-        if (tid < C::ENTRIES) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
-        }
-    };
     if constexpr (EXACT) {
-        fill_table();
+        fill_pair_table<BITS, false>(lut, p.levels, tid);
         if (p.late) {
             griddep_launch_dependents();
             griddep_wait();
@@ -258,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     stage_a(1); commit();
     if constexpr (ALIGNED) stage_q(2);
     commit();
-    if constexpr (!EXACT) fill_table();
+    if constexpr (!EXACT) fill_pair_table<BITS, true>(lut, p.levels, tid);
     // B fragments of the warp's rows
     const int i0 = row0 + warp * 16 + g, i1 = i0 + 8;
     uint32_t bf[RK][4];

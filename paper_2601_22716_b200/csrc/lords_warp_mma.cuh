@@ -62,15 +62,23 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// A level pair's two fp32 words, twice, for the table of pairs; called by whole warps.  (One level a lane and two shuffles: indexed by
-// the pair, the parameters were read again for every copy that is stored, sixteen addresses to a warp: 128 x 128, one token, 3.9 us
-// a call against 2.4.)
-template <int BITS> __device__ __forceinline__ uint4 level_pair(const float (&levels)[16], int pair)
+// The table of level pairs, 128 bytes an entry, one entry a thread (the first 4^BITS of the block; called by whole warps): sixteen copies of
+// two fp32 values, one for each lane of a half warp, or (HALF) 32 of two fp16 values.  Stored as eight words of 16 bytes that rotate over
+// the banks.  (One level a lane and two shuffles: indexed by the pair, the parameters were read again for every copy that is stored,
+// sixteen addresses to a warp: 128 x 128, one token, 3.9 us a call against 2.4.)
+template <int BITS, bool HALF> __device__ __forceinline__ void fill_pair_table(uint32_t table, const float (&levels)[16], int tid)
 {
-    const float mine = levels[threadIdx.x & 15];
-    const uint32_t l0 = __float_as_uint(__shfl_sync(0xffffffffu, mine, pair & ((1 << BITS) - 1)));
-    const uint32_t l1 = __float_as_uint(__shfl_sync(0xffffffffu, mine, (pair >> BITS) & ((1 << BITS) - 1)));
-    return make_uint4(l0, l1, l0, l1);
+    const float mine = levels[tid & 15];
+    const float l0 = __shfl_sync(0xffffffffu, mine, tid & ((1 << BITS) - 1)), l1 = __shfl_sync(0xffffffffu, mine, (tid >> BITS) & ((1 << BITS) - 1));
+    uint4 v = make_uint4(__float_as_uint(l0), __float_as_uint(l1), __float_as_uint(l0), __float_as_uint(l1));
+    if constexpr (HALF) {
+        const __half2 h = __floats2half2_rn(l0, l1);
+        v.x = v.y = v.z = v.w = *reinterpret_cast<const uint32_t *>(&h);
+    }
+    if (tid < 1 << 2 * BITS) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sts_v4(table + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
+    }
 }
 
 // B[i][k], B[i][k + 1] (k even) as one word, zeros outside the matrix

@@ -88,12 +88,6 @@ struct alignas(64) WideParams {
     int *status;
 };
 
-__device__ __forceinline__ void st_async_cluster_2f32(uint32_t addr, float a, float b, uint32_t bar)
-{
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
-                 ::"r"(addr), "r"(__float_as_uint(a)), "r"(__float_as_uint(b)), "r"(bar) : "memory");
-}
-
 // Byte offset of 32-column group c (0..3) of row `row` in a code tile as the tensor-map copy lays it out: 4-bit rows are 64
 // bytes with 16-byte chunks swizzled over four, 2-bit rows 32 bytes (a group is 8 bytes) with chunks swapped
 // every four rows, 3-bit rows 48 bytes as they are; eight consecutive rows fall into different banks.
@@ -249,12 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         // ------------------------------------------------------------------ consumers
         // row group rw (its TMEM quadrant), column quarter ch
         const int g = lane >> 2, t = lane & 3, rw = warp & 3, ch = warp >> 2;
-        // level pairs: one entry per thread, its copies as eight 16-byte stores that rotate over the banks
-        const uint4 v = level_pair<BITS>(p.levels, tid);
-        if (tid < C::ENTRIES) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) sts_v4(lut + (uint32_t)(tid * 128 + ((tid + k) & 7) * 16), v);
-        }
+        fill_pair_table<BITS, false>(lut, p.levels, tid);
         if (!b_by_tma) {
             // rows of B that are not 16-byte multiples: element by element, zeros past rank r and past row m
             griddep_wait();
