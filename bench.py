@@ -73,18 +73,17 @@ def measured_peaks():
     return {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0, "source": "fallback"}
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch from the ncu captures summarised
-# under profiles/ (None until a capture of that case exists).
+# dram__bytes_read.sum + dram__bytes_write.sum per launch, from profiles/kernels.md
 NCU_TRAFFIC_BYTES = {
-    "decode_q_m1": 8976640,         # profiles/decode_kernel_decode_q_m1.md
-    "decode_q_m8": 9029632,         # profiles/decode16_kernel_decode_q_m8_down_m16.md
-    "mlp3_gate_m1": 23850496,       # profiles/decode_kernel_mlp3_gate_m1_down_m1.md
-    "mlp3_down_m1": 23938560,       # same
-    "mlp3_down_m16": 24299520,      # profiles/decode16_kernel_decode_q_m8_down_m16.md
-    "prefill_m2048": 145443072,     # profiles/umma_kernel_prefill_m2048.md (the scale-MMA kernel; the pre-pass moves 73.7 MB more)
-    "quantize_q_nf4": 34120448,     # profiles/quantize_kernel_q_nf4_gate_nf3.md (8.4 MB of codes were still in L2 at the end)
-    "quantize_gate_nf3": 130577408,
-    "backward_q_m512": 19691008,    # profiles/backward_tc_kernel_backward_q_m512.md (the factor-gradient kernel)
+    "decode_q_m1": 8995584,
+    "decode_q_m8": 9061120,
+    "mlp3_gate_m1": 23867136,
+    "mlp3_down_m1": 23887360,
+    "mlp3_down_m16": 25217536,
+    "prefill_m2048": 162462720,     # the pair kernel; the pre-pass moves 75.0 MB more
+    "quantize_q_nf4": 34163200,     # 8.4 MB of codes were still in L2 at the end
+    "quantize_gate_nf3": 130008576,
+    "backward_q_m512": 17395456,    # the factor-gradient kernel; the sum behind it moves 19.6 MB more
 }
 
 
@@ -537,7 +536,7 @@ FP32_ALU_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 def time_backward(name, m, n, r, bits, M, device, min_seconds=0.3):
     """The backward with the codes fixed (Sec. 3.4) on one layer shape: dx = g W^ on the forward
     kernels (transposed codes, made once outside the timed region; the per-call transposition of the
-    factors inside it), then dB and dA on the CUDA cores.  Reported separately."""
+    factors inside it), then dB and dA.  Reported separately."""
     import numpy as np
     import torch
     from paper_2601_22716_b200 import binding as lords
@@ -585,21 +584,21 @@ def time_backward(name, m, n, r, bits, M, device, min_seconds=0.3):
     peaks = measured_peaks()
     flops = 2.0 * M * m * n
     tf_dx = flops / (us_dx * 1e-6) / 1e12
-    # CUDA-core work of the factor gradients: the two folds and the level multiply; with the schedules that
-    # form g^T x on the CUDA cores as well, that product too (once: one CTA per tile of W)
-    alu_flops = 4.0 * m * n * r + m * n + (0.0 if path_f == "backward_tensor" else flops)
-    tf_f = alu_flops / (us_f * 1e-6) / 1e12
+    # the factor gradients: g^T x and its two folds with A and B, all on the tensor cores or all on the CUDA cores
+    on_tensor = path_f == "backward_tensor"
+    tf_f = (flops + 4.0 * m * n * r) / (us_f * 1e-6) / 1e12
+    peak_f = peaks["bf16_tflops"] if on_tensor else FP32_ALU_TFLOPS
     return {"case": name, "path": f"{path_dx}+{path_f}", "us_per_call": us_dx + us_f, "gbs": None, "tflops": None,
             "copies": 1, "rounds": reps_dx, "steps": 1, "status_retries": 0 if status == 0 else 1,
             "input_gradient": {"us": us_dx, "path": path_dx, "tflops": tf_dx,
                                "roofline": {"bound": "tensor", "achieved": tf_dx, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                                             "frac": tf_dx / peaks["bf16_tflops"], "peak_kind": "burst", "traffic": None}},
-            "factor_gradients": {"us": us_f, "path": path_f, "alu_tflops": tf_f,
+            "factor_gradients": {"us": us_f, "path": path_f, "tflops": tf_f,
                                  "tile_product_tflops": flops / (us_f * 1e-6) / 1e12,
-                                 "tile_product_on": "tensor cores" if path_f == "backward_tensor" else "CUDA cores"},
+                                 "tile_product_on": "tensor cores" if on_tensor else "CUDA cores"},
             "qat_gradients": {"us": us_q, "path": path_q},
-            "roofline": {"bound": "alu", "achieved": tf_f, "peak": FP32_ALU_TFLOPS, "unit": "TFLOP/s",
-                         "frac": tf_f / FP32_ALU_TFLOPS, "peak_source": "148 SMs x 128 fp32 lanes x 2 flops x 1.965 GHz",
+            "roofline": {"bound": "tensor" if on_tensor else "alu", "achieved": tf_f, "peak": peak_f, "unit": "TFLOP/s", "frac": tf_f / peak_f,
+                         "peak_source": peaks["source"] if on_tensor else "148 SMs x 128 fp32 lanes x 2 flops x 1.965 GHz",
                          "traffic": NCU_TRAFFIC_BYTES.get(name), "us_per_launch": us_f}}
 
 

@@ -213,10 +213,11 @@ int lords_quantize_codes(const void *W, const void *B, const void *A, const floa
  *   dx: device, bf16 [M][n] (or float [M][n] for _f32).
  * lords_linear_backward_factors: dB (device, float [m][r]) and dA (device, float [r][n]); either may
  *   be NULL.  The product g^T x is formed tile by tile on the tensor cores (bf16 operands as given,
- *   fp32 accumulation) when m and n are multiples of 8, else on the CUDA cores; the level multiply
- *   and the contractions with A and B are fp32 on the CUDA cores.  Every element is summed in a
- *   fixed order (runs are bit-identical).  The tiles' contributions go through the lords_init
- *   workspace; without room there a slower schedule without scratch memory runs.
+ *   fp32 accumulation); dS, the product times the levels in fp32, enters the contractions with A and B, on the
+ *   tensor cores as well, as three bf16 terms that add up to it exactly.  Every element is summed in a
+ *   fixed order (runs are bit-identical).  The tiles' contributions, and padded copies of operands whose rows are no
+ *   multiples of 16 bytes, go through the lords_init workspace; without room there, and for very small
+ *   layers off that grid, slower schedules on the CUDA cores run.
  *   x: device, bf16 [M][n].  Any bits in {2,3,4}, r <= LORDS_R_MAX.
  * All enqueue on `stream` and return without synchronising; all need lords_init.
  */
@@ -323,7 +324,7 @@ int lords_last_cuda_error(void);
 /*
  * Measurement switches.  Keys: "path" = "auto" | "simt" | "decode" (reassociated-form kernel,
  * M <= 2) | "decode16" (scale-MMA form with 128-column k-steps, 3 <= M <= 16) | "umma" (scale-MMA
- * kernel for any M; "prefill" is an alias) | "dense" (weights expanded to fp16 scratch, then a dense product; any shape) | "direct" (weights formed in registers; M <= 128) | "wide" (M <= 16, 64 < r <= 128)
+ * kernel for any M; "prefill" is an alias) | "dense" (weights expanded to scratch, then a dense product; any shape) | "direct" (weights formed in registers; M <= 128) | "wide" (M <= 16, 64 < r <= 128)
  * | "pair" (the scale-MMA kernel on CTA pairs, which "umma" and "auto" use for large calls; reports "umma");
  * "splitk" = "0" (auto) or a positive integer (CTAs sharing one tile's k-range); "bn" = "0" (auto)
  * or the token tile 32, 64, 128, 256 of the scale-MMA kernel for M > 16; "inject_status" = "0" or a

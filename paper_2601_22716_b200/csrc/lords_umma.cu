@@ -693,8 +693,8 @@ int token_tile(const Problem &p, const State &st)
 
 // Whether the kernel on CTA pairs is the faster one: it does a step of 128 columns in about the time that this one needs for a
 // k-step of 64, but divides the work into fewer, larger tiles, and where it cuts them, the meeting of the pieces costs about 15 us,
-// so that it takes the large calls (14336 x 4096, 512 tokens: 68 us against 78; 4096 x 14336, 64 tokens: 38 against 59;
-// 4096 x 4096: 32 against 28 at 512 tokens, 34 against 40 at 1024).  The two estimates below, in microseconds, are least-squares fits to
+// so that it takes the large calls (14336 x 4096, 512 tokens: 60 us against 79; 4096 x 14336, 64 tokens: 32 against 54;
+// 4096 x 4096: 32 against 29 at 512 tokens, 35 against 41 at 1024).  The two estimates below, in microseconds, are least-squares fits to
 // the kernels' times on four layer shapes at 64 to 2048 tokens.  The one for pairs is off by up to 25 %, most where both are short,
 // but on those shapes no call gets a kernel more than 2 % slower than the other.
 bool prefer_pair(const Problem &p, const State &st)

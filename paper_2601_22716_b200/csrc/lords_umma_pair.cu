@@ -3,8 +3,9 @@
 // What bounds the single-CTA kernel at these sizes is the way from L2 into shared memory: 40 KB per 64-column step and SM, about 40
 // bytes a clock, which is also where a plain product with 256 x 256 pair tiles stands (32 KB a step).  Here a pair of CTAs owns 256
 // rows of W^ and up to 256 tokens; each CTA holds half of the tokens' activations, rebuilds its own 128 rows of W^ in TMEM
-// and loads half of the factor tiles: 22 KB per step and SM, most of it activations.  4096 x 14336, 2048 tokens: 282 us with
-// one CTA per tile, 207 now; 14336 x 4096, 512 tokens: 74 -> 64.
+// and loads half of the factor tiles: 22 KB per step and SM, most of it activations.  Calls with their pre-passes, one CTA per tile
+// against pairs, a graph of two or three layers: 4096 x 14336, 2048 tokens 248 us and 206 (239 in longer runs, at the clock that the
+// power cap leaves); 14336 x 4096, 512 tokens 79 and 60.
 //
 // A step is 128 columns (a code stage), two k-steps of 64.  TMEM (512 columns): the accumulator [128 x BN], one buffer of S for a step
 // [128 x 128] fp32 and a ring of four W^ k-steps [128 x 64] fp16.  S and W^ are separate so that neither the scale

@@ -23,7 +23,7 @@
 // sends its partial sums to the CTA that owns the row (asynchronous stores counted on that CTA's barrier), which
 // adds them in a fixed order: deterministic, no atomics, no trip through global memory.
 //
-// Bound: the consumers' instructions (about sixteen a weight: look-up, product, cutting into parts, MMAs) and the latency of their chain, four
+// Bound: the consumers' instructions (13.7 a weight: look-up, product, cutting into parts, MMAs) and the latency of their chain, four
 // warps to a scheduler: 1.6 us a strip of 16384 weights (8192 columns, eight more strips a CTA, take 12.6 us more), of which the strip's
 // arrival (44 KB from L2) and its scale MMAs (8 KB of operands per 16 ranks) are about a third each and overlap.
 //
