@@ -213,7 +213,7 @@ int lords_quantize_codes(const void *W, const void *B, const void *A, const floa
  *   dx: device, bf16 [M][n] (or float [M][n] for _f32).
  * lords_linear_backward_factors: dB (device, float [m][r]) and dA (device, float [r][n]); either may
  *   be NULL.  The product g^T x is formed tile by tile on the tensor cores (bf16 operands as given,
- *   fp32 accumulation); dS, the product times the levels in fp32, enters the contractions with A and B, on the
+ *   fp32 accumulation in sums over a part of the tokens, which are added in fp32); dS, the product times the levels, enters the contractions with A and B, on the
  *   tensor cores as well, as three bf16 terms that add up to it exactly.  Every element is summed in a
  *   fixed order (runs are bit-identical).  The tiles' contributions, and padded copies of operands whose rows are no
  *   multiples of 16 bytes, go through the lords_init workspace; without room there, and for very small

@@ -427,15 +427,20 @@ __global__ void __launch_bounds__(kBwThreads) lords_backward_tile_kernel(const B
 //   G[128 x 128] = sum_t g[t][i] x[t][j]   operands as they lie in memory (MN-major: a shared-memory row is one token), 64 tokens
 //                                          per stage, accumulators in TMEM (two of them: the next tile's product
 //                                          runs while this one is worked on)
-//   dS = G (.) L[Q]                        eight epilogue warps, fp32
+//   dS = G (.) L[Q]                        sixteen epilogue warps, fp32
 //   dB[128 x r] += dS A_tile^T,  dA_tile^T[128 x r] = dS^T B_tile
 // The folds take dS as three bf16 terms, dS = hi + mid + lo exactly (8 bits of the significand each, split by truncation),
-// and the factors are bf16 as given, so every product is exact and the sums are fp32: the precision of the fp32
-// folds on the CUDA cores that this replaces, at the tensor cores' rate.  One shared-memory tile serves both folds,
-// K-major for dB and MN-major (transposed) for dA; likewise the A tile and the B tile.  dB stays in TMEM over the CTA's
-// tiles of a row block; dA_tile goes to scratch, one contribution per row block.
-// 4096 x 4096, r = 32: 512 tokens 119 us with the folds on the CUDA cores (bound by shared memory at two multiply-adds per word
-// read), 43 now; QAT (with 67 MB of dW) 176 -> 74, at 1024 tokens 83.  What bounds it: with many tokens the way of g and x
+// and the factors are bf16 as given, so every product is exact.  Tensor cores cut their sums off instead of rounding them, about 1.5e-8 of
+// the sum an MMA, which adds up where a sum goes through many: so a tile's product leaves TMEM in two sums over half of the tokens
+// each (RAGGED, whose layers ran on the CUDA cores before: 32 or 64 tokens), a fold starts from zero with every tile, its smallest term
+// first, and all these are added up rounding to nearest.  Error of dB and dA against 64 bits, norms: 3.3e-7 at 512 tokens (5.0e-7 with
+// the folds on the CUDA cores and one sum over the tokens, 1.2e-6 with all sums in TMEM), RAGGED 1.6e-7 to 2.2e-7 (CUDA cores 2.0e-7 to
+// 3.1e-7; 0.9e-6 to 3.4e-6); of dW at 1024 tokens 4.7e-7 (9.9e-7), RAGGED 1.0e-7 (2.5e-7; 1.0e-6).
+// One shared-memory tile serves both folds, K-major for dB and MN-major (transposed) for dA; likewise the A tile and the B
+// tile.  A CTA adds its tiles' contributions to dB of a row block in scratch; dA_tile goes there as one contribution per row block.
+// 4096 x 4096, r = 32: 512 tokens 111 us with the folds on the CUDA cores (bound by shared memory at two multiply-adds per word
+// read), 46 now (43 with the long sums in TMEM); QAT (with 67 MB of dW) 165 -> 74 (70), at 1024 tokens 81 (78); 4096 x 4094 at 1024
+// tokens: factors 1361 -> 101 (76), QAT 16253 -> 184 (136).  What bounds it: with many tokens the way of g and x
 // from L2 into shared memory (32 KB per 64 tokens of a tile, about 50 bytes a clock and SM), with few the epilogue (7 thousand cycles a
 // tile; QAT 14, of which 5 for dW's stores and 3 for the quotients) and the first tile, which nothing overlaps.
 //
@@ -460,10 +465,17 @@ template <int RA, bool QAT> struct BwCfg {
     static constexpr int BTILE = RA / 64 * kTcRows * 128;     // 128 rows x RA ranks, 64 ranks per atom
     static constexpr int WSTAGE = QAT && RA == 64 ? kTcEpiWarps * 1024 : 0;       // dW on its way out (with RA = 128 there is no room for it)
     static constexpr int SMEM = 1024 + STAGES * kTcStage + 3 * kTcDsTerm + NA * ATILE + BTILE + WSTAGE + 512;
-    static constexpr uint32_t S_COL = NG * kTcCols, DB_COL = S_COL + (QAT ? kTcCols : 0), DA_COL = DB_COL + RA;
+    static constexpr uint32_t S_COL = NG * kTcCols, DB_COL = S_COL + (QAT ? kTcCols : 0);       // behind it dB and dA of one tile, or of two by turns
     static constexpr uint32_t TMEM = 512;
-    static_assert(SMEM <= 232448 && DA_COL + RA <= 512, "shared memory and TMEM");
+    static_assert(SMEM <= 232448 && DB_COL + 2 * RA <= 512, "shared memory and TMEM");
 };
+
+// Four fp32 sums in global memory, 16-byte aligned, each rounded to nearest.
+__device__ __forceinline__ void red_add_v4(float *at, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(at), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)), "f"(__uint_as_float(c)),
+                 "f"(__uint_as_float(d)) : "memory");
+}
 
 // The division of all 128 x 128 tiles, row block after row block, into one run per CTA.  row_splits 0: equal runs, which may cross from a row
 // block into the next (no CTA idles: 1024 tiles over 148 SMs are 7 rounds, four CTAs per row block 8); else that many runs per row
@@ -493,7 +505,8 @@ struct alignas(64) BwTcParams {
     BwParams b;
     int r4, r_pad;
     Runs runs;            // which tiles a CTA takes
-    int da_bufs;          // TMEM has room for one or two accumulators of dA
+    int fold_bufs;        // TMEM has room for dB and dA of one tile or of two
+    int group;            // MMAs (of 16 tokens) of a tile's product whose sum is taken out of TMEM: 2, 4 or a multiple of 4
     float *part_dB;       // [contribution][m][r4] or null
     float *part_dA;       // [row blocks][r4][n] or null
     int *status;
@@ -618,22 +631,33 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
         const uint32_t hi = (uint32_t)(umma_desc_sw128(0, 1024, (uint32_t)kTcGAtom) >> 32);
         const uint32_t a_lo0 = (uint32_t)umma_desc_sw128(0, 1024, (uint32_t)kTcGAtom) | ((base & 0x3FFFFu) >> 4);
         const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
-        int it = 0;
+        int it = 0, gi = 0;
         for (int t = 0; t < total && !failed; ++t) {
-            const int gb = t % C::NG;
-            if (t >= C::NG && !mbar_wait_warp(bar_g_free + 8 * gb, (uint32_t)((t / C::NG - 1) & 1), status, 47)) { failed = true; break; }
-            tc_fence_after_sync();
-            for (int c = 0; c < chunks; ++c, ++it) {
+            int in_group = 0;                                                      // MMAs of the group so far
+            for (int c = 0; c < chunks && !failed; ++c, ++it) {
                 const int s = it % C::STAGES;
                 if (!mbar_wait_warp(bar_full + 8 * s, (uint32_t)((it / C::STAGES) & 1), status, 42)) { failed = true; break; }
                 tc_fence_after_sync();
                 const uint32_t a_lo = a_lo0 + (uint32_t)((s * kTcStage) >> 4), b_lo = a_lo + (2 * kTcGAtom >> 4);
 #pragma unroll
-                for (int k = 0; k < kTcTok / 16; ++k)      // 16 tokens = 16 rows of 128 bytes
-                    umma_f16_ss(tmem_u + (uint32_t)(gb * kTcCols), umma_desc_pack(a_lo + k * 128, hi), umma_desc_pack(b_lo + k * 128, hi), idesc,
-                                (c > 0 || k > 0) ? 1u : 0u, leader);
+                for (int k = 0; k < kTcTok / 16; k += 2) {      // 16 tokens = 16 rows of 128 bytes
+                    const int gb = gi % C::NG;
+                    if (in_group == 0) {
+                        if (gi >= C::NG && !mbar_wait_warp(bar_g_free + 8 * gb, (uint32_t)((gi / C::NG - 1) & 1), status, 47)) { failed = true; break; }
+                        tc_fence_after_sync();
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        umma_f16_ss(tmem_u + (uint32_t)(gb * kTcCols), umma_desc_pack(a_lo + (k + h) * 128, hi), umma_desc_pack(b_lo + (k + h) * 128, hi), idesc,
+                                    (in_group > 0 || h > 0) ? 1u : 0u, leader);
+                    in_group += 2;
+                    if (in_group == p.group || (c == chunks - 1 && k + 2 == kTcTok / 16)) {
+                        umma_commit(bar_g + 8 * gb, leader);
+                        ++gi;
+                        in_group = 0;
+                    }
+                }
                 umma_commit(bar_empty + 8 * s, leader);
-                if (c == chunks - 1) umma_commit(bar_g + 8 * gb, leader);
             }
         }
     } else if (warp == kTcFoldWarp) {
@@ -673,28 +697,30 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
             if (!mbar_wait_warp2(bar_a + 8 * an, (uint32_t)((t / C::NA) & 1), bar_ds, (uint32_t)(t & 1), status, 50)) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_tile = a_s + (uint32_t)(an * C::ATILE);
-            const bool first = new_rows(t);
-            const uint32_t da_col = tmem_u + C::DA_COL + (uint32_t)(p.da_bufs == 2 && (t & 1) ? p.r_pad : 0);
+            // The smallest term first, each tile onto zero: tensor cores cut sums off instead of rounding them, and this way only the largest
+            // term's eight MMAs do so at the sum's size.
+            const uint32_t db_col = tmem_u + C::DB_COL + (uint32_t)(p.fold_bufs == 2 && (t & 1) ? p.r_pad : 0);
+            const uint32_t da_col = db_col + (uint32_t)(p.fold_bufs * p.r_pad);
             if (p.part_dB) {
                 const uint32_t db = desc_lo(a_tile, 16);
 #pragma unroll 1
-                for (int e = 0; e < 3; ++e) {
+                for (int e = 2; e >= 0; --e) {
                     const uint32_t da = desc_lo(ds0 + (uint32_t)(e * kTcDsTerm), 16);
 #pragma unroll
                     for (int k = 0; k < kTcCols / 16; ++k)
-                        umma_f16_ss(tmem_u + C::DB_COL, umma_desc_pack(da + (k >> 2) * (kTcDsAtom >> 4) + (k & 3) * 2, hi),
-                                    umma_desc_pack(db + (k >> 2) * (C::AATOM >> 4) + (k & 3) * 2, hi), idesc_b, (!first || e > 0 || k > 0) ? 1u : 0u, leader);
+                        umma_f16_ss(db_col, umma_desc_pack(da + (k >> 2) * (kTcDsAtom >> 4) + (k & 3) * 2, hi),
+                                    umma_desc_pack(db + (k >> 2) * (C::AATOM >> 4) + (k & 3) * 2, hi), idesc_b, (e < 2 || k > 0) ? 1u : 0u, leader);
                 }
             }
             if (p.part_dA) {
                 const uint32_t db = desc_lo(b_s, (uint32_t)(kTcRows * 128));
 #pragma unroll 1
-                for (int e = 0; e < 3; ++e) {
+                for (int e = 2; e >= 0; --e) {
                     const uint32_t da = desc_lo(ds0 + (uint32_t)(e * kTcDsTerm), (uint32_t)kTcDsAtom);
 #pragma unroll
                     for (int k = 0; k < kTcRows / 16; ++k)
                         umma_f16_ss(da_col, umma_desc_pack(da + k * 128, hi), umma_desc_pack(db + k * 128, hi), idesc_a,
-                                    (e > 0 || k > 0) ? 1u : 0u, leader);
+                                    (e < 2 || k > 0) ? 1u : 0u, leader);
                 }
             }
             umma_commit(fold_bar(t), leader);
@@ -716,7 +742,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
             if (!p.part_dA) return;
             const int j = col_of(t) * kTcCols + ri;
             float *out = p.part_dA + (size_t)row_of(t) * p.r4 * p.b.n + j;
-            const uint32_t col = C::DA_COL + (uint32_t)(p.da_bufs == 2 && (t & 1) ? p.r_pad : 0);
+            const uint32_t col = C::DB_COL + (uint32_t)(p.fold_bufs * p.r_pad + (p.fold_bufs == 2 && (t & 1) ? p.r_pad : 0));
             for (int k0 = ch * 8; k0 < p.r4; k0 += 32) {          // eight ranks each: all sixteen warps have a part up to rank 32
                 uint32_t v[8];
                 tmem_ld_32x8(lane_addr + col + (uint32_t)k0, v);
@@ -727,24 +753,33 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
             }
             tc_fence_before_sync();
         };
-        // dB of a row block over this CTA's tiles of it (the last one is t): lane = row, TMEM column = rank
+        // a tile's contribution to dB is added to this CTA's contribution to the row block, in scratch (lane = row, TMEM column = rank): only
+        // this thread adds to these values, tile after tile, so the order is fixed.  (Read, added and written back, the way to L2 is waited
+        // for: a fine-tuning step of 4096 x 4096 at 512 tokens 115 us
+        // against 109.)
         auto store_dB = [&](int t) {
             if (!p.part_dB) return;
             const int rb = row_of(t), i = rb * kTcRows + ri;
+            const bool onto = !new_rows(t);
             float *out = p.part_dB + ((size_t)(cta - p.runs.first(rb)) * p.b.m + i) * p.r4;
+            const uint32_t col = C::DB_COL + (uint32_t)(p.fold_bufs == 2 && (t & 1) ? p.r_pad : 0);
             for (int k0 = ch * 16; k0 < p.r4; k0 += 64) {
                 uint32_t v[16];
-                tmem_ld_32x16(lane_addr + C::DB_COL + (uint32_t)k0, v);
+                tmem_ld_32x16(lane_addr + col + (uint32_t)k0, v);
                 tmem_wait_ld(v);
                 if (i < p.b.m)
 #pragma unroll
                     for (int k = 0; k < 16; k += 4)
-                        if (k0 + k < p.r4) __stcg(reinterpret_cast<uint4 *>(out + k0 + k), make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]));
+                        if (k0 + k < p.r4) {
+                            if (onto) red_add_v4(out + k0 + k, v[k], v[k + 1], v[k + 2], v[k + 3]);
+                            else __stcg(reinterpret_cast<uint4 *>(out + k0 + k), make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]));
+                        }
             }
             tc_fence_before_sync();
         };
+        int gi = 0;                  // groups of MMAs so far
         for (int t = 0; t < total; ++t) {
-            const int gb = t % C::NG, i = row_of(t) * kTcRows + ri, jc = col_of(t) * kTcCols + ch * 32;
+            const int i = row_of(t) * kTcRows + ri, jc = col_of(t) * kTcCols + ch * 32;
             // what does not depend on the products is requested first: the thread's codes and latent weights
             // (the last condition holds for every launch without RAGGED; left out, the loads below are scheduled worse: QAT 74 -> 80 us)
             const bool whole = i < p.b.m && jc + 32 <= p.b.n && (RAGGED || (row_bytes & 3) == 0);
@@ -776,49 +811,64 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
                     }
                 }
             }
-            if (!mbar_wait_warp(bar_g + 8 * gb, (uint32_t)((t / C::NG) & 1), status, 43)) { failed = true; break; }
-            tc_fence_after_sync();
+            float gs[32];                                                          // the tile's product, row ri, 32 columns
+#pragma unroll
+            for (int e = 0; e < 32; ++e) gs[e] = 0.0f;
+            for (int c = 0; c < chunks * (kTcTok / 16) && !failed; c += p.group, ++gi) {
+                const int b = gi % C::NG;
+                if (!mbar_wait_warp(bar_g + 8 * b, (uint32_t)((gi / C::NG) & 1), status, 43)) { failed = true; break; }
+                tc_fence_after_sync();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t v[16];
+                    tmem_ld_32x16(lane_addr + (uint32_t)(b * kTcCols + ch * 32 + h * 16), v);
+                    tmem_wait_ld(v);
+#pragma unroll
+                    for (int e = 0; e < 16; e += 2)
+                        f32x2_split(f32x2_add(f32x2(gs[h * 16 + e], gs[h * 16 + e + 1]), f32x2(__uint_as_float(v[e]), __uint_as_float(v[e + 1]))), gs[h * 16 + e],
+                                    gs[h * 16 + e + 1]);
+                }
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_g_free + 8 * b);
+            }
+            if (failed) break;
             if constexpr (QAT) {
                 // Eq. 4: dL/dW = dL/dW^.  Eight rows at a time through the warp's own kilobyte of shared memory, so that a store covers
                 // four rows' 128 bytes: a store takes the load/store unit as many cycles as it touches lines (4096 x 4096, 512 tokens: 4.5
                 // thousand of a tile's 15 thousand cycles with eight rows x 32 bytes per store)
                 if (p.b.dW) {
                     const uint32_t own = w_stage + (uint32_t)(warp * 1024);
-                    const int ir = i - ri + q * 32, lr = lane >> 2, rr = lane >> 3, rc = lane & 7;
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t g[16];
-                        tmem_ld_16x32_frag(lane_addr + ((uint32_t)(hh * 16) << 16) + (uint32_t)(gb * kTcCols + ch * 32), g);
-                        tmem_wait_ld(g);
-                        if constexpr (C::WSTAGE == 0) {
-#pragma unroll
-                            for (int k = 0; k < 8; ++k) {
-                                const int row = ir + hh * 16 + (k & 1) * 8 + lr, col = jc + 2 * (lane & 3) + (k >> 1) * 8;
-                                if (row < p.b.m && col < p.b.n) *reinterpret_cast<uint2 *>(p.b.dW + (size_t)row * p.b.n + col) = make_uint2(g[2 * k], g[2 * k + 1]);
-                            }
-                            continue;
+                    const int ir = i - ri + q * 32, rr = lane >> 3, rc = lane & 7;
+                    auto put = [&](int row, int col, uint4 o) {
+                        if (row >= p.b.m || col >= p.b.n) return;
+                        float *dst = p.b.dW + (size_t)row * p.b.n + col;
+                        if constexpr (!RAGGED) {
+                            __stcs(reinterpret_cast<uint4 *>(dst), o);
+                        } else {                                                   // n is even: 8-byte aligned
+                            *reinterpret_cast<uint2 *>(dst) = make_uint2(o.x, o.y);
+                            if (col + 2 < p.b.n) *reinterpret_cast<uint2 *>(dst + 2) = make_uint2(o.z, o.w);
                         }
+                    };
+                    auto four = [&](int c) {
+                        return make_uint4(__float_as_uint(gs[4 * c]), __float_as_uint(gs[4 * c + 1]), __float_as_uint(gs[4 * c + 2]), __float_as_uint(gs[4 * c + 3]));
+                    };
+                    if constexpr (C::WSTAGE == 0) {
 #pragma unroll
-                        for (int v = 0; v < 2; ++v) {
+                        for (int c = 0; c < 8; ++c) put(i, jc + 4 * c, four(c));
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            // 16-byte chunk c of row l at chunk c ^ l: neither the writes nor the reads meet in a bank
                             __syncwarp();
-                            // 16-byte chunk c of row l at chunk c ^ l: neither the 8-byte writes nor the 16-byte reads meet in a bank
+                            if (rr == v)
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(own + (uint32_t)(lr * 128 + (((2 * u + ((lane >> 1) & 1)) ^ lr) << 4) + (lane & 1) * 8)),
-                                             "r"(g[4 * u + 2 * v]), "r"(g[4 * u + 2 * v + 1]) : "memory");
+                                for (int c = 0; c < 8; ++c) sts_v4(own + (uint32_t)(rc * 128 + ((c ^ rc) << 4)), four(c));
                             __syncwarp();
 #pragma unroll
                             for (int k = 0; k < 2; ++k) {
-                                const int l = k * 4 + rr, row = ir + hh * 16 + v * 8 + l;
-                                const uint4 o = lds_v4(own + (uint32_t)(l * 128 + ((rc ^ l) << 4)));
-                                const int col = jc + 4 * rc;
-                                if constexpr (!RAGGED) {
-                                    if (row < p.b.m && col < p.b.n) __stcs(reinterpret_cast<uint4 *>(p.b.dW + (size_t)row * p.b.n + col), o);
-                                } else if (row < p.b.m && col < p.b.n) {          // n is even: 8-byte aligned
-                                    float *dst = p.b.dW + (size_t)row * p.b.n + col;
-                                    *reinterpret_cast<uint2 *>(dst) = make_uint2(o.x, o.y);
-                                    if (col + 2 < p.b.n) *reinterpret_cast<uint2 *>(dst + 2) = make_uint2(o.z, o.w);
-                                }
+                                const int l = k * 4 + rr;
+                                put(ir + v * 8 + l, jc + 4 * rc, lds_v4(own + (uint32_t)(l * 128 + ((rc ^ l) << 4))));
                             }
                         }
                     }
@@ -831,17 +881,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
             auto level_at = [&](uint32_t code) { return __uint_as_float(lds_table(levels_s + 4u * code)); };
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                uint32_t gacc[16], sv[QAT ? 16 : 1];
-                tmem_ld_32x16(lane_addr + (uint32_t)(gb * kTcCols + ch * 32 + h * 16), gacc);
+                uint32_t sv[QAT ? 16 : 1];
                 if constexpr (QAT) tmem_ld_32x16(lane_addr + C::S_COL + (uint32_t)(ch * 32 + h * 16), sv);
-                tmem_wait_ld(gacc);
-                if constexpr (QAT) tmem_wait_ld(sv);
-                if (h == 1) {
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) {
-                        mbar_arrive(bar_g_free + 8 * gb);
-                        if (QAT) mbar_arrive(bar_s_free);
+                if constexpr (QAT) {
+                    tmem_wait_ld(sv);
+                    if (h == 1) {
+                        tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar_s_free);
                     }
                 }
                 // the factor of dL/dS: the level, or (QAT, Eq. 5) the level minus W (/) S; 0 where S is 0
@@ -867,7 +914,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
                         const int bit = e * W, w = bit >> 5, sh = bit & 31;
                         uint32_t code = cw[w] >> sh;
                         if (sh + W > 32) code |= cw[w + 1 < 4 ? w + 1 : 3] << (32 - sh);
-                        d[e] = __uint_as_float(gacc[e & 15]) * factor(e, level_at(code & ((1u << W) - 1u)));
+                        d[e] = gs[e] * factor(e, level_at(code & ((1u << W) - 1u)));
                     }
                 };
                 if (__all_sync(0xffffffffu, whole)) {
@@ -877,13 +924,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
                 } else {
 #pragma unroll
                     for (int e = 16 * h; e < 16 * h + 16; ++e)
-                        d[e] = (i < p.b.m && jc + e < p.b.n) ? __uint_as_float(gacc[e & 15]) * factor(e, level_at(read_code(p.b.q, row_bytes, i, jc + e, bits))) : 0.0f;
+                        d[e] = (i < p.b.m && jc + e < p.b.n) ? gs[e] * factor(e, level_at(read_code(p.b.q, row_bytes, i, jc + e, bits))) : 0.0f;
                 }
             }
-            // the folds of the tile before have completed: the dS buffer is free, dB and dA of it are in TMEM
+            // the folds of the tile before have completed: the dS buffer is free, its parts of dB and dA are in TMEM
             if (t > 0 && !mbar_wait_warp(fold_bar(t - 1), fold_phase(t - 1), status, 45)) { failed = true; break; }
             tc_fence_after_sync();
-            if (t > 0 && new_rows(t)) store_dB(t - 1);
             // the three terms, eight columns (one 16-byte store each) at a time
 #pragma unroll
             for (int e8 = 0; e8 < 4; ++e8) {
@@ -900,13 +946,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) lords_backward_tc_kernel(const 
 #pragma unroll
                 for (int k = 0; k < 3; ++k) sts_v4(ds_at(ri, k, e8), make_uint4(w[k][0], w[k][1], w[k][2], w[k][3]));
             }
-            // dA of the tile before: with one accumulator it has to leave before this tile's folds begin
-            if (t > 0 && p.da_bufs == 1) store_dA(t - 1);
+            // dA and dB of the tile before: with one accumulator each they have to leave before this tile's folds begin
+            if (t > 0 && p.fold_bufs == 1) {
+                store_dA(t - 1);
+                store_dB(t - 1);
+            }
             fence_proxy_async_smem();
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_ds);
-            if (t > 0 && p.da_bufs == 2) store_dA(t - 1);
+            if (t > 0 && p.fold_bufs == 2) {
+                store_dA(t - 1);
+                store_dB(t - 1);
+            }
         }
         if (!__any_sync(0xffffffffu, failed) && total > 0) {
             if (!mbar_wait_warp(fold_bar(total - 1), fold_phase(total - 1), status, 45)) {
@@ -1056,7 +1108,11 @@ template <int RA, bool QAT, bool RAGGED> static int launch_tc_variant(BwTcParams
         LORDS_CUDA_TRY(cudaFuncSetAttribute(lords_backward_tc_kernel<RA, QAT, RAGGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwCfg<RA, QAT>::SMEM));
         done[dev] = true;
     }
-    k.da_bufs = BwCfg<RA, QAT>::DA_COL + 2 * (uint32_t)k.r_pad <= 512 ? 2 : 1;
+    k.fold_bufs = BwCfg<RA, QAT>::DB_COL + 4 * (uint32_t)k.r_pad <= 512 ? 2 : 1;
+    // (as exact as what these layers ran on before: the CUDA cores with RAGGED, the tensor cores' sum over all tokens and folds on the CUDA cores
+    // without)
+    const int mmas = (k.b.M + kTcTok - 1) / kTcTok * (kTcTok / 16);
+    k.group = RAGGED ? (k.b.M <= 128 ? 2 : 4) : mmas <= 8 ? 4 : (mmas / 2 + 3) / 4 * 4;
     lords_backward_tc_kernel<RA, QAT, RAGGED><<<(unsigned)k.runs.ctas, kTcThreads, BwCfg<RA, QAT>::SMEM, stream>>>(k);
     LORDS_CUDA_TRY(cudaGetLastError());
     return LORDS_OK;
