@@ -83,7 +83,7 @@ NCU_TRAFFIC_BYTES = {
     "prefill_m2048": 162462720,     # the pair kernel; the pre-pass moves 75.0 MB more
     "quantize_q_nf4": 34163200,     # 8.4 MB of codes were still in L2 at the end
     "quantize_gate_nf3": 130008576,
-    "backward_q_m512": 17395456,    # the factor-gradient kernel; the sum behind it moves 19.6 MB more
+    "backward_q_m512": 17399040,    # the factor-gradient kernel; the sum behind it moves 19.6 MB more
 }
 
 
