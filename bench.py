@@ -73,7 +73,7 @@ def measured_peaks():
     return {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0, "source": "fallback"}
 
 
-# dram__bytes_read.sum + dram__bytes_write.sum per launch, from profiles/kernels.md
+# dram__bytes_read.sum + dram__bytes_write.sum per launch, from ncu captures
 NCU_TRAFFIC_BYTES = {
     "decode_q_m1": 8995584,
     "decode_q_m8": 9061120,
