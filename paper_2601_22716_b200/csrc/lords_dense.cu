@@ -20,7 +20,7 @@
 // W^ and x rounded to fp16 3e-4).
 //
 // When it pays: W^ is formed once for all tokens, where the CUDA cores (the only other path for most of these shapes) need r + M
-// multiply-adds a weight: 5952 x 7008, r = 11, 578 tokens: 9160 us there, 255 here (97 with W^ in fp16, a third of the MMAs
+// multiply-adds a weight: 5952 x 7008, r = 11, 578 tokens: 9160 us there, 248 here (81 with W^ in fp16, a third of the MMAs
 // and of the scratch).
 //
 // Every wait is bounded; on expiry the role records LORDS_ERR_TIMEOUT and leaves its loop.
@@ -253,7 +253,7 @@ constexpr int kGEpiWarp0 = 4;                       // warps from 4 on: epilogue
 constexpr uint32_t kGTmemCols = 512;
 
 template <int BN> struct GCfg {
-    static constexpr int EPI = BN >= 256 ? 16 : 8;               // epilogue warps (a k-step's first parts have to be read while the MMAs of its lower parts run: 2816 x 3072, 1024 tokens, 95 us with eight, 85 with sixteen)
+    static constexpr int EPI = BN >= 256 ? 16 : 8;               // epilogue warps (a k-step's first parts have to be read while the MMAs of its lower parts run: 2816 x 3072, 1024 tokens, 95 us with eight, 84 with sixteen)
     static constexpr int THREADS = (kGEpiWarp0 + EPI) * 32;
     static constexpr int ATILE = 128 * 128;                      // this CTA's 128 rows, 64 columns of one part
     static constexpr int BTILE = (BN / 2) * 128;                 // this CTA's half of the tokens
@@ -564,7 +564,7 @@ template <int BN> int run_dense(const Problem &p, State &st, cudaStream_t stream
     if (chunk >= p.m) {
         chunk = p.m;
     } else {
-        // chunks of about equal size: a small last one would leave most pairs idle (5952 x 7008, 578 tokens: 308 us, 255 so)
+        // chunks of about equal size: a small last one would leave most pairs idle (5952 x 7008, 578 tokens: 308 us, 255 with equal ones)
         chunk /= kGRows;
         if (chunk < 1) return LORDS_ERR_WORKSPACE;
         const long long row_tiles = (p.m + kGRows - 1) / kGRows, chunks = (row_tiles + chunk - 1) / chunk;

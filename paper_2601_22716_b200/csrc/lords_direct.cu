@@ -20,7 +20,7 @@
 //
 // Bound: warp instructions -- four per code pair for the table and the product (EXACT: some twenty), the MMAs (2 RK + M / 8, or
 // 3 M / 8, per 16 x 16 weights at the warp-level rate) and the loads around them; codes, factors and activations come by
-// asynchronous copies several strips ahead.  CTAs are small (eight warps, under 110 KB), so that two or more share an SM
+// asynchronous copies several strips ahead.  CTAs are small (eight warps, at most 111 KB), so that two or more share an SM
 // and the next call's CTAs set up (and, where that call is not `late`, load their weights) while this call computes (programmatic
 // dependent launch).
 #include <cuda.h>

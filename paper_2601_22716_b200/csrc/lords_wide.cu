@@ -16,7 +16,7 @@
 // Why a kernel of its own: the factor strip of 128 ranks is 32 KB, which the level table and the rings of the 16-token
 // decode kernel leave no room for, and at 128 ranks the scale product outweighs everything else, so it belongs on
 // tcgen05: with S by warp-level MMAs (the direct kernel) every warp reads the whole factor strip from shared memory
-// again.  4096 x 4096, r = 128, 16 tokens: CUDA cores 585 us, direct kernel 29 us, this kernel 17.5 us (10.4 with W^ in fp16).
+// again.  4096 x 4096, r = 128, 16 tokens: CUDA cores 585 us, direct kernel 31 us, this kernel 17.5 us (10.4 with W^ in fp16).
 //
 // CTA: 128 rows; sixteen consumer warps (32 rows and 32 columns of the strip each), a TMA producer, a warp that makes the copy of the
 // activations without infinities and NaNs, and a scale issuer.  A cluster shares one row tile and splits its strips; every warp
@@ -24,8 +24,8 @@
 // adds them in a fixed order: deterministic, no atomics, no trip through global memory.
 //
 // Bound: the consumers' instructions (13.7 a weight: look-up, product, cutting into parts, MMAs) and the latency of their chain, four
-// warps to a scheduler: 1.6 us a strip of 16384 weights (8192 columns, eight more strips a CTA, take 12.6 us more), of which the strip's
-// arrival (44 KB from L2) and its scale MMAs (8 KB of operands per 16 ranks) are about a third each and overlap.
+// warps to a scheduler: 1.6 us a strip of 16384 weights (8192 columns, eight more strips a CTA, take 12.4 us more), beside which the strip's
+// arrival (44 KB from L2, about a third of that time) and its scale MMAs (a sixth) run.
 //
 // Every wait is bounded; on expiry the role records LORDS_ERR_TIMEOUT and leaves its loop.
 #include <cuda.h>
