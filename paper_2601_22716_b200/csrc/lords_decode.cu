@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
                     // a stage is freed by work that stands behind the dependency point: pass it first, so that
                     // the bounded wait does not run while the previous launch (however long) still works
                     if (!XB && it == SQ) griddep_wait();
-                    if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1), status, 1)) { failed = true; break; }
+                    if (!mbar_wait(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1), status, 1)) { failed = true; break; }
                 }
                 const uint32_t bar = bar_q_full + 8 * sq;
                 mbar_expect_tx(bar, (uint32_t)C::QSTAGE);
@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
             if (!XB) griddep_wait();   // x may be the previous launch's output
             for (int it = 0; it < pre; ++it) load_x(it);
             for (int it = S; it < total; ++it) {
-                if (!mbar_wait<kWaitSlackNs>(bar_mma_done + 8 * ((it - S) % kAF), (uint32_t)(((it - S) / kAF) & 1), status, 2)) { failed = true; break; }
+                if (!mbar_wait(bar_mma_done + 8 * ((it - S) % kAF), (uint32_t)(((it - S) / kAF) & 1), status, 2)) { failed = true; break; }
                 load_a(it);
                 load_x(it);
             }
@@ -399,8 +399,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
         const uint32_t leader = elect_one();
         for (int it = first; it < total; it += kStride) {
             const int s = it % S;
-            if (!mbar_wait<kWaitSpin>(bar_ax_ready + 8 * s, (uint32_t)((it / S) & 1), status, 3) ||
-                !mbar_wait<kWaitSpin>(bar_ready + 8 * (h * S + s), (uint32_t)((it / S) & 1), status, 4)) { failed = true; break; }
+            if (!mbar_wait(bar_ax_ready + 8 * s, (uint32_t)((it / S) & 1), status, 3) ||
+                !mbar_wait(bar_ready + 8 * (h * S + s), (uint32_t)((it / S) & 1), status, 4)) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t wslot = tmem_base + kWCol + (uint32_t)((h * S + s) * kWSlotCols);
             const uint32_t b_lo = desc_lo | ((ax_stage(s) & 0x3FFFFu) >> 4);

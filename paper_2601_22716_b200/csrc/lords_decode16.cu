@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
                     // a stage is freed by work that stands behind the dependency point: pass it first, so that
                     // the bounded wait does not run while the previous launch (however long) still works
                     if (it == SQ) griddep_wait();
-                    if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1))) { failed = true; break; }
+                    if (!mbar_wait(bar_q_empty + 8 * sq, (uint32_t)((it / SQ - 1) & 1))) { failed = true; break; }
                 }
                 const uint32_t bar = bar_q_full + 8 * sq;
                 mbar_expect_tx(bar, (uint32_t)C::QSTAGE);
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             for (int it = 0; it < total; ++it) {
                 const int sa = it % C::SA;
                 if (it == (C::SA > WS ? C::SA : WS)) griddep_wait();
-                if (it >= C::SA && !mbar_wait<kWaitSlackNs>(bar_a_done + 8 * sa, (uint32_t)((it / C::SA - 1) & 1))) { failed = true; break; }
+                if (it >= C::SA && !mbar_wait(bar_a_done + 8 * sa, (uint32_t)((it / C::SA - 1) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_a_full + 8 * sa;
                 mbar_expect_tx(bar, tx);
 #pragma unroll
@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             griddep_wait();
             for (int it = 0; it < total; ++it) {
                 const int sx = it % WS;
-                if (it >= WS && !mbar_wait<kWaitSlackNs>(bar_mma_done + 8 * ((it - WS) % WB), (uint32_t)(((it - WS) / WB) & 1))) { failed = true; break; }
+                if (it >= WS && !mbar_wait(bar_mma_done + 8 * ((it - WS) % WB), (uint32_t)(((it - WS) / WB) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_x_full + 8 * sx;
                 mbar_expect_tx(bar, (uint32_t)kXStage);
 #pragma unroll
@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         for (int it = sj; !BLOCK && it < total && !failed; it += 2) {
             const int sa = it % C::SA, sd = it % SD;
             if (it >= WS && it < WS + 2) griddep_wait();
-            if (!mbar_wait<kWaitSpin>(bar_a_full + 8 * sa, (uint32_t)((it / C::SA) & 1))) { failed = true; break; }
-            if (it >= SD && !mbar_wait<kWaitSpin>(bar_s_empty + 8 * sd, (uint32_t)((it / SD - 1) & 1))) { failed = true; break; }
+            if (!mbar_wait(bar_a_full + 8 * sa, (uint32_t)((it / C::SA) & 1))) { failed = true; break; }
+            if (it >= SD && !mbar_wait(bar_s_empty + 8 * sd, (uint32_t)((it / SD - 1) & 1))) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ASTAGE >> 4));
             for (int k = 0; k < rsteps; ++k)
@@ -400,8 +400,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         const uint32_t acc = tmem_base + (uint32_t)(j * 32);
         for (int it = j; it < total; it += 2) {
             const int ws = it % WS;
-            if (!mbar_wait<kWaitSpin>(bar_x_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1)) ||
-                !mbar_wait<kWaitSpin>(bar_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1))) { failed = true; break; }
+            if (!mbar_wait(bar_x_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1)) ||
+                !mbar_wait(bar_ready + 8 * (it % WB), (uint32_t)((it / WB) & 1))) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t wslot = tmem_base + kWCol + (uint32_t)(ws * 64);
             const uint32_t x_lo = x_lo0 + (uint32_t)(ws * (kXStage >> 4));

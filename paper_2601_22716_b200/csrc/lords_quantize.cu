@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                 }
                 if (failed) break;
                 const int sa = it % kSAQ;
-                if (it >= kSAQ && !mbar_wait<kWaitSlackNs>(bar_a_free + 8 * sa, (uint32_t)((it / kSAQ - 1) & 1), status, 31)) { failed = true; break; }
+                if (it >= kSAQ && !mbar_wait(bar_a_free + 8 * sa, (uint32_t)((it / kSAQ - 1) & 1), status, 31)) { failed = true; break; }
                 mbar_expect_tx(bar_a + 8 * sa, (uint32_t)(p.r_pad * 128));
                 tma_load_2d(a0 + (uint32_t)(sa * C::ATILE), &p.tm_a, st * kColsQ, 0, bar_a + 8 * sa);
                 if (++st == p.steps) { st = 0; ++rt; }

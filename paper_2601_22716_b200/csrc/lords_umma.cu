@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                     if (next_q >= SQ) {
                         const uint32_t par = (uint32_t)((next_q / SQ - 1) & 1);
                         if (blocking) {
-                            if (!mbar_wait<kWaitSlackNs>(bar_q_empty + 8 * sq, par)) return false;
+                            if (!mbar_wait(bar_q_empty + 8 * sq, par)) return false;
                         } else if (!mbar_try_wait(bar_q_empty + 8 * sq, par)) {
                             return true;
                         }
@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
             for (int it = 0; it < total; ++it) {
                 const int sx = it % SX;
                 if (next_q <= (it >> 1) && !issue_q(true)) { failed = true; break; }   // the pair this k-step reads
-                if (it >= SX && !mbar_wait<kWaitSlackNs>(bar_done + 8 * ((it - SX) % DR), (uint32_t)(((it - SX) / DR) & 1))) { failed = true; break; }
+                if (it >= SX && !mbar_wait(bar_done + 8 * ((it - SX) % DR), (uint32_t)(((it - SX) / DR) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_x_full + 8 * sx;
                 mbar_expect_tx(bar, (uint32_t)C::XTILE);
                 tma_load_2d(x0 + sx * C::XTILE, &p.tm_x, (2 * pa + it) * BK, tok0, bar);
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                 // in turn, and no slot barrier can run a phase ahead of it: the scale MMA of k-step
                 // j - SA + SD needs a factor tile that this lane has not loaded yet)
                 if (j >= SA + SD) previous_launch();
-                if (j >= SA && !mbar_wait<kWaitSlackNs>(bar_s_full + 8 * ((j - SA) % SD), (uint32_t)(((j - SA) / SD) & 1))) { failed = true; break; }
+                if (j >= SA && !mbar_wait(bar_s_full + 8 * ((j - SA) % SD), (uint32_t)(((j - SA) / SD) & 1))) { failed = true; break; }
                 const uint32_t bar = bar_a_full + 8 * sa;
                 mbar_expect_tx(bar, tx);
                 tma_load_2d(a0 + sa * kATileBytes, &p.tm_a, (2 * pa + j) * BK, 0, bar);
@@ -310,9 +310,9 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
         for (int j = 0; j < total; ++j) {
             const int sa = j % SA, sd = j % SD;
             if (j >= SD) previous_launch();
-            if (!mbar_wait<kWaitSpin>(bar_a_full + 8 * sa, (uint32_t)((j / SA) & 1))) { failed = true; break; }
+            if (!mbar_wait(bar_a_full + 8 * sa, (uint32_t)((j / SA) & 1))) { failed = true; break; }
             // the slot is free once the main MMAs of k-step j - SD have read their operand out of it
-            if (j >= SD && !mbar_wait<kWaitSpin>(bar_done + 8 * ((j - SD) % DR), (uint32_t)(((j - SD) / DR) & 1))) { failed = true; break; }
+            if (j >= SD && !mbar_wait(bar_done + 8 * ((j - SD) % DR), (uint32_t)(((j - SD) / DR) & 1))) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (kATileBytes >> 4));
             for (int k = 0; k < ksteps; ++k)
@@ -334,8 +334,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
         for (int it = 0; it < total; ++it) {
             const int sx = it % SX, ws = it % SD;
             // W^ of the k-step is in TMEM and its activation tile has landed
-            if (!mbar_wait<kWaitSpin>(bar_w_full + 8 * ws, (uint32_t)((it / SD) & 1))) { failed = true; break; }
-            if (!mbar_wait<kWaitSpin>(bar_x_full + 8 * sx, (uint32_t)((it / SX) & 1))) { failed = true; break; }
+            if (!mbar_wait(bar_w_full + 8 * ws, (uint32_t)((it / SD) & 1))) { failed = true; break; }
+            if (!mbar_wait(bar_x_full + 8 * sx, (uint32_t)((it / SX) & 1))) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t wslot = tmem_base + C::SCOL + (uint32_t)(ws * 64);
             const uint32_t x_lo = x_lo0 + (uint32_t)((sx * C::XTILE) >> 4);

@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
                     previous_launch();                                        // the activations are the pre-pass's
                     for (int h = 0; h < 2; ++h) {
                         const int ks = 2 * st + h, sx = ks % C::SX, prev = ks - C::SX;
-                        if (prev >= 0 && !mbar_wait(bar_done + 8 * (prev % kPDone), (uint32_t)((prev / kPDone) & 1), status, 62)) { failed = true; break; }
+                        if (prev >= 0 && !mbar_wait<kWaitSleepNs>(bar_done + 8 * (prev % kPDone), (uint32_t)((prev / kPDone) & 1), status, 62)) { failed = true; break; }
                         if (rank == 0) mbar_expect_tx(bar_x + 8 * sx, x_tx);
                         tma_load_2d_pair(x0 + (uint32_t)(sx * C::XTILE), &p.tm_x, (2 * k + h) * 64, tt * p.bn + rank * (p.bn / 2), x_pair0 + 8 * sx);
                     }
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             }
             // nothing of this CTA is in flight when it ends
             for (int ks = 2 * st > kPDone ? 2 * st - kPDone : 0; ks < 2 * st && !failed; ++ks)
-                if (!mbar_wait(bar_done + 8 * (ks % kPDone), (uint32_t)((ks / kPDone) & 1), status, 63)) failed = true;
+                if (!mbar_wait<kWaitSleepNs>(bar_done + 8 * (ks % kPDone), (uint32_t)((ks / kPDone) & 1), status, 63)) failed = true;
         }
         __syncwarp();
     } else if (warp == kPTmaA) {
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
                 const int rt = w.tile / p.tok_tiles;
                 if (st > 0) previous_launch();
                 // the scale MMAs of the piece before have read its B
-                if (st > 0 && !mbar_wait(bar_a_free + 8 * ((st - 1) % kPSA), (uint32_t)(((st - 1) / kPSA) & 1), status, 64)) { failed = true; break; }
+                if (st > 0 && !mbar_wait<kWaitSleepNs>(bar_a_free + 8 * ((st - 1) % kPSA), (uint32_t)(((st - 1) / kPSA) & 1), status, 64)) { failed = true; break; }
                 if (rank == 0) mbar_expect_tx(bar_b, 2u * C::BTILE);
                 tma_load_2d_pair(b_tile, &p.tm_b, 0, rt * kPRows + rank * 128, b_pair0);
                 for (int k = w.k0; k < w.k1; ++k, ++st) {
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
                 }
             }
             for (int k = st > kPSA ? st - kPSA : 0; k < st && !failed; ++k)
-                if (!mbar_wait(bar_a_free + 8 * (k % kPSA), (uint32_t)((k / kPSA) & 1), status, 66)) failed = true;
+                if (!mbar_wait<kWaitSleepNs>(bar_a_free + 8 * (k % kPSA), (uint32_t)((k / kPSA) & 1), status, 66)) failed = true;
         }
         __syncwarp();
     } else if (warp == kPScale) {
@@ -210,11 +210,11 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             const int ranks16 = p.r_pad / 16;
             for (int piece = 0; !failed && sched.next(w); ++piece) {
                 if (piece > 0 || !p.b_early) previous_launch();
-                if (!mbar_wait_warp(bar_b, (uint32_t)(piece & 1), status, 69)) { failed = true; break; }
+                if (!mbar_wait_warp<kWaitSleepNs>(bar_b, (uint32_t)(piece & 1), status, 69)) { failed = true; break; }
                 for (int k = w.k0; k < w.k1; ++k, ++st) {
                     const int sa = st % kPSA;
                     if (st >= kPW / 2) previous_launch();                  // the workers stop there, and with them the steps behind
-                    if (!mbar_wait_warp2<kWaitSpin>(bar_a + 8 * sa, (uint32_t)((st / kPSA) & 1), bar_s_free, (uint32_t)((st + 1) & 1), status, 67)) { failed = true; break; }
+                    if (!mbar_wait_warp2(bar_a + 8 * sa, (uint32_t)((st / kPSA) & 1), bar_s_free, (uint32_t)((st + 1) & 1), status, 67)) { failed = true; break; }
                     tc_fence_after_sync();
                     const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ATILE >> 4));
                     for (int c = 0; c < ranks16; ++c)
@@ -236,12 +236,12 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             const uint32_t tmem_u = warp_uniform(tmem_base), leader = elect_one();
             previous_launch();
             for (int piece = 0; !failed && sched.next(w); ++piece) {
-                if (piece > 0 && !mbar_wait_warp(bar_acc_free, (uint32_t)((piece - 1) & 1), status, 70)) { failed = true; break; }
+                if (piece > 0 && !mbar_wait_warp<kWaitSleepNs>(bar_acc_free, (uint32_t)((piece - 1) & 1), status, 70)) { failed = true; break; }
                 for (int k = w.k0; k < w.k1 && !failed; ++k, ++st) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const int ks = 2 * st + h, sx = ks % C::SX, ws = ks % kPW;
-                        if (!mbar_wait_warp2<kWaitSpin>(bar_w + 8 * ws, (uint32_t)((ks / kPW) & 1), bar_x + 8 * sx, (uint32_t)((ks / C::SX) & 1), status, 71)) { failed = true; break; }
+                        if (!mbar_wait_warp2(bar_w + 8 * ws, (uint32_t)((ks / kPW) & 1), bar_x + 8 * sx, (uint32_t)((ks / C::SX) & 1), status, 71)) { failed = true; break; }
                         tc_fence_after_sync();
                         const uint32_t wslot = tmem_u + kPWCol + (uint32_t)(ws * 32), x_lo = x_lo0 + (uint32_t)((sx * C::XTILE) >> 4);
 #pragma unroll
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             for (int k = w.k0; k < w.k1; ++k, ++st) {
                 const int sq = st % kPSQ, ks = 2 * st + g, ws = ks % kPW;
                 if (!p.b_early || 2 * st >= kPW) previous_launch();
-                if (!mbar_wait_warp2(bar_s, (uint32_t)(st & 1), bar_q + 8 * sq, (uint32_t)((st / kPSQ) & 1), status, 73)) { failed = true; break; }
+                if (!mbar_wait_warp2<kWaitSleepNs>(bar_s, (uint32_t)(st & 1), bar_q + 8 * sq, (uint32_t)((st / kPSQ) & 1), status, 73)) { failed = true; break; }
                 tc_fence_after_sync();
                 uint32_t s[32];
                 tmem_ld_32x32(lane_addr + kPSCol + (uint32_t)(g * 64 + ch * 32), s);
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
                 dequant_chunk<BITS>(q0 + (uint32_t)(sq * C::QSTAGE + row * C::QROW), row, g * 2 + ch, lut_lane, s, out);
                 // the ring slot is free once the main MMA of four k-steps ago has read it
                 const int prev = ks - kPW;
-                if (prev >= 0 && !mbar_wait_warp(bar_done + 8 * (prev % kPDone), (uint32_t)((prev / kPDone) & 1), status, 75)) { failed = true; break; }
+                if (prev >= 0 && !mbar_wait_warp<kWaitSleepNs>(bar_done + 8 * (prev % kPDone), (uint32_t)((prev / kPDone) & 1), status, 75)) { failed = true; break; }
                 tc_fence_after_sync();
                 tmem_st_32x16(lane_addr + kPWCol + (uint32_t)(ws * 32 + ch * 16), out);
                 tmem_wait_st();
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(kPThreads, 1) lords_umma_pair_kernel(const __g
             if (failed) break;
             // ---------------------------------------------------------------- epilogue: lane = row, columns = tokens
             previous_launch();
-            if (!mbar_wait_warp(bar_acc, (uint32_t)(piece & 1), status, 76)) { failed = true; break; }
+            if (!mbar_wait_warp<kWaitSleepNs>(bar_acc, (uint32_t)(piece & 1), status, 76)) { failed = true; break; }
             tc_fence_after_sync();
             const int rt = w.tile / p.tok_tiles, tt = w.tile - rt * p.tok_tiles;
             const int i = rt * kPRows + rank * 128 + row;
