@@ -12,11 +12,13 @@
 // them, so S of every 16 ranks and the first parts' products of every 16 columns start from zero and are added on the
 // CUDA cores; the lower parts' products, 2^-8 of the sum, keep to the tensor cores.  Error of the fp32 sums
 // against 64 bits, norms, normal activations, 256 x 256 to 1024 x 14336, ranks 4 to 128: 6e-8 to 1.7e-7 (CUDA cores 8e-8 to 1.6e-7; the
-// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 14.9 us a call (fp16 form 10.7, CUDA cores 67.6).
+// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 13.4 us a call (CUDA cores 67.6).
 //
 // A cluster shares one tile of 128 rows and splits its columns; every CTA sends its partial sums to the CTA that owns
 // the row (asynchronous stores counted on that CTA's barrier), which adds them in rank order: deterministic,
-// no atomics, no trip through global memory.  Tokens beyond sixteen are further groups of CTAs (grid y).
+// no atomics, no trip through global memory.  Tokens that one CTA does not take are further groups of CTAs (grid y), each of which
+// forms W^ again: EXACT takes up to 32 (with groups of 16 and ranks in steps of 32 before, 48 tokens: 4096 x 4094, rank 32, 64.0 us, 44.8 so;
+// 5472 x 10524, rank 11, 170 and 119; 1000 x 2730, rank 10, 15.3 and 13.5).
 //
 // Bound: warp instructions -- four per code pair for the table and the product (EXACT: some twenty), the MMAs (2 RK + M / 8, or
 // 3 M / 8, per 16 x 16 weights at the warp-level rate) and the loads around them; codes, factors and activations come by
@@ -46,17 +48,22 @@ constexpr int kTokenMax = 128;                      // 16 tokens to a group of C
 constexpr int kAPitch = kCols * 2 + 16;             // bytes per rank (or token) row: ldmatrix reads eight rows without bank conflicts
 constexpr int kQPitch = 48;                         // bytes per code row: eight rows in eight different 16-byte bank groups
 
-// BITS: code width.  RK: rank in steps of 16 (zero padded).  MT: tokens (8 or 16, zero padded).
-template <int BITS, int RK, int MT, bool EXACT> struct DirCfg {
+// BITS: code width.  RK: rank in steps of 16 (zero padded).  MT: tokens (8 to 32, zero padded).
+template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirCfg {
     static constexpr int ENTRIES = 1 << 2 * BITS;                             // level pairs
     static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair (EXACT: 16 of 8 bytes)
-    static constexpr int SA = RK <= 4 ? 3 : 2;                                // strips of A and x in flight
-    static constexpr int SQ = 4;                                              // strips of codes in flight
+    static constexpr int SA = RK <= 2 || (RK == 4 && MT < 24) ? 3 : 2;                                // strips of A and x in flight
+    // Strips of codes in flight.  Codes that are not ALIGNED wait in registers instead, and two stages do; the SM so keeps 56 KB of its
+    // 256 as L1 beside two CTAs, not 23, which the words of x that are loaded by turns want (32 tokens, 5472 x 10524, rank 11: 88 us with 23 KB, 60 with 56).
+    static constexpr int SQ = ALIGNED ? 4 : 2;
     static constexpr int ASTAGE = RK * 16 * kAPitch;
     static constexpr int XPART = MT * kAPitch;
     static constexpr int XSTAGE = EXACT ? 2 * XPART : XPART;                  // EXACT: x, and x without infinities and NaNs
     static constexpr int QSTAGE = kRows * kQPitch;
-    static constexpr int RED = (kRows + kClusterMax) * MT * 4;                // partial sums received: cluster x rows owned x tokens
+    // partial sums received: cluster x rows owned x tokens.  The owner's lanes read one token of 32 rows: with rows MT words apart
+    // they met in eight to 32 banks' worth of turns (32 tokens of 4096 x 4094: a third of all shared-memory wavefronts).
+    static constexpr int RPITCH = MT + 2;
+    static constexpr int RED = (kRows + kClusterMax) * RPITCH * 4;
     static constexpr int SMEM = LUT + SA * ASTAGE + 2 * XSTAGE + SQ * QSTAGE + RED + 16;
 };
 
@@ -79,7 +86,7 @@ struct DirectParams {
 template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT>
 __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direct_kernel(const DirectParams p)
 {
-    using C = DirCfg<BITS, RK, MT, EXACT>;
+    using C = DirCfg<BITS, RK, MT, ALIGNED, EXACT>;
     constexpr int TG = MT / 8;                      // groups of eight tokens
     extern __shared__ __align__(1024) uint8_t dir_smem[];
     const uint32_t lut = smem_u32(dir_smem);
@@ -172,18 +179,21 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
             const int col0 = (s_a + it) * kCols;
             constexpr int CB = ALIGNED ? 16 : 4, CH = kCols * 2 / CB;
 #pragma unroll
-            for (int k = 0; k < RK * 16 * CH / kThreads; ++k) {
+            for (int k = 0; k < (RK * 16 * CH + kThreads - 1) / kThreads; ++k) {
                 const int e = tid + k * kThreads, rk = e / CH, ch = e % CH, col = col0 + ch * (CB / 2);
                 const bool in = rk < p.r && col < p.n;
                 const uint16_t *src = p.A + (in ? (size_t)rk * p.n + col : 0);
                 const uint32_t dst = dst0 + (uint32_t)(rk * kAPitch + ch * CB);
-                if constexpr (ALIGNED) cp_async16(dst, src, in ? 16 : 0);
-                else cp_async4(dst, src, in ? 4 : 0);
+                if ((RK * 16 * CH) % kThreads == 0 || rk < RK * 16) {
+                    if constexpr (ALIGNED) cp_async16(dst, src, in ? 16 : 0);
+                    else cp_async4(dst, src, in ? 4 : 0);
+                }
             }
         }
     };
     // activations: eight columns of one token per thread, converted on the way (registers one strip ahead)
-    constexpr int XT = MT * (kCols / 8);             // threads that take part (64 or 128)
+    constexpr int XT = MT * (kCols / 8);             // threads that take part (64 to 256)
+    static_assert(XT <= kThreads && MT % 8 == 0, "one chunk of x per thread");
     const int xt = tid / (kCols / 8), xc = tid % (kCols / 8) * 8;
     auto load_x = [&](int it, uint32_t (&v)[4]) {
         v[0] = v[1] = v[2] = v[3] = 0u;
@@ -231,9 +241,13 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
     // ---- weights first: where the call is not `late` they do not depend on the previous launch.  Copies are committed in the order
     // q0, a0, q1, a1, q2, then per strip a + 2 and q + 3 (or, with two stages of A, q + 3 and a + 2 at its end).
     constexpr int kPending = C::SA == 3 ? 3 : 2;     // youngest copies that strip `it` does not need
+    // What goes through registers (codes that are not ALIGNED, x, the fragments of B) is requested before any of it is waited for: one
+    // way to memory, not three in a row.
+    uint32_t xv[4];
     if constexpr (ALIGNED) stage_q(0);
-    else { load_q(0); store_q(0); load_q(1); }
+    else load_q(0);
     commit();
+    if (EXACT && p.late) load_x(0, xv);
     stage_a(0); commit();
     if constexpr (ALIGNED) stage_q(1);
     commit();
@@ -249,11 +263,12 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
 #pragma unroll
         for (int h = 0; h < 4; ++h) bf[k][h] = load_b_pair(p.B, (h & 1) ? i1 : i0, k * 16 + 2 * t + ((h & 2) ? 8 : 0), p.m, p.r);
 
-    griddep_launch_dependents();
-    griddep_wait();                                  // x may be the previous launch's output
-
-    uint32_t xv[4];
-    load_x(0, xv);
+    if (!(EXACT && p.late)) {
+        griddep_launch_dependents();
+        griddep_wait();                              // x may be the previous launch's output
+        load_x(0, xv);
+    }
+    if constexpr (!ALIGNED) { store_q(0); load_q(1); }
     store_x(0, xv);
     load_x(1, xv);
 
@@ -277,32 +292,37 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
         const uint32_t q_row = q_s + (uint32_t)((it % C::SQ) * C::QSTAGE + (warp * 16 + g) * kQPitch);
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            // S of 16 rows x 32 columns
-            float s[4][4];
+            // S of 16 rows x 16 columns (eight-column tiles 2 h and 2 h + 1 of the 32).  EXACT, which is short of registers, forms it as it is
+            // used, the fp16 form for all 32 columns at once
+            float s[EXACT ? 2 : 4][4];
+            auto form_s = [&](int h, float (&s0)[4], float (&s1)[4]) {
 #pragma unroll
-            for (int k = 0; k < RK; ++k)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                for (int k = 0; k < RK; ++k) {
                     uint32_t v[4];
                     ldmatrix_x4_trans(a_tile + (uint32_t)((k * 16 + (lane & 15)) * kAPitch + c * 64 + (2 * h + (lane >> 4)) * 16), v);
                     if (k == 0) {
-                        mma_bf16_first(s[2 * h], bf[k], v[0], v[1]);
-                        mma_bf16_first(s[2 * h + 1], bf[k], v[2], v[3]);
+                        mma_bf16_first(s0, bf[k], v[0], v[1]);
+                        mma_bf16_first(s1, bf[k], v[2], v[3]);
                     } else if constexpr (EXACT) {
-                        add_mma_bf16(s[2 * h], bf[k], v[0], v[1]);
-                        add_mma_bf16(s[2 * h + 1], bf[k], v[2], v[3]);
+                        add_mma_bf16(s0, bf[k], v[0], v[1]);
+                        add_mma_bf16(s1, bf[k], v[2], v[3]);
                     } else {
-                        mma_bf16(s[2 * h], bf[k], v[0], v[1]);
-                        mma_bf16(s[2 * h + 1], bf[k], v[2], v[3]);
+                        mma_bf16(s0, bf[k], v[0], v[1]);
+                        mma_bf16(s1, bf[k], v[2], v[3]);
                     }
                 }
+            };
+            if constexpr (!EXACT) {
+                form_s(0, s[0], s[1]);
+                form_s(1, s[2], s[3]);
+            }
             CodeWords<BITS> w0, w1;
             w0.read(q_row + (uint32_t)(c * 4 * BITS));
             w1.read(q_row + (uint32_t)(8 * kQPitch + c * 4 * BITS));
             // x of 32 columns: token row lane & 7, 16-byte chunk lane >> 3.  EXACT, which is short of registers, takes it 16 columns at
-            // a time: chunk lane >> 3 & 1, and with two groups of tokens group lane >> 4
+            // a time: chunk lane >> 3 & 1, and of a pair of token groups group lane >> 4
             const uint32_t x_lane = x_tile + (uint32_t)((lane & 7) * kAPitch + c * 64 +
-                                                        (EXACT ? (TG == 2 ? (lane >> 4) * 8 * kAPitch : 0) + ((lane >> 3) & 1) * 16 : (lane >> 3) * 16));
+                                                        (EXACT ? (TG > 1 ? (lane >> 4) * 8 * kAPitch : 0) + ((lane >> 3) & 1) * 16 : (lane >> 3) * 16));
             uint32_t xb[EXACT ? 1 : TG][4];
             if constexpr (!EXACT) {
 #pragma unroll
@@ -311,24 +331,32 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if constexpr (EXACT) {
+                    form_s(h, s[0], s[1]);
                     auto scales = [&](int u, int e) { return f32x2(s[u][e], s[u][e + 1]); };
-                    const uint64_t w[4] = {w0.weights(2 * h, t, lut_lane, scales(2 * h, 0)), w1.weights(2 * h, t, lut_lane, scales(2 * h, 2)),
-                                           w0.weights(2 * h + 1, t, lut_lane, scales(2 * h + 1, 0)), w1.weights(2 * h + 1, t, lut_lane, scales(2 * h + 1, 2))};
+                    const uint64_t w[4] = {w0.weights(2 * h, t, lut_lane, scales(0, 0)), w1.weights(2 * h, t, lut_lane, scales(0, 2)),
+                                           w0.weights(2 * h + 1, t, lut_lane, scales(1, 0)), w1.weights(2 * h + 1, t, lut_lane, scales(1, 2))};
                     uint32_t hi[4], mid[4], lo[4];
                     split_weights(w, hi, mid, lo);
-                    uint32_t xa[2 * TG], xf[2 * TG];
-                    if constexpr (TG == 2) {
-                        ldmatrix_x4(x_lane + (uint32_t)(h * 32), xa);
-                        ldmatrix_x4(x_lane + (uint32_t)(h * 32 + C::XPART), xf);
-                    } else {
-                        ldmatrix_x2(x_lane + (uint32_t)(h * 32), xa);
-                        ldmatrix_x2(x_lane + (uint32_t)(h * 32 + C::XPART), xf);
-                    }
 #pragma unroll
-                    for (int k = 0; k < TG; ++k) {
-                        add_mma_bf16(acc[k], hi, xa[2 * k], xa[2 * k + 1]);
-                        mma_bf16(low[k], mid, xf[2 * k], xf[2 * k + 1]);
-                        mma_bf16(low[k], lo, xf[2 * k], xf[2 * k + 1]);
+                    for (int k0 = 0; k0 < TG; k0 += 2) {
+                        const uint32_t x_pair = x_lane + (uint32_t)(k0 * 8 * kAPitch + h * 32);
+                        uint32_t xa[4], xf[4];
+                        if (k0 + 1 < TG) {
+                            ldmatrix_x4(x_pair, xa);
+                            ldmatrix_x4(x_pair + (uint32_t)C::XPART, xf);
+                        } else {
+                            uint32_t v[2];
+                            ldmatrix_x2(x_pair, v);
+                            xa[0] = v[0]; xa[1] = v[1];
+                            ldmatrix_x2(x_pair + (uint32_t)C::XPART, v);
+                            xf[0] = v[0]; xf[1] = v[1];
+                        }
+#pragma unroll
+                        for (int k = k0; k < (k0 + 2 < TG ? k0 + 2 : TG); ++k) {
+                            add_mma_bf16(acc[k], hi, xa[2 * (k - k0)], xa[2 * (k - k0) + 1]);
+                            mma_bf16(low[k], mid, xf[2 * (k - k0)], xf[2 * (k - k0) + 1]);
+                            mma_bf16(low[k], lo, xf[2 * (k - k0)], xf[2 * (k - k0) + 1]);
+                        }
                     }
                 } else {
                     uint32_t wa[4];
@@ -369,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int row = warp * 16 + g + 8 * h, owner = (int)(((uint32_t)row * p.per_rank_inv) >> 16);
-        const uint32_t dst = map_to_rank(red + (uint32_t)(((rank * per_rank + row - owner * per_rank) * MT + 2 * t) * 4), (uint32_t)owner);
+        const uint32_t dst = map_to_rank(red + (uint32_t)(((rank * per_rank + row - owner * per_rank) * C::RPITCH + 2 * t) * 4), (uint32_t)owner);
         const uint32_t dbar = map_to_rank(bar, (uint32_t)owner);
 #pragma unroll
         for (int k = 0; k < TG; ++k)
@@ -382,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
                 const int tok = e / groups, row = (e - tok * groups) * 32 + lane, i = row0 + own0 + row;
                 if (row < own_n) {
                     float sum = 0.0f;
-                    for (int rr = 0; rr < csize; ++rr) sum += __uint_as_float(lds_u32(red + (uint32_t)(((rr * per_rank + row) * MT + tok) * 4)));
+                    for (int rr = 0; rr < csize; ++rr) sum += __uint_as_float(lds_u32(red + (uint32_t)(((rr * per_rank + row) * C::RPITCH + tok) * 4)));
                     if (i < p.m) store_out(p.y, p.y_f32, (size_t)(tok0 + tok) * p.m + i, sum);
                 }
             }
@@ -394,7 +422,7 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
 }
 
 template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirectVariant {
-    using C = DirCfg<BITS, RK, MT, EXACT>;
+    using C = DirCfg<BITS, RK, MT, ALIGNED, EXACT>;
     static void fill(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int cs, int tiles, int groups, cudaStream_t stream)
     {
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -429,57 +457,86 @@ template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirectVaria
         }
         return cache[dev][cs] > 0 ? cache[dev][cs] : 0;
     }
-    static int launch(DirectParams &k, int tiles, bool ordered, int forced, const State &st, cudaStream_t stream)
+    // The cluster size for this call and an estimate of its time, in strips of sixteen tokens: waves of clusters times (strips of a CTA
+    // x the weight of its tokens + a fixed part worth two and a half).  A strip takes about as long
+    // with two CTAs on an SM as with one (one alone waits for its own loads and MMAs: 4096 x 4096 split 4
+    // ways, one CTA per SM, 16.6 us; split 8 ways, two per SM, 10.0), so what fits at once counts as one wave.
+    static double plan(const DirectParams &k, int tiles, int forced, int dev, int &cs)
     {
-        const int dev = device_slot(st), lim = kClusterMax < k.strips ? kClusterMax : k.strips, groups = (k.M + MT - 1) / MT;
-        int cs = 0;
+        const int lim = kClusterMax < k.strips ? kClusterMax : k.strips, groups = (k.M + MT - 1) / MT;
+        double best = 1e30;
+        cs = 0;
         if (forced > 0) {
             for (cs = forced < lim ? forced : lim; cs > 1 && max_clusters(dev, cs) == 0;) --cs;
+            best = groups;
         } else {
-            // Waves of clusters times (strips of a CTA + a fixed part worth two and a half).  A strip takes about as long
-            // with two CTAs on an SM as with one (one alone waits for its own loads and MMAs: 4096 x 4096 split 4
-            // ways, one CTA per SM, 16.6 us; split 8 ways, two per SM, 10.0), so what fits at once counts as one wave.
-            double best = 1e30;
             for (int c = 1; c <= lim; ++c) {
                 const int res = max_clusters(dev, c);
                 if (res == 0) continue;
-                const double t = (double)((tiles * groups + res - 1) / res) * ((k.strips + c - 1) / c + 2.5);
+                const double t = (double)((tiles * groups + res - 1) / res) * ((k.strips + c - 1) / c * kStripWeight + 2.5);
                 if (t <= best) { best = t; cs = c; }
             }
         }
-        if (cs < 1 || max_clusters(dev, cs) == 0) return LORDS_ERR_UNSUPPORTED;
+        if (cs < 1 || max_clusters(dev, cs) == 0) best = 1e30;
+        return best;
+    }
+    // Forming W^ takes most of a strip; every further group of eight tokens adds its three MMAs and their operands (one group of CTAs, 16,
+    // 24, 32 tokens: 4096 x 4094, rank 32, 22.9, 25.8, 28.5 us; 5472 x 10524, rank 11, 55, 64, 74; 5000 x 4128, rank 60, 35, 42, 47).
+    static constexpr double kStripWeight = MT <= 16 ? 1.0 : 1.0 + 0.2 * (MT / 8 - 2);
+    static int launch(DirectParams &k, int tiles, int cs, bool ordered, cudaStream_t stream)
+    {
         k.per_rank = (kRows + cs - 1) / cs;
         k.per_rank_inv = (uint32_t)((65536 + k.per_rank - 1) / k.per_rank);
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
-        fill(cfg, attr, cs, tiles, groups, stream);
+        fill(cfg, attr, cs, tiles, (k.M + MT - 1) / MT, stream);
         if (ordered) attr[1].val.programmaticStreamSerializationAllowed = 0;
         LORDS_CUDA_TRY(cudaLaunchKernelEx(&cfg, lords_direct_kernel<BITS, RK, MT, ALIGNED, EXACT>, k));
         return LORDS_OK;
     }
 };
 
-template <int BITS, int RK, int MT, bool EXACT> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
+// The first of the token widths MT with the least estimate.
+template <int BITS, int RK, bool ALIGNED, bool EXACT, int... MT>
+int launch_planned(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
+{
+    const int dev = device_slot(st), tiles = (p.m + kRows - 1) / kRows;
+    double best = 1e29;
+    int at = -1, best_cs = 0, i = 0, cs = 0;
+    auto consider = [&](double t) { if (t < best) { best = t; at = i; best_cs = cs; } ++i; };
+    (consider(DirectVariant<BITS, RK, MT, ALIGNED, EXACT>::plan(k, tiles, st.forced_splitk, dev, cs)), ...);
+    int rc = LORDS_ERR_UNSUPPORTED;
+    i = 0;
+    ((i++ == at ? (void)(rc = DirectVariant<BITS, RK, MT, ALIGNED, EXACT>::launch(k, tiles, best_cs, p.ordered, stream)) : (void)0), ...);
+    return rc;
+}
+
+template <int BITS, int RK, bool ALIGNED, bool EXACT> int launch_tokens(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
+{
+    if (p.M <= 8) return launch_planned<BITS, RK, ALIGNED, EXACT, 8>(k, p, st, stream);
+    // more tokens to a group form W^ fewer times (EXACT, up to 64 ranks: beyond, the registers hold B); the fp16 form takes small layers, where CTAs are few
+    if constexpr (EXACT && RK <= 4)
+        if (p.M > 16) return launch_planned<BITS, RK, ALIGNED, EXACT, 16, 24, 32>(k, p, st, stream);
+    return launch_planned<BITS, RK, ALIGNED, EXACT, 16>(k, p, st, stream);
+}
+
+template <int BITS, int RK, bool EXACT> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
     const size_t row_bytes = (size_t)p.n * BITS / 8;
     const bool aligned = row_bytes % (BITS == 3 ? 8 : 16) == 0 && p.n % 8 == 0;
-    const int tiles = (p.m + kRows - 1) / kRows;
     if constexpr (EXACT)
-        if (!aligned) return DirectVariant<BITS, RK, MT, false, true>::launch(k, tiles, p.ordered, st.forced_splitk, st, stream);
+        if (!aligned) return launch_tokens<BITS, RK, false, true>(k, p, st, stream);
     // the fp16 form: n is a multiple of 64 (128 for 3 bits), so its rows are aligned
-    return DirectVariant<BITS, RK, MT, true, EXACT>::launch(k, tiles, p.ordered, st.forced_splitk, st, stream);
-}
-template <int BITS, int RK, bool EXACT> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
-{
-    return p.M <= 8 ? launch_direct<BITS, RK, 8, EXACT>(k, p, st, stream) : launch_direct<BITS, RK, 16, EXACT>(k, p, st, stream);
+    return launch_tokens<BITS, RK, true, EXACT>(k, p, st, stream);
 }
 template <int BITS> int launch_direct(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
     // fp16 operands only where the kernel this one stands in for has them (decode16, umma): what else ran on the CUDA cores in fp32, or,
     // with one or two tokens, on the reassociated form, keeps that range and precision
     if (umma_takes(p) && !decode_takes(p)) return p.r <= 32 ? launch_direct<BITS, 2, false>(k, p, st, stream) : launch_direct<BITS, 4, false>(k, p, st, stream);
-    return p.r <= 32 ? launch_direct<BITS, 2, true>(k, p, st, stream)
-                     : p.r <= 64 ? launch_direct<BITS, 4, true>(k, p, st, stream) : launch_direct<BITS, 8, true>(k, p, st, stream);
+    return p.r <= 16 ? launch_direct<BITS, 1, true>(k, p, st, stream)
+         : p.r <= 32 ? launch_direct<BITS, 2, true>(k, p, st, stream)
+         : p.r <= 64 ? launch_direct<BITS, 4, true>(k, p, st, stream) : launch_direct<BITS, 8, true>(k, p, st, stream);
 }
 
 }  // namespace

@@ -160,15 +160,18 @@ static int validate(const void *x, const uint8_t *q, const void *B, const void *
 //     weights.
 static bool small_for_decode(const Problem &p) { return (long long)p.m * p.n <= (1 << 19); }
 
-// The direct kernel rebuilds W^ for every group of 16 tokens; the two-phase path does it once, at the price of 6 bytes of scratch a weight
-// (which beyond L2's size go to memory and back) and of two launches.  Microseconds, fitted to eight shapes of 0.7 to 58 M weights at 16 to
-// 128 tokens (direct against two-phase: 4096 x 4094, r = 32: 32 tokens 38 : 53, 48 63 : 57; 1000 x 2730, 128 tokens 27 : 40; 2816 x
-// 3072, r = 100: 32 tokens 29 : 37, 64 52 : 41; 5472 x 10524, 48 tokens 170 : 212): the line misses by at most 4 % of a call there.
+// The direct kernel rebuilds W^ for every group of 16 to 32 tokens; the two-phase path does it once, at the price of 6 bytes of scratch a weight
+// (which beyond L2's size go to memory and back) and of two launches.  Microseconds, fitted to seven shapes of 0.3 to 58 M weights at 16 to
+// 128 tokens (direct against two-phase: 4096 x 4094, r = 32: 64 tokens 49 : 57, 80 79 : 62; 1000 x 2730, 128 tokens 21 : 40; 2816 x
+// 3074, r = 50: 64 tokens 41 : 44, 80 54 : 47; 5000 x 4128, r = 60: 48 tokens 76 : 77, 64 86 : 78; 5472 x 10524, r = 11: 64 tokens 138 : 220,
+// 96 204 : 220): the line misses by at most 8 % of a call there.
 static bool direct_first(const Problem &p)
 {
     if (p.M > 128) return false;
-    const double w = (double)p.m * p.n / 1048576.0, groups = (p.M + 15) / 16;
-    return 4.0 + (p.r <= 64 ? 1.15 : 1.55) * groups * w <= 25.0 + (w <= 24.0 ? 1.9 : 3.2) * w;
+    const double w = (double)p.m * p.n / 1048576.0;
+    const int wide = p.r <= 64 ? 32 : 16, groups = (p.M + wide - 1) / wide, tokens = (p.M + groups - 1) / groups;
+    const double strip = tokens <= 16 ? 1.0 : tokens <= 24 ? 1.18 : 1.35, rate = p.r <= 16 ? 0.95 : p.r <= 32 ? 1.15 : p.r <= 64 ? 1.6 : 1.55;
+    return 4.0 + rate * strip * groups * w <= 25.0 + (w <= 24.0 ? 1.9 : 3.5) * w;
 }
 
 static int dispatch(const Problem &p, State &st, cudaStream_t s)

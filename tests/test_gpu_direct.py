@@ -38,6 +38,11 @@ SHAPES = [
     (3, 300, 1024, 64, 16, False),
     (2, 300, 192, 48, 8, True),
 ]
+# groups of up to 24 and 32 tokens, their remainders and several of them; ranks in one fragment and past it; codes in asynchronous copies (n a
+# multiple of 32) and through registers
+GROUP_SHAPES = [(bits, m, n, r, M, M % 2 == 0) for (bits, m, n, r) in
+                ((4, 2700, 2080, 16), (4, 2700, 1002, 17), (3, 2700, 1056, 33), (2, 2700, 1004, 64))
+                for M in (17, 24, 25, 32, 33, 48, 49, 65, 128)]
 
 
 @pytest.fixture(scope="module")
@@ -65,7 +70,7 @@ def _forward(lords, lay, split=0):
     return dl, y32, ybf
 
 
-@pytest.mark.parametrize("bits,m,n,r,M,mixed", SHAPES)
+@pytest.mark.parametrize("bits,m,n,r,M,mixed", SHAPES + GROUP_SHAPES)
 def test_direct_kernel_shapes(lords, bits, m, n, r, M, mixed):
     lay = gen.make_layer(m, n, r, M, bits=bits, seed=m + n + r + M, mixed_sign=mixed)
     dl, y32, ybf = _forward(lords, lay)
