@@ -9,7 +9,7 @@
 // but a k-step of 128 columns (half the barrier traffic per weight element), two main-MMA issuers
 // that take k-steps alternately into accumulators of their own, converter warps for the activation
 // tile, and a thread-block cluster that splits a tile's k-range and adds the partial sums in the
-// leader's shared memory in rank order (deterministic, no atomics).
+// shared memory of the CTA that owns the token, which adds them in rank order (deterministic, no atomics).
 //
 // Warp roles (27 warps):
 //   0..15  two worker groups of eight warps take k-steps alternately: a warp owns 32 rows and one
@@ -90,7 +90,8 @@ template <int BITS, int RP> struct XCfg {
     // offsets OR-ed into the table-size-aligned base.
     static constexpr int LUT_STRIDE = BITS == 4 ? 256 : 128;
     static constexpr int LUT_BYTES = LUT_ENTRIES * LUT_STRIDE;
-    static constexpr int RED_BYTES = kClusterMax * kTok * kRows * 4;   // the cluster's partials, [rank][token][row]
+    // the cluster's partial sums of the tokens that this CTA adds up (ceil(M / cluster) of them), [rank][token][row]
+    static constexpr int RED_BYTES = (kTok + kClusterMax) * kRows * 4;
     static constexpr int BAR_BYTES = 512;
     static constexpr int LOW_BYTES = WS * kXStage + kBTileBytes + SA * ASTAGE + BAR_BYTES;   // before the 4-bit table
     static constexpr int SMEM = BITS == 4 ? 232448
@@ -146,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t lut = (raw + C::LUT_BYTES - 1) & ~(uint32_t)(C::LUT_BYTES - 1);   // table-size aligned
     // x0: activation ring; b_tile: B[128 x 64 ranks]; a0: factor ring; q0: code ring;
-    // red0: [kClusterMax][16 tokens][128 rows] floats (the leader's copy is used)
+    // red0: [cluster][tokens of this CTA][128 rows] floats
     uint32_t x0, b_tile, a0, bars, q0, red0;
     bool fits = true;
     if constexpr (BITS == 4) {
@@ -209,9 +210,10 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         }
         fence_mbar_init();
         __syncwarp();
-        // the leader's reduce barrier counts the bytes of the cluster's partial sums (its one
+        // the reduce barrier counts the bytes of the cluster's partial sums of this CTA's tokens (its one
         // arrival is this one); the stores may come before or after, the phase ends when both are in
-        if (rank == 0 && lane == 0 && csize > 1) mbar_expect_tx(bar_reduce, (uint32_t)(csize * kTok * kRows * 4));
+        const int own_toks = (p.M - rank + csize - 1) / csize;
+        if (own_toks > 0 && lane == 0 && csize > 1) mbar_expect_tx(bar_reduce, (uint32_t)(csize * own_toks * kRows * 4));
         asm volatile("bar.arrive 1, %0;" ::"n"(kThreads) : "memory");   // barriers exist; does not wait for the others
         // split-phase cluster barrier: arrive now (the fence above has published this CTA's barriers
         // cluster-wide, so a relaxed arrival is enough); the wait is in the epilogue
@@ -420,32 +422,44 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
 
         for (int it = g; it < total; it += 2) {
             const int sq = it % SQ, sd = it % SD, ws = it % WS;
-            if (it >= WS && it < WS + 2) griddep_wait();
-            // S and the codes have landed, and the W slot is free: the MMAs of step it - WS have completed
-            const uint32_t bar_first = BLOCK ? bar_q_full + 8 * sq : bar_s_full + 8 * sd, par_q = (uint32_t)((it / SQ) & 1);
-            if (!mbar_wait_warp3(bar_first, BLOCK ? par_q : (uint32_t)((it / SD) & 1), bar_q_full + 8 * sq, par_q,
-                                 bar_mma_done + 8 * ((it + WB - WS) % WB), (uint32_t)(((it - WS) / WB) & 1), it >= WS)) { failed = true; break; }
-            tc_fence_after_sync();
-            // 16 columns of S at a time, the next 16 on their way from TMEM while these are rounded to fp16 pairs and
-            // multiplied by the looked-up level pairs: the conversions, the look-ups and the TMEM loads of a warp overlap
             uint32_t sp[32];
             HalfRow<BITS> codes;
-            if constexpr (BLOCK) {
+            // 2 and 3 bits: the look-ups before the wait for S (two address instructions each overlap its way; 14336 x 4096, 3 bits, rank 48, 16
+            // tokens, 20.8 -> 19.9 us; 2 bits, 8 tokens, 19.5 -> 19.1).  4 bits: among the products below, where the table reads, one address
+            // instruction each, would otherwise come in bursts (18.1 us against 19.0).
+            constexpr bool kLookAhead = BITS != 4 || BLOCK;
+            if constexpr (kLookAhead) {
+                if (!mbar_wait_warp(bar_q_full + 8 * sq, (uint32_t)((it / SQ) & 1))) { failed = true; break; }
                 codes.read(q0 + sq * C::QSTAGE + row * C::QROW, row, ch);
+#pragma unroll
+                for (int P = 0; P < 32; ++P) sp[P] = lds_u32(codes.address(P, lut_lane));
+            }
+            if (it >= WS && it < WS + 2) griddep_wait();
+            // the W slot is free once the MMAs of step it - WS have completed
+            const uint32_t bar_slot = bar_mma_done + 8 * ((it + WB - WS) % WB), par_slot = (uint32_t)(((it - WS) / WB) & 1);
+            if constexpr (BLOCK) {
                 const int i = row0 + row, blkidx = ((ks_a + it) * kStep + ch * 64) / p.blk;
                 const float sc = (i < p.m && blkidx < p.nblk) ? __uint_as_float((uint32_t)p.scales[(size_t)i * p.nblk + blkidx] << 16) : 0.0f;
                 const __half2 s2 = __floats2half2_rn(sc, sc);
 #pragma unroll
-                for (int pp = 0; pp < 32; ++pp) {
-                    const uint32_t lv = lds_table(codes.address(pp, lut_lane));
-                    const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), s2);
-                    sp[pp] = *reinterpret_cast<const uint32_t *>(&wv);
+                for (int P = 0; P < 32; ++P) {
+                    const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&sp[P]), s2);
+                    sp[P] = *reinterpret_cast<const uint32_t *>(&wv);
                 }
+                if (it >= WS && !mbar_wait_warp(bar_slot, par_slot)) { failed = true; break; }
+                tc_fence_after_sync();
             } else {
+                const uint32_t bar_s = bar_s_full + 8 * sd, par_s = (uint32_t)((it / SD) & 1);
+                const bool in = !kLookAhead ? mbar_wait_warp3(bar_s, par_s, bar_q_full + 8 * sq, (uint32_t)((it / SQ) & 1), bar_slot, par_slot, it >= WS)
+                              : it >= WS ? mbar_wait_warp2(bar_s, par_s, bar_slot, par_slot) : mbar_wait_warp(bar_s, par_s);
+                if (!in) { failed = true; break; }
+                tc_fence_after_sync();
+                // 16 columns of S at a time, the next 16 on their way from TMEM while these are rounded to fp16 pairs and
+                // multiplied by the level pairs: the conversions, the look-ups and the TMEM loads of a warp overlap
                 const uint32_t s_addr = lane_addr + kSCol + (uint32_t)(sd * kStep + ch * 64);
                 uint32_t s[2][16];
                 tmem_ld_32x16(s_addr, s[0]);
-                codes.read(q0 + sq * C::QSTAGE + row * C::QROW, row, ch);
+                if constexpr (!kLookAhead) codes.read(q0 + sq * C::QSTAGE + row * C::QROW, row, ch);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     tmem_wait_ld(s[k & 1]);
@@ -457,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
                     }
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const uint32_t lv = lds_table(codes.address(8 * k + e, lut_lane));
+                        const uint32_t lv = kLookAhead ? sp[8 * k + e] : lds_table(codes.address(8 * k + e, lut_lane));
                         const __half2 sv = __floats2half2_rn(__uint_as_float(s[k & 1][2 * e]), __uint_as_float(s[k & 1][2 * e + 1]));
                         const __half2 wv = __hmul2(*reinterpret_cast<const __half2 *>(&lv), sv);
                         sp[8 * k + e] = *reinterpret_cast<const uint32_t *>(&wv);
@@ -476,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
 
         griddep_wait();
         // Epilogue (group 0, column half 0: one thread per row): the two accumulators -> this CTA's
-        // partial y, parked in the cluster leader's shared memory; the leader adds in rank order.
+        // partial y, sent to the CTAs that own the tokens; those add in rank order.
         if (g == 0 && ch == 0 && !failed) {
             const int i = row0 + row;
             // second half of the split-phase cluster barrier, behind the wait for the last MMAs
@@ -513,27 +527,33 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
                     for (int t = 0; t < kTok; ++t)
                         if (t < p.M) store_out(p.y, p.y_f32, (size_t)t * p.m + i, yt[t]);
             } else {
-                // a CTA that gave up still sends its bytes (zeros), so the leader never waits in vain
-                const uint32_t leader_bar = map_to_rank(bar_reduce, 0);
+                // The cluster's partial sums are added up by all of its CTAs: token t by CTA t mod cluster, which so receives M rows of
+                // them in all (with a leader for all tokens, 16 x cluster rows came into one SM: 1024 x 4096, eight tokens, 6.65 us a
+                // call, 5.1 so; 4096 x 4096 9.2 and 8.6).  (Computed here, not above: live through the loop they cost its registers.)
+                const int cta = (int)cluster_ctarank(), red_toks = (p.M + csize - 1) / csize, own_toks = (p.M - cta + csize - 1) / csize;
+                // a CTA that gave up still sends its bytes (zeros), so nobody waits in vain
+                int to = 0, nth = 0;                           // token t goes to CTA `to`, as the `nth` of its tokens
 #pragma unroll
                 for (int t = 0; t < kTok; ++t)
-                    st_async_cluster_f32(map_to_rank(red0 + (uint32_t)(((rank * kTok + t) * kRows + row) * 4), 0), yt[t], leader_bar);
-                if (rank == 0) {
+                    if (t < p.M) {
+                        st_async_cluster_f32(map_to_rank(red0 + (uint32_t)(((cta * red_toks + nth) * kRows + row) * 4), (uint32_t)to), yt[t],
+                                             map_to_rank(bar_reduce, (uint32_t)to));
+                        if (++to == csize) { to = 0; ++nth; }
+                    }
+                if (own_toks > 0) {
                     const bool got = __all_sync(0xffffffffu, mbar_wait_cluster(bar_reduce, 0));
                     if (!got) failed = true;
-                    else if (i < p.m) {
-                        // rank order for every token; the sixteen sums run side by side
-                        float a[kTok];
+                    else if (i < p.m)
+#pragma unroll 1
+                        for (int j = 0; j < own_toks; ++j) {
+                            float v[kClusterMax], a = 0.0f;     // all reads first (they overlap), then the sum in rank order
 #pragma unroll
-                        for (int t = 0; t < kTok; ++t) a[t] = 0.0f;
-                        for (int rr = 0; rr < csize; ++rr)
+                            for (int rr = 0; rr < kClusterMax; ++rr)
+                                v[rr] = rr < csize ? __uint_as_float(lds_u32(red0 + (uint32_t)(((rr * red_toks + j) * kRows + row) * 4))) : 0.0f;
 #pragma unroll
-                            for (int t = 0; t < kTok; ++t)
-                                a[t] += __uint_as_float(lds_u32(red0 + (uint32_t)(((rr * kTok + t) * kRows + row) * 4)));
-#pragma unroll
-                        for (int t = 0; t < kTok; ++t)
-                            if (t < p.M) store_out(p.y, p.y_f32, (size_t)t * p.m + i, a[t]);
-                    }
+                            for (int rr = 0; rr < kClusterMax; ++rr) a += v[rr];
+                            store_out(p.y, p.y_f32, (size_t)(j * csize + cta) * p.m + i, a);
+                        }
                 }
             }
         }
@@ -548,7 +568,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
         asm volatile("ld.shared.u32 %0, [%1];" : "=r"(tmem_base) : "r"(tmem_slot));
         tmem_dealloc(tmem_base, kTmemCols);
     }
-    // No CTA of the cluster leaves before the leader has received every partial sum: the asynchronous
+    // No CTA of the cluster leaves before every CTA has received its partial sums: the asynchronous
     // stores of a CTA must not be in flight when it exits (with programmatic dependent launch a CTA
     // of the next launch can take over the SM at once).
     if (csize > 1) {
