@@ -416,41 +416,64 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
             const int i = row0 + row;
             if (!ok) failed = true;
             if (BN > 16 || csize == 1) {
-                float *const part = p.pair_scratch + (size_t)pair_index * BN * BM;
-                if (pair_split && rank == 0) {
-                    // the partner's half of the k-range comes through global scratch; its arrival on
-                    // this CTA's barrier (release / acquire at cluster scope) orders the data
-                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(bar_reduce, 0))) { ok = false; failed = true; }
-                }
-                if (ok && total > 0) {
-#pragma unroll 1
-                    for (int c0 = cg * CPG; c0 < (cg + 1) * CPG; c0 += 16) {
-                        uint32_t v[16];
-                        tmem_ld_32x16(lane_addr + (uint32_t)c0, v);
-                        tmem_wait_ld();
-                        if (pair_split && rank == 1) {
+                auto store_tokens = [&](int c0, const float (&sum)[16]) {
+                    if (i < p.m)
 #pragma unroll
-                            for (int c = 0; c < 16; ++c) part[(size_t)(c0 + c) * BM + row] = __uint_as_float(v[c]);
-                        } else if (i < p.m) {
-                            // the partner's sums of the chunk are all requested before the first store to y (which
-                            // the compiler must assume may alias them: load and store by turns would pay the way to
-                            // L2 sixteen times)
-                            float pv[16];
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) pv[c] = pair_split ? __ldcg(part + (size_t)(c0 + c) * BM + row) : 0.0f;
-#pragma unroll
-                            for (int c = 0; c < 16; ++c) {
-                                const int t = tok0 + c0 + c;
-                                if (t < p.M) store_out(p.y, p.y_f32, (size_t)t * p.m + i, __uint_as_float(v[c]) + pv[c]);   // fixed order: first half + second half
-                            }
+                        for (int c = 0; c < 16; ++c) {
+                            const int t = tok0 + c0 + c;
+                            if (t < p.M) store_out(p.y, p.y_f32, (size_t)t * p.m + i, sum[c]);
                         }
-                    }
-                }
-                if (pair_split && rank == 1) {
+                };
+                // this CTA's sums of 16 tokens (zeros where it had no k-step)
+                auto sums = [&](int c0, float (&sum)[16]) {
+                    uint32_t v[16];
+                    tmem_ld_32x16(lane_addr + (uint32_t)c0, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) sum[c] = total > 0 ? __uint_as_float(v[c]) : 0.0f;
+                };
+                if (BN > 16 && pair_split) {
+                    // The two CTAs exchange their sums through global scratch: each sends those of the other's half of the tokens, then adds
+                    // and stores its own half (with one CTA sending all and the other adding all, the exchange was twice as long: 4096 x 4096,
+                    // 512 tokens, 28.7 us a call, 24.6 so; 300 tokens, 3 bits, rank 48, 29.0 and 24.6).  The arrivals on the partner's barrier (release / acquire at cluster scope)
+                    // order the data; a CTA that gave up arrives as well.
+                    constexpr int kHalf = BN / 2, kChunks = kHalf / 16;
+                    float *const part = p.pair_scratch + (size_t)pair_index * BN * BM + row;
+                    if (ok)
+#pragma unroll 1
+                        for (int k = cg; k < kChunks; k += 4) {
+                            const int c0 = (1 - rank) * kHalf + 16 * k;
+                            float sum[16];
+                            sums(c0, sum);
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) part[(size_t)(c0 + c) * BM] = sum[c];
+                        }
                     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // the partner's barrier exists
                     cluster_waited = true;
                     __syncwarp();
-                    if (lane == 0) mbar_arrive_cluster(map_to_rank(bar_reduce, 0));
+                    if (lane == 0) mbar_arrive_cluster(map_to_rank(bar_reduce, (uint32_t)(1 - rank)));
+                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(bar_reduce, 0))) { ok = false; failed = true; }
+                    if (ok)
+#pragma unroll 1
+                        for (int k = cg; k < kChunks; k += 4) {
+                            const int c0 = rank * kHalf + 16 * k;
+                            // all of the partner's sums are requested before the first store to y (which the compiler must assume may
+                            // alias them: load and store by turns would pay the way to L2 sixteen times)
+                            float theirs[16], sum[16];
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) theirs[c] = __ldcg(part + (size_t)(c0 + c) * BM);
+                            sums(c0, sum);
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) sum[c] += theirs[c];
+                            store_tokens(c0, sum);
+                        }
+                } else if (ok && total > 0) {
+#pragma unroll 1
+                    for (int c0 = cg * CPG; c0 < (cg + 1) * CPG; c0 += 16) {
+                        float sum[16];
+                        sums(c0, sum);
+                        store_tokens(c0, sum);
+                    }
                 }
             } else {
                 // BN == 16 with the k-range split over the cluster: park the partials in the leader's
