@@ -700,44 +700,51 @@ template <int BITS, int BN, int RP> int launch_variant(UmmaParams &k, const Prob
     return LORDS_OK;
 }
 
-// Token tile: the largest that still gives CTAs for most of the SMs (tiles that fill at most half of the
-// SMs are split over two CTAs each, see launch_variant).
-int token_tile(const Problem &p, const State &st)
-{
-    const long long row_tiles = (p.m + BM - 1) / BM;
-    auto ctas = [&](int b) {
-        const long long t = row_tiles * ((p.M + b - 1) / b);
-        return (2 * t <= st.sm_count && p.n > 128) ? 2 * t : t;
-    };
-    int bn = 256;
-    while (bn > 32 && (p.M <= bn / 2 || 5 * ctas(bn) < 3 * (long long)st.sm_count)) bn /= 2;
-    return bn;
-}
+// Estimates of a call's time in microseconds, least-squares fits to the kernels' times on eighteen layer shapes (0.3 to 59 M weights) at 20 to
+// 2048 tokens, off by 4 (this kernel, every token tile) and 5 % (the one on CTA pairs) on average.  What they choose is 0.7 % slower than the best of
+// the five on average, 18 % at most (5120 x 5120, 256 tokens: 33 us against 28); with the largest token tile that gave CTAs for most of the
+// SMs, and a line between the kernels from four shapes, it was 5.4 and 43 % (2560 x 1024, 512 tokens: 18.4 us in tiles of 32 tokens, 11.2 in tiles of 256;
+// 11008 x 1536, 64 tokens: 23 and 14).
+double fixed_us(const Problem &p) { return 0.053e-6 * (double)p.m * p.n + 0.91e-6 * (double)p.M * ((double)p.m + p.n); }    // weights, activations
 
-// Whether the kernel on CTA pairs is the faster one: it does a step of 128 columns in about the time that this one needs for a
-// k-step of 64, but divides the work into fewer, larger tiles, and where it cuts them, the meeting of the pieces costs about 15 us,
-// so that it takes the large calls (14336 x 4096, 512 tokens: 60 us against 79; 4096 x 14336, 64 tokens: 32 against 54;
-// 4096 x 4096: 32 against 29 at 512 tokens, 35 against 41 at 1024).  The two estimates below, in microseconds, are least-squares fits to
-// the kernels' times on four layer shapes at 64 to 2048 tokens.  The one for pairs is off by up to 25 %, most where both are short,
-// but on those shapes no call gets a kernel more than 2 % slower than the other.
-bool prefer_pair(const Problem &p, const State &st)
+// This kernel with tiles of `bn` tokens: a wave is k-steps of 64 columns, as long as the look-ups whatever the tile, and an epilogue.
+double single_us(const Problem &p, const State &st, int bn)
 {
     const double rank = p.r > 32 ? 1.0 : 0.0;
-    const int bn = token_tile(p, st);
     const long long tiles = (long long)((p.m + BM - 1) / BM) * ((p.M + bn - 1) / bn), sms = st.sm_count;
     double ksteps = (double)((p.n + BK - 1) / BK), waves = (double)((tiles + sms - 1) / sms);
-    const bool halves = 2 * tiles <= sms;                                        // every tile's k-range over two CTAs
+    const bool halves = 2 * tiles <= sms && p.n > 128;                           // every tile's k-range over two CTAs
     if (halves) ksteps *= 0.5;
     else if (tiles > sms && 2 * ((long long)waves * sms - tiles) >= sms) waves -= 0.5;     // the last wave's are
-    const double single = 2.9 + (halves ? 4.8 : 0.0) + (0.319 + 0.0011 * bn + 0.015 * rank) * ksteps * waves;
-
-    const long long tok_tiles = (p.M + 255) / 256, bn2 = ((p.M + tok_tiles - 1) / tok_tiles + 31) / 32 * 32;
-    const long long tiles2 = (long long)((p.m + 255) / 256) * tok_tiles;
-    if (tiles2 > 0x3fffffffLL) return false;
-    const Division d = divide_tiles((int)tiles2, (p.n + 127) / 128, (int)(sms / 2), 2, kMeetSteps);
-    const double paired = 2.4 + (d.whole < (int)tiles2 ? 15.0 : 0.0) + (0.436 + 0.0021 * (double)bn2 + 0.097 * rank) * d.per_pair;
-    return paired < single;
+    return 0.1 + (halves ? 1.4 : 0.0) + ((0.412 + 0.00008 * bn + 0.012 * rank) * ksteps + 2.43 + 0.0100 * bn) * waves + fixed_us(p);
 }
+
+// The kernel on CTA pairs: it does a step of 128 columns in about the time that this one needs for a
+// k-step of 64, but divides the work into fewer, larger tiles, has a longer set-up, and where it cuts tiles, their pieces have to meet, so
+// that it takes the large calls (14336 x 4096, 512 tokens: 60 us against 73; 4096 x 14336, 64 tokens: 33 against 55;
+// 4096 x 4096: 33 against 25 at 512 tokens, 35 against 41 at 1024; 2048 x 2048, 64 tokens: 18 against 11).
+double pair_us(const Problem &p, const State &st)
+{
+    const long long tok_tiles = (p.M + 255) / 256, bn = ((p.M + tok_tiles - 1) / tok_tiles + 31) / 32 * 32;
+    const long long tiles = (long long)((p.m + 255) / 256) * tok_tiles;
+    if (tiles > 0x3fffffffLL) return 1e30;
+    const Division d = divide_tiles((int)tiles, (p.n + 127) / 128, st.sm_count / 2, 2, kMeetSteps);
+    return 3.6 + (d.whole < (int)tiles ? 8.7 : 0.0) + (0.604 + 0.00032 * (double)bn + (p.r > 32 ? 0.037 : 0.0)) * d.per_pair + 0.012 * (double)bn + fixed_us(p);
+}
+
+// Token tile: 32, 64, 128 or 256, whichever has the shortest estimate.
+int token_tile(const Problem &p, const State &st)
+{
+    int best = 32;
+    double best_us = single_us(p, st, 32);
+    for (int bn = 64; bn <= 256 && bn < 2 * p.M; bn *= 2) {
+        const double us = single_us(p, st, bn);
+        if (us < best_us) { best = bn; best_us = us; }
+    }
+    return best;
+}
+
+bool prefer_pair(const Problem &p, const State &st) { return pair_us(p, st) < single_us(p, st, token_tile(p, st)); }
 
 template <int BITS, int RP> int launch_bits_rank(UmmaParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
@@ -788,7 +795,7 @@ int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t s
 int launch_umma(const Problem &p, State &st, cudaStream_t stream)
 {
     if (!umma_takes(p)) return LORDS_ERR_UNSUPPORTED;
-    if (p.M > 32 && st.forced_bn == 0 && prefer_pair(p, st)) {
+    if (p.M > 16 && st.forced_bn == 0 && prefer_pair(p, st)) {
         const int prc = launch_umma_pair(p, st, stream);
         if (prc != LORDS_ERR_UNSUPPORTED && prc != LORDS_ERR_WORKSPACE) return prc;
     }

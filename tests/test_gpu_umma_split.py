@@ -1,11 +1,12 @@
-"""The scale-MMA kernel where the two CTAs of a cluster share a tile's columns and exchange halves of its tokens: every token tile, token
-counts around its half and its whole, ragged rows.  Sums of small integers are exact in any order."""
+"""The scale-MMA kernels.  Where the two CTAs of a cluster share a tile's columns and exchange halves of its tokens: every token tile, token
+counts around its half and its whole, ragged rows; sums of small integers are exact in any order.  And what the dispatch chooses by its
+estimates: the kernel on CTA pairs from 17 tokens on, and small and large token tiles."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2601_22716_b200 import inputs as gen
-from _util import DeviceLayer
+from _util import DeviceLayer, check_against_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +35,12 @@ def test_halves_of_the_tokens(lords, bits, bn, M):
         lords.lords_set_option("path", "auto")
         lords.lords_set_option("bn", "0")
     assert np.array_equal(y32.astype(np.float64), oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits))
+
+
+@pytest.mark.parametrize("bits,m,n,r,M", [(4, 500, 8192, 20, 17), (3, 512, 8192, 48, 32), (4, 640, 1024, 8, 256), (2, 1100, 1536, 32, 140), (4, 390, 768, 16, 300)])
+def test_estimates_choose(lords, bits, m, n, r, M):
+    lay = gen.make_layer(m, n, r, M, bits=bits, seed=m + M)
+    dl = DeviceLayer(lay)
+    y32, ybf = dl.forward()
+    assert lords.lords_last_path() == "umma"
+    check_against_oracle(y32, ybf, oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits))
