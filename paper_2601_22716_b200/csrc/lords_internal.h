@@ -74,6 +74,8 @@ int launch_simt(const Problem &p, State &st, cudaStream_t stream);
 // Tensor-core path (TMA + tcgen05/TMEM), scale matrix rebuilt per tile by a small MMA.
 // LORDS_ERR_UNSUPPORTED for shapes outside its rules.
 int launch_umma(const Problem &p, State &st, cudaStream_t stream);
+// Estimate of its time in microseconds (more than 16 tokens).
+double umma_us(const Problem &p, const State &st);
 
 // The same on CTA pairs, for large calls, and the pre-pass that both share.
 int launch_umma_pair(const Problem &p, State &st, cudaStream_t stream);

@@ -790,6 +790,12 @@ int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t s
     return LORDS_OK;
 }
 
+double umma_us(const Problem &p, const State &st)
+{
+    const double single = single_us(p, st, token_tile(p, st)), pairs = pair_us(p, st);
+    return single < pairs ? single : pairs;
+}
+
 // Rules of this path: r <= 64; n a multiple of 64 (2- and 4-bit codes) or 128 (3-bit), which makes
 // every TMA row pitch a multiple of 16 bytes.  Anything else: LORDS_ERR_UNSUPPORTED.
 int launch_umma(const Problem &p, State &st, cudaStream_t stream)
