@@ -54,7 +54,7 @@ template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirCfg {
     static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair (EXACT: 16 of 8 bytes)
     static constexpr int SA = RK <= 2 || (RK == 4 && MT < 24) ? 3 : 2;                                // strips of A and x in flight
     // Strips of codes in flight.  Codes that are not ALIGNED wait in registers instead, and two stages do; the SM so keeps 56 KB of its
-    // 256 as L1 beside two CTAs, not 23, which the words of x that are loaded by turns want (32 tokens, 5472 x 10524, rank 11: 88 us with 23 KB, 60 with 56).
+    // 256 as L1 beside two CTAs, not 23, which the words of x that are loaded by turns want (32 tokens, 5472 x 10524, rank 11: 88 us with 23 KB, 74 with 56).
     static constexpr int SQ = ALIGNED ? 4 : 2;
     static constexpr int ASTAGE = RK * 16 * kAPitch;
     static constexpr int XPART = MT * kAPitch;
