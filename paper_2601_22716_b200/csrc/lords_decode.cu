@@ -714,9 +714,11 @@ template <int BITS, int NTOK, int H> int choose_cluster(int dev, int tiles, int 
     const int resident = V::max_clusters(dev, cs) > 0 ? V::max_clusters(dev, cs) : 1;
     const int waves = (tiles + resident - 1) / resident;
     const int steps = (ksteps + cs - 1) / cs;
-    // a two-half step covers twice the rows in about 1.4 times the time of a one-half step (1400 cycles against 1000: converting the
-    // factor tile costs both the same), and every launch pays a fixed prologue + reduction worth a few steps
-    cost = (double)waves * ((double)steps * (H == 2 ? 1.4 : 1.0) + 2.0);
+    // A two-half step covers twice the rows in 1.3 to 1.4 times the time of a one-half step (converting the
+    // factor tile costs both the same), and every launch pays a fixed prologue + reduction worth a few steps.  1.3: the taller tile's grid also leaves
+    // SMs free, where the next launch's CTAs start before this one's end (4096 x 2048, 4 x 32 CTAs of one half against 6 x 16 of two: 6.0 : 5.5 us,
+    // two tokens 7.1 : 6.3; 4096 x 4096 7.5 : 7.3, two tokens 8.9 : 8.8).
+    cost = (double)waves * ((double)steps * (H == 2 ? 1.3 : 1.0) + 2.0);
     return cs;
 }
 
