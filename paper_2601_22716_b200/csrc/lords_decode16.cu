@@ -428,13 +428,19 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             // tokens, 20.8 -> 19.9 us; 2 bits, 8 tokens, 19.5 -> 19.1).  4 bits: among the products below, where the table reads, one address
             // instruction each, would otherwise come in bursts (18.1 us against 19.0).
             constexpr bool kLookAhead = BITS != 4 || BLOCK;
+            // The dependency point comes before the first wait for something that stands behind it in another role: the W slot of step WS,
+            // and the codes of step SQ, whose TMA lane passes it there.  Only a ring that holds the codes of both groups' first steps from
+            // WS on lets their look-ups go ahead of it.
+            constexpr bool kPointFirst = SQ < WS + 2;
+            const bool at_point = it >= WS && it < WS + 2;
+            if (kPointFirst && at_point) griddep_wait();
             if constexpr (kLookAhead) {
                 if (!mbar_wait_warp(bar_q_full + 8 * sq, (uint32_t)((it / SQ) & 1))) { failed = true; break; }
                 codes.read(q0 + sq * C::QSTAGE + row * C::QROW, row, ch);
 #pragma unroll
                 for (int P = 0; P < 32; ++P) sp[P] = lds_u32(codes.address(P, lut_lane));
             }
-            if (it >= WS && it < WS + 2) griddep_wait();
+            if (!kPointFirst && at_point) griddep_wait();
             // the W slot is free once the MMAs of step it - WS have completed
             const uint32_t bar_slot = bar_mma_done + 8 * ((it + WB - WS) % WB), par_slot = (uint32_t)(((it - WS) / WB) & 1);
             if constexpr (BLOCK) {
