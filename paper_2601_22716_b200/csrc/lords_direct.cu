@@ -60,10 +60,13 @@ template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirCfg {
     static constexpr int XPART = MT * kAPitch;
     static constexpr int XSTAGE = EXACT ? 2 * XPART : XPART;                  // EXACT: x, and x without infinities and NaNs
     static constexpr int QSTAGE = kRows * kQPitch;
-    // partial sums received: cluster x rows owned x tokens.  The owner's lanes read one token of 32 rows: with rows MT words apart
-    // they met in eight to 32 banks' worth of turns (32 tokens of 4096 x 4094: a third of all shared-memory wavefronts).
-    static constexpr int RPITCH = MT + 2;
-    static constexpr int RED = (kRows + kClusterMax) * RPITCH * 4;
+    // Partial sums received: cluster x rows owned x tokens.  The owner's lanes read one token of 32 rows, which with the pairs of tokens in
+    // order would meet in two to eight banks: pair u of a row sits at u ^ red_swizzle(row).  A remote store of four pairs keeps to
+    // one 32-byte sector; rows padded by a pair instead, which stores then straddle, took 2 % longer with eight tokens (1344 x 704, rank 5:
+    // 3.41 us, 3.20 so) and gained less with more (2880 x 1792, rank 9, 14 tokens: 7.7 us in order, 6.9 padded, 6.4 so).
+    static constexpr int RED_SHIFT = MT == 32 ? 0 : MT == 16 ? 1 : 2, RED_MASK = MT == 32 ? 15 : MT == 16 ? 7 : 3;
+    static __device__ __forceinline__ int red_swizzle(int row) { return row >> RED_SHIFT & RED_MASK; }
+    static constexpr int RED = (kRows + kClusterMax) * MT * 4;
     static constexpr int SMEM = LUT + SA * ASTAGE + 2 * XSTAGE + SQ * QSTAGE + RED + 16;
 };
 
@@ -295,26 +298,26 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
             // S of 16 rows x 16 columns (eight-column tiles 2 h and 2 h + 1 of the 32).  EXACT, which is short of registers, forms it as it is
             // used, the fp16 form for all 32 columns at once
             float s[EXACT ? 2 : 4][4];
-            auto form_s = [&](int h, float (&s0)[4], float (&s1)[4]) {
-#pragma unroll
-                for (int k = 0; k < RK; ++k) {
-                    uint32_t v[4];
-                    ldmatrix_x4_trans(a_tile + (uint32_t)((k * 16 + (lane & 15)) * kAPitch + c * 64 + (2 * h + (lane >> 4)) * 16), v);
-                    if (k == 0) {
-                        mma_bf16_first(s0, bf[k], v[0], v[1]);
-                        mma_bf16_first(s1, bf[k], v[2], v[3]);
-                    } else if constexpr (EXACT) {
-                        add_mma_bf16(s0, bf[k], v[0], v[1]);
-                        add_mma_bf16(s1, bf[k], v[2], v[3]);
-                    } else {
-                        mma_bf16(s0, bf[k], v[0], v[1]);
-                        mma_bf16(s1, bf[k], v[2], v[3]);
-                    }
+            auto add_ranks = [&](int k, int h, float (&s0)[4], float (&s1)[4]) {      // 16 ranks from 16 k on
+                uint32_t v[4];
+                ldmatrix_x4_trans(a_tile + (uint32_t)((k * 16 + (lane & 15)) * kAPitch + c * 64 + (2 * h + (lane >> 4)) * 16), v);
+                if (k == 0) {
+                    mma_bf16_first(s0, bf[k], v[0], v[1]);
+                    mma_bf16_first(s1, bf[k], v[2], v[3]);
+                } else if constexpr (EXACT) {
+                    add_mma_bf16(s0, bf[k], v[0], v[1]);
+                    add_mma_bf16(s1, bf[k], v[2], v[3]);
+                } else {
+                    mma_bf16(s0, bf[k], v[0], v[1]);
+                    mma_bf16(s1, bf[k], v[2], v[3]);
                 }
             };
             if constexpr (!EXACT) {
-                form_s(0, s[0], s[1]);
-                form_s(1, s[2], s[3]);
+                // ranks outermost: four chains of MMAs side by side
+#pragma unroll
+                for (int k = 0; k < RK; ++k)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) add_ranks(k, h, s[2 * h], s[2 * h + 1]);
             }
             CodeWords<BITS> w0, w1;
             w0.read(q_row + (uint32_t)(c * 4 * BITS));
@@ -331,7 +334,8 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 if constexpr (EXACT) {
-                    form_s(h, s[0], s[1]);
+#pragma unroll
+                    for (int k = 0; k < RK; ++k) add_ranks(k, h, s[0], s[1]);
                     auto scales = [&](int u, int e) { return f32x2(s[u][e], s[u][e + 1]); };
                     const uint64_t w[4] = {w0.weights(2 * h, t, lut_lane, scales(0, 0)), w1.weights(2 * h, t, lut_lane, scales(0, 2)),
                                            w0.weights(2 * h + 1, t, lut_lane, scales(1, 0)), w1.weights(2 * h + 1, t, lut_lane, scales(1, 2))};
@@ -397,11 +401,12 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int row = warp * 16 + g + 8 * h, owner = (int)(((uint32_t)row * p.per_rank_inv) >> 16);
-        const uint32_t dst = map_to_rank(red + (uint32_t)(((rank * per_rank + row - owner * per_rank) * C::RPITCH + 2 * t) * 4), (uint32_t)owner);
+        const int own_row = row - owner * per_rank, swz = C::red_swizzle(own_row);
+        const uint32_t dst = map_to_rank(red + (uint32_t)((rank * per_rank + own_row) * MT * 4), (uint32_t)owner);
         const uint32_t dbar = map_to_rank(bar, (uint32_t)owner);
 #pragma unroll
         for (int k = 0; k < TG; ++k)
-            if (k * 8 + 2 * t < ntok) st_async_cluster_2f32(dst + (uint32_t)(k * 32), acc[k][2 * h], acc[k][2 * h + 1], dbar);
+            if (k * 8 + 2 * t < ntok) st_async_cluster_2f32(dst + (uint32_t)(((k * 4 + t) ^ swz) * 8), acc[k][2 * h], acc[k][2 * h + 1], dbar);
     }
     if (own_n > 0) {
         if (!mbar_wait_cluster(bar, 0, p.status, 61)) failed = true;
@@ -409,8 +414,9 @@ __global__ void __launch_bounds__(kThreads, EXACT || RK > 4 ? 2 : 3) lords_direc
             for (int e = warp, groups = (own_n + 31) / 32; e < ntok * groups; e += kWarps) {
                 const int tok = e / groups, row = (e - tok * groups) * 32 + lane, i = row0 + own0 + row;
                 if (row < own_n) {
+                    const int word = ((tok >> 1) ^ C::red_swizzle(row)) * 2 + (tok & 1);
                     float sum = 0.0f;
-                    for (int rr = 0; rr < csize; ++rr) sum += __uint_as_float(lds_u32(red + (uint32_t)(((rr * per_rank + row) * C::RPITCH + tok) * 4)));
+                    for (int rr = 0; rr < csize; ++rr) sum += __uint_as_float(lds_u32(red + (uint32_t)(((rr * per_rank + row) * MT + word) * 4)));
                     if (i < p.m) store_out(p.y, p.y_f32, (size_t)(tok0 + tok) * p.m + i, sum);
                 }
             }
