@@ -732,14 +732,15 @@ double pair_us(const Problem &p, const State &st)
     return 3.6 + (d.whole < (int)tiles ? 8.7 : 0.0) + (0.604 + 0.00032 * (double)bn + (p.r > 32 ? 0.037 : 0.0)) * d.per_pair + 0.012 * (double)bn + fixed_us(p);
 }
 
-// Token tile: 32, 64, 128 or 256, whichever has the shortest estimate.
-int token_tile(const Problem &p, const State &st)
+// Token tile: 32, 64, 128 or 256, whichever has the shortest estimate of those that are not in `tried` (a sum of tiles); 0 if all are.
+int token_tile(const Problem &p, const State &st, int tried = 0)
 {
-    int best = 32;
-    double best_us = single_us(p, st, 32);
-    for (int bn = 64; bn <= 256 && bn < 2 * p.M; bn *= 2) {
+    int best = 0;
+    double best_us = 0.0;
+    for (int bn = 32; bn == 32 || (bn <= 256 && bn < 2 * p.M); bn *= 2) {
+        if (tried & bn) continue;
         const double us = single_us(p, st, bn);
-        if (us < best_us) { best = bn; best_us = us; }
+        if (best == 0 || us < best_us) { best = bn; best_us = us; }
     }
     return best;
 }
@@ -749,14 +750,19 @@ bool prefer_pair(const Problem &p, const State &st) { return pair_us(p, st) < si
 template <int BITS, int RP> int launch_bits_rank(UmmaParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
     if (p.M <= 16) return launch_variant<BITS, 16, RP>(k, p, st, stream);
-    int bn = token_tile(p, st);
-    if (st.forced_bn > 0) bn = st.forced_bn;   // measurement switch
-    switch (bn) {
-        case 32: return launch_variant<BITS, 32, RP>(k, p, st, stream);
-        case 64: return launch_variant<BITS, 64, RP>(k, p, st, stream);
-        case 128: return launch_variant<BITS, 128, RP>(k, p, st, stream);
-        default: return launch_variant<BITS, 256, RP>(k, p, st, stream);
-    }
+    auto launch_tile = [&](int bn) {
+        switch (bn) {
+            case 32: return launch_variant<BITS, 32, RP>(k, p, st, stream);
+            case 64: return launch_variant<BITS, 64, RP>(k, p, st, stream);
+            case 128: return launch_variant<BITS, 128, RP>(k, p, st, stream);
+            default: return launch_variant<BITS, 256, RP>(k, p, st, stream);
+        }
+    };
+    if (st.forced_bn > 0) return launch_tile(st.forced_bn);   // measurement switch
+    // how much scratch a tile takes depends on how many of them share their columns: one that does not find room leaves the call to the others
+    int rc = LORDS_ERR_WORKSPACE;
+    for (int tried = 0, bn; rc == LORDS_ERR_WORKSPACE && (bn = token_tile(p, st, tried)) > 0; tried |= bn) rc = launch_tile(bn);
+    return rc;
 }
 
 template <int BITS> int launch_bits(UmmaParams &k, const Problem &p, State &st, cudaStream_t stream)
@@ -801,9 +807,12 @@ double umma_us(const Problem &p, const State &st)
 int launch_umma(const Problem &p, State &st, cudaStream_t stream)
 {
     if (!umma_takes(p)) return LORDS_ERR_UNSUPPORTED;
-    if (p.M > 16 && st.forced_bn == 0 && prefer_pair(p, st)) {
-        const int prc = launch_umma_pair(p, st, stream);
-        if (prc != LORDS_ERR_UNSUPPORTED && prc != LORDS_ERR_WORKSPACE) return prc;
+    // a kernel that does not find room for its scratch leaves the call to the other
+    const bool may_pair = p.M > 16 && st.forced_bn == 0, pair_first = may_pair && prefer_pair(p, st);
+    int rc = LORDS_ERR_UNSUPPORTED;
+    if (pair_first) {
+        rc = launch_umma_pair(p, st, stream);
+        if (rc != LORDS_ERR_UNSUPPORTED && rc != LORDS_ERR_WORKSPACE) return rc;
     }
 
     UmmaParams k;
@@ -814,7 +823,8 @@ int launch_umma(const Problem &p, State &st, cudaStream_t stream)
     k.npairs = (p.n + 127) / 128;
     k.y = p.y; k.y_f32 = p.y_f32;
     k.status = st.status_word;
-    const int rc = p.bits == 4 ? launch_bits<4>(k, p, st, stream) : p.bits == 3 ? launch_bits<3>(k, p, st, stream) : launch_bits<2>(k, p, st, stream);
+    rc = p.bits == 4 ? launch_bits<4>(k, p, st, stream) : p.bits == 3 ? launch_bits<3>(k, p, st, stream) : launch_bits<2>(k, p, st, stream);
+    if (rc == LORDS_ERR_WORKSPACE && may_pair && !pair_first) return launch_umma_pair(p, st, stream);
     if (rc != LORDS_OK) return rc;
     st.last_path = "umma";
     return LORDS_OK;

@@ -44,3 +44,17 @@ def test_estimates_choose(lords, bits, m, n, r, M):
     y32, ybf = dl.forward()
     assert lords.lords_last_path() == "umma"
     check_against_oracle(y32, ybf, oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits))
+
+
+# m, n, r, M and the scratch beyond the fp16 activations: too little for the pieces that the preferred tile's or kernel's CTAs exchange
+@pytest.mark.parametrize("m,n,r,M,room", [(2560, 1024, 32, 512, 1 << 20), (512, 8192, 48, 300, 700 << 10)])
+def test_tight_scratch_keeps_the_path(lords, m, n, r, M, room):
+    lay = gen.make_layer(m, n, r, M, bits=4, seed=m + M)
+    dl = DeviceLayer(lay)
+    lords.lords_init(0, M * n * 2 + room)
+    try:
+        y32, ybf = dl.forward()
+        assert lords.lords_last_path() == "umma"
+    finally:
+        lords.lords_init(0, 0)
+    check_against_oracle(y32, ybf, oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, 4))
