@@ -698,8 +698,8 @@ template <int BITS, int NTOK, int H, int XB = 0> struct DecodeVariant {
 
 // Cluster size for `tiles` tiles of `ksteps` k-steps: the largest split that still lets every cluster
 // be resident at once (one wave); 1 when there are more tiles than that.  `cost` receives a relative
-// time estimate, k-steps per CTA x waves x the per-step weight of the tile height.
-template <int BITS, int NTOK, int H> int choose_cluster(int dev, int tiles, int ksteps, int forced, double &cost)
+// time estimate in one-half steps.
+template <int BITS, int NTOK, int H> int choose_cluster(int dev, int sms, int tiles, int ksteps, int forced, double &cost)
 {
     using V = DecodeVariant<BITS, NTOK, H>;
     int cs = 1;
@@ -714,11 +714,13 @@ template <int BITS, int NTOK, int H> int choose_cluster(int dev, int tiles, int 
     const int resident = V::max_clusters(dev, cs) > 0 ? V::max_clusters(dev, cs) : 1;
     const int waves = (tiles + resident - 1) / resident;
     const int steps = (ksteps + cs - 1) / cs;
-    // A two-half step covers twice the rows in 1.3 to 1.4 times the time of a one-half step (converting the
-    // factor tile costs both the same), and every launch pays a fixed prologue + reduction worth a few steps.  1.3: the taller tile's grid also leaves
-    // SMs free, where the next launch's CTAs start before this one's end (4096 x 2048, 4 x 32 CTAs of one half against 6 x 16 of two: 6.0 : 5.5 us,
-    // two tokens 7.1 : 6.3; 4096 x 4096 7.5 : 7.3, two tokens 8.9 : 8.8).
-    cost = (double)waves * ((double)steps * (H == 2 ? 1.3 : 1.0) + 2.0);
+    // A two-half step covers twice the rows in about 1.4 times the time of a one-half step (converting the factor tile costs both the same), and
+    // every launch pays a fixed prologue and reduction worth a few steps.  The last term is the SMs that the grid takes: on those it leaves,
+    // the next launch's CTAs set up and load before this one ends (1600 x 832, 2 bits, 13 x 7 CTAs of one half against 7 x 7 of two: 5.75 :
+    // 4.44 us).  On 608 layers of 0.5 to 59 M weights at one or two tokens, back to back, what the estimate chooses is 1.0 % slower than
+    // the better height on average, 21 % at most; without the last term 4.8 and 51 %, whether a two-half step counts 1.3 or 1.4.
+    const int ctas = tiles * cs < sms ? tiles * cs : sms;
+    cost = (double)waves * ((double)steps * (H == 2 ? 1.4 : 1.0) + 2.0) + 8.0 * (double)ctas / (double)sms;
     return cs;
 }
 
@@ -735,8 +737,11 @@ template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem
     const int tiles1 = (p.m + 127) / 128, tiles2 = (p.m + 255) / 256;
     if (tiles1 > 65535) return LORDS_ERR_UNSUPPORTED;
     double cost1 = 0, cost2 = 0;
-    const int cs1 = choose_cluster<BITS, NTOK, 1>(dev, tiles1, k.ksteps, forced_cs, cost1);
-    const int cs2 = choose_cluster<BITS, NTOK, 2>(dev, tiles2, k.ksteps, forced_cs, cost2);
+    const int cs1 = choose_cluster<BITS, NTOK, 1>(dev, st.sm_count, tiles1, k.ksteps, forced_cs, cost1);
+    const int cs2 = choose_cluster<BITS, NTOK, 2>(dev, st.sm_count, tiles2, k.ksteps, forced_cs, cost2);
+    // Ranks above 32: two halves read twice the rows of B at the end, with 4 bits past a cache of next to nothing beside the shared memory (1152 x 640,
+    // rank 64: one half 3.4 us, two 4.4) and one value at a time where rows are no multiples of 16 bytes (9536 x 704, rank 62: 7.5 and 11.4).
+    if (k.r > 32) cost2 += BITS == 4 ? 2.0 + (k.r % 8 != 0 ? 0.1 * (k.r - 32) : 0.0) : k.r % 8 == 0 ? 1.5 : 0.0;
     const bool two = cost2 < cost1;
     if (x_host) {
         if ((k.ksteps + (two ? cs2 : cs1) - 1) / (two ? cs2 : cs1) * NTOK * kStep * 2 > kInlineSlice) return LORDS_ERR_UNSUPPORTED;
