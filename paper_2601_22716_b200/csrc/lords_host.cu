@@ -152,29 +152,21 @@ static int validate(const void *x, const uint8_t *q, const void *B, const void *
 //   - shapes whose row pitches TMA can express, ranks up to 64: the reassociated decode kernel (up to two tokens), the 16-token
 //     kernel, the scale-MMA kernel -- except where the layer is so small that their set-up (a 64 KB table, 27 warps,
 //     TMEM) is most of the call: there the direct kernel stands in for them, under their name (the two-token kernel sets up less: level at
-//     1024 x 1024; small_for_decode16 and direct_us say where the others' lines lie);
+//     1024 x 1024; for the others the kernels' estimates are compared);
 //   - ranks above 64 with up to 16 tokens: the wide-rank kernel, or for small layers the direct kernel (r = 128, 16 tokens: 512 x 512 4.8
 //     against 5.2 us, 768 x 768 5.8 against 5.3);
 //   - everything else: the direct kernel or the two-phase path, whichever an estimate puts first; the CUDA cores for a handful of
 //     weights.
 static bool small_for_decode(const Problem &p) { return (long long)p.m * p.n <= (1 << 19); }
 
-// Up to eight tokens the direct kernel's groups are half as wide.  Microseconds, direct against the 16-token kernel: eight tokens, 512 x 512 3.2 : 3.6,
-// 1024 x 1024 3.8 : 4.1, 2048 x 1024 4.7 : 4.7, 512 x 4096 5.1 : 4.4, 3072 x 1024 6.1 : 4.7; sixteen, 256 x 256 3.6 : 4.1,
-// 512 x 512 4.0 : 3.9, 1024 x 1024 4.9 : 4.4; rank 48, eight tokens, 1024 x 2048 5.9 : 4.2.
-static bool small_for_decode16(const Problem &p)
+// Three to sixteen tokens: whichever of the two has the shorter estimate.  On 300 layers that the estimates were not fitted to it is 0.7 %
+// slower than the better one on average, 19 % at most (2048 x 1024, 3 bits, rank 4, three tokens, direct 3.7 and 16-token kernel 4.1 us; 1024 x
+// 1024 with ranks above 32, eight tokens, 5.9 and 4.2; 3072 x 1024 6.1 and 4.7).  All layers but one (rank 61) below 2^17 weights were
+// the direct kernel's and none above 2^23: those are not asked about, which keeps the smallest calls' host path short.
+static bool direct_for_decode16(const Problem &p, const State &st)
 {
     const long long weights = (long long)p.m * p.n;
-    return weights <= (p.M > 8 ? 1 << 17 : p.r <= 32 ? 3 << 19 : 1 << 20);
-}
-
-// The direct kernel's fp16 form at 17 to 128 tokens, microseconds: fitted to nine shapes of 0.06 to 4 M weights, within 15 % (24 M token groups x weights 25).  Against the estimate of the scale-MMA
-// kernels: 1024 x 4096, rank 16, 64 tokens 11.6 : 17.2; 512 x 4096, 128 tokens 11.6 : 17.3; 1024 x 1024, 64 tokens 6.1 : 7.1, 96 7.4 : 7.1;
-// 1024 x 2048, rank 48, 64 tokens 12.2 : 10.4; 2048 x 2048, 64 tokens 11.5 : 10.9.
-static double direct_us(const Problem &p)
-{
-    const double grouped = 1e-6 * ((p.M + 15) / 16) * (double)p.m * p.n;
-    return p.r <= 32 ? 4.6 + 0.43 * grouped : 5.0 + 0.76 * grouped;
+    return weights <= 1 << 17 || (weights <= 1 << 23 && direct_us(p, st) < decode16_us(p, st));
 }
 
 // The direct kernel rebuilds W^ for every group of 16 to 32 tokens; the two-phase path does it once, at the price of 6 bytes of scratch a weight
@@ -216,7 +208,7 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
         if (rc != LORDS_ERR_UNSUPPORTED) return rc;
     }
     if (decode16_takes(p)) {
-        if (small_for_decode16(p)) {
+        if (direct_for_decode16(p, st)) {
             rc = launch_direct(p, st, s);
             if (rc == LORDS_OK) st.last_path = "decode16";
         } else {
@@ -225,7 +217,7 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
         if (rc != LORDS_ERR_UNSUPPORTED) return rc;
     }
     if (umma_takes(p)) {
-        if (p.M > 16 && p.M <= 128 && direct_us(p) <= umma_us(p, st)) {
+        if (p.M > 16 && p.M <= 128 && direct_us(p, st) < umma_us(p, st)) {
             rc = launch_direct(p, st, s);
             if (rc == LORDS_OK) st.last_path = "umma";
         } else {

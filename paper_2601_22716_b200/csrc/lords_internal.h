@@ -86,6 +86,8 @@ int launch_wide(const Problem &p, State &st, cudaStream_t stream);
 
 // Up to 128 tokens, any shape: weights formed in registers and multiplied there (warp-level MMAs).
 int launch_direct(const Problem &p, State &st, cudaStream_t stream);
+// Estimate of its time in microseconds where it stands in for the 16-token or the scale-MMA kernel (fp16 operands).
+double direct_us(const Problem &p, const State &st);
 
 // Two-phase tensor-core path for any shape: W^ expanded once into scratch, then a dense product.
 // LORDS_ERR_WORKSPACE when the scratch memory does not hold it.
@@ -100,6 +102,8 @@ int launch_decode_inline(const Problem &p, const void *x_host, State &st, cudaSt
 // Tensor-core decode path for 3 .. 16 tokens, scale-MMA form with 128-column k-steps.
 // LORDS_ERR_UNSUPPORTED for shapes outside its rules.
 int launch_decode16(const Problem &p, State &st, cudaStream_t stream);
+// Estimate of its time in microseconds.
+double decode16_us(const Problem &p, const State &st);
 
 // Up to three matrices of 16-bit values copied to rows of `pitch` (a multiple of 8) values, zeros behind.
 struct PadJob {

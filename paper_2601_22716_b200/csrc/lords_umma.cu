@@ -700,23 +700,24 @@ template <int BITS, int BN, int RP> int launch_variant(UmmaParams &k, const Prob
     return LORDS_OK;
 }
 
-// Estimates of a call's time in microseconds, least-squares fits to the kernels' times on eighteen layer shapes (0.3 to 59 M weights) at 20 to
-// 2048 tokens, off by 4 (this kernel, every token tile) and 5 % (the one on CTA pairs) on average.  What they choose is 0.7 % slower than the best of
-// the five on average, 18 % at most (5120 x 5120, 256 tokens: 33 us against 28); with the largest token tile that gave CTAs for most of the
-// SMs, and a line between the kernels from four shapes, it was 5.4 and 43 % (2560 x 1024, 512 tokens: 18.4 us in tiles of 32 tokens, 11.2 in tiles of 256;
-// 11008 x 1536, 64 tokens: 23 and 14).
-double fixed_us(const Problem &p) { return 0.053e-6 * (double)p.m * p.n + 0.91e-6 * (double)p.M * ((double)p.m + p.n); }    // weights, activations
+// Estimates of a call's time in microseconds: least-squares fits to the kernels' times on 1170 layers of 0.06 to 59 M weights at 17 to
+// 2048 tokens, calls back to back, off by 5 (this kernel, every token tile) and 3 % (the one on CTA pairs) on average.  What they choose
+// (and direct_us, up to 128 tokens) is 0.8 % slower than the best of the kernels and tiles on average, 27 % at most, on 600 layers that they were
+// not fitted to.  The terms in CTAs are the SMs that a grid takes: on those it leaves, the next launch's CTAs set up before this one ends.
 
 // This kernel with tiles of `bn` tokens: a wave is k-steps of 64 columns, as long as the look-ups whatever the tile, and an epilogue.
 double single_us(const Problem &p, const State &st, int bn)
 {
-    const double rank = p.r > 32 ? 1.0 : 0.0;
     const long long tiles = (long long)((p.m + BM - 1) / BM) * ((p.M + bn - 1) / bn), sms = st.sm_count;
     double ksteps = (double)((p.n + BK - 1) / BK), waves = (double)((tiles + sms - 1) / sms);
     const bool halves = 2 * tiles <= sms && p.n > 128;                           // every tile's k-range over two CTAs
+    const bool last_halves = tiles > sms && 2 * ((long long)waves * sms - tiles) >= sms;   // the last wave's are
     if (halves) ksteps *= 0.5;
-    else if (tiles > sms && 2 * ((long long)waves * sms - tiles) >= sms) waves -= 0.5;     // the last wave's are
-    return 0.1 + (halves ? 1.4 : 0.0) + ((0.412 + 0.00008 * bn + 0.012 * rank) * ksteps + 2.43 + 0.0100 * bn) * waves + fixed_us(p);
+    if (last_halves) waves -= 0.5;
+    const long long ctas = halves ? 2 * tiles : tiles < sms ? tiles : sms;
+    return -1.9 + (halves ? 1.6 - 0.0029 * bn : 0.0) + (last_halves ? 2.8 + 0.0025 * bn : 0.0) +
+           ((0.370 + 0.000216 * bn + (p.r > 32 ? 0.0305 : 0.0)) * ksteps + 3.18 + 0.0162 * bn) * waves + 0.87e-6 * (double)p.M * p.n +
+           2.5 * (double)ctas / (double)sms;
 }
 
 // The kernel on CTA pairs: it does a step of 128 columns in about the time that this one needs for a
@@ -728,8 +729,11 @@ double pair_us(const Problem &p, const State &st)
     const long long tok_tiles = (p.M + 255) / 256, bn = ((p.M + tok_tiles - 1) / tok_tiles + 31) / 32 * 32;
     const long long tiles = (long long)((p.m + 255) / 256) * tok_tiles;
     if (tiles > 0x3fffffffLL) return 1e30;
-    const Division d = divide_tiles((int)tiles, (p.n + 127) / 128, st.sm_count / 2, 2, kMeetSteps);
-    return 3.6 + (d.whole < (int)tiles ? 8.7 : 0.0) + (0.604 + 0.00032 * (double)bn + (p.r > 32 ? 0.037 : 0.0)) * d.per_pair + 0.012 * (double)bn + fixed_us(p);
+    const int pairs = st.sm_count / 2;
+    const Division d = divide_tiles((int)tiles, (p.n + 127) / 128, pairs, 2, kMeetSteps);
+    return -0.5 + (d.whole < (int)tiles ? 7.7 + 0.0205 * (double)bn : 0.0) + (0.617 + 0.00029 * (double)bn + (p.r > 32 ? 0.034 : 0.0)) * d.per_pair +
+           0.0112 * (double)bn + 3.4 * ((d.whole + pairs - 1) / pairs) + 0.048e-6 * (double)p.m * p.n + 0.75e-6 * (double)p.M * p.n +
+           1.9 * (double)d.pairs / (double)pairs + (p.r % 8 != 0 ? 1.2 : 0.0);     // (B padded first)
 }
 
 // Token tile: 32, 64, 128 or 256, whichever has the shortest estimate of those that are not in `tried` (a sum of tiles); 0 if all are.
