@@ -83,3 +83,15 @@ def test_direct_kernel_cluster_splits(lords, split):
     dl, y32, ybf = _forward(lords, lay, split)
     want = oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, 4)
     assert np.array_equal(y32.astype(np.float64), want)
+
+
+# Under a forced split the fewest groups win and of those the narrowest: groups of 24 tokens, 24, 32, 32, two of 24, two of 32; 16 with ranks
+# above 64 and with fp16 operands
+@pytest.mark.parametrize("bits,m,n,r", [(4, 300, 1100, 9), (3, 260, 1056, 30), (2, 200, 1000, 60), (4, 257, 1152, 40), (4, 200, 1100, 70)])
+@pytest.mark.parametrize("M", [17, 24, 25, 32, 47, 63])
+@pytest.mark.parametrize("split", [1, 3])
+def test_direct_kernel_group_widths(lords, bits, m, n, r, M, split):
+    lay = gen.make_integer_layer(m, n, r, M, bits=bits, seed=M + split)
+    dl, y32, ybf = _forward(lords, lay, split)
+    want = oracle.forward(lay.x, dl.packed_host, lay.B, lay.A, lay.codebook, bits)
+    assert np.array_equal(y32.astype(np.float64), want)
