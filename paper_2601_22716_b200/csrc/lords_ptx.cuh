@@ -70,8 +70,8 @@ __device__ __forceinline__ WaitLimit wait_limit_start()
     return w;
 }
 // called after every 64 unsuccessful tries; `status` is the library's device status word (may be null).
-// Every 16th call (about every hundred microseconds of waiting) it looks at the status word and at the
-// clock.  The first wait of a grid that runs out by itself (not because the status word was already
+// Every 16th call it looks at the status word and at the clock (a try that fails takes 7.8 thousand cycles, about 4 us: after
+// every four milliseconds of waiting).  The first wait of a grid that runs out by itself (not because the status word was already
 // set) leaves a record behind the status word, for diagnosis: {tag | parity << 8 | warp << 16 |
 // CTA << 32, barrier address | rounds of 64 tries << 32}.
 __device__ __forceinline__ bool wait_limit_expired(WaitLimit &w, const int *status, uint32_t bar, uint32_t parity, uint32_t tag)
@@ -103,7 +103,10 @@ __device__ __forceinline__ void record_give_up(int *status, int code)
 // passed, so tries one after the other (SLEEP 0, four instructions each) take few issue slots and end with the phase; a sleep of 40 ns
 // before each try, which ends later than the phase more often than not, cost 4096 x 1024, one token, 0.12 us of 4.25, a block of seven
 // projections 73.1 us against 70.6, a rank of 128 17.3 against 16.9.  (The hint of a suspension time compiles to sleeps as well.)
-// Kernels that run at the power limit keep the sleep: 4096 x 14336, 2048 tokens, 230 us with it, 232 without.
+// The scale-MMA kernel on CTA pairs, which runs at the power limit, keeps the sleep: 4096 x 14336, 2048 tokens, 230 us with it, 232
+// without.  So does the code assignment: 2216 x 12576, 3 bits, rank 65, 59 us with it, 74 without; rank 100, 70 and 92 (most of its forms are level).
+// Level either way are the dense product (ten layers of 3 to 60 M weights, 130 to 2048 tokens) and the factor gradients, within 1 %.  The
+// QAT gradients are faster without: 4096 x 4096, 512 tokens, 76.3 us and 79.3; 4096 x 14336, 256 tokens, 234 and 238.
 template <int SLEEP> __device__ __forceinline__ bool mbar_try_wait_64(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
@@ -149,8 +152,8 @@ template <int SLEEP> __device__ __forceinline__ bool mbar_try_wait_64(uint32_t b
 
 // Bounded wait: gives up after kWaitLimitNs of polling (or as soon as the status word is set) and
 // reports failure, so that no role of a kernel can spin forever on a shared GPU.  Callers record
-// LORDS_ERR_TIMEOUT and drain.  SLEEP: 0 ordinarily; in kernels that run at the power limit kWaitSleepNs, and kWaitSlackNs for producers that run
-// several steps ahead.
+// LORDS_ERR_TIMEOUT and drain.  SLEEP: 0 ordinarily; in the kernels named above kWaitSleepNs, and kWaitSlackNs for producers
+// that run several steps ahead.
 constexpr int kWaitSleepNs = 40, kWaitSlackNs = 200;
 template <int SLEEP = 0>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const int *status = nullptr, uint32_t tag = 0)
