@@ -169,6 +169,14 @@ static bool direct_for_decode16(const Problem &p, const State &st)
     return weights <= 1 << 17 || (weights <= 1 << 23 && direct_us(p, st) < decode16_us(p, st));
 }
 
+// 17 to 128 tokens: the same against the scale-MMA kernels.  Up to 2^19 weights x groups of 16 tokens the direct kernel took 5.6 us at most (over
+// 100 layers), less than the host needs for the others' two launches: those are not asked about.
+static bool direct_for_umma(const Problem &p, const State &st)
+{
+    if (p.M <= 16 || p.M > 128) return false;
+    return (p.M + 15) / 16 * ((long long)p.m * p.n) <= 1 << 19 || direct_us(p, st) < umma_us(p, st);
+}
+
 // The direct kernel rebuilds W^ for every group of 16 to 32 tokens; the two-phase path does it once, at the price of 6 bytes of scratch a weight
 // (which beyond L2's size go to memory and back) and of two launches.  Microseconds, fitted to seven shapes of 0.3 to 58 M weights at 16 to
 // 128 tokens (direct against two-phase: 4096 x 4094, r = 32: 64 tokens 49 : 57, 80 79 : 62; 1000 x 2730, 128 tokens 21 : 40; 2816 x
@@ -217,7 +225,7 @@ static int dispatch(const Problem &p, State &st, cudaStream_t s)
         if (rc != LORDS_ERR_UNSUPPORTED) return rc;
     }
     if (umma_takes(p)) {
-        if (p.M > 16 && p.M <= 128 && direct_us(p, st) < umma_us(p, st)) {
+        if (direct_for_umma(p, st)) {
             rc = launch_direct(p, st, s);
             if (rc == LORDS_OK) st.last_path = "umma";
         } else {

@@ -87,7 +87,8 @@ struct alignas(64) UmmaParams {
     int tok_tiles;
     int whole_pairs;      // pair mode (BN > 16, clusters of 2): clusters below this index run two whole tiles,
                           // the others share one tile, half of its k-range each; -1 = no pair mode
-    float *pair_scratch;  // pair mode: [shared tile][BN][128] partial sums of the second half
+    float *pair_scratch;  // pair mode: [shared tile][BN][128] partial sums, each of the half of the tokens that the other CTA stores:
+                          // tokens [0, BN / 2) hold the second CTA's part of the k-range, the others the first one's
     void *y;
     int y_f32;
     int *status;
@@ -435,8 +436,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_umma_kernel(const __grid_co
                 if (BN > 16 && pair_split) {
                     // The two CTAs exchange their sums through global scratch: each sends those of the other's half of the tokens, then adds
                     // and stores its own half (with one CTA sending all and the other adding all, the exchange was twice as long: 4096 x 4096,
-                    // 512 tokens, 28.7 us a call, 24.6 so; 300 tokens, 3 bits, rank 48, 29.0 and 24.6).  The arrivals on the partner's barrier (release / acquire at cluster scope)
-                    // order the data; a CTA that gave up arrives as well.
+                    // 512 tokens, 28.7 us a call, 24.6 so; 300 tokens, 3 bits, rank 48, 29.0 and 24.6).  The arrivals on the partner's
+                    // barrier (release / acquire at cluster scope) order the data; a CTA that gave up arrives as well.
                     constexpr int kHalf = BN / 2, kChunks = kHalf / 16;
                     float *const part = p.pair_scratch + (size_t)pair_index * BN * BM + row;
                     if (ok)
@@ -802,8 +803,10 @@ int launch_umma_prepass(const Problem &p, void *x16, void *b_pad, cudaStream_t s
 
 double umma_us(const Problem &p, const State &st)
 {
-    const double single = single_us(p, st, token_tile(p, st)), pairs = pair_us(p, st);
-    return single < pairs ? single : pairs;
+    const double single = single_us(p, st, token_tile(p, st)), pairs = pair_us(p, st), us = single < pairs ? single : pairs;
+    // calls back to back are no shorter than their two launches take the host (2112 x 256, 2 bits, rank 55, 24 tokens: estimated 4.7, 5.9 us; the
+    // direct kernel 4.8)
+    return us > 5.8 ? us : 5.8;
 }
 
 // Rules of this path: r <= 64; n a multiple of 64 (2- and 4-bit codes) or 128 (3-bit), which makes
