@@ -152,7 +152,7 @@ template <int SLEEP> __device__ __forceinline__ bool mbar_try_wait_64(uint32_t b
 
 // Bounded wait: gives up after kWaitLimitNs of polling (or as soon as the status word is set) and
 // reports failure, so that no role of a kernel can spin forever on a shared GPU.  Callers record
-// LORDS_ERR_TIMEOUT and drain.  SLEEP: 0 ordinarily; in the kernels named above kWaitSleepNs, and kWaitSlackNs for producers
+// LORDS_ERR_TIMEOUT and drain.  SLEEP: 0 ordinarily; kWaitSleepNs where a measurement stands for it, and there kWaitSlackNs for producers
 // that run several steps ahead.
 constexpr int kWaitSleepNs = 40, kWaitSlackNs = 200;
 template <int SLEEP = 0>

@@ -228,7 +228,10 @@ __global__ void __launch_bounds__(kThreads, 1) lords_wide_kernel(const __grid_co
         if (b_by_tma && !mbar_wait_warp(bar_b, 0, status, 77)) failed = true;
         for (int it = 0; it < total && !failed; ++it) {
             const int sa = it % D, sd = it % DS;
-            if (!mbar_wait_warp2(bar_a + 8 * sa, (uint32_t)((it / D) & 1), bar_s_free + 8 * sd, (uint32_t)((it / DS + 1) & 1), status, 78)) { failed = true; break; }
+            // Up to eight tokens this wait sleeps between tries: without, layers were up to 7 % slower (5646 x 512, 2 bits, rank 71, two tokens:
+            // 9.7 us and 10.4; 72 layers 1.0 % on average).  With more tokens it costs 0.3 % (4096 x 4096, rank 128, 16 tokens: 17.5 us, 17.3 without).
+            if (!mbar_wait_warp2<TG == 1 ? kWaitSleepNs : 0>(bar_a + 8 * sa, (uint32_t)((it / D) & 1), bar_s_free + 8 * sd,
+                                                            (uint32_t)((it / DS + 1) & 1), status, 78)) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_lo = a_lo0 + (uint32_t)(sa * ((2 * kAAtom) >> 4));
             for (int k = 0; k < rsteps; ++k)                                   // 64 ranks per atom of the B tile, and per sum
