@@ -343,9 +343,9 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode_kernel(const __grid_
     // let a dependent launch (the next layer) begin its own weight prefetch as SMs become free
     griddep_launch_dependents();
     // What works on x waits here for the previous launch to finish.  What works on weights alone runs on: the streams of packed codes and
-    // factor tiles as far as their rings go, and the workers until the W ring is full (with the 16-token kernel: a block at one token 76.1 -> 75.0 us, at eight 89.6 -> 85.6).  Each passes the dependency point before its
-    // first wait for something that x is needed for, so that no bounded wait runs while the previous launch (however
-    // long) still works.
+    // factor tiles as far as their rings go, and the workers until the W ring is full (with the 16-token kernel: a block at one token
+    // 76.1 -> 75.0 us, at eight 89.6 -> 85.6).  Each passes the dependency point before its first wait for something that x is needed
+    // for, so that no bounded wait runs while the previous launch (however long) still works.
     if (!XB && warp >= kConvWarp0 && warp < kTmaQWarp) griddep_wait();
 
     if (warp == kTmaQWarp) {
@@ -739,8 +739,9 @@ template <int BITS, int NTOK> int launch_bits_tok(DecodeParams &k, const Problem
     double cost1 = 0, cost2 = 0;
     const int cs1 = choose_cluster<BITS, NTOK, 1>(dev, st.sm_count, tiles1, k.ksteps, forced_cs, cost1);
     const int cs2 = choose_cluster<BITS, NTOK, 2>(dev, st.sm_count, tiles2, k.ksteps, forced_cs, cost2);
-    // Ranks above 32: two halves read twice the rows of B at the end, with 4 bits past a cache of next to nothing beside the shared memory (1152 x 640,
-    // rank 64: one half 3.4 us, two 4.4) and one value at a time where rows are no multiples of 16 bytes (9536 x 704, rank 62: 7.5 and 11.4).
+    // Ranks above 32: two halves read twice the rows of B at the end, with 4 bits past a cache of next to nothing beside the shared
+    // memory (1152 x 640, rank 64: one half 3.4 us, two 4.4) and one value at a time where rows are no multiples of 16 bytes (9536 x
+    // 704, rank 62: 7.5 and 11.4).
     if (k.r > 32) cost2 += BITS == 4 ? 2.0 + (k.r % 8 != 0 ? 0.1 * (k.r - 32) : 0.0) : k.r % 8 == 0 ? 1.5 : 0.0;
     const bool two = cost2 < cost1;
     if (x_host) {

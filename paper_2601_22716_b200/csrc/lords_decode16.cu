@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
     // let a dependent launch (the next layer) begin its own weight prefetch as SMs become free
     griddep_launch_dependents();
     // What works on x waits here for the previous launch to finish.  What works on weights alone (codes, factor tiles, scale MMAs, workers)
-    // runs on until the W ring is full (a block at eight tokens 89.6 -> 85.6 us); each passes the dependency point before its first wait for something that x is needed
-    // for, so that no bounded wait runs while the previous launch (however long) still works.
+    // runs on until the W ring is full (a block at eight tokens 89.6 -> 85.6 us); each passes the dependency point before its first
+    // wait for something that x is needed for, so that no bounded wait runs while the previous launch (however long) still works.
     if (warp == kTmaXWarp || (warp >= kConvWarp0 && warp < kScaleWarp0)) griddep_wait();
 
     if (warp == kTmaQWarp) {
@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, 1) lords_decode16_kernel(const __gri
             } else {
                 // The cluster's partial sums are added up by all of its CTAs: token t by CTA t mod cluster, which so receives M rows of
                 // them in all (with a leader for all tokens, 16 x cluster rows came into one SM: 1024 x 4096, eight tokens, 6.65 us a
-                // call, 5.1 so; 4096 x 4096 9.2 and 8.6).  (Computed here, not above: live through the loop they cost its registers.)
+                // call, 5.1 so; 4096 x 4096 9.2 and 8.4).  (Computed here, not above: live through the loop they cost its registers.)
                 const int cta = (int)cluster_ctarank(), red_toks = (p.M + csize - 1) / csize, own_toks = (p.M - cta + csize - 1) / csize;
                 // a CTA that gave up still sends its bytes (zeros), so nobody waits in vain
                 int to = 0, nth = 0;                           // token t goes to CTA `to`, as the `nth` of its tokens

@@ -12,13 +12,13 @@
 // them, so S of every 16 ranks and the first parts' products of every 16 columns start from zero and are added on the
 // CUDA cores; the lower parts' products, 2^-8 of the sum, keep to the tensor cores.  Error of the fp32 sums
 // against 64 bits, norms, normal activations, 256 x 256 to 1024 x 14336, ranks 4 to 128: 6e-8 to 1.7e-7 (CUDA cores 8e-8 to 1.6e-7; the
-// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 13.4 us a call (CUDA cores 67.6).
+// fp16 form 2e-4 to 3.3e-4).  37 tokens of 1000 x 2730, rank 10: 12.7 us a call (CUDA cores 67.6).
 //
 // A cluster shares one tile of 128 rows and splits its columns; every CTA sends its partial sums to the CTA that owns
 // the row (asynchronous stores counted on that CTA's barrier), which adds them in rank order: deterministic,
 // no atomics, no trip through global memory.  Tokens that one CTA does not take are further groups of CTAs (grid y), each of which
 // forms W^ again: EXACT takes up to 32 (with groups of 16 and ranks in steps of 32 before, 48 tokens: 4096 x 4094, rank 32, 64.0 us, 44.8 so;
-// 5472 x 10524, rank 11, 170 and 119; 1000 x 2730, rank 10, 15.3 and 13.5).
+// 5472 x 10524, rank 11, 170 and 119; 37 tokens of 1000 x 2730, rank 10, 15.0 and 12.7).
 //
 // Bound: warp instructions -- four per code pair for the table and the product (EXACT: some twenty), the MMAs (2 RK + M / 8, or
 // 3 M / 8, per 16 x 16 weights at the warp-level rate) and the loads around them; codes, factors and activations come by
@@ -44,7 +44,7 @@ constexpr int kWarps = 8, kThreads = kWarps * 32;
 constexpr int kRows = kWarps * 16;                  // rows of W^ per CTA
 constexpr int kCols = 64;                           // columns per strip
 constexpr int kClusterMax = 16;
-constexpr int kTokenMax = 128;                      // 16 tokens to a group of CTAs
+constexpr int kTokenMax = 128;                      // beyond, the two-phase and the scale-MMA kernels, which form W^ less often
 constexpr int kAPitch = kCols * 2 + 16;             // bytes per rank (or token) row: ldmatrix reads eight rows without bank conflicts
 constexpr int kQPitch = 48;                         // bytes per code row: eight rows in eight different 16-byte bank groups
 
@@ -52,9 +52,10 @@ constexpr int kQPitch = 48;                         // bytes per code row: eight
 template <int BITS, int RK, int MT, bool ALIGNED, bool EXACT> struct DirCfg {
     static constexpr int ENTRIES = 1 << 2 * BITS;                             // level pairs
     static constexpr int LUT = ENTRIES * 128;                                 // 32 lane-private copies of every pair (EXACT: 16 of 8 bytes)
-    static constexpr int SA = RK <= 2 || (RK == 4 && MT < 24) ? 3 : 2;                                // strips of A and x in flight
+    static constexpr int SA = RK <= 2 || (RK == 4 && MT < 24) ? 3 : 2;        // strips of A and x in flight
     // Strips of codes in flight.  Codes that are not ALIGNED wait in registers instead, and two stages do; the SM so keeps 56 KB of its
-    // 256 as L1 beside two CTAs, not 23, which the words of x that are loaded by turns want (32 tokens, 5472 x 10524, rank 11: 88 us with 23 KB, 74 with 56).
+    // 256 as L1 beside two CTAs, not 23, which the words of x that are loaded by turns want (32 tokens, 5472 x 10524, rank 11: 88 us
+    // with 23 KB, 74 with 56).
     static constexpr int SQ = ALIGNED ? 4 : 2;
     static constexpr int ASTAGE = RK * 16 * kAPitch;
     static constexpr int XPART = MT * kAPitch;
@@ -520,7 +521,9 @@ int launch_planned(DirectParams &k, const Problem &p, State &st, cudaStream_t st
 template <int BITS, int RK, bool ALIGNED, bool EXACT> int launch_tokens(DirectParams &k, const Problem &p, State &st, cudaStream_t stream)
 {
     if (p.M <= 8) return launch_planned<BITS, RK, ALIGNED, EXACT, 8>(k, p, st, stream);
-    // more tokens to a group form W^ fewer times (EXACT, up to 64 ranks: beyond, the registers hold B); the fp16 form takes small layers, where CTAs are few
+    // More tokens to a group form W^ fewer times (EXACT, up to 64 ranks: beyond, the registers hold B); the fp16 form takes small
+    // layers, where CTAs are few.  Without groups of 24, 55 layers off the grid took 4 % longer on average (6897 x 834, rank 42, 44 tokens:
+    // 26.9 us, 34.4 without), without those of 32 3 % (3670 x 6944, rank 6, 32 tokens: 37.4 us, 58.0 without).
     if constexpr (EXACT && RK <= 4)
         if (p.M > 16) return launch_planned<BITS, RK, ALIGNED, EXACT, 16, 24, 32>(k, p, st, stream);
     return launch_planned<BITS, RK, ALIGNED, EXACT, 16>(k, p, st, stream);

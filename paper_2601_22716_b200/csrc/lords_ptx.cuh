@@ -104,9 +104,8 @@ __device__ __forceinline__ void record_give_up(int *status, int code)
 // before each try, which ends later than the phase more often than not, cost 4096 x 1024, one token, 0.12 us of 4.25, a block of seven
 // projections 73.1 us against 70.6, a rank of 128 17.3 against 16.9.  (The hint of a suspension time compiles to sleeps as well.)
 // The scale-MMA kernel on CTA pairs, which runs at the power limit, keeps the sleep: 4096 x 14336, 2048 tokens, 230 us with it, 232
-// without.  So does the code assignment: 2216 x 12576, 3 bits, rank 65, 59 us with it, 74 without; rank 100, 70 and 92 (most of its forms are level).
-// Level either way are the dense product (ten layers of 3 to 60 M weights, 130 to 2048 tokens) and the factor gradients, within 1 %.  The
-// QAT gradients are faster without: 4096 x 4096, 512 tokens, 76.3 us and 79.3; 4096 x 14336, 256 tokens, 234 and 238.
+// without.  Level either way are the dense product (ten layers of 3 to 60 M weights, 130 to 2048 tokens) and the factor gradients,
+// within 1 %.  The QAT gradients are faster without: 4096 x 4096, 512 tokens, 76.3 us and 79.3; 4096 x 14336, 256 tokens, 234 and 238.
 template <int SLEEP> __device__ __forceinline__ bool mbar_try_wait_64(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;

@@ -206,6 +206,9 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
     const uint32_t bar_w = bars, bar_w_free = bar_w + 8 * kSWQ, bar_a = bar_w_free + 8 * kSWQ, bar_a_free = bar_a + 8 * kSAQ;
     const uint32_t bar_s = bar_a_free + 8 * kSAQ, bar_s_free = bar_s + 8 * kSDQ, bar_b = bar_s_free + 8 * kSDQ, tmem_slot = bar_b + 8;
     static_assert(16 * (kSWQ + kSAQ + kSDQ) + 8 + 4 <= 256, "barrier area");
+    // SURE: with tries one after the other 3 bits take 24 to 31 % longer (2216 x 12576, rank 65: 59 us, 74 so; rank 100: 70 and 92; 2 and 4 bits are
+    // level).  The other forms, alone, are within 1 % either way; a training step of 4096 x 4096 at 1024 tokens takes 205.5 us so, 207.2 with sleeps.
+    constexpr int kSleep = SURE ? kWaitSleepNs : 0;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // this CTA's run of steps, across row tiles (step `st` of row tile `rt` is number rt * steps + st)
@@ -275,7 +278,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
             int rt = rt0, st = st0;
             for (int it = 0; it < total; ++it) {
                 if (b_by_tma && (it == 0 || st == 0)) {      // a new row tile: its B once nothing reads the last one's
-                    if (it > 0 && !mbar_wait<kWaitSleepNs>(bar_a_free + 8 * ((it - 1) % kSAQ), (uint32_t)(((it - 1) / kSAQ) & 1), status, 29)) { failed = true; break; }
+                    if (it > 0 && !mbar_wait<kSleep>(bar_a_free + 8 * ((it - 1) % kSAQ), (uint32_t)(((it - 1) / kSAQ) & 1), status, 29)) { failed = true; break; }
                     mbar_expect_tx(bar_b, (uint32_t)C::BTILE);
                     for (int h = 0; h < RA / 64; ++h) tma_load_2d(b_tile + (uint32_t)(h * kRowsQ * 128), &p.tm_b, h * 64, rt * kRowsQ, bar_b);
                 }
@@ -284,7 +287,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                     if (next_w >= kSWQ) {
                         const uint32_t par = (uint32_t)((next_w / kSWQ - 1) & 1);
                         if (next_w > it) { if (!mbar_try_wait(bar_w_free + 8 * s, par)) break; }
-                        else if (!mbar_wait<kWaitSleepNs>(bar_w_free + 8 * s, par, status, 30)) { failed = true; break; }
+                        else if (!mbar_wait<kSleep>(bar_w_free + 8 * s, par, status, 30)) { failed = true; break; }
                     }
                     mbar_expect_tx(bar_w + 8 * s, (uint32_t)kWTileQ);
                     tma_load_2d(w0 + (uint32_t)(s * kWTileQ), &p.tm_w, w_st * kColsQ, w_rt * kRowsQ, bar_w + 8 * s);
@@ -293,7 +296,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                 }
                 if (failed) break;
                 const int sa = it % kSAQ;
-                if (it >= kSAQ && !mbar_wait<kWaitSlackNs>(bar_a_free + 8 * sa, (uint32_t)((it / kSAQ - 1) & 1), status, 31)) { failed = true; break; }
+                if (it >= kSAQ && !mbar_wait<kSleep>(bar_a_free + 8 * sa, (uint32_t)((it / kSAQ - 1) & 1), status, 31)) { failed = true; break; }
                 mbar_expect_tx(bar_a + 8 * sa, (uint32_t)(p.r_pad * 128));
                 tma_load_2d(a0 + (uint32_t)(sa * C::ATILE), &p.tm_a, st * kColsQ, 0, bar_a + 8 * sa);
                 if (++st == p.steps) { st = 0; ++rt; }
@@ -310,12 +313,12 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
         int st = st0;
         for (int it = 0; it < total; ++it) {
             if (b_by_tma && (it == 0 || st == 0)) {
-                if (!mbar_wait_warp<kWaitSleepNs>(bar_b, b_phase, status, 36)) { failed = true; break; }
+                if (!mbar_wait_warp<kSleep>(bar_b, b_phase, status, 36)) { failed = true; break; }
                 b_phase ^= 1;
             }
             if (++st == p.steps) st = 0;
             const int sa = it % kSAQ, sd = it % kSDQ;
-            if (!mbar_wait_warp2<kWaitSleepNs>(bar_a + 8 * sa, (uint32_t)((it / kSAQ) & 1), bar_s_free + 8 * sd, (uint32_t)((it / kSDQ + 1) & 1), status, 32)) { failed = true; break; }
+            if (!mbar_wait_warp2<kSleep>(bar_a + 8 * sa, (uint32_t)((it / kSAQ) & 1), bar_s_free + 8 * sd, (uint32_t)((it / kSDQ + 1) & 1), status, 32)) { failed = true; break; }
             tc_fence_after_sync();
             const uint32_t a_lo = a_lo0 + (uint32_t)(sa * (C::ATILE >> 4));
             for (int k = 0; k < p.r_pad / 16; ++k)
@@ -325,7 +328,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
             umma_commit(bar_a_free + 8 * sa, leader);
         }
         // no commit is still on its way to a barrier when the CTA ends
-        if (!failed && total > 0 && !mbar_wait_warp<kWaitSleepNs>(bar_a_free + 8 * ((total - 1) % kSAQ), (uint32_t)(((total - 1) / kSAQ) & 1), status, 34)) failed = true;
+        if (!failed && total > 0 && !mbar_wait_warp<kSleep>(bar_a_free + 8 * ((total - 1) % kSAQ), (uint32_t)(((total - 1) / kSAQ) & 1), status, 34)) failed = true;
     } else {
         const int q = warp & 3, ch = (warp >> 2) & 1, row = q * 32 + lane;
         const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(ch * 32);
@@ -353,7 +356,7 @@ __global__ void __launch_bounds__(kThreadsQ, 1) lords_quantize_kernel(const __gr
                 least_s = off * p.least_scale;
             }
             st += kGroupsQ;
-            if (!mbar_wait_warp2<kWaitSleepNs>(bar_s + 8 * sd, (uint32_t)((it / kSDQ) & 1), bar_w + 8 * sw, (uint32_t)((it / kSWQ) & 1), status, 35)) { failed = true; break; }
+            if (!mbar_wait_warp2<kSleep>(bar_s + 8 * sd, (uint32_t)((it / kSDQ) & 1), bar_w + 8 * sw, (uint32_t)((it / kSWQ) & 1), status, 35)) { failed = true; break; }
             tc_fence_after_sync();
             const float past = EDGE && (i >= p.m || col0 >= p.n) ? 1.0f : 0.0f;
             uint32_t packed[BITS];
